@@ -221,3 +221,95 @@ def tolerance(case):
     # Sums of FP4 products are exact in FP32 but for blocks of very different scale, MXFP8 sums differ from 64-bit ones by
     # 2.4e-7; what remains is one rounding to BF16: measured against 64-bit products 1.7e-3 in norm, half a unit (3.9e-3) at most.
     return {"rel": 2e-3, "max": 8e-3}
+
+
+# ---- the same passes in 64 bits: quantizers and products from their definitions, in plain torch
+
+_E2M1 = (0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 6.0)
+
+
+def _exact_bytes(rows, cols, seed, tensor_id):
+    """One random byte per element: byte idx % 16 of Philox4x32-10 at counter idx / 16, idx the row-major index."""
+    mask = 0xFFFFFFFF
+    n = (rows * cols + 15) // 16
+    c0 = torch.arange(n, dtype=torch.int64, device=DEVICE)
+    c = [c0 & mask, c0 >> 32, torch.full_like(c0, tensor_id), torch.zeros_like(c0)]
+    k0, k1 = seed & mask, (seed >> 32) & mask
+
+    def mul(m, x):   # 32 x 32 bits -> (high, low) without leaving int64
+        lo, hi = m * (x & 0xFFFF), m * (x >> 16)
+        low = lo + ((hi & 0xFFFF) << 16)
+        return (hi >> 16) + (low >> 32), low & mask
+
+    for _ in range(10):
+        h0, l0 = mul(0xD2511F53, c[0])
+        h1, l1 = mul(0xCD9E8D57, c[2])
+        c = [h1 ^ c[1] ^ k0, l1, h0 ^ c[3] ^ k1, l0]
+        k0, k1 = (k0 + 0x9E3779B9) & mask, (k1 + 0xBB67AE85) & mask
+    words = torch.stack(c, dim=1)
+    b = torch.stack([(words >> (8 * i)) & 0xFF for i in range(4)], dim=2)
+    return b.reshape(-1)[:rows * cols].reshape(rows, cols)
+
+
+def _exact_scale(x, br, bc, top):
+    """2^e per element, e the least with top * 2^e >= the largest magnitude of the element's br x bc block."""
+    rows, cols = x.shape
+    p = torch.nn.functional.pad(x.abs(), (0, -cols % bc, 0, -rows % br))
+    m = p.view(p.shape[0] // br, br, p.shape[1] // bc, bc).amax(dim=(1, 3))
+    f, e = torch.frexp(m / top)   # m / top = f 2^e, 0.5 <= f < 1
+    e = torch.where(f == 0.5, e - 1, e).clamp(min=-127)
+    s = torch.ldexp(torch.ones_like(m), torch.where(m == 0, torch.zeros_like(e), e))
+    return s.repeat_interleave(br, 0)[:rows].repeat_interleave(bc, 1)[:, :cols]
+
+
+def _exact_fp4(x, br=32, bc=32, sr=None):
+    """x rounded to E2M1 in br x bc blocks, dequantized; sr = (seed, tensor_id): stochastically."""
+    x = x.detach().to(torch.bfloat16).double()
+    s = _exact_scale(x, br, bc, 6.0)
+    v, grid = (x / s).abs(), torch.tensor(_E2M1, dtype=torch.float64, device=DEVICE)
+    lo = (torch.searchsorted(grid, v, right=True) - 1).clamp(0, 6)
+    pos = (v - grid[lo]) / (grid[lo + 1] - grid[lo])
+    if sr is None:
+        up = (pos > 0.5) | ((pos == 0.5) & (lo % 2 == 1))
+    else:
+        up = torch.floor(256 * pos) + _exact_bytes(x.shape[0], x.shape[1], *sr) >= 256
+    return torch.copysign(grid[lo + up.long()], x) * s
+
+
+def _exact_mxfp8(x):
+    x = x.detach().double()
+    s = _exact_scale(x, 1, 32, 448.0)
+    return (x / s).float().to(torch.float8_e4m3fn).double() * s
+
+
+def exact(case, seed):
+    c, kind = case, case["kind"]
+    if kind in ("quantize", "fused"):
+        return None   # codes and scales
+    sr = seed & 0x7FFFFFFF
+    if kind == "moe":
+        s = prepare(case, seed)
+        offs, outs = s["offsets"].tolist(), []
+        groups = list(zip(offs[:-1], offs[1:]))
+        for name in ("gate", "down"):
+            w, x, dy = _exact_fp4(s["w_" + name]), _exact_fp4(s["x_" + name]), _exact_fp4(s["dy_" + name], sr=(sr, 2))
+            w = w.view(c["experts"], -1, w.shape[1])
+            outs.append(torch.cat([x[a:b] @ w[e].T for e, (a, b) in enumerate(groups)]))
+            outs.append(torch.cat([dy[a:b] @ w[e] for e, (a, b) in enumerate(groups)]))
+            outs.append(torch.cat([dy[a:b].T @ x[a:b] for a, b in groups]))
+        return outs
+    w, x, dy = _dense_inputs(c, seed)
+    if kind == "mxfp8":
+        wk = workloads.weights(c["N"], c["K"], 3 * seed + 7_000_001, DEVICE)
+        q = _exact_mxfp8(x)
+        return (q @ _exact_mxfp8(w).T, q @ _exact_mxfp8(wk).T, _exact_mxfp8(dy) @ _exact_mxfp8(w.T.contiguous()).T,
+                _exact_mxfp8(dy.T.contiguous()) @ _exact_mxfp8(x.T.contiguous()).T)
+    if kind == "layer":
+        w, x, dy = (_exact_fp4(t, sr=(sr, i)) for i, t in enumerate((w, x, dy)))
+        return x @ w.T, dy @ w, dy.T @ x
+    if kind == "act1d":
+        w, dy = _exact_fp4(w), _exact_fp4(dy, sr=(sr, 1))
+        return _exact_fp4(x, 1, 32) @ w.T, dy @ w, dy.T @ _exact_fp4(x, 32, 1)
+    b = 16 if kind == "block16" else 32
+    w, x, dy = _exact_fp4(w, b, b), _exact_fp4(x, b, b), _exact_fp4(dy, b, b, sr=(sr, 1))
+    return x @ w.T, dy @ w, dy.T @ x   # linear, microbatch (its first pass: the sum starts at zero), block16
