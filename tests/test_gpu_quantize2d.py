@@ -219,3 +219,24 @@ def test_ragged_outputs_do_not_write_outside_their_extent():
         o_rm, o_t, o_s = oracle.quantize2d(workloads.bf16_bits(x), oracle.MODE_STOCHASTIC, 3, 1)
         assert np.array_equal(q.scale.cpu().numpy()[:, :o_s.shape[1]], o_s)
         assert np.array_equal(q.q_rm.cpu().numpy()[:, :o_rm.shape[1]], o_rm) and np.array_equal(q.q_t.cpu().numpy()[:, :o_t.shape[1]], o_t)
+
+
+@pytest.mark.parametrize("rows,cols,pitch,offset", [(1, 17, 17, 0), (129, 131, 131, 0), (33, 129, 143, 7), (300, 391, 401, 3), (160, 256, 264, 4),
+                                                    (127, 1000, 1000, 0), (64, 272, 273, 1)])
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("block", [32, 16, 64])
+def test_rows_that_start_anywhere(rows, cols, pitch, offset, mode, block):
+    # every offset of a row into its first 16-byte piece and of a segment into its Philox block, tiles that end in any
+    # column, at the tensor's first and last element; the elements between the rows are NaN and must not be read as data
+    g = torch.Generator(device="cuda").manual_seed(rows * cols)
+    flat = torch.full((offset + rows * pitch + 64,), float("nan"), device="cuda", dtype=torch.bfloat16)
+    x = flat[offset:offset + rows * pitch].view(rows, pitch)[:, :cols]
+    x.copy_(torch.randn(rows, cols, generator=g, device="cuda") * torch.exp(2 * torch.randn(rows, 1, generator=g, device="cuda")))
+    flags = {16: binding.BLOCK_16, 32: 0, 64: binding.BLOCK_64}[block]
+    qt = gpu_quantize(x, mode, seed=31, tensor_id=5, flags=flags)
+    o_rm, o_t, o_s = oracle.quantize2d_block(workloads.bf16_bits(x), block, mode, 31, 5)
+    s = qt.scale.cpu().numpy()
+    if block == 64:   # the scale matrix stays 32-granular: each block's scale in its (up to) four entries
+        o_s = np.repeat(np.repeat(o_s, 2, 0), 2, 1)[:s.shape[0], :s.shape[1]]
+    assert np.array_equal(s, o_s)
+    assert np.array_equal(qt.q_rm.cpu().numpy()[:, :(cols + 1) // 2], o_rm) and np.array_equal(qt.q_t.cpu().numpy()[:, :(rows + 1) // 2], o_t)
