@@ -1,15 +1,18 @@
-"""Builds libfp4q.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libfp4q.so (the C-ABI CUDA library, nvcc, sm_100a) and _host.so (the binding's native marshalling, g++) in-tree."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libfp4q.so")
+HOST_SRC = os.path.join(CSRC, "host", "marshal.cpp")
+HOST = os.path.join(HERE, "_host.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I" + INCLUDE, "-I" + CSRC]
@@ -27,8 +30,45 @@ def stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def host_stale() -> bool:
+    if not os.path.exists(HOST):
+        return True
+    t = os.path.getmtime(HOST)
+    return any(os.path.getmtime(d) > t for d in [HOST_SRC] + glob.glob(os.path.join(INCLUDE, "*.h")))
+
+
+def start_host_build():
+    """g++ of the marshalling module, against the headers and libraries of the torch that is imported."""
+    import torch
+    root = os.path.dirname(torch.__file__)
+    inc = [INCLUDE, sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
+    sysinc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include")]
+    tmp = HOST + ".%d.tmp" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi())]
+    cmd += ["-I" + d for d in inc] + [a for d in sysinc for a in ("-isystem", d)]
+    cmd += ["-o", tmp, HOST_SRC, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    return tmp, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+
+
+def finish_host_build(tmp, pr):
+    out, _ = pr.communicate()
+    if pr.returncode != 0:
+        sys.stderr.write(out)
+        raise RuntimeError("g++ failed on %s" % HOST_SRC)
+    os.replace(tmp, HOST)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every csrc/*.cu and link libfp4q.so. Returns the library path."""
+    """Compile every csrc/*.cu and link libfp4q.so, and the marshalling module. Returns the library path."""
+    host = start_host_build() if force or host_stale() else None
+    try:
+        return build_library(force, verbose)
+    finally:
+        if host:
+            finish_host_build(*host)
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
     if not force and not stale():
         return LIB
     objdir = os.path.join(HERE, "build")

@@ -1,0 +1,533 @@
+// Native argument marshalling for binding.py (module paper_2607_24953_b200._host).
+//
+// The kernels of a small layer run a few microseconds each, less than a ctypes call spends on turning tensors into
+// pointers: 20 us for a quantizer call and 18 us for a product, of which the launch itself is about 3.  These functions
+// take the Python arguments as they are, allocate the outputs, and call the C entry points through the addresses that
+// binding.py hands over once (so that a library chosen by FP4Q_LIB stays the one that is used): 8 and 7 us.  No state is
+// kept from one call to the next.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <algorithm>
+#include <vector>
+
+#include <ATen/ATen.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "fp4q.h"
+
+namespace {
+
+struct Entry {
+    decltype(&fp4q_quantize2d) quantize2d;
+    decltype(&fp4q_quantize2d_multi) quantize2d_multi;
+    decltype(&fp4q_mxfp8_quantize1d) mxfp8_quantize1d, mxfp8_quantize1d_t;
+    decltype(&fp4q_quantize1d) quantize1d;
+    decltype(&fp4q_quantize1d_t) quantize1d_t;
+    decltype(&fp4q_gemm_fwd) gemm_fwd, gemm_dgrad;
+    decltype(&fp4q_gemm_wgrad) gemm_wgrad;
+    decltype(&fp4q_gemm_fwd_b16) gemm_fwd_b16, gemm_dgrad_b16;
+    decltype(&fp4q_gemm_wgrad_b16) gemm_wgrad_b16;
+    decltype(&fp4q_gemm_fwd_quantized) gemm_fwd_quantized, gemm_dgrad_quantized;
+    decltype(&fp4q_gemm_fwd_act1d) gemm_fwd_act1d;
+    decltype(&fp4q_gemm_wgrad_act1d) gemm_wgrad_act1d;
+    decltype(&fp4q_mxfp8_qk) mxfp8_qk;
+    decltype(&fp4q_mxfp8_gemm) mxfp8_gemm;
+} lib;
+
+PyObject *g_qtensor = nullptr, *g_fail = nullptr;   // binding.QTensor; binding._check
+PyObject *s_rows, *s_cols, *s_q_rm, *s_q_t, *s_scale, *s_granularity;
+
+// A Python exception is set: unwinds to the entry point, which returns NULL.
+struct PyError {};
+
+struct Ref {   // owned reference
+    PyObject *p;
+    explicit Ref(PyObject *o) : p(o) { if (!p) throw PyError(); }
+    ~Ref() { Py_DECREF(p); }
+    Ref(const Ref &) = delete;
+    Ref &operator=(const Ref &) = delete;
+};
+
+// The interpreter lock is given up around allocations and library calls, as torch.empty and ctypes do.
+struct Unlock {
+    PyThreadState *state = PyEval_SaveThread();
+    ~Unlock() { PyEval_RestoreThread(state); }
+};
+template <typename F, typename... A>
+fp4q_status unlocked(F fn, A... args)
+{
+    Unlock u;
+    return fn(args...);
+}
+
+[[noreturn]] void value_error(const char *text) { PyErr_SetString(PyExc_ValueError, text); throw PyError(); }
+
+int64_t as_i64(PyObject *o)
+{
+    const long long v = PyLong_AsLongLong(o);
+    if (v == -1 && PyErr_Occurred()) throw PyError();
+    return v;
+}
+uint64_t as_bits(PyObject *o)   // seeds and ids: reduced modulo 2^64, as ctypes does
+{
+    if (!PyLong_Check(o)) { PyErr_Format(PyExc_TypeError, "int expected instead of %s instance", Py_TYPE(o)->tp_name); throw PyError(); }
+    const unsigned long long v = PyLong_AsUnsignedLongLongMask(o);
+    if (v == (unsigned long long)-1 && PyErr_Occurred()) throw PyError();
+    return v;
+}
+int as_int(PyObject *o) { return (int)(uint32_t)as_bits(o); }
+bool as_bool(PyObject *o)
+{
+    const int v = PyObject_IsTrue(o);
+    if (v < 0) throw PyError();
+    return v != 0;
+}
+const at::Tensor &as_tensor(PyObject *o)
+{
+    if (!THPVariable_Check(o)) { PyErr_Format(PyExc_TypeError, "expected a tensor, got %s", Py_TYPE(o)->tp_name); throw PyError(); }
+    return THPVariable_Unpack(o);
+}
+void *as_stream(PyObject *o)   // None: the current stream of the current device
+{
+    return o == Py_None ? (void *)c10::cuda::getCurrentCUDAStream().stream() : PyLong_AsVoidPtr(o);
+}
+uint8_t *bytes_of(const at::Tensor &t) { return static_cast<uint8_t *>(t.data_ptr()); }
+
+// Error status: binding._check raises.
+void check(fp4q_status st, const char *where)
+{
+    if (st == FP4Q_OK) return;
+    Ref r(PyObject_CallFunction(g_fail, "is", (int)st, where));
+}
+
+int64_t pad16(int64_t n) { return (n + 15) / 16 * 16; }
+int64_t ceil_to(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+at::Tensor empty2(int64_t r, int64_t c, at::ScalarType dt, const at::Tensor &like)
+{
+    Unlock u;
+    return at::empty({r, c}, at::TensorOptions().dtype(dt).device(like.device()));
+}
+
+// x: BF16 [rows, cols], unit stride along the columns.
+const at::Tensor &as_matrix(PyObject *o, const char *name, const char *what)
+{
+    const at::Tensor &x = as_tensor(o);
+    if (!x.is_cuda()) { PyErr_Format(PyExc_ValueError, "%s must live on a CUDA device (there is no CPU path)", name); throw PyError(); }
+    if (x.scalar_type() != at::kBFloat16 || x.dim() != 2 || (x.numel() && x.stride(1) != 1)) value_error(what);
+    return x;
+}
+const char kXText[] = "x must be a 2-D BF16 tensor with contiguous rows";
+int64_t pitch(const at::Tensor &x) { return x.size(0) ? x.stride(0) : x.size(1); }
+
+// Leading dimensions the C interface asks for, as in binding.alloc_qtensor.
+struct QBuffers { at::Tensor q_rm, q_t, scale; };
+QBuffers alloc_q(int64_t rows, int64_t cols, const at::Tensor &like, bool want_t, int64_t g)
+{
+    QBuffers b;
+    b.q_rm = empty2(rows, std::max<int64_t>(pad16(ceil_to(cols, 32) * 16), 16), at::kByte, like);
+    if (want_t) b.q_t = empty2(cols, std::max<int64_t>(pad16(ceil_to(rows, 32) * 16), 16), at::kByte, like);
+    b.scale = empty2(ceil_to(rows, g), std::max<int64_t>(ceil_to(cols, g), 1), at::kByte, like);
+    return b;
+}
+fp4q_tensor c_tensor(int64_t rows, int64_t cols, const at::Tensor &q_rm, const at::Tensor &q_t, const at::Tensor &scale)
+{
+    fp4q_tensor t;
+    t.rows = rows; t.cols = cols;
+    t.q_rm = bytes_of(q_rm); t.ld_rm = q_rm.stride(0);
+    t.q_t = q_t.defined() ? bytes_of(q_t) : nullptr; t.ld_t = q_t.defined() ? q_t.stride(0) : 0;
+    t.scale = bytes_of(scale); t.ld_s = scale.stride(0);
+    return t;
+}
+PyObject *new_qtensor(int64_t rows, int64_t cols, const QBuffers &b, int64_t g)
+{
+    Ref r(PyLong_FromLongLong(rows)), c(PyLong_FromLongLong(cols)), rm(THPVariable_Wrap(b.q_rm));
+    Ref t(b.q_t.defined() ? THPVariable_Wrap(b.q_t) : Py_NewRef(Py_None)), s(THPVariable_Wrap(b.scale)), gr(PyLong_FromLongLong(g));
+    PyObject *args[6] = {r.p, c.p, rm.p, t.p, s.p, gr.p};
+    PyObject *q = PyObject_Vectorcall(g_qtensor, args, 6, nullptr);
+    if (!q) throw PyError();
+    return q;
+}
+// The C view of a QTensor; granularity: the scale granularity the callee expects (0 = any).
+fp4q_tensor from_qtensor(PyObject *q, long granularity)
+{
+    if (granularity) {
+        Ref g(PyObject_GetAttr(q, s_granularity));
+        const long have = PyLong_AsLong(g.p);
+        if (have == -1 && PyErr_Occurred()) throw PyError();
+        if (have != granularity) {
+            PyErr_Format(PyExc_ValueError, "this call takes tensors quantized in %ld x %ld blocks (scale matrix of that granularity); got %ld",
+                         granularity, granularity, have);
+            throw PyError();
+        }
+    }
+    Ref r(PyObject_GetAttr(q, s_rows)), c(PyObject_GetAttr(q, s_cols)), rm(PyObject_GetAttr(q, s_q_rm)), t(PyObject_GetAttr(q, s_q_t)),
+        s(PyObject_GetAttr(q, s_scale));
+    return c_tensor(as_i64(r.p), as_i64(c.p), as_tensor(rm.p), t.p == Py_None ? at::Tensor() : as_tensor(t.p), as_tensor(s.p));
+}
+at::Tensor qtensor_payload(PyObject *q)
+{
+    Ref rm(PyObject_GetAttr(q, s_q_rm));
+    return as_tensor(rm.p);
+}
+
+// An output matrix: rows padded to whole 16 bytes, the padding cut off the returned view.
+at::Tensor out_buffer(int64_t rows, int64_t cols, int dt, const at::Tensor &like)
+{
+    const int64_t per16 = dt == FP4Q_OUT_BF16 ? 8 : 4, ld = std::max(ceil_to(cols, per16) * per16, per16);
+    at::Tensor t = empty2(rows, ld, dt == FP4Q_OUT_BF16 ? at::kBFloat16 : at::kFloat, like);
+    return ld == cols ? t : t.slice(1, 0, cols);
+}
+int64_t out_pitch(const at::Tensor &out, int64_t cols) { return out.numel() ? out.stride(0) : cols; }
+
+struct Groups {
+    fp4q_groups g;
+    const fp4q_groups *ptr = nullptr;
+    Groups(PyObject *row_offsets, int alignment)
+    {
+        if (row_offsets == Py_None) return;
+        const at::Tensor &t = as_tensor(row_offsets);
+        if (!t.is_cuda()) value_error("row_offsets must live on a CUDA device (there is no CPU path)");
+        if (t.scalar_type() != at::kLong || !t.is_contiguous()) value_error("row_offsets must be a contiguous int64 device tensor");
+        g.n_groups = (int32_t)(t.numel() - 1);
+        g.row_alignment = alignment;
+        g.row_offsets = static_cast<const int64_t *>(t.data_ptr());
+        ptr = &g;
+    }
+};
+
+typedef PyObject *const *Args;
+
+void want(Py_ssize_t got, Py_ssize_t n)
+{
+    if (got != n) { PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", n, got); throw PyError(); }
+}
+
+// x, out | None, mode, seed, tensor_id, flags, want_t, stream
+PyObject *quantize2d(Args a, Py_ssize_t n)
+{
+    want(n, 8);
+    const at::Tensor &x = as_matrix(a[0], "x", kXText);
+    const int64_t rows = x.size(0), cols = x.size(1);
+    const uint32_t flags = (uint32_t)as_bits(a[5]);
+    const int64_t g = (flags & FP4Q_BLOCK_16) ? 16 : 32;
+    fp4q_tensor t;
+    QBuffers b;
+    if (a[1] == Py_None) {
+        b = alloc_q(rows, cols, x, as_bool(a[6]), g);
+        t = c_tensor(rows, cols, b.q_rm, b.q_t, b.scale);
+    } else {
+        t = from_qtensor(a[1], 0);
+    }
+    check(unlocked(lib.quantize2d, x.data_ptr(), rows, cols, pitch(x), &t, (fp4q_round)as_int(a[2]), as_bits(a[3]), (uint32_t)as_bits(a[4]), flags,
+                         as_stream(a[7])), "fp4q_quantize2d");
+    return a[1] == Py_None ? new_qtensor(rows, cols, b, g) : Py_NewRef(a[1]);
+}
+
+// xs, outs | None, mode, seed, tensor_ids | None, flags, want_t, stream
+PyObject *quantize2d_multi(Args a, Py_ssize_t n)
+{
+    want(n, 8);
+    Ref xs(PySequence_Fast(a[0], "xs must be a sequence of tensors"));
+    const Py_ssize_t k = PySequence_Fast_GET_SIZE(xs.p);
+    Ref ids(a[4] == Py_None ? Py_NewRef(Py_None) : PySequence_Fast(a[4], "tensor_ids must be a sequence of ints"));
+    const bool own = a[1] == Py_None;
+    Ref outs(own ? PyList_New(0) : PySequence_Fast(a[1], "outs must be a sequence of QTensor"));
+    const uint32_t flags = (uint32_t)as_bits(a[5]);
+    const bool want_t = as_bool(a[6]);
+    if ((!own && PySequence_Fast_GET_SIZE(outs.p) < k) || (ids.p != Py_None && PySequence_Fast_GET_SIZE(ids.p) < k)) {
+        PyErr_SetString(PyExc_IndexError, "list index out of range");
+        throw PyError();
+    }
+    std::vector<fp4q_tensor> ts((size_t)k);
+    std::vector<fp4q_quantize_job> jobs((size_t)(k > 0 ? k : 1));
+    for (Py_ssize_t j = 0; j < k; j++) {
+        char name[32];
+        snprintf(name, sizeof name, "xs[%zd]", j);
+        const at::Tensor &x = as_matrix(PySequence_Fast_GET_ITEM(xs.p, j), name, "every input must be a 2-D BF16 tensor with contiguous rows");
+        if (own) {
+            const QBuffers b = alloc_q(x.size(0), x.size(1), x, want_t, 32);
+            Ref q(new_qtensor(x.size(0), x.size(1), b, 32));
+            if (PyList_Append(outs.p, q.p) < 0) throw PyError();
+            ts[j] = c_tensor(x.size(0), x.size(1), b.q_rm, b.q_t, b.scale);
+        } else {
+            ts[j] = from_qtensor(PySequence_Fast_GET_ITEM(outs.p, j), 32);
+        }
+        jobs[j].x_bf16 = x.data_ptr();
+        jobs[j].rows = x.size(0); jobs[j].cols = x.size(1); jobs[j].ld_x = pitch(x);
+        jobs[j].out = &ts[j];
+        jobs[j].tensor_id = ids.p == Py_None ? (uint32_t)j : (uint32_t)as_bits(PySequence_Fast_GET_ITEM(ids.p, j));
+        jobs[j].flags = flags;
+    }
+    check(unlocked(lib.quantize2d_multi, jobs.data(), (int32_t)k, (fp4q_round)as_int(a[2]), as_bits(a[3]), as_stream(a[7])), "fp4q_quantize2d_multi");
+    return own ? Py_NewRef(outs.p) : Py_NewRef(a[1]);
+}
+
+PyObject *pair(const at::Tensor &q, const at::Tensor &s)
+{
+    Ref x(THPVariable_Wrap(q)), y(THPVariable_Wrap(s));
+    return PyTuple_Pack(2, x.p, y.p);
+}
+
+// x, stream; transposed: the encoding of x^T
+template <bool T>
+PyObject *mxfp8_quantize1d(Args a, Py_ssize_t n)
+{
+    want(n, 2);
+    const at::Tensor &x = as_matrix(a[0], "x", kXText);
+    const int64_t rows = x.size(0), cols = x.size(1), along = T ? rows : cols, across = T ? cols : rows;
+    const at::Tensor q = empty2(across, std::max<int64_t>(ceil_to(along, 32) * 32, 32), at::kByte, x);
+    const at::Tensor s = empty2(across, std::max<int64_t>(ceil_to(along, 32), 1), at::kByte, x);
+    check(unlocked(T ? lib.mxfp8_quantize1d_t : lib.mxfp8_quantize1d, x.data_ptr(), rows, cols, pitch(x), bytes_of(q), q.stride(0), bytes_of(s),
+                                                              s.stride(0), as_stream(a[1])),
+          T ? "fp4q_mxfp8_quantize1d_t" : "fp4q_mxfp8_quantize1d");
+    return pair(q, s);
+}
+
+// x, mode, seed, tensor_id, stream
+PyObject *quantize1d(Args a, Py_ssize_t n)
+{
+    want(n, 5);
+    const at::Tensor &x = as_matrix(a[0], "x", kXText);
+    const int64_t rows = x.size(0), cols = x.size(1);
+    const at::Tensor q = empty2(rows, std::max<int64_t>(pad16(ceil_to(cols, 32) * 16), 16), at::kByte, x);
+    const at::Tensor s = empty2(rows, std::max<int64_t>(ceil_to(cols, 32), 1), at::kByte, x);
+    check(unlocked(lib.quantize1d, x.data_ptr(), rows, cols, pitch(x), bytes_of(q), q.stride(0), bytes_of(s), s.stride(0), (fp4q_round)as_int(a[1]),
+                         as_bits(a[2]), (uint32_t)as_bits(a[3]), as_stream(a[4])), "fp4q_quantize1d");
+    return pair(q, s);
+}
+
+// x, stream
+PyObject *quantize1d_t(Args a, Py_ssize_t n)
+{
+    want(n, 2);
+    const at::Tensor &x = as_matrix(a[0], "x", kXText);
+    const int64_t rows = x.size(0), cols = x.size(1);
+    const at::Tensor q = empty2(cols, std::max<int64_t>(pad16(ceil_to(rows, 32) * 16), 16), at::kByte, x);
+    const at::Tensor s = empty2(cols, std::max<int64_t>(ceil_to(rows, 32), 1), at::kByte, x);
+    check(unlocked(lib.quantize1d_t, x.data_ptr(), rows, cols, pitch(x), bytes_of(q), q.stride(0), bytes_of(s), s.stride(0), as_stream(a[1])),
+          "fp4q_quantize1d_t");
+    return pair(q, s);
+}
+
+// which (0 fwd, 1 dgrad, 2 wgrad), a, b, out_rows, out_cols, out | None, dt, accumulate, row_offsets | None, row_alignment, ws, stream
+PyObject *gemm(Args a, Py_ssize_t n)
+{
+    want(n, 12);
+    static const char *const names[3] = {"fp4q_gemm_fwd", "fp4q_gemm_dgrad", "fp4q_gemm_wgrad"};
+    const int which = as_int(a[0]), dt = as_int(a[6]);
+    const int64_t rows = as_i64(a[3]), cols = as_i64(a[4]);
+    const at::Tensor out = a[5] == Py_None ? out_buffer(rows, cols, dt, qtensor_payload(a[1])) : as_tensor(a[5]);
+    const fp4q_tensor ta = from_qtensor(a[1], 32), tb = from_qtensor(a[2], 32);
+    const Groups g(a[8], as_int(a[9]));
+    const at::Tensor &ws = as_tensor(a[10]);
+    void *st = as_stream(a[11]);
+    const int64_t ld = out_pitch(out, cols);
+    const fp4q_status s =
+        which == 2 ? unlocked(lib.gemm_wgrad, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, as_int(a[7]), g.ptr, ws.data_ptr(), (size_t)ws.numel(), st)
+                   : unlocked(which == 1 ? lib.gemm_dgrad : lib.gemm_fwd, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, g.ptr, ws.data_ptr(),
+                                                                  (size_t)ws.numel(), st);
+    check(s, names[which]);
+    return a[5] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[5]);
+}
+
+// which, a, b, out_rows, out_cols, out | None, dt, accumulate, ws, stream
+PyObject *gemm_b16(Args a, Py_ssize_t n)
+{
+    want(n, 10);
+    static const char *const names[3] = {"fp4q_gemm_fwd_b16", "fp4q_gemm_dgrad_b16", "fp4q_gemm_wgrad_b16"};
+    const int which = as_int(a[0]), dt = as_int(a[6]), accumulate = as_int(a[7]);
+    const int64_t rows = as_i64(a[3]), cols = as_i64(a[4]);
+    const at::Tensor out = a[5] == Py_None ? out_buffer(rows, cols, dt, qtensor_payload(a[1])) : as_tensor(a[5]);
+    if (a[5] == Py_None && accumulate) out.zero_();
+    const fp4q_tensor ta = from_qtensor(a[1], 16), tb = from_qtensor(a[2], 16);
+    const at::Tensor &ws = as_tensor(a[8]);
+    void *st = as_stream(a[9]);
+    const int64_t ld = out_pitch(out, cols);
+    const fp4q_status s =
+        which == 2 ? unlocked(lib.gemm_wgrad_b16, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, accumulate, ws.data_ptr(), (size_t)ws.numel(), st)
+                   : unlocked(which == 1 ? lib.gemm_dgrad_b16 : lib.gemm_fwd_b16, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, ws.data_ptr(),
+                                                                          (size_t)ws.numel(), st);
+    check(s, names[which]);
+    return a[5] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[5]);
+}
+
+// which (0 fwd, 1 dgrad), a, b, out_rows, out_cols, out | None, mode, seed, tensor_id, want_t, row_offsets | None, ws, stream
+PyObject *gemm_quantized(Args a, Py_ssize_t n)
+{
+    want(n, 13);
+    const int which = as_int(a[0]);
+    const Groups g(a[10], 256);
+    const int64_t rows = as_i64(a[3]), cols = as_i64(a[4]);
+    QBuffers b;
+    fp4q_tensor tc;
+    if (a[5] == Py_None) {
+        b = alloc_q(rows, cols, qtensor_payload(a[1]), as_bool(a[9]), 32);
+        tc = c_tensor(rows, cols, b.q_rm, b.q_t, b.scale);
+    }
+    const fp4q_tensor ta = from_qtensor(a[1], 32), tb = from_qtensor(a[2], 32);
+    if (a[5] != Py_None) tc = from_qtensor(a[5], 32);
+    const at::Tensor &ws = as_tensor(a[11]);
+    check(unlocked(which ? lib.gemm_dgrad_quantized : lib.gemm_fwd_quantized, &ta, &tb, &tc, (fp4q_round)as_int(a[6]), as_bits(a[7]),
+                                                                      (uint32_t)as_bits(a[8]), g.ptr, ws.data_ptr(), (size_t)ws.numel(),
+                                                                      as_stream(a[12])),
+          which ? "fp4q_gemm_dgrad_quantized" : "fp4q_gemm_fwd_quantized");
+    return a[5] == Py_None ? new_qtensor(rows, cols, b, 32) : Py_NewRef(a[5]);
+}
+
+// xq, xs, T, W, out | None, dt, ws, stream
+PyObject *gemm_fwd_act1d(Args a, Py_ssize_t n)
+{
+    want(n, 8);
+    const at::Tensor &xq = as_tensor(a[0]), &xs = as_tensor(a[1]);
+    const int64_t T = as_i64(a[2]);
+    const int dt = as_int(a[5]);
+    Ref wr(PyObject_GetAttr(a[3], s_rows));
+    const at::Tensor out = a[4] == Py_None ? out_buffer(T, as_i64(wr.p), dt, xq) : as_tensor(a[4]);
+    const fp4q_tensor w = from_qtensor(a[3], 32);
+    const at::Tensor &ws = as_tensor(a[6]);
+    check(unlocked(lib.gemm_fwd_act1d, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), T, &w, out.data_ptr(), out.stride(0), (fp4q_out)dt,
+                             ws.data_ptr(), (size_t)ws.numel(), as_stream(a[7])), "fp4q_gemm_fwd_act1d");
+    return a[4] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[4]);
+}
+
+// dY, xtq, xts, K, out | None, dt, accumulate, ws, stream
+PyObject *gemm_wgrad_act1d(Args a, Py_ssize_t n)
+{
+    want(n, 9);
+    const at::Tensor &xq = as_tensor(a[1]), &xs = as_tensor(a[2]);
+    const int64_t K = as_i64(a[3]);
+    const int dt = as_int(a[5]), accumulate = as_bool(a[6]) ? 1 : 0;
+    Ref dc(PyObject_GetAttr(a[0], s_cols));
+    const at::Tensor out = a[4] == Py_None ? out_buffer(as_i64(dc.p), K, dt, xq) : as_tensor(a[4]);
+    if (a[4] == Py_None && accumulate) out.zero_();
+    const fp4q_tensor d = from_qtensor(a[0], 32);
+    const at::Tensor &ws = as_tensor(a[7]);
+    check(unlocked(lib.gemm_wgrad_act1d, &d, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), K, out.data_ptr(), out.stride(0), (fp4q_out)dt,
+                               accumulate, ws.data_ptr(), (size_t)ws.numel(), as_stream(a[8])), "fp4q_gemm_wgrad_act1d");
+    return a[4] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[4]);
+}
+
+// aq, as, bq, bs, M, N, K, dt, ws, stream
+PyObject *mxfp8_gemm(Args a, Py_ssize_t n)
+{
+    want(n, 10);
+    const at::Tensor &aq = as_tensor(a[0]), &as = as_tensor(a[1]), &bq = as_tensor(a[2]), &bs = as_tensor(a[3]);
+    const int64_t M = as_i64(a[4]), N = as_i64(a[5]), K = as_i64(a[6]);
+    const int dt = as_int(a[7]);
+    const at::Tensor out = out_buffer(M, N, dt, aq);
+    const at::Tensor &ws = as_tensor(a[8]);
+    const int64_t per16 = dt == FP4Q_OUT_BF16 ? 8 : 4, ld = std::max(ceil_to(N, per16) * per16, per16);
+    check(unlocked(lib.mxfp8_gemm, bytes_of(aq), aq.stride(0), bytes_of(as), as.stride(0), M, bytes_of(bq), bq.stride(0), bytes_of(bs), bs.stride(0), N,
+                         K, out.data_ptr(), ld, (fp4q_out)dt, ws.data_ptr(), (size_t)ws.numel(), as_stream(a[9])), "fp4q_mxfp8_gemm");
+    return THPVariable_Wrap(out);
+}
+
+// xq, xs, wq_q | None, wq_s | None, wk_q | None, wk_s | None, T, K, N, dt, ws, stream
+PyObject *mxfp8_qk(Args a, Py_ssize_t n)
+{
+    want(n, 12);
+    const at::Tensor &xq = as_tensor(a[0]), &xs = as_tensor(a[1]);
+    at::Tensor w[4];
+    uint8_t *p[4];
+    for (int i = 0; i < 4; i++) {
+        if (a[2 + i] != Py_None) w[i] = as_tensor(a[2 + i]);
+        p[i] = w[i].defined() ? bytes_of(w[i]) : nullptr;
+    }
+    const int64_t T = as_i64(a[6]), K = as_i64(a[7]), N = as_i64(a[8]);
+    const int dt = as_int(a[9]);
+    const int64_t per16 = dt == FP4Q_OUT_BF16 ? 8 : 4, ld = std::max(ceil_to(N, per16) * per16, per16);
+    at::Tensor out[2];
+    for (int i = 0; i < 2; i++) if (w[2 * i].defined()) out[i] = out_buffer(T, N, dt, xq);
+    const at::Tensor &wref = w[0].defined() ? w[0] : w[2], &sref = w[0].defined() ? w[1] : w[3];
+    if (!wref.defined() || !sref.defined()) { PyErr_SetString(PyExc_AttributeError, "'NoneType' object has no attribute 'stride'"); throw PyError(); }
+    const at::Tensor &ws = as_tensor(a[10]);
+    check(unlocked(lib.mxfp8_qk, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), T, K, p[0], p[1], p[2], p[3], wref.stride(0), sref.stride(0), N,
+                       out[0].defined() ? out[0].data_ptr() : nullptr, out[1].defined() ? out[1].data_ptr() : nullptr, ld, (fp4q_out)dt,
+                       ws.data_ptr(), (size_t)ws.numel(), as_stream(a[11])), "fp4q_mxfp8_qk");
+    Ref q(out[0].defined() ? THPVariable_Wrap(out[0]) : Py_NewRef(Py_None)), k(out[1].defined() ? THPVariable_Wrap(out[1]) : Py_NewRef(Py_None));
+    return PyTuple_Pack(2, q.p, k.p);
+}
+
+template <typename F>
+void set_entry(PyObject *addresses, const char *name, F &slot)
+{
+    PyObject *v = PyDict_GetItemString(addresses, name);
+    if (!v) { PyErr_Format(PyExc_KeyError, "%s", name); throw PyError(); }
+    slot = reinterpret_cast<F>(PyLong_AsVoidPtr(v));
+    if (PyErr_Occurred()) throw PyError();
+}
+
+// {name: address of the C entry point}, QTensor, _check
+PyObject *init(Args a, Py_ssize_t n)
+{
+    want(n, 3);
+    set_entry(a[0], "fp4q_quantize2d", lib.quantize2d);
+    set_entry(a[0], "fp4q_quantize2d_multi", lib.quantize2d_multi);
+    set_entry(a[0], "fp4q_mxfp8_quantize1d", lib.mxfp8_quantize1d);
+    set_entry(a[0], "fp4q_mxfp8_quantize1d_t", lib.mxfp8_quantize1d_t);
+    set_entry(a[0], "fp4q_quantize1d", lib.quantize1d);
+    set_entry(a[0], "fp4q_quantize1d_t", lib.quantize1d_t);
+    set_entry(a[0], "fp4q_gemm_fwd", lib.gemm_fwd);
+    set_entry(a[0], "fp4q_gemm_dgrad", lib.gemm_dgrad);
+    set_entry(a[0], "fp4q_gemm_wgrad", lib.gemm_wgrad);
+    set_entry(a[0], "fp4q_gemm_fwd_b16", lib.gemm_fwd_b16);
+    set_entry(a[0], "fp4q_gemm_dgrad_b16", lib.gemm_dgrad_b16);
+    set_entry(a[0], "fp4q_gemm_wgrad_b16", lib.gemm_wgrad_b16);
+    set_entry(a[0], "fp4q_gemm_fwd_quantized", lib.gemm_fwd_quantized);
+    set_entry(a[0], "fp4q_gemm_dgrad_quantized", lib.gemm_dgrad_quantized);
+    set_entry(a[0], "fp4q_gemm_fwd_act1d", lib.gemm_fwd_act1d);
+    set_entry(a[0], "fp4q_gemm_wgrad_act1d", lib.gemm_wgrad_act1d);
+    set_entry(a[0], "fp4q_mxfp8_qk", lib.mxfp8_qk);
+    set_entry(a[0], "fp4q_mxfp8_gemm", lib.mxfp8_gemm);
+    Py_XSETREF(g_qtensor, Py_NewRef(a[1]));
+    Py_XSETREF(g_fail, Py_NewRef(a[2]));
+    return Py_NewRef(Py_None);
+}
+
+// What a call throws becomes a Python exception: its own, or torch's (out of memory, a failed CUDA call).
+template <PyObject *(*F)(Args, Py_ssize_t)>
+PyObject *entry(PyObject *, Args a, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    try {
+        return F(a, n);
+    } catch (const PyError &) {
+        return nullptr;
+    }
+    END_HANDLE_TH_ERRORS
+}
+
+#define METHOD(name, fn) {name, (PyCFunction)(void (*)(void))entry<fn>, METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {METHOD("init", init),
+                         METHOD("quantize2d", quantize2d),
+                         METHOD("quantize2d_multi", quantize2d_multi),
+                         METHOD("mxfp8_quantize1d", mxfp8_quantize1d<false>),
+                         METHOD("mxfp8_quantize1d_t", mxfp8_quantize1d<true>),
+                         METHOD("quantize1d", quantize1d),
+                         METHOD("quantize1d_t", quantize1d_t),
+                         METHOD("gemm", gemm),
+                         METHOD("gemm_b16", gemm_b16),
+                         METHOD("gemm_quantized", gemm_quantized),
+                         METHOD("gemm_fwd_act1d", gemm_fwd_act1d),
+                         METHOD("gemm_wgrad_act1d", gemm_wgrad_act1d),
+                         METHOD("mxfp8_gemm", mxfp8_gemm),
+                         METHOD("mxfp8_qk", mxfp8_qk),
+                         {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_host", "argument marshalling of binding.py", -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__host(void)
+{
+    s_rows = PyUnicode_InternFromString("rows");
+    s_cols = PyUnicode_InternFromString("cols");
+    s_q_rm = PyUnicode_InternFromString("q_rm");
+    s_q_t = PyUnicode_InternFromString("q_t");
+    s_scale = PyUnicode_InternFromString("scale");
+    s_granularity = PyUnicode_InternFromString("scale_granularity");
+    return PyModule_Create(&module);
+}
