@@ -10,12 +10,14 @@
 // tile through cta_group::2 MMAs (each CTA holds 128 rows of the accumulator, loads its own 128 A rows and half of
 // the B rows); grouped products and MXFP8 use one CTA per 128x256 tile.
 //   warp 0      TMA producer: per stage the A tile (128 rows x 128 B) and the B tile (256 or 128 rows x 128 B),
-//               128B swizzle; polls all free slots first, then issues their loads back to back
+//               128B swizzle
 //   warp 1      MMA issuer: stays converged, one elected lane issues per stage 6 tcgen05.cp (scale images -> TMEM),
-//               4 tcgen05.mma and the tcgen05.commit that frees the slot; it never reads shared memory in the loop
-//   warp 2      watcher: polls the slots' "full" barriers (several at a time), the scale images and the
-//               accumulator's "empty" barrier and meets the MMA warp at a named barrier per stage
-//   warp 3      scale image builder: per unit of 16 (FP4) or 8 (MXFP8) stages gathers the scale bytes and writes the
+//               4 tcgen05.mma and the tcgen05.commit that frees the slot; in the second CTA of a pair it reports
+//               that CTA's per-row scale images to the leader
+//   warp 2      dense FP4 and MXFP8 pairs: watcher, polls the slots' "full" barriers (several at a time), the scale images
+//               and the accumulator's "empty" barrier and meets the MMA warp at a named barrier per stage (elsewhere the
+//               MMA warp looks for itself); per-row FP4 kinds: second scale image builder
+//   warp 3      scale image builder: per unit of 16 stages (4 or 2 with per-row images) gathers the scale bytes and writes the
 //               images tcgen05.cp reads in place (double-buffered); 2D-block scales as replicated 8-row images,
 //               per-row scales as real 32-row images
 //   warps 4-11  epilogue: tcgen05.ld of the 128x256 FP32 accumulator (each warp 32 lanes x 128 columns),
@@ -49,22 +51,22 @@ constexpr int kCacheChunks = 32;             // chunks per unit
 constexpr int kUnitStagesMxf4 = kCacheChunks / 2;
 // Per-row scales (MXFP8): a stage covers 4 contraction blocks; its three images (A rows, B rows 0..127, B rows
 // 128..255) are real 32-row x 16-byte images (512 B each), row l holding rows l, l+32, l+64, l+96 of the operand.
-// A unit is 8 stages, so that a buffer has the same size as for 2D-block scales.
-constexpr int kUnitStagesMxf8 = 8;
+// A unit is 4 stages (16 blocks, one 16-byte piece of every row's scales): half of the other kinds' 12 KB buffers, which
+// pays for one more ring stage.
+constexpr int kUnitStagesMxf8 = 4;
 constexpr int kImageStageBytesMxf8 = 1536;
 constexpr int kCompactBytes = kCacheChunks * 48;
 constexpr int kImageStageBytes = 768;        // A chunk 0, A chunk 1, B chunk 0 (rows 0..127, 128..255), B chunk 1 (same)
 constexpr int kCacheBufBytes = kUnitStagesMxf4 * kImageStageBytes;
-static_assert(kUnitStagesMxf8 * kImageStageBytesMxf8 == kCacheBufBytes, "both kinds share the image buffers");
 // mxf4 with per-row scales: a stage has two chunks of four blocks; A 2 x 512 B, B (256 rows) 4 x 512 B per stage
 constexpr int kUnitStagesMxf4R = 4;
 constexpr int kImageStageBytesMxf4R = 3072;
-static_assert(kUnitStagesMxf4R * kImageStageBytesMxf4R == kCacheBufBytes, "all kinds share the image buffers");
+static_assert(kUnitStagesMxf4R * kImageStageBytesMxf4R == kCacheBufBytes, "the FP4 kinds share the size of an image buffer");
 // mxf4nvf4 with 16-element scale vectors (tensors quantized in 16 x 16 blocks): every MMA (64 contraction elements)
 // has its own image per 128 operand rows - four scale bytes per row - so a stage holds A 4 x 512 B and B 8 x 512 B
 constexpr int kUnitStagesMxf4B16 = 2;
 constexpr int kImageStageBytesMxf4B16 = 6144;
-static_assert(kUnitStagesMxf4B16 * kImageStageBytesMxf4B16 == kCacheBufBytes, "all kinds share the image buffers");
+static_assert(kUnitStagesMxf4B16 * kImageStageBytesMxf4B16 == kCacheBufBytes, "the FP4 kinds share the size of an image buffer");
 // Epilogue staging of the pair kernel: each of the 8 epilogue warps owns 32 rows x 128 bytes, written from registers
 // (128-byte swizzle: the 16-byte pieces of 8 rows fall into different banks) and drained by a TMA store, which keeps
 // the output off the load/store unit that the MMA warp's instructions also pass through.
@@ -81,29 +83,33 @@ constexpr int kStagingWarpBytes = 32 * 128;
 enum { KIND_MXF4 = 0, KIND_MXF8 = 1, KIND_MXF4R = 2, KIND_MXF4B16 = 3 };
 __host__ __device__ constexpr bool kind_fp4(int kind) { return kind != KIND_MXF8; }
 
-// Per-row scale images are rebuilt every 4 (FP4) or 8 (MXFP8) stages from 12 KB of scale bytes, whose global-memory
-// latency under the operand traffic (about 3000 cycles) exceeds the time such a unit runs.  The kernels for those
-// kinds therefore fetch the bytes two units ahead with cp.async into raw buffers (no registers are held meanwhile)
-// and pay for the buffers with one ring stage; the pair kernel also keeps a third image buffer, because the way
+// Per-row scale images are rebuilt every 4 stages (2 with 16 x 16 blocks) from 12 KB (MXFP8: 6 KB) of scale bytes, whose
+// global-memory latency under the operand traffic (about 3000 cycles) exceeds the time such a unit runs.  The kernels for
+// those kinds therefore fetch the bytes two units ahead with cp.async into raw buffers (no registers are held meanwhile);
+// the FP4 kinds pay for the buffers with one ring stage; the pair kernel also keeps a third image buffer, because the way
 // from "the MMAs have finished with a buffer" to "the leader may copy the next unit out of it" (commit to both
 // CTAs, build, report to the leader) is longer than one unit as well.
 template <int KIND, int CTAS>
 struct Cfg {
     static constexpr bool kRowImages = KIND != KIND_MXF4;
-    static constexpr int kImageBufs = (CTAS == 2 && kRowImages) ? 3 : 2;
-    static constexpr int kRawBufs = kRowImages ? 2 : 0;
+    // Image builder warps: the per-row FP4 kinds, whose units are 4 or 2 stages, have two that take turns (one warp needs
+    // 1500-2500 cycles for a unit, all of it latency); their MMA warp waits for itself and needs no watcher.
+    static constexpr int kBuilders = (KIND == KIND_MXF4R || KIND == KIND_MXF4B16) ? 2 : 1;
+    static constexpr int kImageBufs = (CTAS == 2 && kRowImages) ? (KIND == KIND_MXF4B16 ? 4 : 3) : 2;
+    static constexpr int kRawBufs = kRowImages ? (KIND == KIND_MXF4B16 ? 4 : 2) : 0;
     // The output leaves through staging rows and TMA stores wherever shared memory allows (everything but the
     // one-CTA kernel of the per-row kinds).  In the one-CTA kernel of the 2D kind - grouped products with short
     // contractions - plain stores of the 64 KB tile filled the SM's path to L2 and the TMA loads issued meanwhile
     // took 6500-8000 cycles instead of 3000; the staging costs that kernel its fourth ring stage.
     static constexpr bool kTmaStores = CTAS == 2 || !kRowImages;
-    // One-CTA kernel of the 2D kind (grouped products): its 48 KB stages keep the TMA unit busy ~740 of every ~800 cycles,
-    // so a producer that also polls (a poll queues behind the loads the same warp has just issued) leaves gaps.  There
-    // the producer is split: warp 2 waits for free slots and arms their barriers, warp 0 only issues loads; the MMA warp
-    // waits on its barriers itself (measured: MoE expert layer 1.95 -> 2.07 PFLOP/s; no gain for the pair kernel).
-    static constexpr bool kSplitProducer = KIND == KIND_MXF4 && CTAS == 1;
-    static constexpr int kStages = (CTAS == 2 ? 5 : (kTmaStores ? 3 : 4)) - (kRowImages ? 1 : 0);
-    static constexpr int kSmemCache = kCompactBytes + (kImageBufs + kRawBufs) * kCacheBufBytes;
+    static constexpr int kStages = (CTAS == 2 ? 5 : (kTmaStores ? 3 : 4)) - (kRowImages && KIND != KIND_MXF8 ? 1 : 0);
+    static constexpr int kBufBytes = KIND == KIND_MXF8 ? kUnitStagesMxf8 * kImageStageBytesMxf8 : kCacheBufBytes;   // an image buffer
+    static constexpr int kUnitBlocks = KIND == KIND_MXF8 ? 16 : 32;   // per-row kinds: contraction blocks of a unit = scale bytes of a row
+    // a raw buffer: 32 lanes' scale bytes per slot, 4 slots of A rows and 8 of B rows; with 16 x 16 blocks both operands are
+    // compact and need one slot each
+    static constexpr int kRawSlotB = KIND == KIND_MXF4B16 ? 1 : 4;
+    static constexpr int kRawBytes = (kRawSlotB + (KIND == KIND_MXF4B16 ? 1 : 8)) * 32 * kUnitBlocks;
+    static constexpr int kSmemCache = (kRowImages ? 0 : kCompactBytes) + kImageBufs * kBufBytes + kRawBufs * kRawBytes;
     static constexpr int kBRows = CTAS == 2 ? 128 : 256;
     static constexpr int kBStageBytes = kBRows * 128;
     static constexpr int kSmemOperands = kStages * (kAStageBytes + kBStageBytes);
@@ -268,11 +274,6 @@ __device__ __noinline__ bool mbar_wait_lazy(uint32_t bar, uint32_t parity, volat
 }
 // For barriers that another CTA of the cluster completes (a multicast tcgen05.commit): probe instead of try_wait,
 // whose suspended thread is not reliably woken early by a remote arrival.
-__device__ __noinline__ bool mbar_poll(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status, uint64_t limit,
-                                       uint32_t where)
-{
-    return mbar_wait_impl<0, true>(bar, parity, abort_flag, status, limit, where);
-}
 __device__ __noinline__ bool mbar_poll_relaxed(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status,
                                                uint64_t limit, uint32_t where)
 {
@@ -645,11 +646,11 @@ __device__ __forceinline__ void ldg_v4(const uint8_t *ptr, uint32_t *w)
 }
 
 template <int KIND>
-__device__ __forceinline__ void store_row_scale_images(const uint32_t (&w)[12][8], int n_stages, uint8_t *images, int lane)
+__device__ __forceinline__ void store_row_scale_images(const uint32_t (&w)[12][KIND == KIND_MXF8 ? 4 : 8], int n_stages, uint8_t *images, int lane)
 {
-    if (KIND == KIND_MXF8) {
+    if constexpr (KIND == KIND_MXF8) {
 #pragma unroll
-        for (int st = 0; st < 8; st++) {
+        for (int st = 0; st < 4; st++) {
             if (st < n_stages) {
                 uint4 *img = reinterpret_cast<uint4 *>(images + st * kImageStageBytesMxf8);
                 img[lane] = make_uint4(w[0][st], w[1][st], w[2][st], w[3][st]);           // A
@@ -657,7 +658,7 @@ __device__ __forceinline__ void store_row_scale_images(const uint32_t (&w)[12][8
                 img[64 + lane] = make_uint4(w[8][st], w[9][st], w[10][st], w[11][st]);    // B rows 128..255
             }
         }
-    } else if (KIND == KIND_MXF4B16) {
+    } else if constexpr (KIND == KIND_MXF4B16) {
         // word j of a row = the four scale bytes of MMA j of the unit (stage j / 4, MMA j % 4)
 #pragma unroll
         for (int st = 0; st < 2; st++) {
@@ -832,7 +833,11 @@ struct UnitIter {
         seek(p);
     }
     __device__ __forceinline__ bool valid(const GemmParams &p) const { return tile < p.n_tile_total; }
-    __device__ __forceinline__ void next(const GemmParams &p, int unit_elems) { k0 += unit_elems; seek(p); }
+    __device__ __forceinline__ void next(const GemmParams &p, int unit_elems)
+    {
+        k0 += unit_elems;
+        if (k0 >= t.k_len) { tile += step; k0 = 0; seek(p); }   // a tile is decoded once: its three divisions took longer than a unit's images
+    }
 };
 
 __device__ __forceinline__ void cp_async(uint32_t dst, const void *src, int bytes, int src_bytes)
@@ -842,25 +847,25 @@ __device__ __forceinline__ void cp_async(uint32_t dst, const void *src, int byte
     else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
 
-// Raw scale bytes of one unit (32 contraction blocks from k0), asynchronously into `raw` (12 KB): slot q (1 KB,
-// q < 4: A rows 32q.., q >= 4: B rows 32(q-4)..) holds 32 bytes per lane, the scale bytes of the lane's operand row.
+// Raw scale bytes of one unit (BLOCKS contraction blocks from k0: 32, or 16 for MXFP8), asynchronously into `raw`: slot q
+// (q < 4: A rows 32q.., q >= 4: B rows 32(q-4)..) holds BLOCKS bytes per lane, the scale bytes of the lane's operand row.
 // A 2D-block operand (row_shift 5) needs only 32 bytes per row tile: they are packed at the start of the operand's
 // first slot; if its view is transposed (blocks stride_kb apart, row tiles contiguous) lane l fetches block l's
 // bytes for the operand's 4 or 8 row tiles into the first 8 bytes of its entry of that slot.  With 16 x 16 blocks
 // (row_shift 4, KB_SHIFT 4: a block is 16 contraction elements and a row tile 16 rows) the unit still has 32 blocks but
 // the operand has 8 or 16 row tiles.  Bytes beyond the tensor arrive as zero.  Every lane commits exactly one
 // cp.async group per call.
-template <int KB_SHIFT>
+template <int KB_SHIFT, int BLOCKS, int SLOT_B>
 __device__ __forceinline__ void issue_raw_scales(const GemmParams &p, const Tile &t, int k0, uint8_t *raw, int lane)
 {
 #pragma unroll
     for (int op = 0; op < 2; op++) {
         const ScaleView &v = op == 0 ? p.sfa : p.sfb;
-        const int nq = op == 0 ? 4 : 8, q0 = op == 0 ? 0 : 4;
+        const int nq = op == 0 ? 4 : 8, q0 = op == 0 ? 0 : SLOT_B;
         const int row0 = op == 0 ? t.a_row0 : t.b_row0;
         const int kb0 = ((op == 0 ? t.a_k0 : t.b_k0) + k0) >> KB_SHIFT;
         const int n_tiles = v.row_shift != 0 ? nq << (5 - v.row_shift) : 0;   // row tiles of a 2D-block operand
-        if (v.row_shift != 0 && v.stride_kb != 1) {
+        if (BLOCKS == 32 && v.row_shift != 0 && v.stride_kb != 1) {
             const int rt0 = row0 >> v.row_shift, kb = kb0 + lane, nbytes = n_tiles;   // 4 .. 16 row tiles, one byte each
             uint8_t *dst = raw + q0 * 1024 + lane * 32;
             const uint8_t *src = v.ptr + (int64_t)kb * v.stride_kb + rt0;
@@ -876,7 +881,7 @@ __device__ __forceinline__ void issue_raw_scales(const GemmParams &p, const Tile
             }
             continue;
         }
-        if (v.row_shift != 0) {
+        if (BLOCKS == 32 && v.row_shift != 0) {
             // 2D-block operand, blocks contiguous: the 32 bytes of each of the operand's row tiles once (two lanes
             // per row tile copy 16 bytes each), packed at the start of the operand's first slot
             if (lane < 2 * n_tiles) {
@@ -900,16 +905,16 @@ __device__ __forceinline__ void issue_raw_scales(const GemmParams &p, const Tile
 #pragma unroll
         for (int q = 0; q < nq; q++) {
             const int row = row0 + lane + 32 * q;
-            uint8_t *dst = raw + (q0 + q) * 1024 + lane * 32;
+            uint8_t *dst = raw + (q0 + q) * 32 * BLOCKS + lane * BLOCKS;
             const uint8_t *src = v.ptr + (int64_t)row * v.stride_row + kb0;
             if (v.stride_kb == 1 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-                const int valid = row < v.n_row ? max(0, min(32, v.n_kb - kb0)) : 0;
+                const int valid = row < v.n_row ? max(0, min(BLOCKS, v.n_kb - kb0)) : 0;
                 const uint8_t *safe = v.ptr - (reinterpret_cast<uintptr_t>(v.ptr) & 15);
                 cp_async(smem_u32(dst), valid > 0 ? src : safe, 16, min(valid, 16));
-                cp_async(smem_u32(dst + 16), valid > 16 ? src + 16 : safe, 16, max(valid - 16, 0));
+                if (BLOCKS == 32) cp_async(smem_u32(dst + 16), valid > 16 ? src + 16 : safe, 16, max(valid - 16, 0));
             } else {
 #pragma unroll
-                for (int st = 0; st < 8; st++) {
+                for (int st = 0; st < BLOCKS / 4; st++) {
                     uint32_t word;
                     load_scale_word(v, row, kb0 + 4 * st, word);
                     reinterpret_cast<uint32_t *>(dst)[st] = word;
@@ -923,19 +928,28 @@ __device__ __forceinline__ void issue_raw_scales(const GemmParams &p, const Tile
 // The unit's scale words from a raw buffer whose copies have completed: w[q][j] = the four scale bytes of the
 // lane's row of slot q for blocks 4j..4j+3.  Lanes read bytes other lanes copied: the caller synchronizes the warp
 // after its cp.async wait.
-__device__ __forceinline__ void read_raw_scales(const GemmParams &p, const uint8_t *raw, int lane, uint32_t (&w)[12][8])
+template <int BLOCKS, int SLOT_B>
+__device__ __forceinline__ void read_raw_scales(const GemmParams &p, const uint8_t *raw, int lane, uint32_t (&w)[12][BLOCKS / 4])
 {
+    if constexpr (BLOCKS == 16) {
+#pragma unroll
+        for (int q = 0; q < 12; q++) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(raw + q * 512 + lane * 16);
+            w[q][0] = v.x; w[q][1] = v.y; w[q][2] = v.z; w[q][3] = v.w;
+        }
+        return;
+    } else {
 #pragma unroll
     for (int op = 0; op < 2; op++) {
         const ScaleView &v = op == 0 ? p.sfa : p.sfb;
-        const int nq = op == 0 ? 4 : 8, q0 = op == 0 ? 0 : 4;
+        const int nq = op == 0 ? 4 : 8, q0 = op == 0 ? 0 : 4, s0 = op == 0 ? 0 : SLOT_B;
         if (v.row_shift != 0 && v.stride_kb != 1) {
             // lane l holds block l's bytes [row tile 0..]: words of four consecutive lanes, transposed as 4x4 bytes,
             // are the four row tiles' words of one chunk
             if (v.row_shift == 4) {
                 // 16-row tiles: 8 (A) or 16 (B) bytes per lane; operand rows l + 32 q of image row l lie in row tile
                 // 2 q + (l >> 4), so the two halves of the warp pick different tiles of each transposed word
-                const uint4 mine4 = *reinterpret_cast<const uint4 *>(raw + q0 * 1024 + lane * 32);
+                const uint4 mine4 = *reinterpret_cast<const uint4 *>(raw + s0 * 1024 + lane * 32);
                 const bool hi = lane >= 16;
 #pragma unroll
                 for (int h = 0; h < (op == 0 ? 2 : 4); h++) {
@@ -950,7 +964,7 @@ __device__ __forceinline__ void read_raw_scales(const GemmParams &p, const uint8
                 }
                 continue;
             }
-            const uint2 mine = *reinterpret_cast<const uint2 *>(raw + q0 * 1024 + lane * 32);
+            const uint2 mine = *reinterpret_cast<const uint2 *>(raw + s0 * 1024 + lane * 32);
 #pragma unroll
             for (int h = 0; h < (op == 0 ? 1 : 2); h++) {
                 const uint32_t m = h == 0 ? mine.x : mine.y;
@@ -966,17 +980,54 @@ __device__ __forceinline__ void read_raw_scales(const GemmParams &p, const uint8
 #pragma unroll
         for (int q = 0; q < nq; q++) {
             const int tile = v.row_shift == 4 ? 2 * q + (lane >> 4) : q;   // row tile of operand row lane + 32 q
-            const uint4 *src = reinterpret_cast<const uint4 *>(v.row_shift != 0 ? raw + q0 * 1024 + tile * 32 : raw + (q0 + q) * 1024 + lane * 32);
+            const uint4 *src = reinterpret_cast<const uint4 *>(v.row_shift != 0 ? raw + s0 * 1024 + tile * 32 : raw + (s0 + q) * 1024 + lane * 32);
             const uint4 lo = src[0], hi = src[1];
             w[q0 + q][0] = lo.x; w[q0 + q][1] = lo.y; w[q0 + q][2] = lo.z; w[q0 + q][3] = lo.w;
             w[q0 + q][4] = hi.x; w[q0 + q][5] = hi.y; w[q0 + q][6] = hi.z; w[q0 + q][7] = hi.w;
         }
     }
+    }
 }
+
+// MXFP8: the lane's twelve scale rows of a tile (4 of A, 8 of B).  A unit's fetch is then one 16-byte copy per row with
+// nothing to compute but the address step.
+struct RowFetch {
+    const uint8_t *src[12];
+    uint32_t valid;   // bit q: the row exists
+    bool fast;        // every copy starts on a 16-byte boundary
+    __device__ __forceinline__ void set(const GemmParams &p, const Tile &t, int lane)
+    {
+        valid = 0;
+        fast = true;
+#pragma unroll
+        for (int q = 0; q < 12; q++) {
+            const ScaleView &v = q < 4 ? p.sfa : p.sfb;
+            const int row = q < 4 ? t.a_row0 + lane + 32 * q : t.b_row0 + lane + 32 * (q - 4), kb = (q < 4 ? t.a_k0 : t.b_k0) >> 5;
+            const bool ok = row < v.n_row;
+            valid |= ok ? 1u << q : 0u;
+            src[q] = ok ? v.ptr + (int64_t)row * v.stride_row + kb : v.ptr;
+            fast = fast && v.stride_kb == 1 && v.stride_row % 16 == 0 && (reinterpret_cast<uintptr_t>(v.ptr) & 15) == 0 && (kb & 15) == 0;
+        }
+    }
+    __device__ __forceinline__ void issue(const GemmParams &p, const Tile &t, int k0, uint32_t raw, int lane) const
+    {
+        const int kb0 = k0 >> 5;   // both operands of an MXFP8 product have the same number of blocks
+        const int n = max(0, min(16, p.sfa.n_kb - (t.a_k0 >> 5) - kb0));
+#pragma unroll
+        for (int q = 0; q < 12; q++) {
+            const bool ok = (valid >> q & 1) && n > 0;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(raw + q * 512 + lane * 16), "l"(ok ? src[q] + kb0 : src[q]),
+                         "r"(ok ? n : 0) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+};
 
 // ---------------------------------------------------------------------------------------- kernel
 
-template <int KIND, int CTAS, int EPI>
+// WATCH: warp 2 looks at the ring's barriers for the MMA warp and the two meet at a named barrier per stage; otherwise the
+// MMA warp looks for itself, at the next stage's before it issues a stage.  launch_gemm() says which is used where.
+template <int KIND, int CTAS, int EPI, bool WATCH>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmD,
@@ -989,6 +1040,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     constexpr int kBStageBytes = Cfg<KIND, CTAS>::kBStageBytes;
     constexpr int kUnitStages = KIND == KIND_MXF4 ? kUnitStagesMxf4 : KIND == KIND_MXF8 ? kUnitStagesMxf8
                                 : KIND == KIND_MXF4R ? kUnitStagesMxf4R : kUnitStagesMxf4B16;   // stages whose scale images are built together
+    constexpr int kBufBytes = Cfg<KIND, CTAS>::kBufBytes;
+    constexpr int kUnitBlocks = Cfg<KIND, CTAS>::kUnitBlocks;
     constexpr int kKbShift = KIND == KIND_MXF4B16 ? 4 : 5;    // log2 of the scale vector's length (contraction elements per scale byte)
 
     extern __shared__ uint8_t smem_raw[];
@@ -996,8 +1049,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     uint8_t *smem_a = smem;
     uint8_t *smem_b = smem + kStages * kAStageBytes;
     uint8_t *smem_compact = smem + Cfg<KIND, CTAS>::kSmemOperands;   // 2D blocks: compact scale rows of the unit being built ...
-    uint8_t *smem_images = smem_compact + kCompactBytes;        // ... and the buffers of ready scale images (any kind)
-    uint8_t *smem_raw_scales = smem_images + Cfg<KIND, CTAS>::kImageBufs * kCacheBufBytes;   // per-row scales: bytes in flight
+    uint8_t *smem_images = smem_compact + (Cfg<KIND, CTAS>::kRowImages ? 0 : kCompactBytes);   // ... and the buffers of ready scale images (any kind)
+    uint8_t *smem_raw_scales = smem_images + Cfg<KIND, CTAS>::kImageBufs * kBufBytes;   // per-row scales: bytes in flight
     uint8_t *smem_staging = smem_compact + Cfg<KIND, CTAS>::kSmemScales;   // 1024-byte aligned (pair kernel only)
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem_staging + Cfg<KIND, CTAS>::kSmemStaging);
     // bars[0..5] full, bars[6..11] empty, bars[12] accumulator full, bars[13] accumulator empty,
@@ -1005,6 +1058,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     // bars[32..35] (leader of a pair) the second CTA's scale images full - one of each per image buffer
     uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(bars + 21);
     volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(bars + 21) + 1;
+    volatile uint32_t *acc_seen = reinterpret_cast<volatile uint32_t *>(bars + 22);   // the epilogue's verdict on its wait for the accumulator
     int32_t *goffs_smem = reinterpret_cast<int32_t *>(reinterpret_cast<uint8_t *>(bars) + kSmemTail);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1077,90 +1131,63 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        // A shared-memory access of this warp (the poll of the next "empty" barrier) queues behind the TMA
-        // instructions it has just issued and waits ~450 cycles, which would limit one warp to a stage per
-        // ~900 cycles.  So every round first polls - it waits for the next slot and then probes up to two
-        // more - and only then issues the loads of all slots found free, back to back.
-        constexpr int kBatch = 3;
-        StageIter pr;
-        pr.init(p, first_tile, tile_step, rank, kStageElems, goffs, true);
+        // One stage at a time: wait for its slot (the suspending form, by the whole warp: a wait in a lane-0 branch cost
+        // 2-4 % of a dense product, probing three slots per round as much again), then issue its loads.
+        const uint32_t lbar0 = CTAS == 1 ? bar_full : cluster_addr(bar_full, 0), a0 = smem_u32(smem_a), b0 = smem_u32(smem_b);
         uint32_t stage = 0, phase = 0;
         bool ok = true;
         const bool issuer = elect_one();
-        TRACE_DECL(c_empty); TRACE_DECL(c_issue); TRACE_DECL(c_rounds);
+        TRACE_DECL(c_empty); TRACE_DECL(c_issue);
         TRACE_T0(tt);
         int ev_j = 0;
-        while (Cfg<KIND, CTAS>::kSplitProducer && pr.valid(p)) {
-            asm volatile("bar.sync %0, 64;" ::"r"(8 + stage) : "memory");   // the poller (warp 2) has seen the slot free and armed its barrier
-            if (issuer && !(withhold_load != 0u && (uint32_t)ev_j + 1u == withhold_load)) {
-                const Tile &t = pr.t;
-                const int xa = (t.a_k0 + pr.it * kStageElems) / kElemsPerByte, xb = (t.b_k0 + pr.it * kStageElems) / kElemsPerByte;
-                tma_load_2d(smem_u32(smem_a + stage * kAStageBytes), &tmA, xa, t.a_row0, bar_full + 8 * stage);
-                tma_load_2d(smem_u32(smem_b + stage * kBStageBytes), &tmB, xb, t.b_load_row0, bar_full + 8 * stage);
-            }
-            ev_j++;
-            if (++stage == kStages) { stage = 0; phase ^= 1u; }
-            pr.next(p, kStageElems);
-        }
-        while (ok && pr.valid(p)) {
-            int n_free = 0;
-#ifdef FP4Q_TRACE
-            c_rounds++;
-#endif
-            if (lane == 0) {
-                ok = mbar_wait_impl<0, true>(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status, wait_limit, 0x100u + stage);
-                if (ok) {
-                    n_free = 1;
-                    uint32_t s2 = stage, ph2 = phase;
-                    while (n_free < kBatch) {
-                        if (++s2 == kStages) { s2 = 0; ph2 ^= 1u; }
-                        if (!mbar_test_wait(bar_empty + 8 * s2, ph2 ^ 1u)) break;
-                        n_free++;
-                    }
-                }
-            }
-            n_free = __shfl_sync(0xFFFFFFFFu, n_free, 0);
-            ok = n_free > 0;
-            TRACE_ADD(c_empty, tt);
-            for (int b = 0; b < n_free && pr.valid(p); b++) {
+        for (int tile = first_tile; ok && tile < p.n_tile_total; tile += tile_step) {
+            Tile t;
+            decode_tile(p, tile, rank, t, goffs);
+            const int n_it = (t.k_len + kStageElems - 1) / kStageElems;
+            int xa = t.a_k0 / kElemsPerByte, xb = t.b_k0 / kElemsPerByte;
+#pragma unroll 1
+            for (int it = 0; it < n_it; it++, xa += 128, xb += 128) {
+                ok = mbar_wait_impl<0>(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status, wait_limit, 0x100u + stage);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok) break;
+                TRACE_ADD(c_empty, tt);
                 if (lane == 0) TRACE_EV(0, ev_j);
                 if (issuer && !(withhold_load != 0u && (uint32_t)ev_j + 1u == withhold_load)) {
-                    const Tile &t = pr.t;
-                    const int xa = (t.a_k0 + pr.it * kStageElems) / kElemsPerByte, xb = (t.b_k0 + pr.it * kStageElems) / kElemsPerByte;
+                    const uint32_t lbar = lbar0 + 8 * stage;
                     if (CTAS == 1) {
-                        mbar_arrive_expect_tx(bar_full + 8 * stage, kAStageBytes + kBStageBytes);
-                        tma_load_2d(smem_u32(smem_a + stage * kAStageBytes), &tmA, xa, t.a_row0, bar_full + 8 * stage);
-                        tma_load_2d(smem_u32(smem_b + stage * kBStageBytes), &tmB, xb, t.b_load_row0, bar_full + 8 * stage);
+                        mbar_arrive_expect_tx(lbar, kAStageBytes + kBStageBytes);
+                        tma_load_2d(a0 + stage * kAStageBytes, &tmA, xa, t.a_row0, lbar);
+                        tma_load_2d(b0 + stage * kBStageBytes, &tmB, xb, t.b_load_row0, lbar);
                     } else {
                         // Both CTAs' bytes are counted on the leader's barrier, which the leader arms for all of them.
                         // (A remote mbarrier.arrive per stage by a thread of the second CTA costs ~1200 cycles each
                         // and cannot be pipelined; letting the TMA unit signal the remote barrier costs nothing.)
                         if (leader) mbar_arrive_expect_tx(bar_full + 8 * stage, 2 * (kAStageBytes + kBStageBytes));
-                        const uint32_t lbar = cluster_addr(bar_full + 8 * stage, 0);
-                        tma_load_2d_pair(smem_u32(smem_a + stage * kAStageBytes), &tmA, xa, t.a_row0, lbar);
-                        tma_load_2d_pair(smem_u32(smem_b + stage * kBStageBytes), &tmB, xb, t.b_load_row0, lbar);
+                        tma_load_2d_pair(a0 + stage * kAStageBytes, &tmA, xa, t.a_row0, lbar);
+                        tma_load_2d_pair(b0 + stage * kBStageBytes, &tmB, xb, t.b_load_row0, lbar);
                     }
                 }
                 if (lane == 0) TRACE_EV(1, ev_j);
                 ev_j++;
                 if (++stage == kStages) { stage = 0; phase ^= 1u; }
-                pr.next(p, kStageElems);
+                TRACE_ADD(c_issue, tt);
             }
-            TRACE_ADD(c_issue, tt);
         }
         if (!ok) {   // give copies already in flight time to land before the CTA's shared memory is released
             for (int i = 0; i < 200; i++) __nanosleep(1000);
         }
-        if (lane == 0) { TRACE_OUT(p, 0, c_empty); TRACE_OUT(p, 1, c_issue); TRACE_OUT(p, 5, c_rounds); }
+        if (lane == 0) { TRACE_OUT(p, 0, c_empty); TRACE_OUT(p, 1, c_issue); }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (the leader CTA of a pair)
         // The warp stays converged and one elected lane issues the tcgen05 instructions: their descriptors then live
-        // in uniform registers, and a scale copy costs about ten cycles of the issuing thread instead of fifty.  The
-        // warp never reads shared memory inside the loop: a shared-memory access of this warp queues behind its own
-        // pending MMAs and stalls the tensor pipe for ~200 cycles per poll.  A watcher warp polls the stage's "full"
-        // barrier (and, for 2D scales, the accumulator's "empty" barrier) and hands over through a named barrier.
+        // in uniform registers, and a scale copy costs about ten cycles of the issuing thread instead of fifty.
+        // A shared-memory access of this warp queues behind its own pending MMAs: a wait for the next stage right after a
+        // stage was issued stalls the tensor pipe for 200-300 cycles even when the stage is there.  So either a watcher warp
+        // looks at the barriers and hands over through a named barrier (WATCH), or this warp probes the next stage's
+        // barriers BEFORE it issues a stage and waits afterwards only if they were not complete.  All lanes wait: a
+        // lane-0 branch around the wait costs as much as the wait.
         uint32_t stage = 0, full_phase = 0, acc_empty_phase = 0;
-        bool mma_ok = true;   // split producer only: this warp's own waits have not run out
+        bool mma_ok = true, ready = false;   // !WATCH: this warp's waits have not run out; the next stage has been seen complete
         BufRing ring;   // image buffer of the current unit
         const bool issuer = elect_one();
         int ev_j = 0;
@@ -1173,18 +1200,30 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             if (n_it == 0) continue;
             TRACE_ADD(c_acc, tt);
             for (int it = 0; it < n_it; it++) {
-                if (Cfg<KIND, CTAS>::kSplitProducer) {
-                    // no watcher: the elected lane waits for the accumulator, the unit's scale images and the operands itself
-                    if (lane == 0 && mma_ok) {
-                        if (it == 0) mma_ok = mbar_wait_impl<0, true>(bar_acc_empty, acc_empty_phase ^ 1u, abort_flag, p.status, wait_limit, 0x200u);
-                        if (mma_ok && (it & (kUnitStages - 1)) == 0)
-                            mma_ok = mbar_wait_impl<0, true>(bar_cache_full + 8 * ring.buf, ring.phase, abort_flag, p.status, wait_limit, 0x510u + ring.buf);
-                        if (mma_ok) mma_ok = mbar_wait_impl<0, true>(bar_full + 8 * stage, full_phase, abort_flag, p.status, wait_limit, 0x300u + stage);
-                    }
-                    if (it == 0) acc_empty_phase ^= 1u;
-                    __syncwarp();
-                } else {
+                if (WATCH) {
                     named_sync(1 + stage);   // the watcher has seen the operands and both scale images of this stage
+                } else {
+                    if (it == 0) {
+                        if (mma_ok) mma_ok = mbar_wait_impl<0>(bar_acc_empty, acc_empty_phase ^ 1u, abort_flag, p.status, wait_limit, 0x200u);
+                        acc_empty_phase ^= 1u;
+                    }
+                    if (!ready) {
+                        if ((it & (kUnitStages - 1)) == 0) {
+                            if (mma_ok) mma_ok = mbar_wait_impl<0>(bar_cache_full + 8 * ring.buf, ring.phase, abort_flag, p.status, wait_limit, 0x510u + ring.buf);
+                            if (CTAS == 2 && mma_ok)
+                                mma_ok = mbar_wait_impl<0>(bar_peer_cache_full + 8 * ring.buf, ring.phase, abort_flag, p.status, wait_limit, 0x520u + ring.buf);
+                        }
+                        if (mma_ok) mma_ok = mbar_wait_impl<0>(bar_full + 8 * stage, full_phase, abort_flag, p.status, wait_limit, 0x300u + stage);
+                    }
+                    const uint32_t ns = stage + 1 == kStages ? 0u : stage + 1;
+                    ready = mbar_test_wait(bar_full + 8 * ns, ns == 0 ? full_phase ^ 1u : full_phase);
+                    if (it == n_it - 1 || ((it + 1) & (kUnitStages - 1)) == 0) {   // the next stage starts a unit
+                        BufRing nu = ring;
+                        nu.next(kImageBufs);
+                        ready = ready && mbar_test_wait(bar_cache_full + 8 * nu.buf, nu.phase);
+                        if (CTAS == 2) ready = ready && mbar_test_wait(bar_peer_cache_full + 8 * nu.buf, nu.phase);
+                    }
+                    __syncwarp();
                 }
                 tcgen05_fence_after();
                 TRACE_ADD(c_sync, tt);
@@ -1192,7 +1231,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 if (issuer) {
                     const uint32_t sf_tmem = tmem_base + kTmemSfBase + stage * SfCols<KIND>::kStride;
                     if (KIND == KIND_MXF4) {
-                        const uint32_t img = smem_u32(smem_images + ring.buf * kCacheBufBytes + (it & (kUnitStages - 1)) * kImageStageBytes);
+                        const uint32_t img = smem_u32(smem_images + ring.buf * kBufBytes + (it & (kUnitStages - 1)) * kImageStageBytes);
 #pragma unroll
                         for (int c = 0; c < 2; c++) {
                             tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 4 * c, smem_desc_scale_image_rep(img + 128 * c));
@@ -1200,7 +1239,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                             tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 12 + 8 * c, smem_desc_scale_image_rep(img + 384 + 256 * c));
                         }
                     } else if (KIND == KIND_MXF4B16) {
-                        const uint32_t img = smem_u32(smem_images + ring.buf * kCacheBufBytes + (it & (kUnitStages - 1)) * kImageStageBytesMxf4B16);
+                        const uint32_t img = smem_u32(smem_images + ring.buf * kBufBytes + (it & (kUnitStages - 1)) * kImageStageBytesMxf4B16);
 #pragma unroll
                         for (int i = 0; i < 4; i++) {
                             tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 4 * i, smem_desc_scale_image(img + 512 * i));
@@ -1208,7 +1247,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                             tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 20 + 8 * i, smem_desc_scale_image(img + 2560 + 1024 * i));
                         }
                     } else if (KIND == KIND_MXF4R) {
-                        const uint32_t img = smem_u32(smem_images + ring.buf * kCacheBufBytes + (it & (kUnitStages - 1)) * kImageStageBytesMxf4R);
+                        const uint32_t img = smem_u32(smem_images + ring.buf * kBufBytes + (it & (kUnitStages - 1)) * kImageStageBytesMxf4R);
 #pragma unroll
                         for (int c = 0; c < 2; c++) {
                             tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 4 * c, smem_desc_scale_image(img + 512 * c));
@@ -1216,7 +1255,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                             tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 12 + 8 * c, smem_desc_scale_image(img + 1536 + 1024 * c));
                         }
                     } else {
-                        const uint32_t img = smem_u32(smem_images + ring.buf * kCacheBufBytes + (it & (kUnitStages - 1)) * kImageStageBytesMxf8);
+                        const uint32_t img = smem_u32(smem_images + ring.buf * kBufBytes + (it & (kUnitStages - 1)) * kImageStageBytesMxf8);
                         tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem, smem_desc_scale_image(img));
                         tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 8, smem_desc_scale_image(img + 512));
                         tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 12, smem_desc_scale_image(img + 1024));
@@ -1252,9 +1291,21 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 if (++stage == kStages) { stage = 0; full_phase ^= 1u; }
             }
         }
+        if (KIND != KIND_MXF4 && CTAS == 2 && !leader) {
+            // Per-row scales, second CTA of a pair, whose MMA warp has nothing else to do: report each unit of scale images the
+            // builders have finished to the leader, which issues the scale copies of both CTAs.
+            bool fwd_ok = true;
+            BufRing fr;
+            UnitIter un;
+            for (un.init(p, first_tile, tile_step, rank, goffs); fwd_ok && un.valid(p); un.next(p, kUnitStages * kStageElems), fr.next(kImageBufs)) {
+                fwd_ok = __all_sync(0xFFFFFFFFu, mbar_wait_impl<0>(bar_cache_full + 8 * fr.buf, fr.phase, abort_flag, p.status, wait_limit, 0x530u + fr.buf));
+                if (fwd_ok && issuer) mbar_arrive_cluster_release(cluster_addr(bar_peer_cache_full + 8 * fr.buf, 0));
+            }
+            __syncwarp();
+        }
         if (leader && *abort_flag) {
-            // Some role gave up: the watchers then release every remaining stage unseen, and this warp has run
-            // through them.  Wait (bounded) until the tensor pipe is idle before tensor memory is freed.
+            // Some role gave up: the watcher then releases every remaining stage unseen (or this warp has stopped waiting), and
+            // this warp has run through them.  Wait (bounded) until the tensor pipe is idle before tensor memory is freed.
             if (issuer) tcgen05_commit<CTAS>(bar_drain);
             __syncwarp();
             if (lane == 0) mbar_wait_lazy(bar_drain, 0u, abort_flag, p.status, wait_limit, 0x220u);   // gives up after 256 polls (abort is set)
@@ -1264,7 +1315,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             for (int i = 0; i < 200; i++) __nanosleep(1000);
         }
         if (lane == 0) { TRACE_OUT(p, 2, c_acc); TRACE_OUT(p, 3, c_sync); TRACE_OUT(p, 4, c_issue); }
-    } else if (warp == 3) {
+    } else if (warp == 3 || (warp == 2 && Cfg<KIND, CTAS>::kBuilders == 2)) {
         // ------------------------------------------------------------------ scale image builder
         // 2D-block scales: per unit (up to 16 stages of one tile) gathers the compact scale bytes from global memory
         // into 16-byte rows and replicates each row into its image; per-row scales: loads the unit's scale words and
@@ -1276,49 +1327,64 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         BufRing ring;
         bool ok = true;
         if (KIND != KIND_MXF4) {
-            // per-row scales: the raw bytes of the next kRawBufs units are in flight (cp.async) while a unit is
-            // turned into images.  In a pair an image buffer is released by the leader's multicast commit: probe
-            // (a suspended try_wait is not reliably woken early by a remote arrival).
-            constexpr int kRawBufs = Cfg<KIND, CTAS>::kRawBufs > 0 ? Cfg<KIND, CTAS>::kRawBufs : 1;
+            // per-row scales: the raw bytes of the next kOwnRaw units are in flight (cp.async) while a unit is turned into
+            // images.  Two builders take every other unit and have raw buffers of their own.
+            constexpr int kBuilders = Cfg<KIND, CTAS>::kBuilders, kRawBytes = Cfg<KIND, CTAS>::kRawBytes, kSlotB = Cfg<KIND, CTAS>::kRawSlotB;
+            constexpr int kOwnRaw = Cfg<KIND, CTAS>::kRawBufs > 0 ? Cfg<KIND, CTAS>::kRawBufs / kBuilders : 1;
+            uint8_t *raw = smem_raw_scales + (3 - warp) * kOwnRaw * kRawBytes;
             UnitIter ahead, cur;
             ahead.init(p, first_tile, tile_step, rank, goffs);
             cur.init(p, first_tile, tile_step, rank, goffs);
-            uint32_t raw_fill = 0, raw_read = 0;
-            for (int i = 0; i < kRawBufs; i++) {
-                if (ahead.valid(p)) {
-                    issue_raw_scales<kKbShift>(p, ahead.t, ahead.k0, smem_raw_scales + raw_fill * kCacheBufBytes, lane);
-                    ahead.next(p, kUnitStages * kStageElems);
-                } else {
-                    asm volatile("cp.async.commit_group;" ::: "memory");
-                }
-                if (++raw_fill == kRawBufs) raw_fill = 0;
+            if (warp == 2) {   // the second builder starts with the second unit
+                if (ahead.valid(p)) ahead.next(p, kUnitStages * kStageElems);
+                if (cur.valid(p)) cur.next(p, kUnitStages * kStageElems);
+                ring.next(kImageBufs);
             }
+            RowFetch rows;
+            int rows_tile = -1;
+            uint32_t raw_buf = 0;
+            auto fetch = [&](uint32_t buf) {   // the unit `ahead` points at, into raw buffer buf; one cp.async group in any case
+                if (!ahead.valid(p)) {
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                    return;
+                }
+                if constexpr (KIND == KIND_MXF8) {
+                    if (ahead.tile != rows_tile) {
+                        rows.set(p, ahead.t, lane);
+                        rows_tile = ahead.tile;
+                    }
+                    if (rows.fast) rows.issue(p, ahead.t, ahead.k0, smem_u32(raw + buf * kRawBytes), lane);
+                    else issue_raw_scales<kKbShift, kUnitBlocks, kSlotB>(p, ahead.t, ahead.k0, raw + buf * kRawBytes, lane);
+                } else {
+                    issue_raw_scales<kKbShift, kUnitBlocks, kSlotB>(p, ahead.t, ahead.k0, raw + buf * kRawBytes, lane);
+                }
+#pragma unroll
+                for (int i = 0; i < kBuilders; i++)
+                    if (ahead.valid(p)) ahead.next(p, kUnitStages * kStageElems);
+            };
+            for (int i = 0; i < kOwnRaw; i++) fetch(i);
             while (cur.valid(p)) {
-                asm volatile("cp.async.wait_group %0;" ::"n"(kRawBufs - 1) : "memory");   // this unit's bytes have landed
+                asm volatile("cp.async.wait_group %0;" ::"n"(kOwnRaw - 1) : "memory");   // this unit's bytes have landed
                 __syncwarp();
-                uint32_t w[12][8];
-                read_raw_scales(p, smem_raw_scales + raw_read * kCacheBufBytes, lane, w);
-                if (lane == 0)
-                    ok = mbar_wait_impl<kRelaxedNs, CTAS == 2>(bar_cache_empty + 8 * ring.buf, ring.phase ^ 1u, abort_flag, p.status, wait_limit, 0x500u + ring.buf);
-                ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+                uint32_t w[12][kUnitBlocks / 4];
+                read_raw_scales<kUnitBlocks, kSlotB>(p, raw + raw_buf * kRawBytes, lane, w);
+                ok = mbar_wait_impl<0>(bar_cache_empty + 8 * ring.buf, ring.phase ^ 1u, abort_flag, p.status, wait_limit, 0x500u + ring.buf);
+                ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 store_row_scale_images<KIND>(w, min(kUnitStages, (cur.t.k_len - cur.k0 + kStageElems - 1) / kStageElems),
-                                             smem_images + ring.buf * kCacheBufBytes, lane);
+                                             smem_images + ring.buf * kBufBytes, lane);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tcgen05.cp
                 __syncwarp();
-                // In the second CTA of a pair the arrival is forwarded to the leader by warp 2: the remote arrival
+                // In the second CTA of a pair the arrival is forwarded to the leader by warp 1: the remote arrival
                 // stalls its issuing thread for about a thousand cycles, which this warp spends on the next unit.
                 if (lane == 0) mbar_arrive(bar_cache_full + 8 * ring.buf);
-                ring.next(kImageBufs);
-                cur.next(p, kUnitStages * kStageElems);
-                // the raw buffer just read is free: fetch the unit kRawBufs ahead into it
-                if (ahead.valid(p)) {
-                    issue_raw_scales<kKbShift>(p, ahead.t, ahead.k0, smem_raw_scales + raw_read * kCacheBufBytes, lane);
-                    ahead.next(p, kUnitStages * kStageElems);
-                } else {
-                    asm volatile("cp.async.commit_group;" ::: "memory");
+                fetch(raw_buf);   // the raw buffer just read is free
+                if (++raw_buf == kOwnRaw) raw_buf = 0;
+#pragma unroll
+                for (int i = 0; i < kBuilders; i++) {
+                    ring.next(kImageBufs);
+                    if (cur.valid(p)) cur.next(p, kUnitStages * kStageElems);
                 }
-                if (++raw_read == kRawBufs) raw_read = 0;
             }
             asm volatile("cp.async.wait_all;" ::: "memory");
         }
@@ -1327,7 +1393,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             decode_tile(p, tile, rank, t, goffs);
             for (int k0 = 0; ok && k0 < t.k_len; k0 += kUnitStages * kStageElems, ring.next(kImageBufs)) {
                 const int buf = ring.buf;
-                uint8_t *images = smem_images + buf * kCacheBufBytes;
+                uint8_t *images = smem_images + buf * kBufBytes;
                 {
                     const int n_chunks = min(kCacheChunks, (((t.k_len - k0 + 127) >> 7) + 1) & ~1);   // whole stages; pad rows beyond the tensor
                     uint32_t *compact = reinterpret_cast<uint32_t *>(smem_compact);
@@ -1379,28 +1445,14 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         TRACE_DECL(c_meet); TRACE_DECL(c_poll);
         TRACE_T0(tt);
         int ev_j = 0;
-        bool unit_seen = false;   // lane 0: the next unit's scale images have been seen complete
+        bool unit_seen = false;   // the next unit's scale images have been seen complete
         uint32_t ahead = 0;   // stages after the current one whose "full" barrier is already known to be complete
-        if (Cfg<KIND, CTAS>::kSplitProducer) {
-            // poller half of the split producer: waits for each slot to be free, arms its barrier for the stage's bytes and
-            // releases the issuing warp; after a timeout it keeps releasing, so that warp 0 always reaches its end
-            while (sg.valid(p)) {
-                if (lane == 0) {
-                    if (ok) ok = mbar_wait_impl<0, true>(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status, wait_limit, 0x100u + stage);
-                    mbar_arrive_expect_tx(bar_full + 8 * stage, kAStageBytes + kBStageBytes);
-                }
-                __syncwarp();
-                asm volatile("bar.sync %0, 64;" ::"r"(8 + stage) : "memory");
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
-                sg.next(p, kStageElems);
-            }
-        }
-        while (!Cfg<KIND, CTAS>::kSplitProducer && leader && sg.valid(p)) {
+        while (WATCH && leader && sg.valid(p)) {
             if (lane == 0) TRACE_EV(4, ev_j);
             if (ahead > 0) {
                 ahead--;
             } else {
-                if (ok && lane == 0) {
+                if (ok) {   // all lanes probe (a lane-0 branch and the broadcast of its result slowed the hand-over by 2-4 %)
                     if ((sg.it & (kUnitStages - 1)) == 0 && !unit_seen) {
                         // both CTAs' images of this unit: the two barriers probed together (the latencies overlap)
                         const uint32_t b0 = bar_cache_full + 8 * ring.buf, b1 = (CTAS == 2 ? bar_peer_cache_full : bar_cache_full) + 8 * ring.buf;
@@ -1485,9 +1537,9 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                         if (r4 && r5) unit_seen = true;
                     }
                 }
-                ahead = __shfl_sync(0xFFFFFFFFu, ahead, 0);
+                ahead = __reduce_min_sync(0xFFFFFFFFu, ahead);   // what every lane has seen
             }
-            ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+            ok = __all_sync(0xFFFFFFFFu, ok);
             TRACE_ADD(c_poll, tt);
             if (lane == 0) TRACE_EV(6, ev_j);
             ev_j++;
@@ -1497,17 +1549,6 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             if ((sg.it & (kUnitStages - 1)) == kUnitStages - 1 || sg.it == sg.n_it - 1) ring.next(kImageBufs);
             if (++stage == kStages) { stage = 0; phase ^= 1u; }
             sg.next(p, kStageElems);
-        }
-        if (KIND != KIND_MXF4 && CTAS == 2 && !leader && lane == 0) {
-            // Per-row scales, second CTA of a pair: report each unit of scale images the builder has finished to the
-            // leader, which issues the scale copies of both CTAs.
-            bool fwd_ok = true;
-            BufRing fr;
-            UnitIter un;
-            for (un.init(p, first_tile, tile_step, rank, goffs); fwd_ok && un.valid(p); un.next(p, kUnitStages * kStageElems), fr.next(kImageBufs)) {
-                fwd_ok = mbar_wait_impl<kRelaxedNs>(bar_cache_full + 8 * fr.buf, fr.phase, abort_flag, p.status, wait_limit, 0x530u + fr.buf);
-                if (fwd_ok) mbar_arrive_cluster_release(cluster_addr(bar_peer_cache_full + 8 * fr.buf, 0));
-            }
         }
         __syncwarp();
         if (lane == 0) { TRACE_OUT(p, 6, c_meet); TRACE_OUT(p, 7, c_poll); }
@@ -1531,10 +1572,15 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 // this wait spans a whole tile (every other one spans a few stages at most): its limit grows with the
                 // tile's contraction length, so that a very long contraction cannot run into it on a healthy run
                 const uint64_t tile_limit = wait_limit * (uint64_t)(1 + (t.k_len >> 12));
-                if (lane == 0)
-                    ok = CTAS == 2 ? mbar_poll(bar_acc_full, acc_phase, abort_flag, p.status, tile_limit, 0x400u + warp)
-                                   : mbar_wait_relaxed(bar_acc_full, acc_phase, abort_flag, p.status, tile_limit, 0x400u + warp);
-                ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+                // One thread waits and the warps meet at a named barrier: eight lanes polling the barrier kept the shared-memory
+                // unit busy enough to slow every other role's waits (a probe took 475 cycles), 2-3 % of a dense product.
+                if (warp == 4 && lane == 0) {
+                    ok = mbar_wait(bar_acc_full, acc_phase, abort_flag, p.status, tile_limit, 0x404u);
+                    acc_seen[acc_phase] = ok ? 1u : 0u;   // one word per phase: a warp is at most one tile behind
+                }
+                __syncwarp();
+                asm volatile("bar.sync 15, 256;" ::: "memory");
+                ok = acc_seen[acc_phase] != 0u;
                 TRACE_ADD(c_wait, tt);
                 if (lane == 0) TRACE_EV(7, 16 * ev_t + 2 * (warp - 4));
                 if (!ok) break;
@@ -1782,7 +1828,7 @@ static int sm_count(int dev)
     return n[dev];
 }
 
-template <int KIND, int CTAS, int EPI = EPI_STORE>
+template <int KIND, int CTAS, int EPI, bool WATCH>
 static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmParams &p, void *stream)
 {
     CUtensorMap tmA, tmB, tmC;
@@ -1808,7 +1854,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     if (dev < 0) return FP4Q_ERR_CUDA;
     static bool attr_set[kMaxDevices];   // the attribute is a property of (kernel, device): one flag per device and instantiation
     if (!attr_set[dev]) {
-        if (cudaFuncSetAttribute(gemm_block_scaled_kernel<KIND, CTAS, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  Cfg<KIND, CTAS>::kSmemBytes) != cudaSuccess)
             return FP4Q_ERR_CUDA;
         attr_set[dev] = true;
@@ -1830,7 +1876,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = CTAS == 2 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, gemm_block_scaled_kernel<KIND, CTAS, EPI>, tmA, tmB, tmC, tmD, p) == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH>, tmA, tmB, tmC, tmD, p) == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
 }
 
 // Argument checks common to every product: everything that can be refused is refused here, before any work is enqueued.
@@ -1861,8 +1907,17 @@ static fp4q_status launch_gemm(const Operand &A, const Operand &B, GemmParams &p
     // caller states that every token group starts on a multiple of 256 rows.
     static const bool use_pairs = [] { const char *e = getenv("FP4Q_CTA_PAIRS"); return !(e && e[0] == '0'); }();
     const bool pair_mode = p.mode == MODE_DENSE || p.mode == MODE_GROUPED_K || (p.mode == MODE_GROUPED_ROWS && p.rows_pair_aligned);
-    if (use_pairs && pair_mode && p.M > BM) return launch_gemm_impl<KIND, 2>(A, B, p, stream);
-    return launch_gemm_impl<KIND, 1>(A, B, p, stream);
+    // The watcher pays in the dense FP4 and MXFP8 products on pairs (16384 x 4096 x 4096, with and without: FP4 weight gradient
+    // 98.4 and 102.7 us, forward 100.7 both; MXFP8 forward 213 and 218 us, weight gradient 228 and 236 us).  Everything else is
+    // faster without it: the short contractions of grouped products (expert weight gradients 222 and 225 us without, 228
+    // and 230 us with), the quantizing epilogue, whose warps it competes with (113 and 116 us), and the per-row FP4
+    // kinds, where its warp builds scale images instead.
+    constexpr bool kWatchDense = KIND == KIND_MXF4 || KIND == KIND_MXF8;
+    if (use_pairs && pair_mode && p.M > BM) {
+        if (kWatchDense && p.mode == MODE_DENSE) return launch_gemm_impl<KIND, 2, EPI_STORE, kWatchDense>(A, B, p, stream);
+        return launch_gemm_impl<KIND, 2, EPI_STORE, KIND == KIND_MXF8>(A, B, p, stream);
+    }
+    return launch_gemm_impl<KIND, 1, EPI_STORE, false>(A, B, p, stream);
 }
 
 static bool tensor_ok(const fp4q_tensor *t) { return t && t->rows >= 0 && t->cols >= 0; }
@@ -1987,7 +2042,7 @@ static fp4q_status launch_gemm_quantized(const Operand &A, const Operand &B, int
         p.rows_pair_aligned = 1;
         p.b_rows_per_group = b_rows_per_group; p.b_k_per_group = b_k_per_group;
     }
-    return launch_gemm_impl<KIND_MXF4, 2, EPI_QUANT>(A, B, p, stream);
+    return launch_gemm_impl<KIND_MXF4, 2, EPI_QUANT, false>(A, B, p, stream);
 }
 
 extern "C" fp4q_status fp4q_gemm_fwd_quantized(const fp4q_tensor *X, const fp4q_tensor *W, const fp4q_tensor *Yq, fp4q_round mode,
