@@ -40,6 +40,7 @@ constexpr int BM = 128, BN = 256;            // per-CTA accumulator: 128 rows x 
 constexpr int kMaxStages = 6;
 constexpr int kAStageBytes = BM * 128;
 constexpr int kMaxGroupsShared = 1023;       // grouped contraction: boundaries kept in shared memory up to this many groups
+constexpr int kMaxGroupsSorted = 256;        // grouped contraction: groups are taken longest first up to this many
 constexpr int kMaxRowTilesShared = 2048;     // grouped rows: group of each 128-row tile kept in shared memory up to this many tiles
 constexpr int kSmemTail = 512;               // barriers, TMEM base, abort flag, scale scratch (one per loader warp)
 // 2D-block scales: the scale images of a whole unit (up to 16 stages = 4096 contraction elements of one tile) are
@@ -115,12 +116,15 @@ struct Cfg {
     static constexpr int kSmemOperands = kStages * (kAStageBytes + kBStageBytes);
     static constexpr int kSmemScales = (kSmemCache + 1023) / 1024 * 1024;
     static constexpr int kSmemStaging = kTmaStores ? 8 * kStagingWarpBytes : 0;
-    static constexpr int kSmemGroups = (CTAS == 1 || KIND == KIND_MXF4) ? (kMaxGroupsShared + 1) * 4 : 0;   // grouped products: group table
-    static_assert(kSmemGroups == 0 || kSmemGroups >= kMaxRowTilesShared * 2, "group table");
+    static constexpr int kSmemGroups = (CTAS == 1 || KIND == KIND_MXF4) ? (kMaxGroupsShared + 1) * 4 + kMaxGroupsSorted * 2 : 0;   // grouped products: group tables
+    static_assert(kSmemGroups == 0 || (kMaxGroupsShared + 1) * 4 >= kMaxRowTilesShared * 2, "group table");
     static constexpr int kSmemBytes = 1024 + kSmemOperands + kSmemScales + kSmemStaging + kSmemTail + kSmemGroups;
     static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 };
-constexpr int kRasterM = 16;                 // dense products: row tiles per rasterisation group
+// Dense products and grouped rows: row tiles per rasterisation group.  With grouped rows a group's A rows and the weights of the
+// few experts they belong to stay in L2 for the whole sweep over the columns (expert layer, 139520 rows, one group of all
+// row tiles -> groups of 16: 768 x 2048 fwd/dgrad 148/207 -> 132/170 us, 2048 x 768 201/149 -> 164/134 us; 8 and 32 within 2 %).
+constexpr int kRasterM = 16;
 constexpr int kThreads = 384;
 constexpr int kTmemCols = 512;
 constexpr int kTmemSfBase = 256;
@@ -451,11 +455,11 @@ __device__ __forceinline__ int find_group(const int64_t *offs, const int32_t *go
 // producer and the scale builder need - the MMA issuer, the watcher and the epilogue use the contraction length and
 // the output position alone, and a lookup in the MMA warp (shared-memory reads behind its pending MMAs) costs
 // about 1900 cycles per tile.
-__device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int rank, Tile &t, const int32_t *goffs, bool need_b = true)
+__device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int rank, Tile &t, const int32_t *goffs, const uint16_t *gorder, bool need_b = true)
 {
     const int per_problem = p.m_tiles * p.n_tiles;
-    const int g = p.mode == MODE_GROUPED_K ? tile / per_problem : 0;
-    const int local = tile - g * per_problem;
+    const int nth = p.mode == MODE_GROUPED_K ? tile / per_problem : 0, g = p.mode == MODE_GROUPED_K && gorder ? (int)gorder[nth] : nth;
+    const int local = tile - nth * per_problem;
     // Tiles that run at the same time (consecutive indices) cover raster_m row tiles x a few column tiles, and
     // the sweep over column tiles finishes before the next group of row tiles starts: the group's A rows stay
     // in L2 for the whole sweep instead of the whole A operand being streamed once per wave.
@@ -506,12 +510,13 @@ __device__ __forceinline__ void load_scale(const ScaleView &v, int row, int kb, 
 struct StageIter {
     int tile, step, rank, it, n_it;
     const int32_t *goffs;
+    const uint16_t *gorder;
     bool need_b;
     Tile t;
     __device__ __forceinline__ void seek(const GemmParams &p, int stage_elems)
     {
         while (tile < p.n_tile_total) {
-            decode_tile(p, tile, rank, t, goffs, need_b);
+            decode_tile(p, tile, rank, t, goffs, gorder, need_b);
             n_it = (t.k_len + stage_elems - 1) / stage_elems;
             if (n_it > 0) { it = 0; return; }
             tile += step;
@@ -519,9 +524,9 @@ struct StageIter {
         n_it = 0;
     }
     __device__ __forceinline__ void init(const GemmParams &p, int first, int step_, int rank_, int stage_elems, const int32_t *goffs_,
-                                         bool need_b_)
+                                         const uint16_t *gorder_, bool need_b_)
     {
-        tile = first; step = step_; rank = rank_; it = 0; goffs = goffs_; need_b = need_b_;
+        tile = first; step = step_; rank = rank_; it = 0; goffs = goffs_; gorder = gorder_; need_b = need_b_;
         seek(p, stage_elems);
     }
     __device__ __forceinline__ bool valid(const GemmParams &p) const { return tile < p.n_tile_total; }
@@ -817,19 +822,20 @@ struct BufRing {
 struct UnitIter {
     int tile, step, rank, k0;
     const int32_t *goffs;
+    const uint16_t *gorder;
     Tile t;
     __device__ __forceinline__ void seek(const GemmParams &p)
     {
         while (tile < p.n_tile_total) {
-            decode_tile(p, tile, rank, t, goffs);
+            decode_tile(p, tile, rank, t, goffs, gorder);
             if (k0 < t.k_len) return;
             tile += step;
             k0 = 0;
         }
     }
-    __device__ __forceinline__ void init(const GemmParams &p, int first, int step_, int rank_, const int32_t *goffs_)
+    __device__ __forceinline__ void init(const GemmParams &p, int first, int step_, int rank_, const int32_t *goffs_, const uint16_t *gorder_)
     {
-        tile = first; step = step_; rank = rank_; k0 = 0; goffs = goffs_;
+        tile = first; step = step_; rank = rank_; k0 = 0; goffs = goffs_; gorder = gorder_;
         seek(p);
     }
     __device__ __forceinline__ bool valid(const GemmParams &p) const { return tile < p.n_tile_total; }
@@ -1122,6 +1128,24 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         for (int i = threadIdx.x; i < n_row_tiles; i += kThreads)
             reinterpret_cast<uint16_t *>(goffs_smem)[i] = (uint16_t)find_group(p.row_offsets, nullptr, p.n_groups, (int64_t)i * BM);
     const int32_t *goffs = goffs_ok ? goffs_smem : nullptr;
+    // Grouped contraction: the groups longest first.  Their tiles go round the CTAs in turn, so that in any other order a CTA
+    // that meets several of the long ones finishes last (expert layer, 128 groups of
+    // 256 .. 15616 tokens in four random orders: 235-262 -> 222-226 us).
+    uint16_t *gorder = nullptr;
+    if (goffs_ok && p.mode == MODE_GROUPED_K && p.n_groups <= kMaxGroupsSorted) {
+        gorder = reinterpret_cast<uint16_t *>(goffs_smem + kMaxGroupsShared + 1);
+        __syncthreads();
+        for (int g = threadIdx.x; g < p.n_groups; g += kThreads) {
+            const int len = goffs_smem[g + 1] - goffs_smem[g];
+            int before = 0;
+#pragma unroll 4
+            for (int h = 0; h < p.n_groups; h++) {
+                const int other = goffs_smem[h + 1] - goffs_smem[h];
+                before += other > len || (other == len && h < g);
+            }
+            gorder[before] = (uint16_t)g;
+        }
+    }
     tcgen05_fence_before();
     __syncwarp();
     if (CTAS == 2) cluster_sync_all();   // the peer's barriers must exist before anything is signalled across CTAs
@@ -1142,7 +1166,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         int ev_j = 0;
         for (int tile = first_tile; ok && tile < p.n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile(p, tile, rank, t, goffs);
+            decode_tile(p, tile, rank, t, goffs, gorder);
             const int n_it = (t.k_len + kStageElems - 1) / kStageElems;
             int xa = t.a_k0 / kElemsPerByte, xb = t.b_k0 / kElemsPerByte;
 #pragma unroll 1
@@ -1195,7 +1219,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         TRACE_T0(tt);
         for (int tile = first_tile; leader && tile < p.n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile(p, tile, rank, t, goffs, false);
+            decode_tile(p, tile, rank, t, goffs, gorder, false);
             const int n_it = (t.k_len + kStageElems - 1) / kStageElems;
             if (n_it == 0) continue;
             TRACE_ADD(c_acc, tt);
@@ -1297,7 +1321,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             bool fwd_ok = true;
             BufRing fr;
             UnitIter un;
-            for (un.init(p, first_tile, tile_step, rank, goffs); fwd_ok && un.valid(p); un.next(p, kUnitStages * kStageElems), fr.next(kImageBufs)) {
+            for (un.init(p, first_tile, tile_step, rank, goffs, gorder); fwd_ok && un.valid(p); un.next(p, kUnitStages * kStageElems), fr.next(kImageBufs)) {
                 fwd_ok = __all_sync(0xFFFFFFFFu, mbar_wait_impl<0>(bar_cache_full + 8 * fr.buf, fr.phase, abort_flag, p.status, wait_limit, 0x530u + fr.buf));
                 if (fwd_ok && issuer) mbar_arrive_cluster_release(cluster_addr(bar_peer_cache_full + 8 * fr.buf, 0));
             }
@@ -1333,8 +1357,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             constexpr int kOwnRaw = Cfg<KIND, CTAS>::kRawBufs > 0 ? Cfg<KIND, CTAS>::kRawBufs / kBuilders : 1;
             uint8_t *raw = smem_raw_scales + (3 - warp) * kOwnRaw * kRawBytes;
             UnitIter ahead, cur;
-            ahead.init(p, first_tile, tile_step, rank, goffs);
-            cur.init(p, first_tile, tile_step, rank, goffs);
+            ahead.init(p, first_tile, tile_step, rank, goffs, gorder);
+            cur.init(p, first_tile, tile_step, rank, goffs, gorder);
             if (warp == 2) {   // the second builder starts with the second unit
                 if (ahead.valid(p)) ahead.next(p, kUnitStages * kStageElems);
                 if (cur.valid(p)) cur.next(p, kUnitStages * kStageElems);
@@ -1390,7 +1414,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         }
         for (int tile = first_tile; KIND == KIND_MXF4 && ok && tile < p.n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile(p, tile, rank, t, goffs);
+            decode_tile(p, tile, rank, t, goffs, gorder);
             for (int k0 = 0; ok && k0 < t.k_len; k0 += kUnitStages * kStageElems, ring.next(kImageBufs)) {
                 const int buf = ring.buf;
                 uint8_t *images = smem_images + buf * kBufBytes;
@@ -1438,7 +1462,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         // stage is released unseen, so that the MMA warp, which cannot time out on a named barrier, always runs
         // to its end.
         StageIter sg;
-        sg.init(p, first_tile, tile_step, rank, kStageElems, goffs, false);
+        sg.init(p, first_tile, tile_step, rank, kStageElems, goffs, gorder, false);
         uint32_t stage = 0, phase = 0, acc_phase = 0;
         BufRing ring;   // image buffer of the current unit
         bool ok = true;
@@ -1563,7 +1587,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         TRACE_T0(tt);
         for (int tile = first_tile; ok && tile < p.n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile(p, tile, rank, t, goffs, false);
+            decode_tile(p, tile, rank, t, goffs, gorder, false);
             const int row_in_tile = 32 * quarter + lane;
             const int64_t row = (int64_t)t.c_row0 + row_in_tile;
             const bool row_ok = row_in_tile < t.m_valid;
@@ -1845,7 +1869,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     p.ctas = CTAS;
     p.m_tiles = (int32_t)ceil_div(p.M, BM * CTAS);
     p.n_tile_total = p.m_tiles * p.n_tiles * (p.mode == MODE_GROUPED_K ? p.n_groups : 1);
-    p.raster_m = p.mode == MODE_DENSE ? (p.m_tiles < kRasterM ? p.m_tiles : kRasterM) : p.m_tiles;
+    p.raster_m = p.mode != MODE_GROUPED_K ? (p.m_tiles < kRasterM ? p.m_tiles : kRasterM) : p.m_tiles;
 #ifdef FP4Q_TRACE
     if (const char *g = getenv("FP4Q_DEBUG_RASTER")) { p.raster_m = atoi(g); if (p.raster_m > p.m_tiles) p.raster_m = p.m_tiles; }
 #endif

@@ -136,3 +136,24 @@ def test_block_sizes_must_match_the_product():
         binding.fp4q_gemm_fwd_b16(binding.fp4q_quantize2d(x), X)      # and the 16-block products a 32-block one
     with pytest.raises(binding.Fp4qError):
         binding.fp4q_quantize2d(x, flags=binding.BLOCK_16 | binding.BLOCK_64)
+
+
+@pytest.mark.parametrize("T,N,K", [(4864, 4096, 1280), (1280, 4096, 4864)])
+def test_two_builders_of_16x16_scales_over_several_tiles(T, N, K):
+    # several pair tiles per pair, tiles of an odd number of scale units (5 stages: units of 2 + 2 + 1)
+    x = workloads.activations_gauss_outliers(T, K, seed=31, device="cuda")
+    w = workloads.weights(N, K, seed=32, device="cuda")
+    qx, qw = (binding.fp4q_quantize2d(t, flags=binding.BLOCK_16) for t in (x, w))
+    y = binding.fp4q_gemm_fwd_b16(qx, qw, dt=binding.OUT_F32)
+    dw = binding.fp4q_gemm_wgrad_b16(qx, qx, dt=binding.OUT_F32)          # X^T X: both operands transposed views
+    torch.cuda.synchronize()
+
+    def dequantized(q):
+        cols = (q.cols + 1) // 2
+        d = oracle.dequantize2d_block(np.ascontiguousarray(q.q_rm.cpu().numpy()[:, :cols]), q.scale.cpu().numpy(), 16, q.rows, q.cols)
+        return torch.from_numpy(d).cuda()
+
+    xd, wd = dequantized(qx), dequantized(qw)
+    for got, ref in ((y, xd @ wd.T), (dw, xd.T @ xd)):
+        err = (got.double() - ref).norm() / ref.norm()
+        assert float(err) <= 1e-6, float(err)      # FP32 accumulation of exact products: 2^-24 per addition at the worst

@@ -342,3 +342,26 @@ def test_seeded_random_grouped_cases(ws):
         H = int(rng.choice([64, 256, 320, 1024]))
         F = int(rng.choice([64, 128, 192, 448]))
         _moe_case(ws, E=E, H=H, F=F, counts=counts, seed=200 + n, pad=128 if n & 1 else 256)
+
+
+@pytest.mark.parametrize("E", [5, 256, 257])
+def test_grouped_weight_gradient_with_groups_in_any_order_of_length(ws, E):
+    # up to 256 groups are taken longest first, more in the given order: lengths that rise, fall, repeat and vanish
+    rng = np.random.default_rng(E)
+    counts = rng.permutation(np.resize([0, 1, 128, 128, 300, 700, 129, 640], E))
+    _moe_case(ws, E=E, H=96, F=64, counts=counts, seed=E)
+
+
+@pytest.mark.parametrize("T,N,K", [(300, 520, 2560),     # scale rows on 16-byte boundaries, five units of 512, rows past the end
+                                   (640, 264, 1056),     # 33 blocks a row: the general fetch; the last unit is one block
+                                   (257, 300, 544),      # 17 blocks
+                                   (4864, 4096, 1280)])  # several tiles per CTA, a short last unit in each
+def test_mxfp8_scale_units(ws, T, N, K):
+    g = torch.Generator(device="cuda").manual_seed(T + K)
+    x = (torch.randn(T, K, generator=g, device="cuda") * torch.exp(2 * torch.randn(T, 1, generator=g, device="cuda"))).to(torch.bfloat16)
+    w = (torch.randn(N, K, generator=g, device="cuda") * 0.02).to(torch.bfloat16)
+    (xq, xs, xd), (wq, wsc, wd) = _mxfp8_operand(x), _mxfp8_operand(w)
+    y = binding.fp4q_mxfp8_gemm(xq, xs, wq, wsc, T, N, K, dt=binding.OUT_F32, ws=ws)
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
+    check(y, (torch.from_numpy(xd).cuda() @ torch.from_numpy(wd).cuda().T).cpu().numpy(), "MXFP8 product")

@@ -149,3 +149,23 @@ def test_seeded_random_shapes_with_1d_activations():
         assert binding.fp4q_workspace_status(ws) == 0
         check(y, oracle.gemm_fwd(x_hat, dequant_from_gpu(W)), "forward, 1D activations, shape %d" % n)
         check(dw, oracle.gemm_wgrad(dequant_from_gpu(dY), x_hat_t), "wgrad, 1D activations, shape %d" % n)
+
+
+@pytest.mark.parametrize("T,N,K", [(4864, 4096, 1280), (1280, 4864, 4096)])
+def test_two_builders_over_several_tiles(T, N, K):
+    # 304 pair tiles, four or five per pair, with an odd number of scale units in a tile (5 stages: units of 4 + 1), so that the
+    # builders' turns shift from tile to tile; forward (1D activations x 2D weights) and weight gradient
+    x = workloads.activations_gauss_outliers(T, K, seed=21, device="cuda")
+    w = workloads.weights(N, K, seed=22, device="cuda")
+    xq, xs, x_hat = act1d(x)
+    W = assert_matches_oracle(w, binding.ROUND_NEAREST)
+    y = binding.fp4q_gemm_fwd_act1d(xq, xs, T, W, dt=binding.OUT_F32)
+    dy = workloads.gradients_rowscaled(K, N, seed=23, device="cuda")      # contraction over K tokens this time
+    xt = workloads.activations_gauss_outliers(K, T, seed=24, device="cuda")
+    D = assert_matches_oracle(dy, binding.ROUND_STOCHASTIC, seed=3, tensor_id=1)
+    tq, ts, t_hat = act1d_t(xt)
+    dw = binding.fp4q_gemm_wgrad_act1d(D, tq, ts, T)
+    torch.cuda.synchronize()
+    gpu = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    check(y, (gpu(x_hat) @ gpu(dequant_from_gpu(W)).T).cpu().numpy(), "forward")
+    check(dw, (gpu(dequant_from_gpu(D)).T @ gpu(t_hat)).cpu().numpy(), "weight gradient")
