@@ -23,4 +23,33 @@ struct Workspace {
     uint32_t pad[60];
 };
 
+// Short launches overlap their predecessor's end: quantizers of up to kShortGrid CTAs and short products (launch_gemm_impl says
+// which) are launched as the programmatic dependents of the kernel before them in their stream (after a copy or a foreign
+// kernel the attribute changes nothing), so their CTAs may be placed, and set up barriers and tensor memory, while the last
+// CTAs of that kernel still run.  Before it touches global memory - reads an input or writes an output - every thread
+// waits until that kernel has completed and its writes are visible: streams keep their order.  A kernel lets its own successor
+// in only after that wait, so that whoever skips the wait (the later tensors of a multi-tensor quantizer call) still
+// runs behind everything before the call.  Long grids do not take part: in a dependent launch the wait costs every CTA of the
+// grid, not only the first ones (expert layer with all quantizers dependent 1662 -> 1844 us).
+constexpr int64_t kShortGrid = 2 * 4 * 148;   // two waves of four CTAs per SM
+// A launch of `kernel` with one parameter block; always: as a dependent whatever its size.
+template <typename P>
+inline cudaError_t launch_dependent(void (*kernel)(const P), dim3 grid, int threads, cudaStream_t stream, const P &p, bool always = false)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = always || (int64_t)grid.x * grid.y <= kShortGrid ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void admit_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 }  // namespace fp4q

@@ -1068,11 +1068,6 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     int32_t *goffs_smem = reinterpret_cast<int32_t *>(reinterpret_cast<uint8_t *>(bars) + kSmemTail);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // Poll limit of every bounded wait (workspace word 2; 0 = the default) and the development hook of word 3 (n > 0:
-    // the producer of CTA 0 leaves out its n-th stage load, so that a test can watch a wait run out and the kernel
-    // leave through its timeout path without anything faulting or spinning for long).
-    const uint32_t wait_limit_word = __ldg(p.status + 2), withhold_load = blockIdx.x == 0 ? __ldg(p.status + 3) : 0u;
-    const uint64_t wait_limit = wait_limit_word != 0u ? wait_limit_word : kWaitLimit;
     const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + kMaxStages);
     const uint32_t bar_acc_full = smem_u32(bars + 12), bar_acc_empty = smem_u32(bars + 13);
     const uint32_t bar_cache_full = smem_u32(bars + 24), bar_cache_empty = smem_u32(bars + 28);
@@ -1117,6 +1112,14 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
         }
     }
+    // Everything above touches this CTA only; from here on the kernel reads what its predecessor in the stream wrote.
+    wait_for_predecessor();
+    admit_successor();
+    // Poll limit of every bounded wait (workspace word 2; 0 = the default) and the development hook of word 3 (n > 0:
+    // the producer of CTA 0 leaves out its n-th stage load, so that a test can watch a wait run out and the kernel
+    // leave through its timeout path without anything faulting or spinning for long).
+    const uint32_t wait_limit_word = __ldg(p.status + 2), withhold_load = blockIdx.x == 0 ? __ldg(p.status + 3) : 0u;
+    const uint64_t wait_limit = wait_limit_word != 0u ? wait_limit_word : kWaitLimit;
     // grouped products: a 32-bit copy of the group boundaries for the per-tile lookups of every role
     const int n_row_tiles = (p.M + BM - 1) / BM;
     const bool goffs_ok = Cfg<KIND, CTAS>::kSmemGroups > 0 &&
@@ -1893,13 +1896,26 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = Cfg<KIND, CTAS>::kSmemBytes;
     cfg.stream = static_cast<cudaStream_t>(stream);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CTAS;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    // Short products start beside their predecessor's end (up to 48 stages, about 25 us, per CTA or pair: a 2048 x 4096 x 4096
+    // microbatch of five calls 111 -> 106 us, 16 x 16 blocks at 8192 x 2048 x 2048 134 -> 129 us).  Long ones do not: their CTAs
+    // would be placed as SMs fall free instead of in order, and tiles that share operands end up far apart (all three products of
+    // 16384 x 11008 x 4096 with their quantizers 1039 -> 1084 us, 1D activations at 8192 x 5632 x 2048 241 -> 251 us).
+    constexpr int kElems = kind_fp4(KIND) ? 256 : 128;
+    const int64_t tile_stages = ceil_div(p.K, kElems);   // a grouped contraction: of one output tile over all groups
+    const int64_t n_stages = p.mode == MODE_GROUPED_K ? (int64_t)p.m_tiles * p.n_tiles * (tile_stages + p.n_groups) : p.n_tile_total * tile_stages;
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = CTAS == 2 ? 1 : 0;
+    if (CTAS == 2) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = CTAS;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.numAttrs = 1;
+    }
+    if (n_stages <= 48 * (int64_t)slots) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
     return cudaLaunchKernelEx(&cfg, gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH>, tmA, tmB, tmC, tmD, p) == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
 }
 

@@ -28,6 +28,8 @@ __device__ __forceinline__ uint32_t cvt_rn_e4m3x2(float hi, float lo)
 
 __global__ void __launch_bounds__(256) mxfp8_quantize1d_kernel(const __grid_constant__ Mxfp8QuantParams p)
 {
+    wait_for_predecessor();
+    admit_successor();
     // one whole block of 32 elements per thread: four 128-bit loads, two 128-bit stores, no exchange between lanes
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t blocks_per_row = p.segs_per_row >> 1, total = p.rows * blocks_per_row;
@@ -103,6 +105,8 @@ __global__ void __launch_bounds__(256) mxfp8_quantize1d_kernel(const __grid_cons
 // column (one whole sector each).
 __global__ void __launch_bounds__(128) mxfp8_quantize1d_t_kernel(const __grid_constant__ Mxfp8QuantParams p)
 {
+    wait_for_predecessor();
+    admit_successor();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t rb = (int64_t)blockIdx.y * 4 + warp;            // block of 32 rows
     const int64_t i0 = rb * 32, c0 = (int64_t)blockIdx.x * 64 + 2 * lane;
@@ -192,6 +196,8 @@ __global__ void __launch_bounds__(128) mxfp8_quantize1d_t_kernel(const __grid_co
 // column's group) and leave as 128 contiguous bytes per column; the four scale bytes of a column as one word.
 __global__ void __launch_bounds__(128, 4) mxfp8_quantize1d_t_tile_kernel(const __grid_constant__ Mxfp8QuantParams p)
 {
+    wait_for_predecessor();
+    admit_successor();
     __shared__ uint4 stage[128 * 8];         // 128 output rows (columns of x) x 128 B
     __shared__ uint32_t sc_stage[128];       // per column of x: the scale codes of the CTA's four row blocks
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -318,7 +324,7 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d(const void *x_bf16, int64_t rows, i
     const int64_t total = rows * (p.segs_per_row / 2);
     const int64_t n_cta = ceil_div(total, 256);
     if (n_cta > 0x7FFFFFFF) return FP4Q_ERR_UNSUPPORTED;
-    mxfp8_quantize1d_kernel<<<(unsigned)n_cta, 256, 0, static_cast<cudaStream_t>(stream)>>>(p);
+    launch_dependent(mxfp8_quantize1d_kernel, dim3((unsigned)n_cta), 256, static_cast<cudaStream_t>(stream), p);
     return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
 }
 
@@ -341,11 +347,11 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d_t(const void *x_bf16, int64_t rows,
     // full 128x128 tiles and aligned rows: the tile kernel (coalesced 128-byte column stores)
     if (rows % 128 == 0 && cols % 128 == 0 && aligned(x_bf16, 32) && ld_x % 16 == 0 && ld_s % 4 == 0 && aligned(scale, 4) &&
         (rows / 128) * (cols / 128) <= 0x7FFFFFFF) {
-        mxfp8_quantize1d_t_tile_kernel<<<(unsigned)((rows / 128) * (cols / 128)), 128, 0, static_cast<cudaStream_t>(stream)>>>(p);
+        launch_dependent(mxfp8_quantize1d_t_tile_kernel, dim3((unsigned)((rows / 128) * (cols / 128))), 128, static_cast<cudaStream_t>(stream), p);
         return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
     }
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;
-    mxfp8_quantize1d_t_kernel<<<dim3((unsigned)gx, (unsigned)gy), 128, 0, static_cast<cudaStream_t>(stream)>>>(p);
+    launch_dependent(mxfp8_quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p);
     return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
 }

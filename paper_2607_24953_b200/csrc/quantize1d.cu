@@ -32,6 +32,8 @@ struct Quant1dParams {
 template <int MODE>
 __global__ void __launch_bounds__(256) quantize1d_kernel(const __grid_constant__ Quant1dParams p)
 {
+    wait_for_predecessor();
+    admit_successor();
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t blocks_per_row = p.segs_per_row >> 1, total = p.rows * blocks_per_row;
     if (gid >= total) return;
@@ -106,6 +108,8 @@ __global__ void __launch_bounds__(256) quantize1d_kernel(const __grid_constant__
 // a lane keeps its two columns' 32 values in registers, and writes the 16 payload bytes of each column's block.
 __global__ void __launch_bounds__(128) quantize1d_t_kernel(const __grid_constant__ Quant1dParams p)
 {
+    wait_for_predecessor();
+    admit_successor();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t rb = (int64_t)blockIdx.y * 4 + warp;   // block of 32 rows
     const int64_t i0 = rb * 32, c0 = (int64_t)blockIdx.x * 64 + 2 * lane;
@@ -201,6 +205,8 @@ __device__ __noinline__ uint32_t round_column_scalar(uint4 rows, float inv)
 // one 32-bit store.
 __global__ void __launch_bounds__(128, 4) quantize1d_t_tile_kernel(const __grid_constant__ Quant1dParams p)
 {
+    wait_for_predecessor();
+    admit_successor();
     __shared__ uint4 qt_stage[128 * 4];      // 128 output rows (columns of x) x 64 B, 16-byte chunks XOR-swizzled
     __shared__ uint32_t sc_stage[128];       // per column of x: the scale codes of the CTA's four row blocks
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -333,8 +339,8 @@ extern "C" fp4q_status fp4q_quantize1d(const void *x_bf16, int64_t rows, int64_t
     const int64_t n_cta = ceil_div(rows * (p.segs_per_row / 2), 256);
     if (n_cta > 0x7FFFFFFF) return FP4Q_ERR_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (mode == FP4Q_ROUND_STOCHASTIC) quantize1d_kernel<FP4Q_ROUND_STOCHASTIC><<<(unsigned)n_cta, 256, 0, s>>>(p);
-    else quantize1d_kernel<FP4Q_ROUND_NEAREST><<<(unsigned)n_cta, 256, 0, s>>>(p);
+    if (mode == FP4Q_ROUND_STOCHASTIC) launch_dependent(quantize1d_kernel<FP4Q_ROUND_STOCHASTIC>, dim3((unsigned)n_cta), 256, s, p);
+    else launch_dependent(quantize1d_kernel<FP4Q_ROUND_NEAREST>, dim3((unsigned)n_cta), 256, s, p);
     return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
 }
 
@@ -354,11 +360,11 @@ extern "C" fp4q_status fp4q_quantize1d_t(const void *x_bf16, int64_t rows, int64
     // full 128x128 tiles and aligned rows: the tile kernel (coalesced 64-byte column stores)
     if (rows % 128 == 0 && cols % 128 == 0 && aligned(x_bf16, 32) && ld_x % 16 == 0 && ld_s % 4 == 0 && aligned(scale, 4) &&
         (rows / 128) * (cols / 128) <= 0x7FFFFFFF) {
-        quantize1d_t_tile_kernel<<<(unsigned)((rows / 128) * (cols / 128)), 128, 0, static_cast<cudaStream_t>(stream)>>>(p);
+        launch_dependent(quantize1d_t_tile_kernel, dim3((unsigned)((rows / 128) * (cols / 128))), 128, static_cast<cudaStream_t>(stream), p);
         return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
     }
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;
-    quantize1d_t_kernel<<<dim3((unsigned)gx, (unsigned)gy), 128, 0, static_cast<cudaStream_t>(stream)>>>(p);
+    launch_dependent(quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p);
     return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
 }

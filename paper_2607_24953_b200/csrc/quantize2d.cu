@@ -42,6 +42,7 @@ struct Quant2dParams {
     uint32_t tensor_id;
     uint32_t flags;
     int x_vec_ok;             // 2: x 32-byte aligned, ld_x % 16 == 0 (256-bit loads); 1: 16-byte aligned, ld_x % 8 == 0
+    int waits;                // the kernel waits for its predecessor before it reads (0: a later tensor of a multi-tensor call)
     int rng_aligned;          // nearest, or cols % 16 == 0 and index not transposed: one Philox block per 16-element segment
     PhiloxRoundKeys keys;
 };
@@ -454,18 +455,16 @@ __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_kernel(
     __shared__ uint4 qt_stage[128 * 4];   // 128 transposed rows x 64 B (four 16-byte chunks, XOR-swizzled)
     __shared__ uint4 rnd_stage[MODE == FP4Q_ROUND_STOCHASTIC ? 8 * 128 : 1];   // per thread: 8 rows x 16 random bytes
     __shared__ uint32_t xchg[BLK == 64 ? 16 : 1];   // 64x64 blocks: maxima of the four warps' two half blocks
-    // Programmatic dependent launch (used by fp4q_quantize2d_multi to chain the launches of independent tensors in
-    // one stream): a launch configured as this one's dependent may start filling SMs as soon as every CTA of this
-    // grid is resident, i.e. beside this grid's last wave.  Without such a configuration both instructions do nothing.
-    asm volatile("griddepcontrol.launch_dependents;");
+    if (p.waits) wait_for_predecessor();
+    admit_successor();
     const int64_t bx = (int64_t)blockIdx.x % p.grid_x, by = (int64_t)blockIdx.x / p.grid_x;
     const bool full = p.x_vec_ok == 2 && p.rng_aligned && (by + 1) * 128 <= p.rows && (bx + 1) * 128 <= p.cols;
     if (full) quantize_tile<MODE, true, BLK>(p, qt_stage, rnd_stage, xchg);
     else quantize_tile<MODE, false, BLK>(p, qt_stage, rnd_stage, xchg);
-    // A dependent grid does not read what its predecessor wrote (different tensors), so it never waited for it; it
-    // waits here, after its own stores, so that the grids of a chain still COMPLETE in launch order and whatever is
-    // enqueued after the chain sees every tensor of it.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The later tensors of a multi-tensor call do not read what the call's earlier ones wrote, so they did not wait; they
+    // wait here, after their own stores, so that the grids still COMPLETE in launch order and whatever is enqueued after the
+    // call sees every tensor of it.
+    if (!p.waits) wait_for_predecessor();
 }
 
 // Every tile of a tensor for which quantize2d_kernel has no check-free one.  Static shared memory (44 KB with the
@@ -476,9 +475,10 @@ __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_staged_
     __shared__ uint4 qt_stage[128 * 4];
     __shared__ uint4 stage[4 * kStageWarpBytes / 16];
     __shared__ uint32_t xchg[BLK == 64 ? 16 : 1];
-    asm volatile("griddepcontrol.launch_dependents;");
+    if (p.waits) wait_for_predecessor();
+    admit_successor();
     quantize_tile<MODE, false, BLK, true>(p, qt_stage, stage, xchg);
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // as in quantize2d_kernel
+    if (!p.waits) wait_for_predecessor();   // as in quantize2d_kernel
 }
 
 typedef void (*Quant2dKernel)(const Quant2dParams);
@@ -548,8 +548,9 @@ extern "C" fp4q_status fp4q_quantize2d(const void *x_bf16, int64_t rows, int64_t
     if (fp4q_status st = prepare_quantize2d(x_bf16, rows, cols, ld_x, out, mode, seed, tensor_id, flags, p, &n_cta)) return st;
     if (n_cta == 0) return FP4Q_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC)<<<(unsigned)n_cta, 128, 0, s>>>(p);
-    return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
+    p.waits = 1;
+    return launch_dependent(quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC), dim3((unsigned)n_cta), 128, s, p) == cudaSuccess
+               ? FP4Q_OK : FP4Q_ERR_CUDA;
 }
 
 extern "C" fp4q_status fp4q_quantize2d_multi(const fp4q_quantize_job *jobs, int32_t n_jobs, fp4q_round mode, uint64_t seed,
@@ -567,9 +568,8 @@ extern "C" fp4q_status fp4q_quantize2d_multi(const fp4q_quantize_job *jobs, int3
             return st;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // One launch of the one-tensor kernel per tensor, each after the first configured as the programmatic dependent of
-    // the one before it: the tensors are independent, so a launch may begin beside its predecessor's last wave instead
-    // of after it (what two streams would give, in one stream).
+    // One launch of the one-tensor kernel per tensor; the tensors are independent, so a launch after the first does not wait
+    // for the one before it and begins beside its last wave instead of after it (what two streams would give, in one stream).
     bool first = true;
     for (int32_t j = 0; j < n_jobs; j++) {
         Quant2dParams p;
@@ -577,16 +577,9 @@ extern "C" fp4q_status fp4q_quantize2d_multi(const fp4q_quantize_job *jobs, int3
         prepare_quantize2d(jobs[j].x_bf16, jobs[j].rows, jobs[j].cols, jobs[j].ld_x, jobs[j].out, mode, seed, jobs[j].tensor_id,
                            jobs[j].flags, p, &n_cta);
         if (n_cta == 0) continue;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)n_cta);
-        cfg.blockDim = dim3(128);
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = first ? 0 : 1;
-        if (cudaLaunchKernelEx(&cfg, quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC), p) != cudaSuccess) return FP4Q_ERR_CUDA;
+        p.waits = first;
+        if (launch_dependent(quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC), dim3((unsigned)n_cta), 128, s, p, !first) != cudaSuccess)
+            return FP4Q_ERR_CUDA;
         first = false;
     }
     return FP4Q_OK;
