@@ -71,14 +71,18 @@ int64_t as_i64(PyObject *o)
     if (v == -1 && PyErr_Occurred()) throw PyError();
     return v;
 }
-uint64_t as_bits(PyObject *o)   // seeds and ids: reduced modulo 2^64, as ctypes does
+uint64_t as_bits(PyObject *o)   // seeds and modes: anything with __index__ (NumPy's and torch's whole numbers), modulo 2^64, as ctypes does
 {
-    if (!PyLong_Check(o)) { PyErr_Format(PyExc_TypeError, "int expected instead of %s instance", Py_TYPE(o)->tp_name); throw PyError(); }
     const unsigned long long v = PyLong_AsUnsignedLongLongMask(o);
     if (v == (unsigned long long)-1 && PyErr_Occurred()) throw PyError();
     return v;
 }
 int as_int(PyObject *o) { return (int)(uint32_t)as_bits(o); }
+uint32_t id_at(PyObject *ids, Py_ssize_t j)   // int(ids[j]), of a list, an array or a tensor
+{
+    Ref index(PyLong_FromSsize_t(j)), item(PyObject_GetItem(ids, index.p)), number(PyNumber_Long(item.p));
+    return (uint32_t)as_bits(number.p);
+}
 bool as_bool(PyObject *o)
 {
     const int v = PyObject_IsTrue(o);
@@ -233,12 +237,11 @@ PyObject *quantize2d_multi(Args a, Py_ssize_t n)
     want(n, 8);
     Ref xs(PySequence_Fast(a[0], "xs must be a sequence of tensors"));
     const Py_ssize_t k = PySequence_Fast_GET_SIZE(xs.p);
-    Ref ids(a[4] == Py_None ? Py_NewRef(Py_None) : PySequence_Fast(a[4], "tensor_ids must be a sequence of ints"));
     const bool own = a[1] == Py_None;
     Ref outs(own ? PyList_New(0) : PySequence_Fast(a[1], "outs must be a sequence of QTensor"));
     const uint32_t flags = (uint32_t)as_bits(a[5]);
     const bool want_t = as_bool(a[6]);
-    if ((!own && PySequence_Fast_GET_SIZE(outs.p) < k) || (ids.p != Py_None && PySequence_Fast_GET_SIZE(ids.p) < k)) {
+    if (!own && PySequence_Fast_GET_SIZE(outs.p) < k) {
         PyErr_SetString(PyExc_IndexError, "list index out of range");
         throw PyError();
     }
@@ -259,7 +262,7 @@ PyObject *quantize2d_multi(Args a, Py_ssize_t n)
         jobs[j].x_bf16 = x.data_ptr();
         jobs[j].rows = x.size(0); jobs[j].cols = x.size(1); jobs[j].ld_x = pitch(x);
         jobs[j].out = &ts[j];
-        jobs[j].tensor_id = ids.p == Py_None ? (uint32_t)j : (uint32_t)as_bits(PySequence_Fast_GET_ITEM(ids.p, j));
+        jobs[j].tensor_id = a[4] == Py_None ? (uint32_t)j : id_at(a[4], j);
         jobs[j].flags = flags;
     }
     check(unlocked(lib.quantize2d_multi, jobs.data(), (int32_t)k, (fp4q_round)as_int(a[2]), as_bits(a[3]), as_stream(a[7])), "fp4q_quantize2d_multi");
