@@ -29,7 +29,9 @@ struct Workspace {
 // CTAs of that kernel still run.  Before it touches global memory - reads an input or writes an output - every thread
 // waits until that kernel has completed and its writes are visible: streams keep their order.  A kernel lets its own successor
 // in only after that wait, so that whoever skips the wait (the later tensors of a multi-tensor quantizer call) still
-// runs behind everything before the call.  Long grids do not take part: in a dependent launch the wait costs every CTA of the
+// runs behind everything before the call.  What the predecessor wrote is read with ordinary loads: the non-coherent path
+// (ld.global.nc, __ldg) is for memory that nothing writes while the kernel runs, and a dependent kernel runs before its
+// inputs are complete.  Long grids do not take part: in a dependent launch the wait costs every CTA of the
 // grid, not only the first ones (expert layer with all quantizers dependent 1662 -> 1844 us).
 constexpr int64_t kShortGrid = 2 * 4 * 148;   // two waves of four CTAs per SM
 // A launch of `kernel` with one parameter block; always: as a dependent whatever its size.
@@ -49,6 +51,9 @@ inline cudaError_t launch_dependent(void (*kernel)(const P), dim3 grid, int thre
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// An ordinary load; it stays below wait_for_predecessor(), which clobbers memory.
+template <typename T>
+__device__ __forceinline__ T load_global(const T *p) { return *p; }
 __device__ __forceinline__ void admit_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 

@@ -445,7 +445,7 @@ __device__ __forceinline__ int find_group(const int64_t *offs, const int32_t *go
     int lo = 0, hi = n_groups;      // largest g with offs[g] <= row
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        const int64_t v = goffs ? (int64_t)goffs[mid] : __ldg(offs + mid);
+        const int64_t v = goffs ? (int64_t)goffs[mid] : load_global(offs + mid);
         if (v <= row) lo = mid; else hi = mid;
     }
     return lo;
@@ -455,10 +455,14 @@ __device__ __forceinline__ int find_group(const int64_t *offs, const int32_t *go
 // producer and the scale builder need - the MMA issuer, the watcher and the epilogue use the contraction length and
 // the output position alone, and a lookup in the MMA warp (shared-memory reads behind its pending MMAs) costs
 // about 1900 cycles per tile.
+// GROUPED = false: a kernel that only dense products use.  Their tiles are decoded without the group branches, which cost
+// the builders of the per-row kinds 3-8 % of a product (1D activations at 4096 x 4096 x 4096: 45.8 us without, 49.7 us with).
+template <bool GROUPED>
 __device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int rank, Tile &t, const int32_t *goffs, const uint16_t *gorder, bool need_b = true)
 {
+    const int mode = GROUPED ? p.mode : MODE_DENSE;
     const int per_problem = p.m_tiles * p.n_tiles;
-    const int nth = p.mode == MODE_GROUPED_K ? tile / per_problem : 0, g = p.mode == MODE_GROUPED_K && gorder ? (int)gorder[nth] : nth;
+    const int nth = mode == MODE_GROUPED_K ? tile / per_problem : 0, g = mode == MODE_GROUPED_K && gorder ? (int)gorder[nth] : nth;
     const int local = tile - nth * per_problem;
     // Tiles that run at the same time (consecutive indices) cover raster_m row tiles x a few column tiles, and
     // the sweep over column tiles finishes before the next group of row tiles starts: the group's A rows stay
@@ -476,15 +480,15 @@ __device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int r
     t.c_col0 = t.b_row0;
     t.m_valid = min(BM, p.M - t.a_row0);
     t.n_valid = min(BN, p.N - t.b_row0);
-    if (p.mode == MODE_GROUPED_ROWS) {
+    if (mode == MODE_GROUPED_ROWS) {
         if (!need_b) return;
         const int grp = goffs ? (int)reinterpret_cast<const uint16_t *>(goffs)[t.a_row0 / BM]
                               : find_group(p.row_offsets, nullptr, p.n_groups, (int64_t)t.a_row0);
         t.b_row0 += grp * p.b_rows_per_group;
         t.b_load_row0 += grp * p.b_rows_per_group;
         t.b_k0 = grp * p.b_k_per_group;
-    } else if (p.mode == MODE_GROUPED_K) {
-        const int64_t k0 = goffs ? (int64_t)goffs[g] : __ldg(p.row_offsets + g), k1 = goffs ? (int64_t)goffs[g + 1] : __ldg(p.row_offsets + g + 1);
+    } else if (mode == MODE_GROUPED_K) {
+        const int64_t k0 = goffs ? (int64_t)goffs[g] : load_global(p.row_offsets + g), k1 = goffs ? (int64_t)goffs[g + 1] : load_global(p.row_offsets + g + 1);
         t.a_k0 = t.b_k0 = (int32_t)k0;
         t.k_len = (int32_t)(k1 - k0);
         t.c_row0 = g * p.M + t.a_row0;
@@ -503,30 +507,26 @@ __device__ __forceinline__ void load_scale(const ScaleView &v, int row, int kb, 
 {
     const uint8_t *ptr = (row < v.n_row && kb < v.n_kb) ? v.ptr + (int64_t)row * v.stride_row + (int64_t)kb * v.stride_kb
                                                         : g_scale_pad;
-    asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(dst) : "l"(ptr));
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(dst) : "l"(ptr));
 }
 
-// The stream of ring stages one CTA works through: its tiles in order, each with its contraction stages.
+// The stream of ring stages one CTA of a dense product works through: its tiles in order, each with its contraction stages.
 struct StageIter {
     int tile, step, rank, it, n_it;
-    const int32_t *goffs;
-    const uint16_t *gorder;
-    bool need_b;
     Tile t;
     __device__ __forceinline__ void seek(const GemmParams &p, int stage_elems)
     {
         while (tile < p.n_tile_total) {
-            decode_tile(p, tile, rank, t, goffs, gorder, need_b);
+            decode_tile<false>(p, tile, rank, t, nullptr, nullptr, false);
             n_it = (t.k_len + stage_elems - 1) / stage_elems;
             if (n_it > 0) { it = 0; return; }
             tile += step;
         }
         n_it = 0;
     }
-    __device__ __forceinline__ void init(const GemmParams &p, int first, int step_, int rank_, int stage_elems, const int32_t *goffs_,
-                                         const uint16_t *gorder_, bool need_b_)
+    __device__ __forceinline__ void init(const GemmParams &p, int first, int step_, int rank_, int stage_elems)
     {
-        tile = first; step = step_; rank = rank_; it = 0; goffs = goffs_; gorder = gorder_; need_b = need_b_;
+        tile = first; step = step_; rank = rank_; it = 0;
         seek(p, stage_elems);
     }
     __device__ __forceinline__ bool valid(const GemmParams &p) const { return tile < p.n_tile_total; }
@@ -538,7 +538,7 @@ struct StageIter {
 
 __device__ __forceinline__ void ldg_b32(const uint8_t *ptr, uint32_t &w)
 {
-    asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(w) : "l"(ptr));
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(w) : "l"(ptr));
 }
 
 // Rows of a 4x4 byte matrix given by its columns: w[k] holds byte rt of column k in byte lane rt.
@@ -632,7 +632,7 @@ __device__ __forceinline__ void load_scale_word(const ScaleView &v, int row, int
 {
     const uint8_t *ptr = v.ptr + (int64_t)row * v.stride_row + kb0;
     if (row < v.n_row && kb0 + 4 <= v.n_kb && v.stride_kb == 1 && (reinterpret_cast<uintptr_t>(ptr) & 3) == 0) {
-        asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(dst) : "l"(ptr));   // the common case: nothing depends on it yet
+        asm volatile("ld.global.b32 %0, [%1];" : "=r"(dst) : "l"(ptr));   // the common case: nothing depends on it yet
         return;
     }
     uint32_t word = 0;
@@ -643,11 +643,6 @@ __device__ __forceinline__ void load_scale_word(const ScaleView &v, int row, int
         word |= b << (8 * kb);
     }
     dst = word;
-}
-
-__device__ __forceinline__ void ldg_v4(const uint8_t *ptr, uint32_t *w)
-{
-    asm volatile("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(ptr));
 }
 
 template <int KIND>
@@ -818,24 +813,22 @@ struct BufRing {
     __device__ __forceinline__ void next(uint32_t n) { if (++buf == n) { buf = 0; phase ^= 1u; } }
 };
 
-// The stream of scale units (kUnitStages stages of one tile) a CTA works through.
+// The stream of scale units (kUnitStages stages of one tile) a CTA works through; per-row scales, dense products.
 struct UnitIter {
     int tile, step, rank, k0;
-    const int32_t *goffs;
-    const uint16_t *gorder;
     Tile t;
     __device__ __forceinline__ void seek(const GemmParams &p)
     {
         while (tile < p.n_tile_total) {
-            decode_tile(p, tile, rank, t, goffs, gorder);
+            decode_tile<false>(p, tile, rank, t, nullptr, nullptr);
             if (k0 < t.k_len) return;
             tile += step;
             k0 = 0;
         }
     }
-    __device__ __forceinline__ void init(const GemmParams &p, int first, int step_, int rank_, const int32_t *goffs_, const uint16_t *gorder_)
+    __device__ __forceinline__ void init(const GemmParams &p, int first, int step_, int rank_)
     {
-        tile = first; step = step_; rank = rank_; k0 = 0; goffs = goffs_; gorder = gorder_;
+        tile = first; step = step_; rank = rank_; k0 = 0;
         seek(p);
     }
     __device__ __forceinline__ bool valid(const GemmParams &p) const { return tile < p.n_tile_total; }
@@ -1031,6 +1024,9 @@ struct RowFetch {
 
 // ---------------------------------------------------------------------------------------- kernel
 
+// Grouped products exist for 2D-block scales only, and their kernels have no watcher.
+template <int KIND, bool WATCH> constexpr bool kGroupedKernel = KIND == KIND_MXF4 && !WATCH;
+
 // WATCH: warp 2 looks at the ring's barriers for the MMA warp and the two meet at a named barrier per stage; otherwise the
 // MMA warp looks for itself, at the next stage's before it issues a stage.  launch_gemm() says which is used where.
 template <int KIND, int CTAS, int EPI, bool WATCH>
@@ -1048,6 +1044,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                                 : KIND == KIND_MXF4R ? kUnitStagesMxf4R : kUnitStagesMxf4B16;   // stages whose scale images are built together
     constexpr int kBufBytes = Cfg<KIND, CTAS>::kBufBytes;
     constexpr int kUnitBlocks = Cfg<KIND, CTAS>::kUnitBlocks;
+    constexpr bool kGrouped = kGroupedKernel<KIND, WATCH>;
     constexpr int kKbShift = KIND == KIND_MXF4B16 ? 4 : 5;    // log2 of the scale vector's length (contraction elements per scale byte)
 
     extern __shared__ uint8_t smem_raw[];
@@ -1118,15 +1115,15 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     // Poll limit of every bounded wait (workspace word 2; 0 = the default) and the development hook of word 3 (n > 0:
     // the producer of CTA 0 leaves out its n-th stage load, so that a test can watch a wait run out and the kernel
     // leave through its timeout path without anything faulting or spinning for long).
-    const uint32_t wait_limit_word = __ldg(p.status + 2), withhold_load = blockIdx.x == 0 ? __ldg(p.status + 3) : 0u;
+    const uint32_t wait_limit_word = load_global(p.status + 2), withhold_load = blockIdx.x == 0 ? load_global(p.status + 3) : 0u;
     const uint64_t wait_limit = wait_limit_word != 0u ? wait_limit_word : kWaitLimit;
     // grouped products: a 32-bit copy of the group boundaries for the per-tile lookups of every role
     const int n_row_tiles = (p.M + BM - 1) / BM;
-    const bool goffs_ok = Cfg<KIND, CTAS>::kSmemGroups > 0 &&
+    const bool goffs_ok = kGrouped && Cfg<KIND, CTAS>::kSmemGroups > 0 &&
                           ((p.mode == MODE_GROUPED_K && p.n_groups <= kMaxGroupsShared) ||
                            (p.mode == MODE_GROUPED_ROWS && n_row_tiles <= kMaxRowTilesShared && p.n_groups <= 65535));
     if (goffs_ok && p.mode == MODE_GROUPED_K)
-        for (int g = threadIdx.x; g <= p.n_groups; g += kThreads) goffs_smem[g] = (int32_t)__ldg(p.row_offsets + g);
+        for (int g = threadIdx.x; g <= p.n_groups; g += kThreads) goffs_smem[g] = (int32_t)load_global(p.row_offsets + g);
     if (goffs_ok && p.mode == MODE_GROUPED_ROWS)
         for (int i = threadIdx.x; i < n_row_tiles; i += kThreads)
             reinterpret_cast<uint16_t *>(goffs_smem)[i] = (uint16_t)find_group(p.row_offsets, nullptr, p.n_groups, (int64_t)i * BM);
@@ -1169,7 +1166,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         int ev_j = 0;
         for (int tile = first_tile; ok && tile < p.n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile(p, tile, rank, t, goffs, gorder);
+            decode_tile<kGrouped>(p, tile, rank, t, goffs, gorder);
             const int n_it = (t.k_len + kStageElems - 1) / kStageElems;
             int xa = t.a_k0 / kElemsPerByte, xb = t.b_k0 / kElemsPerByte;
 #pragma unroll 1
@@ -1222,7 +1219,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         TRACE_T0(tt);
         for (int tile = first_tile; leader && tile < p.n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile(p, tile, rank, t, goffs, gorder, false);
+            decode_tile<kGrouped>(p, tile, rank, t, goffs, gorder, false);
             const int n_it = (t.k_len + kStageElems - 1) / kStageElems;
             if (n_it == 0) continue;
             TRACE_ADD(c_acc, tt);
@@ -1324,7 +1321,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             bool fwd_ok = true;
             BufRing fr;
             UnitIter un;
-            for (un.init(p, first_tile, tile_step, rank, goffs, gorder); fwd_ok && un.valid(p); un.next(p, kUnitStages * kStageElems), fr.next(kImageBufs)) {
+            for (un.init(p, first_tile, tile_step, rank); fwd_ok && un.valid(p); un.next(p, kUnitStages * kStageElems), fr.next(kImageBufs)) {
                 fwd_ok = __all_sync(0xFFFFFFFFu, mbar_wait_impl<0>(bar_cache_full + 8 * fr.buf, fr.phase, abort_flag, p.status, wait_limit, 0x530u + fr.buf));
                 if (fwd_ok && issuer) mbar_arrive_cluster_release(cluster_addr(bar_peer_cache_full + 8 * fr.buf, 0));
             }
@@ -1360,8 +1357,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             constexpr int kOwnRaw = Cfg<KIND, CTAS>::kRawBufs > 0 ? Cfg<KIND, CTAS>::kRawBufs / kBuilders : 1;
             uint8_t *raw = smem_raw_scales + (3 - warp) * kOwnRaw * kRawBytes;
             UnitIter ahead, cur;
-            ahead.init(p, first_tile, tile_step, rank, goffs, gorder);
-            cur.init(p, first_tile, tile_step, rank, goffs, gorder);
+            ahead.init(p, first_tile, tile_step, rank);
+            cur.init(p, first_tile, tile_step, rank);
             if (warp == 2) {   // the second builder starts with the second unit
                 if (ahead.valid(p)) ahead.next(p, kUnitStages * kStageElems);
                 if (cur.valid(p)) cur.next(p, kUnitStages * kStageElems);
@@ -1417,7 +1414,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         }
         for (int tile = first_tile; KIND == KIND_MXF4 && ok && tile < p.n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile(p, tile, rank, t, goffs, gorder);
+            decode_tile<kGrouped>(p, tile, rank, t, goffs, gorder);
             for (int k0 = 0; ok && k0 < t.k_len; k0 += kUnitStages * kStageElems, ring.next(kImageBufs)) {
                 const int buf = ring.buf;
                 uint8_t *images = smem_images + buf * kBufBytes;
@@ -1465,7 +1462,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         // stage is released unseen, so that the MMA warp, which cannot time out on a named barrier, always runs
         // to its end.
         StageIter sg;
-        sg.init(p, first_tile, tile_step, rank, kStageElems, goffs, gorder, false);
+        sg.init(p, first_tile, tile_step, rank, kStageElems);
         uint32_t stage = 0, phase = 0, acc_phase = 0;
         BufRing ring;   // image buffer of the current unit
         bool ok = true;
@@ -1590,7 +1587,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         TRACE_T0(tt);
         for (int tile = first_tile; ok && tile < p.n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile(p, tile, rank, t, goffs, gorder, false);
+            decode_tile<kGrouped>(p, tile, rank, t, goffs, gorder, false);
             const int row_in_tile = 32 * quarter + lane;
             const int64_t row = (int64_t)t.c_row0 + row_in_tile;
             const bool row_ok = row_in_tile < t.m_valid;
@@ -1859,6 +1856,7 @@ template <int KIND, int CTAS, int EPI, bool WATCH>
 static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmParams &p, void *stream)
 {
     CUtensorMap tmA, tmB, tmC;
+    if (!kGroupedKernel<KIND, WATCH> && p.mode != MODE_DENSE) return FP4Q_ERR_UNSUPPORTED;
     const int64_t out_rows = p.mode == MODE_GROUPED_K ? (int64_t)p.n_groups * p.M : p.M;
     if (!make_operand_map(&tmA, A.payload, A.rows, A.row_bytes, A.ld_bytes, BM)) return FP4Q_ERR_CUDA;
     CUtensorMap tmD = tmA;   // second output map: only the quantizing epilogue has one

@@ -49,14 +49,14 @@ __global__ void __launch_bounds__(256) mxfp8_quantize1d_kernel(const __grid_cons
     if (p.x_vec_ok && j0 + 32 <= p.cols) {
 #pragma unroll
         for (int q = 0; q < 4; q++) {
-            const uint4 a = __ldg(reinterpret_cast<const uint4 *>(src) + q);
+            const uint4 a = load_global(reinterpret_cast<const uint4 *>(src) + q);
             raw[4 * q] = a.x; raw[4 * q + 1] = a.y; raw[4 * q + 2] = a.z; raw[4 * q + 3] = a.w;
         }
     } else {
 #pragma unroll
         for (int k = 0; k < 16; k++) {
-            const uint32_t lo = (j0 + 2 * k < p.cols) ? (uint32_t)__ldg(src + 2 * k) : 0u;
-            const uint32_t hi = (j0 + 2 * k + 1 < p.cols) ? (uint32_t)__ldg(src + 2 * k + 1) : 0u;
+            const uint32_t lo = (j0 + 2 * k < p.cols) ? (uint32_t)load_global(src + 2 * k) : 0u;
+            const uint32_t hi = (j0 + 2 * k + 1 < p.cols) ? (uint32_t)load_global(src + 2 * k + 1) : 0u;
             raw[k] = lo | (hi << 16);
         }
     }
@@ -117,14 +117,14 @@ __global__ void __launch_bounds__(128) mxfp8_quantize1d_t_kernel(const __grid_co
         const uint32_t *src = reinterpret_cast<const uint32_t *>(p.x + i0 * p.ld_x + c0);
         const int64_t step = p.ld_x >> 1;
 #pragma unroll
-        for (int r = 0; r < 32; r++) raw[r] = __ldg(src + r * step);
+        for (int r = 0; r < 32; r++) raw[r] = load_global(src + r * step);
     } else {
 #pragma unroll
         for (int r = 0; r < 32; r++) {
             raw[r] = 0u;
             if (i0 + r < p.rows) {
                 const uint16_t *src = p.x + (i0 + r) * p.ld_x + c0;
-                raw[r] = (uint32_t)__ldg(src) | (two ? (uint32_t)__ldg(src + 1) << 16 : 0u);
+                raw[r] = (uint32_t)load_global(src) | (two ? (uint32_t)load_global(src + 1) << 16 : 0u);
             }
         }
     }
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(128, 4) mxfp8_quantize1d_t_tile_kernel(const _
         const uint16_t *src = p.x + row0 * p.ld_x + col0;
 #pragma unroll
         for (int r = 0; r < 8; r++)
-            asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                          : "=r"(raw[r][0]), "=r"(raw[r][1]), "=r"(raw[r][2]), "=r"(raw[r][3]), "=r"(raw[r][4]),
                            "=r"(raw[r][5]), "=r"(raw[r][6]), "=r"(raw[r][7])
                          : "l"(src + r * p.ld_x));

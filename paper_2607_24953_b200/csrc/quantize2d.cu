@@ -89,20 +89,20 @@ __device__ __forceinline__ void load_segment(const Quant2dParams &p, int64_t i, 
     }
     const uint16_t *src = p.x + i * p.ld_x + j0;
     if (p.x_vec_ok == 2 && j0 + 16 <= p.cols) {
-        asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                      : "=r"(out[0]), "=r"(out[1]), "=r"(out[2]), "=r"(out[3]), "=r"(out[4]), "=r"(out[5]), "=r"(out[6]),
                        "=r"(out[7])
                      : "l"(src));
     } else if (p.x_vec_ok && j0 + 16 <= p.cols) {
-        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(src));
-        const uint4 b = __ldg(reinterpret_cast<const uint4 *>(src) + 1);
+        const uint4 a = load_global(reinterpret_cast<const uint4 *>(src));
+        const uint4 b = load_global(reinterpret_cast<const uint4 *>(src) + 1);
         out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w;
         out[4] = b.x; out[5] = b.y; out[6] = b.z; out[7] = b.w;
     } else {
 #pragma unroll
         for (int k = 0; k < 8; k++) {
-            const uint32_t lo = (j0 + 2 * k < p.cols) ? (uint32_t)__ldg(src + 2 * k) : 0u;
-            const uint32_t hi = (j0 + 2 * k + 1 < p.cols) ? (uint32_t)__ldg(src + 2 * k + 1) : 0u;
+            const uint32_t lo = (j0 + 2 * k < p.cols) ? (uint32_t)load_global(src + 2 * k) : 0u;
+            const uint32_t hi = (j0 + 2 * k + 1 < p.cols) ? (uint32_t)load_global(src + 2 * k + 1) : 0u;
             out[k] = lo | (hi << 16);
         }
     }
@@ -146,7 +146,7 @@ __device__ __forceinline__ void stage_tile_rows(const Quant2dParams &p, int64_t 
 #pragma unroll 1
             for (int e = 0; e < 8; e++) {
                 const uintptr_t s = g + 2 * e;
-                if (s >= lo && s < hi) reinterpret_cast<uint16_t *>(dst)[e] = __ldg(reinterpret_cast<const uint16_t *>(s));
+                if (s >= lo && s < hi) reinterpret_cast<uint16_t *>(dst)[e] = load_global(reinterpret_cast<const uint16_t *>(s));
             }
         }
     }
@@ -252,7 +252,7 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
         const uint16_t *src = p.x + row0 * p.ld_x + col0;
 #pragma unroll
         for (int r = 0; r < 8; r++)
-            asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                          : "=r"(raw[r][0]), "=r"(raw[r][1]), "=r"(raw[r][2]), "=r"(raw[r][3]), "=r"(raw[r][4]),
                            "=r"(raw[r][5]), "=r"(raw[r][6]), "=r"(raw[r][7])
                          : "l"(src + r * p.ld_x));
