@@ -238,23 +238,17 @@ def fp4q_mxfp8_quantize1d_t(x: torch.Tensor, stream=None):
 
 def fp4q_mxfp8_gemm(aq, a_s, bq, b_s, M: int, N: int, Kdim: int, dt: int = OUT_BF16, ws=None, stream=None):
     """C[M,N] = A^ B^^T on MXFP8 operands (rows along the contraction axis) from the two MXFP8 quantizers."""
-    if ws is None:
-        ws = alloc_workspace(aq.device)
     return _host().mxfp8_gemm(aq, a_s, bq, b_s, M, N, Kdim, dt, ws, _handle(stream))
 
 
 def fp4q_gemm_fwd_act1d(xq, xs, T: int, W: QTensor, out=None, dt: int = OUT_BF16, ws=None, stream=None):
     """Y[T,N] = X^ W^^T with X in 1D blocks along the contraction axis (fp4q_quantize1d) and W in 2D blocks."""
-    if ws is None:
-        ws = alloc_workspace(xq.device)
     return _host().gemm_fwd_act1d(xq, xs, T, W, out, dt, ws, _handle(stream))
 
 
 def fp4q_gemm_wgrad_act1d(dY: QTensor, xtq, xts, K: int, out=None, dt: int = OUT_F32, accumulate: bool = False,
                           ws=None, stream=None):
     """dW[N,K] (+)= dY^^T X^_t with X^_t the 1D-block encoding of X^T (fp4q_quantize1d_t) and dY in 2D blocks."""
-    if ws is None:
-        ws = alloc_workspace(xtq.device)
     return _host().gemm_wgrad_act1d(dY, xtq, xts, K, out, dt, accumulate, ws, _handle(stream))
 
 
@@ -284,8 +278,6 @@ _FWD, _DGRAD, _WGRAD = 0, 1, 2
 
 
 def _gemm(which, a: QTensor, b: QTensor, out_rows, out_cols, out, dt, row_offsets, ws, stream, accumulate=False, row_alignment: int = 128):
-    if ws is None:
-        ws = alloc_workspace(a.q_rm.device)
     return _host().gemm(which, a, b, out_rows, out_cols, out, dt, int(accumulate), row_offsets, row_alignment, ws, _handle(stream))
 
 
@@ -301,8 +293,6 @@ def fp4q_gemm_fwd_quantized(X: QTensor, W: QTensor, out: Optional[QTensor] = Non
                             row_offsets=None) -> QTensor:
     """Yq = 2D-block FP4 of the BF16-rounded product X^ W^^T, quantized in the GEMM's epilogue.  Grouped when
     row_offsets is given (every group then starts on a multiple of 256 rows)."""
-    if ws is None:
-        ws = alloc_workspace(X.q_rm.device)
     n = W.rows if row_offsets is None else W.rows // (row_offsets.numel() - 1)
     return _host().gemm_quantized(_FWD, X, W, X.rows, n, out, mode, seed, tensor_id, want_t, row_offsets, ws, _handle(stream))
 
@@ -312,8 +302,6 @@ def fp4q_gemm_dgrad_quantized(dY: QTensor, W: QTensor, out: Optional[QTensor] = 
                               row_offsets=None) -> QTensor:
     """dXq = 2D-block FP4 of the BF16-rounded product dY^ W^, quantized in the GEMM's epilogue.  Grouped when
     row_offsets is given (every group then starts on a multiple of 256 rows)."""
-    if ws is None:
-        ws = alloc_workspace(dY.q_rm.device)
     return _host().gemm_quantized(_DGRAD, dY, W, dY.rows, W.cols, out, mode, seed, tensor_id, want_t, row_offsets, ws, _handle(stream))
 
 
@@ -345,8 +333,6 @@ def fp4q_gemm_wgrad(dY: QTensor, X: QTensor, out=None, dt: int = OUT_F32, accumu
 
 
 def _gemm_b16(which, a: QTensor, b: QTensor, out_rows, out_cols, out, dt, ws, stream, accumulate=False):
-    if ws is None:
-        ws = alloc_workspace(a.q_rm.device)
     return _host().gemm_b16(which, a, b, out_rows, out_cols, out, dt, int(accumulate), ws, _handle(stream))
 
 
@@ -368,6 +354,4 @@ def fp4q_gemm_wgrad_b16(dY: QTensor, X: QTensor, out=None, dt: int = OUT_F32, ac
 def fp4q_mxfp8_qk(xq, xs, wq_q, wq_s, wk_q, wk_s, T: int, K: int, N: int, dt: int = OUT_BF16, ws=None,
                   stream=None):
     """Q = X^ Wq^^T and K = X^ Wk^^T on MXFP8 operands from fp4q_mxfp8_quantize1d."""
-    if ws is None:
-        ws = alloc_workspace(xq.device)
     return _host().mxfp8_qk(xq, xs, wq_q, wq_s, wk_q, wk_s, T, K, N, dt, ws, _handle(stream))

@@ -4,14 +4,17 @@
 // pointers: 20 us for a quantizer call and 18 us for a product, of which the launch itself is about 3.  These functions
 // take the Python arguments as they are, allocate the outputs, and call the C entry points through the addresses that
 // binding.py hands over once (so that a library chosen by FP4Q_LIB stays the one that is used): 8 and 7 us.  No state is
-// kept from one call to the next.
+// kept from one call to the next.  Whatever a call allocates or clears is allocated and cleared in the order of the stream that
+// its kernels run in (OnStream).
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
 #include <algorithm>
+#include <optional>
 #include <vector>
 
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -35,6 +38,7 @@ struct Entry {
     decltype(&fp4q_gemm_wgrad_act1d) gemm_wgrad_act1d;
     decltype(&fp4q_mxfp8_qk) mxfp8_qk;
     decltype(&fp4q_mxfp8_gemm) mxfp8_gemm;
+    decltype(&fp4q_workspace_bytes) workspace_bytes;
 } lib;
 
 PyObject *g_qtensor = nullptr, *g_fail = nullptr;   // binding.QTensor; binding._check
@@ -94,10 +98,36 @@ const at::Tensor &as_tensor(PyObject *o)
     if (!THPVariable_Check(o)) { PyErr_Format(PyExc_TypeError, "expected a tensor, got %s", Py_TYPE(o)->tp_name); throw PyError(); }
     return THPVariable_Unpack(o);
 }
-void *as_stream(PyObject *o)   // None: the current stream of the current device
-{
-    return o == Py_None ? (void *)c10::cuda::getCurrentCUDAStream().stream() : PyLong_AsVoidPtr(o);
-}
+// The stream a call runs in: the current stream of the current device (None) or another one, given by its handle.  In the
+// second case that stream is made current while the call lasts: outputs, their zero fill and the default workspace belong to its
+// order and, freed, to its pool.  What the call returns is also recorded for the caller's stream, where it is likely to be
+// read and dropped.
+struct OnStream {
+    void *handle;
+    std::optional<c10::cuda::CUDAStream> caller;
+    std::optional<c10::cuda::CUDAStreamGuard> guard;
+    OnStream(PyObject *o, const at::Tensor *like)
+    {
+        if (o == Py_None) {
+            handle = c10::cuda::getCurrentCUDAStream().stream();
+            return;
+        }
+        handle = PyLong_AsVoidPtr(o);
+        if (PyErr_Occurred()) throw PyError();
+        if (!like || !like->is_cuda()) return;
+        const auto device = like->device().index();
+        const auto raw = handle == (void *)cudaStreamLegacy ? nullptr : static_cast<cudaStream_t>(handle);
+        const auto now = c10::cuda::getCurrentCUDAStream(device);
+        if (raw == now.stream()) return;
+        caller.emplace(now);
+        guard.emplace(c10::cuda::getStreamFromExternal(raw, device));
+    }
+    const at::Tensor &returned(const at::Tensor &t) const
+    {
+        if (caller && t.defined()) t.record_stream(caller->unwrap());
+        return t;
+    }
+};
 uint8_t *bytes_of(const at::Tensor &t) { return static_cast<uint8_t *>(t.data_ptr()); }
 
 // Error status: binding._check raises.
@@ -124,17 +154,25 @@ const at::Tensor &as_matrix(PyObject *o, const char *name, const char *what)
     if (x.scalar_type() != at::kBFloat16 || x.dim() != 2 || (x.numel() && x.stride(1) != 1)) value_error(what);
     return x;
 }
+// The caller's workspace, or one that lasts for this call: its memory is reused in the order of the call's stream.
+at::Tensor workspace(PyObject *o, const at::Tensor &like)
+{
+    if (o != Py_None) return as_tensor(o);
+    Unlock u;
+    return at::zeros({(int64_t)lib.workspace_bytes()}, at::TensorOptions().dtype(at::kByte).device(like.device()));
+}
 const char kXText[] = "x must be a 2-D BF16 tensor with contiguous rows";
 int64_t pitch(const at::Tensor &x) { return x.size(0) ? x.stride(0) : x.size(1); }
 
 // Leading dimensions the C interface asks for, as in binding.alloc_qtensor.
 struct QBuffers { at::Tensor q_rm, q_t, scale; };
-QBuffers alloc_q(int64_t rows, int64_t cols, const at::Tensor &like, bool want_t, int64_t g)
+QBuffers alloc_q(const OnStream &on, int64_t rows, int64_t cols, const at::Tensor &like, bool want_t, int64_t g)
 {
     QBuffers b;
     b.q_rm = empty2(rows, std::max<int64_t>(pad16(ceil_to(cols, 32) * 16), 16), at::kByte, like);
     if (want_t) b.q_t = empty2(cols, std::max<int64_t>(pad16(ceil_to(rows, 32) * 16), 16), at::kByte, like);
     b.scale = empty2(ceil_to(rows, g), std::max<int64_t>(ceil_to(cols, g), 1), at::kByte, like);
+    for (const at::Tensor *t : {&b.q_rm, &b.q_t, &b.scale}) on.returned(*t);
     return b;
 }
 fp4q_tensor c_tensor(int64_t rows, int64_t cols, const at::Tensor &q_rm, const at::Tensor &q_t, const at::Tensor &scale)
@@ -179,10 +217,11 @@ at::Tensor qtensor_payload(PyObject *q)
 }
 
 // An output matrix: rows padded to whole 16 bytes, the padding cut off the returned view.
-at::Tensor out_buffer(int64_t rows, int64_t cols, int dt, const at::Tensor &like)
+at::Tensor out_buffer(const OnStream &on, int64_t rows, int64_t cols, int dt, const at::Tensor &like)
 {
     const int64_t per16 = dt == FP4Q_OUT_BF16 ? 8 : 4, ld = std::max(ceil_to(cols, per16) * per16, per16);
     at::Tensor t = empty2(rows, ld, dt == FP4Q_OUT_BF16 ? at::kBFloat16 : at::kFloat, like);
+    on.returned(t);
     return ld == cols ? t : t.slice(1, 0, cols);
 }
 int64_t out_pitch(const at::Tensor &out, int64_t cols) { return out.numel() ? out.stride(0) : cols; }
@@ -218,16 +257,17 @@ PyObject *quantize2d(Args a, Py_ssize_t n)
     const int64_t rows = x.size(0), cols = x.size(1);
     const uint32_t flags = (uint32_t)as_bits(a[5]);
     const int64_t g = (flags & FP4Q_BLOCK_16) ? 16 : 32;
+    const OnStream on(a[7], &x);
     fp4q_tensor t;
     QBuffers b;
     if (a[1] == Py_None) {
-        b = alloc_q(rows, cols, x, as_bool(a[6]), g);
+        b = alloc_q(on, rows, cols, x, as_bool(a[6]), g);
         t = c_tensor(rows, cols, b.q_rm, b.q_t, b.scale);
     } else {
         t = from_qtensor(a[1], 0);
     }
     check(unlocked(lib.quantize2d, x.data_ptr(), rows, cols, pitch(x), &t, (fp4q_round)as_int(a[2]), as_bits(a[3]), (uint32_t)as_bits(a[4]), flags,
-                         as_stream(a[7])), "fp4q_quantize2d");
+                         on.handle), "fp4q_quantize2d");
     return a[1] == Py_None ? new_qtensor(rows, cols, b, g) : Py_NewRef(a[1]);
 }
 
@@ -245,6 +285,7 @@ PyObject *quantize2d_multi(Args a, Py_ssize_t n)
         PyErr_SetString(PyExc_IndexError, "list index out of range");
         throw PyError();
     }
+    const OnStream on(a[7], k > 0 ? &as_tensor(PySequence_Fast_GET_ITEM(xs.p, 0)) : nullptr);
     std::vector<fp4q_tensor> ts((size_t)k);
     std::vector<fp4q_quantize_job> jobs((size_t)(k > 0 ? k : 1));
     for (Py_ssize_t j = 0; j < k; j++) {
@@ -252,7 +293,7 @@ PyObject *quantize2d_multi(Args a, Py_ssize_t n)
         snprintf(name, sizeof name, "xs[%zd]", j);
         const at::Tensor &x = as_matrix(PySequence_Fast_GET_ITEM(xs.p, j), name, "every input must be a 2-D BF16 tensor with contiguous rows");
         if (own) {
-            const QBuffers b = alloc_q(x.size(0), x.size(1), x, want_t, 32);
+            const QBuffers b = alloc_q(on, x.size(0), x.size(1), x, want_t, 32);
             Ref q(new_qtensor(x.size(0), x.size(1), b, 32));
             if (PyList_Append(outs.p, q.p) < 0) throw PyError();
             ts[j] = c_tensor(x.size(0), x.size(1), b.q_rm, b.q_t, b.scale);
@@ -265,13 +306,13 @@ PyObject *quantize2d_multi(Args a, Py_ssize_t n)
         jobs[j].tensor_id = a[4] == Py_None ? (uint32_t)j : id_at(a[4], j);
         jobs[j].flags = flags;
     }
-    check(unlocked(lib.quantize2d_multi, jobs.data(), (int32_t)k, (fp4q_round)as_int(a[2]), as_bits(a[3]), as_stream(a[7])), "fp4q_quantize2d_multi");
+    check(unlocked(lib.quantize2d_multi, jobs.data(), (int32_t)k, (fp4q_round)as_int(a[2]), as_bits(a[3]), on.handle), "fp4q_quantize2d_multi");
     return own ? Py_NewRef(outs.p) : Py_NewRef(a[1]);
 }
 
-PyObject *pair(const at::Tensor &q, const at::Tensor &s)
+PyObject *pair(const OnStream &on, const at::Tensor &q, const at::Tensor &s)
 {
-    Ref x(THPVariable_Wrap(q)), y(THPVariable_Wrap(s));
+    Ref x(THPVariable_Wrap(on.returned(q))), y(THPVariable_Wrap(on.returned(s)));
     return PyTuple_Pack(2, x.p, y.p);
 }
 
@@ -282,12 +323,13 @@ PyObject *mxfp8_quantize1d(Args a, Py_ssize_t n)
     want(n, 2);
     const at::Tensor &x = as_matrix(a[0], "x", kXText);
     const int64_t rows = x.size(0), cols = x.size(1), along = T ? rows : cols, across = T ? cols : rows;
+    const OnStream on(a[1], &x);
     const at::Tensor q = empty2(across, std::max<int64_t>(ceil_to(along, 32) * 32, 32), at::kByte, x);
     const at::Tensor s = empty2(across, std::max<int64_t>(ceil_to(along, 32), 1), at::kByte, x);
     check(unlocked(T ? lib.mxfp8_quantize1d_t : lib.mxfp8_quantize1d, x.data_ptr(), rows, cols, pitch(x), bytes_of(q), q.stride(0), bytes_of(s),
-                                                              s.stride(0), as_stream(a[1])),
+                                                              s.stride(0), on.handle),
           T ? "fp4q_mxfp8_quantize1d_t" : "fp4q_mxfp8_quantize1d");
-    return pair(q, s);
+    return pair(on, q, s);
 }
 
 // x, mode, seed, tensor_id, stream
@@ -296,11 +338,12 @@ PyObject *quantize1d(Args a, Py_ssize_t n)
     want(n, 5);
     const at::Tensor &x = as_matrix(a[0], "x", kXText);
     const int64_t rows = x.size(0), cols = x.size(1);
+    const OnStream on(a[4], &x);
     const at::Tensor q = empty2(rows, std::max<int64_t>(pad16(ceil_to(cols, 32) * 16), 16), at::kByte, x);
     const at::Tensor s = empty2(rows, std::max<int64_t>(ceil_to(cols, 32), 1), at::kByte, x);
     check(unlocked(lib.quantize1d, x.data_ptr(), rows, cols, pitch(x), bytes_of(q), q.stride(0), bytes_of(s), s.stride(0), (fp4q_round)as_int(a[1]),
-                         as_bits(a[2]), (uint32_t)as_bits(a[3]), as_stream(a[4])), "fp4q_quantize1d");
-    return pair(q, s);
+                         as_bits(a[2]), (uint32_t)as_bits(a[3]), on.handle), "fp4q_quantize1d");
+    return pair(on, q, s);
 }
 
 // x, stream
@@ -309,79 +352,84 @@ PyObject *quantize1d_t(Args a, Py_ssize_t n)
     want(n, 2);
     const at::Tensor &x = as_matrix(a[0], "x", kXText);
     const int64_t rows = x.size(0), cols = x.size(1);
+    const OnStream on(a[1], &x);
     const at::Tensor q = empty2(cols, std::max<int64_t>(pad16(ceil_to(rows, 32) * 16), 16), at::kByte, x);
     const at::Tensor s = empty2(cols, std::max<int64_t>(ceil_to(rows, 32), 1), at::kByte, x);
-    check(unlocked(lib.quantize1d_t, x.data_ptr(), rows, cols, pitch(x), bytes_of(q), q.stride(0), bytes_of(s), s.stride(0), as_stream(a[1])),
+    check(unlocked(lib.quantize1d_t, x.data_ptr(), rows, cols, pitch(x), bytes_of(q), q.stride(0), bytes_of(s), s.stride(0), on.handle),
           "fp4q_quantize1d_t");
-    return pair(q, s);
+    return pair(on, q, s);
 }
 
-// which (0 fwd, 1 dgrad, 2 wgrad), a, b, out_rows, out_cols, out | None, dt, accumulate, row_offsets | None, row_alignment, ws, stream
+// which (0 fwd, 1 dgrad, 2 wgrad), a, b, out_rows, out_cols, out | None, dt, accumulate, row_offsets | None, row_alignment, ws | None, stream
 PyObject *gemm(Args a, Py_ssize_t n)
 {
     want(n, 12);
     static const char *const names[3] = {"fp4q_gemm_fwd", "fp4q_gemm_dgrad", "fp4q_gemm_wgrad"};
     const int which = as_int(a[0]), dt = as_int(a[6]);
     const int64_t rows = as_i64(a[3]), cols = as_i64(a[4]);
-    const at::Tensor out = a[5] == Py_None ? out_buffer(rows, cols, dt, qtensor_payload(a[1])) : as_tensor(a[5]);
+    const at::Tensor like = qtensor_payload(a[1]);
+    const OnStream on(a[11], &like);
+    const at::Tensor out = a[5] == Py_None ? out_buffer(on, rows, cols, dt, like) : as_tensor(a[5]);
     const fp4q_tensor ta = from_qtensor(a[1], 32), tb = from_qtensor(a[2], 32);
     const Groups g(a[8], as_int(a[9]));
-    const at::Tensor &ws = as_tensor(a[10]);
-    void *st = as_stream(a[11]);
+    const at::Tensor ws = workspace(a[10], like);
     const int64_t ld = out_pitch(out, cols);
     const fp4q_status s =
-        which == 2 ? unlocked(lib.gemm_wgrad, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, as_int(a[7]), g.ptr, ws.data_ptr(), (size_t)ws.numel(), st)
+        which == 2 ? unlocked(lib.gemm_wgrad, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, as_int(a[7]), g.ptr, ws.data_ptr(), (size_t)ws.numel(), on.handle)
                    : unlocked(which == 1 ? lib.gemm_dgrad : lib.gemm_fwd, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, g.ptr, ws.data_ptr(),
-                                                                  (size_t)ws.numel(), st);
+                                                                  (size_t)ws.numel(), on.handle);
     check(s, names[which]);
     return a[5] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[5]);
 }
 
-// which, a, b, out_rows, out_cols, out | None, dt, accumulate, ws, stream
+// which, a, b, out_rows, out_cols, out | None, dt, accumulate, ws | None, stream
 PyObject *gemm_b16(Args a, Py_ssize_t n)
 {
     want(n, 10);
     static const char *const names[3] = {"fp4q_gemm_fwd_b16", "fp4q_gemm_dgrad_b16", "fp4q_gemm_wgrad_b16"};
     const int which = as_int(a[0]), dt = as_int(a[6]), accumulate = as_int(a[7]);
     const int64_t rows = as_i64(a[3]), cols = as_i64(a[4]);
-    const at::Tensor out = a[5] == Py_None ? out_buffer(rows, cols, dt, qtensor_payload(a[1])) : as_tensor(a[5]);
+    const at::Tensor like = qtensor_payload(a[1]);
+    const OnStream on(a[9], &like);
+    const at::Tensor out = a[5] == Py_None ? out_buffer(on, rows, cols, dt, like) : as_tensor(a[5]);
     if (a[5] == Py_None && accumulate) out.zero_();
     const fp4q_tensor ta = from_qtensor(a[1], 16), tb = from_qtensor(a[2], 16);
-    const at::Tensor &ws = as_tensor(a[8]);
-    void *st = as_stream(a[9]);
+    const at::Tensor ws = workspace(a[8], like);
     const int64_t ld = out_pitch(out, cols);
     const fp4q_status s =
-        which == 2 ? unlocked(lib.gemm_wgrad_b16, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, accumulate, ws.data_ptr(), (size_t)ws.numel(), st)
+        which == 2 ? unlocked(lib.gemm_wgrad_b16, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, accumulate, ws.data_ptr(), (size_t)ws.numel(), on.handle)
                    : unlocked(which == 1 ? lib.gemm_dgrad_b16 : lib.gemm_fwd_b16, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, ws.data_ptr(),
-                                                                          (size_t)ws.numel(), st);
+                                                                          (size_t)ws.numel(), on.handle);
     check(s, names[which]);
     return a[5] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[5]);
 }
 
-// which (0 fwd, 1 dgrad), a, b, out_rows, out_cols, out | None, mode, seed, tensor_id, want_t, row_offsets | None, ws, stream
+// which (0 fwd, 1 dgrad), a, b, out_rows, out_cols, out | None, mode, seed, tensor_id, want_t, row_offsets | None, ws | None, stream
 PyObject *gemm_quantized(Args a, Py_ssize_t n)
 {
     want(n, 13);
     const int which = as_int(a[0]);
     const Groups g(a[10], 256);
     const int64_t rows = as_i64(a[3]), cols = as_i64(a[4]);
+    const at::Tensor like = qtensor_payload(a[1]);
+    const OnStream on(a[12], &like);
     QBuffers b;
     fp4q_tensor tc;
     if (a[5] == Py_None) {
-        b = alloc_q(rows, cols, qtensor_payload(a[1]), as_bool(a[9]), 32);
+        b = alloc_q(on, rows, cols, like, as_bool(a[9]), 32);
         tc = c_tensor(rows, cols, b.q_rm, b.q_t, b.scale);
     }
     const fp4q_tensor ta = from_qtensor(a[1], 32), tb = from_qtensor(a[2], 32);
     if (a[5] != Py_None) tc = from_qtensor(a[5], 32);
-    const at::Tensor &ws = as_tensor(a[11]);
+    const at::Tensor ws = workspace(a[11], like);
     check(unlocked(which ? lib.gemm_dgrad_quantized : lib.gemm_fwd_quantized, &ta, &tb, &tc, (fp4q_round)as_int(a[6]), as_bits(a[7]),
                                                                       (uint32_t)as_bits(a[8]), g.ptr, ws.data_ptr(), (size_t)ws.numel(),
-                                                                      as_stream(a[12])),
+                                                                      on.handle),
           which ? "fp4q_gemm_dgrad_quantized" : "fp4q_gemm_fwd_quantized");
     return a[5] == Py_None ? new_qtensor(rows, cols, b, 32) : Py_NewRef(a[5]);
 }
 
-// xq, xs, T, W, out | None, dt, ws, stream
+// xq, xs, T, W, out | None, dt, ws | None, stream
 PyObject *gemm_fwd_act1d(Args a, Py_ssize_t n)
 {
     want(n, 8);
@@ -389,15 +437,16 @@ PyObject *gemm_fwd_act1d(Args a, Py_ssize_t n)
     const int64_t T = as_i64(a[2]);
     const int dt = as_int(a[5]);
     Ref wr(PyObject_GetAttr(a[3], s_rows));
-    const at::Tensor out = a[4] == Py_None ? out_buffer(T, as_i64(wr.p), dt, xq) : as_tensor(a[4]);
+    const OnStream on(a[7], &xq);
+    const at::Tensor out = a[4] == Py_None ? out_buffer(on, T, as_i64(wr.p), dt, xq) : as_tensor(a[4]);
     const fp4q_tensor w = from_qtensor(a[3], 32);
-    const at::Tensor &ws = as_tensor(a[6]);
+    const at::Tensor ws = workspace(a[6], xq);
     check(unlocked(lib.gemm_fwd_act1d, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), T, &w, out.data_ptr(), out.stride(0), (fp4q_out)dt,
-                             ws.data_ptr(), (size_t)ws.numel(), as_stream(a[7])), "fp4q_gemm_fwd_act1d");
+                             ws.data_ptr(), (size_t)ws.numel(), on.handle), "fp4q_gemm_fwd_act1d");
     return a[4] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[4]);
 }
 
-// dY, xtq, xts, K, out | None, dt, accumulate, ws, stream
+// dY, xtq, xts, K, out | None, dt, accumulate, ws | None, stream
 PyObject *gemm_wgrad_act1d(Args a, Py_ssize_t n)
 {
     want(n, 9);
@@ -405,31 +454,33 @@ PyObject *gemm_wgrad_act1d(Args a, Py_ssize_t n)
     const int64_t K = as_i64(a[3]);
     const int dt = as_int(a[5]), accumulate = as_bool(a[6]) ? 1 : 0;
     Ref dc(PyObject_GetAttr(a[0], s_cols));
-    const at::Tensor out = a[4] == Py_None ? out_buffer(as_i64(dc.p), K, dt, xq) : as_tensor(a[4]);
+    const OnStream on(a[8], &xq);
+    const at::Tensor out = a[4] == Py_None ? out_buffer(on, as_i64(dc.p), K, dt, xq) : as_tensor(a[4]);
     if (a[4] == Py_None && accumulate) out.zero_();
     const fp4q_tensor d = from_qtensor(a[0], 32);
-    const at::Tensor &ws = as_tensor(a[7]);
+    const at::Tensor ws = workspace(a[7], xq);
     check(unlocked(lib.gemm_wgrad_act1d, &d, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), K, out.data_ptr(), out.stride(0), (fp4q_out)dt,
-                               accumulate, ws.data_ptr(), (size_t)ws.numel(), as_stream(a[8])), "fp4q_gemm_wgrad_act1d");
+                               accumulate, ws.data_ptr(), (size_t)ws.numel(), on.handle), "fp4q_gemm_wgrad_act1d");
     return a[4] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[4]);
 }
 
-// aq, as, bq, bs, M, N, K, dt, ws, stream
+// aq, as, bq, bs, M, N, K, dt, ws | None, stream
 PyObject *mxfp8_gemm(Args a, Py_ssize_t n)
 {
     want(n, 10);
     const at::Tensor &aq = as_tensor(a[0]), &as = as_tensor(a[1]), &bq = as_tensor(a[2]), &bs = as_tensor(a[3]);
     const int64_t M = as_i64(a[4]), N = as_i64(a[5]), K = as_i64(a[6]);
     const int dt = as_int(a[7]);
-    const at::Tensor out = out_buffer(M, N, dt, aq);
-    const at::Tensor &ws = as_tensor(a[8]);
+    const OnStream on(a[9], &aq);
+    const at::Tensor out = out_buffer(on, M, N, dt, aq);
+    const at::Tensor ws = workspace(a[8], aq);
     const int64_t per16 = dt == FP4Q_OUT_BF16 ? 8 : 4, ld = std::max(ceil_to(N, per16) * per16, per16);
     check(unlocked(lib.mxfp8_gemm, bytes_of(aq), aq.stride(0), bytes_of(as), as.stride(0), M, bytes_of(bq), bq.stride(0), bytes_of(bs), bs.stride(0), N,
-                         K, out.data_ptr(), ld, (fp4q_out)dt, ws.data_ptr(), (size_t)ws.numel(), as_stream(a[9])), "fp4q_mxfp8_gemm");
+                         K, out.data_ptr(), ld, (fp4q_out)dt, ws.data_ptr(), (size_t)ws.numel(), on.handle), "fp4q_mxfp8_gemm");
     return THPVariable_Wrap(out);
 }
 
-// xq, xs, wq_q | None, wq_s | None, wk_q | None, wk_s | None, T, K, N, dt, ws, stream
+// xq, xs, wq_q | None, wq_s | None, wk_q | None, wk_s | None, T, K, N, dt, ws | None, stream
 PyObject *mxfp8_qk(Args a, Py_ssize_t n)
 {
     want(n, 12);
@@ -443,14 +494,15 @@ PyObject *mxfp8_qk(Args a, Py_ssize_t n)
     const int64_t T = as_i64(a[6]), K = as_i64(a[7]), N = as_i64(a[8]);
     const int dt = as_int(a[9]);
     const int64_t per16 = dt == FP4Q_OUT_BF16 ? 8 : 4, ld = std::max(ceil_to(N, per16) * per16, per16);
+    const OnStream on(a[11], &xq);
     at::Tensor out[2];
-    for (int i = 0; i < 2; i++) if (w[2 * i].defined()) out[i] = out_buffer(T, N, dt, xq);
+    for (int i = 0; i < 2; i++) if (w[2 * i].defined()) out[i] = out_buffer(on, T, N, dt, xq);
     const at::Tensor &wref = w[0].defined() ? w[0] : w[2], &sref = w[0].defined() ? w[1] : w[3];
     if (!wref.defined() || !sref.defined()) { PyErr_SetString(PyExc_AttributeError, "'NoneType' object has no attribute 'stride'"); throw PyError(); }
-    const at::Tensor &ws = as_tensor(a[10]);
+    const at::Tensor ws = workspace(a[10], xq);
     check(unlocked(lib.mxfp8_qk, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), T, K, p[0], p[1], p[2], p[3], wref.stride(0), sref.stride(0), N,
                        out[0].defined() ? out[0].data_ptr() : nullptr, out[1].defined() ? out[1].data_ptr() : nullptr, ld, (fp4q_out)dt,
-                       ws.data_ptr(), (size_t)ws.numel(), as_stream(a[11])), "fp4q_mxfp8_qk");
+                       ws.data_ptr(), (size_t)ws.numel(), on.handle), "fp4q_mxfp8_qk");
     Ref q(out[0].defined() ? THPVariable_Wrap(out[0]) : Py_NewRef(Py_None)), k(out[1].defined() ? THPVariable_Wrap(out[1]) : Py_NewRef(Py_None));
     return PyTuple_Pack(2, q.p, k.p);
 }
@@ -486,6 +538,7 @@ PyObject *init(Args a, Py_ssize_t n)
     set_entry(a[0], "fp4q_gemm_wgrad_act1d", lib.gemm_wgrad_act1d);
     set_entry(a[0], "fp4q_mxfp8_qk", lib.mxfp8_qk);
     set_entry(a[0], "fp4q_mxfp8_gemm", lib.mxfp8_gemm);
+    set_entry(a[0], "fp4q_workspace_bytes", lib.workspace_bytes);
     Py_XSETREF(g_qtensor, Py_NewRef(a[1]));
     Py_XSETREF(g_fail, Py_NewRef(a[2]));
     return Py_NewRef(Py_None);
