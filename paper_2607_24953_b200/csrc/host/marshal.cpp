@@ -365,17 +365,18 @@ PyObject *gemm(Args a, Py_ssize_t n)
 {
     want(n, 12);
     static const char *const names[3] = {"fp4q_gemm_fwd", "fp4q_gemm_dgrad", "fp4q_gemm_wgrad"};
-    const int which = as_int(a[0]), dt = as_int(a[6]);
+    const int which = as_int(a[0]), dt = as_int(a[6]), accumulate = as_int(a[7]);
     const int64_t rows = as_i64(a[3]), cols = as_i64(a[4]);
     const at::Tensor like = qtensor_payload(a[1]);
     const OnStream on(a[11], &like);
     const at::Tensor out = a[5] == Py_None ? out_buffer(on, rows, cols, dt, like) : as_tensor(a[5]);
+    if (a[5] == Py_None && accumulate) out.zero_();
     const fp4q_tensor ta = from_qtensor(a[1], 32), tb = from_qtensor(a[2], 32);
     const Groups g(a[8], as_int(a[9]));
     const at::Tensor ws = workspace(a[10], like);
     const int64_t ld = out_pitch(out, cols);
     const fp4q_status s =
-        which == 2 ? unlocked(lib.gemm_wgrad, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, as_int(a[7]), g.ptr, ws.data_ptr(), (size_t)ws.numel(), on.handle)
+        which == 2 ? unlocked(lib.gemm_wgrad, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, accumulate, g.ptr, ws.data_ptr(), (size_t)ws.numel(), on.handle)
                    : unlocked(which == 1 ? lib.gemm_dgrad : lib.gemm_fwd, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, g.ptr, ws.data_ptr(),
                                                                   (size_t)ws.numel(), on.handle);
     check(s, names[which]);

@@ -365,3 +365,16 @@ def test_mxfp8_scale_units(ws, T, N, K):
     torch.cuda.synchronize()
     assert binding.fp4q_workspace_status(ws) == 0
     check(y, (torch.from_numpy(xd).cuda() @ torch.from_numpy(wd).cuda().T).cpu().numpy(), "MXFP8 product")
+
+
+@pytest.mark.parametrize("grouped", [False, True])
+def test_accumulating_without_an_output_starts_from_zero(ws, grouped):
+    T, N, K = 384, 256, 320
+    qd, qx = (binding.fp4q_quantize2d(torch.randn(T, n, device="cuda").to(torch.bfloat16)) for n in (N, K))
+    offs = torch.tensor([0, 128, 384], device="cuda") if grouped else None
+    want = binding.fp4q_gemm_wgrad(qd, qx, row_offsets=offs, ws=ws)
+    dirty = [torch.full_like(want, 1e6) for _ in range(8)]          # the blocks that the next output of this size is one of
+    del dirty
+    got = binding.fp4q_gemm_wgrad(qd, qx, accumulate=True, row_offsets=offs, ws=ws)
+    torch.cuda.synchronize()
+    assert torch.equal(got, want)

@@ -30,6 +30,7 @@ def _calls():
         "gemm_fwd": lambda s: b.fp4q_gemm_fwd(qx, qw, stream=s),
         "gemm_dgrad": lambda s: b.fp4q_gemm_dgrad(qd, qw, stream=s),
         "gemm_wgrad": lambda s: b.fp4q_gemm_wgrad(qd, qx, stream=s),
+        "gemm_wgrad added": lambda s: b.fp4q_gemm_wgrad(qd, qx, accumulate=True, stream=s),
         "gemm_fwd grouped": lambda s: b.fp4q_gemm_fwd(qx, stack, row_offsets=offs, stream=s),
         "gemm_fwd_quantized": lambda s: fields(b.fp4q_gemm_fwd_quantized(qx, qw, stream=s)),
         "gemm_dgrad_quantized": lambda s: fields(b.fp4q_gemm_dgrad_quantized(qd, qw, seed=4, stream=s)),
