@@ -275,30 +275,32 @@ PyObject *quantize2d(Args a, Py_ssize_t n)
 PyObject *quantize2d_multi(Args a, Py_ssize_t n)
 {
     want(n, 8);
-    Ref xs(PySequence_Fast(a[0], "xs must be a sequence of tensors"));
-    const Py_ssize_t k = PySequence_Fast_GET_SIZE(xs.p);
+    // Copies of the lists: the loop below lets other threads and the caller's own attributes run, which may change them.
+    if (PyObject_Size(a[0]) < 0) throw PyError();
+    Ref xs(PySequence_Tuple(a[0]));
+    const Py_ssize_t k = PyTuple_GET_SIZE(xs.p);
     const bool own = a[1] == Py_None;
-    Ref outs(own ? PyList_New(0) : PySequence_Fast(a[1], "outs must be a sequence of QTensor"));
+    Ref outs(own ? PyList_New(0) : PySequence_Tuple(a[1]));
     const uint32_t flags = (uint32_t)as_bits(a[5]);
     const bool want_t = as_bool(a[6]);
-    if (!own && PySequence_Fast_GET_SIZE(outs.p) < k) {
+    if (!own && PyTuple_GET_SIZE(outs.p) < k) {
         PyErr_SetString(PyExc_IndexError, "list index out of range");
         throw PyError();
     }
-    const OnStream on(a[7], k > 0 ? &as_tensor(PySequence_Fast_GET_ITEM(xs.p, 0)) : nullptr);
+    const OnStream on(a[7], k > 0 ? &as_tensor(PyTuple_GET_ITEM(xs.p, 0)) : nullptr);
     std::vector<fp4q_tensor> ts((size_t)k);
     std::vector<fp4q_quantize_job> jobs((size_t)(k > 0 ? k : 1));
     for (Py_ssize_t j = 0; j < k; j++) {
         char name[32];
         snprintf(name, sizeof name, "xs[%zd]", j);
-        const at::Tensor &x = as_matrix(PySequence_Fast_GET_ITEM(xs.p, j), name, "every input must be a 2-D BF16 tensor with contiguous rows");
+        const at::Tensor &x = as_matrix(PyTuple_GET_ITEM(xs.p, j), name, "every input must be a 2-D BF16 tensor with contiguous rows");
         if (own) {
             const QBuffers b = alloc_q(on, x.size(0), x.size(1), x, want_t, 32);
             Ref q(new_qtensor(x.size(0), x.size(1), b, 32));
             if (PyList_Append(outs.p, q.p) < 0) throw PyError();
             ts[j] = c_tensor(x.size(0), x.size(1), b.q_rm, b.q_t, b.scale);
         } else {
-            ts[j] = from_qtensor(PySequence_Fast_GET_ITEM(outs.p, j), 32);
+            ts[j] = from_qtensor(PyTuple_GET_ITEM(outs.p, j), 32);
         }
         jobs[j].x_bf16 = x.data_ptr();
         jobs[j].rows = x.size(0); jobs[j].cols = x.size(1); jobs[j].ld_x = pitch(x);
@@ -306,6 +308,7 @@ PyObject *quantize2d_multi(Args a, Py_ssize_t n)
         jobs[j].tensor_id = a[4] == Py_None ? (uint32_t)j : id_at(a[4], j);
         jobs[j].flags = flags;
     }
+    for (Py_ssize_t j = k; !own && j < PyTuple_GET_SIZE(outs.p); j++) from_qtensor(PyTuple_GET_ITEM(outs.p, j), 32);   // refused as a whole
     check(unlocked(lib.quantize2d_multi, jobs.data(), (int32_t)k, (fp4q_round)as_int(a[2]), as_bits(a[3]), on.handle), "fp4q_quantize2d_multi");
     return own ? Py_NewRef(outs.p) : Py_NewRef(a[1]);
 }

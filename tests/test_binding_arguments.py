@@ -25,6 +25,38 @@ def test_other_things_than_whole_numbers_are_refused(what, value):
         binding.fp4q_quantize2d_multi([], stream=0, **{what: value})
 
 
+def test_lists_of_tensors_need_a_length():
+    with pytest.raises(TypeError):
+        binding.fp4q_quantize2d_multi((t for t in ()), stream=0)
+    assert binding.fp4q_quantize2d_multi((), outs=[], stream=0) == []
+    with pytest.raises(ValueError):       # a surplus output of the wrong granularity is refused like any other
+        binding.fp4q_quantize2d_multi([], outs=[binding.alloc_qtensor(32, 32, "cpu", True, 16)], stream=0)
+
+
+class _Meddling:
+    """A QTensor whose first reader empties the lists that the call was given."""
+
+    def __init__(self, q, lists):
+        self._q, self._lists = q, lists
+
+    def __getattr__(self, name):
+        for l in self._lists:
+            l.clear()
+        return getattr(self._q, name)
+
+
+@pytest.mark.gpu
+def test_lists_may_change_while_the_call_runs():
+    want = [torch.randn(96, 64, device="cuda").to(torch.bfloat16) for _ in range(3)]
+    ref = binding.fp4q_quantize2d_multi(want)
+    got = [binding.alloc_qtensor(96, 64, "cuda") for _ in want]
+    xs, ids, outs = [t.clone() for t in want], [0, 1, 2], []
+    outs += [_Meddling(got[0], [xs, outs])] + got[1:]
+    assert binding.fp4q_quantize2d_multi(xs, outs, tensor_ids=ids) is outs and not xs
+    for a, c in zip(ref, got):
+        assert torch.equal(a.q_rm, c.q_rm) and torch.equal(a.q_t, c.q_t) and torch.equal(a.scale, c.scale)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("ids", [np.arange(5, 7), torch.tensor([5, 6]), (5, np.int64(6)), range(5, 7), [5.0, "6"], {0: 5, 1: 6}])
 def test_tensor_ids_of_any_kind_name_the_same_rounding_streams(ids):
