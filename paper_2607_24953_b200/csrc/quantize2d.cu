@@ -9,9 +9,9 @@
 // hardware converts, the row-major payload goes straight to global memory (8 B per lane and row,
 // 64 B contiguous per row and warp) and the transposed payload is built with an in-register 8x8
 // nibble transpose, staged through 8 KB of shared memory and written as 64 B contiguous segments.
-// CTAs whose tile lies fully inside an aligned tensor run a check-free body, its ragged edges a general body with
-// the same arithmetic; tensors whose rows do not start on vector boundaries have a kernel that stages its tile
-// (quantize2d_staged_kernel).
+// CTAs whose tile lies fully inside a 32-byte aligned tensor run a check-free body, its ragged edges and tensors on 16-byte
+// boundaries a general body with the same arithmetic; tensors whose rows start anywhere have a kernel that stages its
+// tile (quantize2d_staged_kernel).
 //
 // Rounding: x 2^-e (exact in FP32) goes through the hardware converts cvt.rn.satfinite.e2m1x2.f32
 // (nearest even) or cvt.rs.satfinite.e2m1x4.f32 (stochastic).  The stochastic convert adds 16 random bits
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_kernel(
     if (!p.waits) wait_for_predecessor();
 }
 
-// Every tile of a tensor for which quantize2d_kernel has no check-free one.  Static shared memory (44 KB with the
+// Every tile of a tensor whose rows start anywhere or whose segments straddle Philox blocks.  Static shared memory (44 KB with the
 // transposed payload's staging) and 128 registers allow four CTAs per SM, like the aligned kernel.
 template <int MODE, int BLK = 32>
 __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_staged_kernel(const __grid_constant__ Quant2dParams p)
@@ -483,11 +483,14 @@ __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_staged_
 
 typedef void (*Quant2dKernel)(const Quant2dParams);
 
-// Rows on 32-byte boundaries and, with stochastic rounding, segments on Philox blocks: the kernel with the check-free
-// body.  Anything else is staged, except for the transposed index, whose random bytes run down the columns.
+// Rows on vector boundaries and, with stochastic rounding, segments on Philox blocks are read directly: on 32-byte boundaries
+// by the check-free body, on 16-byte ones by the general body's 128-bit loads.  Staging costs those more than it gives
+// (nearest / stochastic, us, direct and staged: 4096 x 4096 in a pitch of 4104 14.7 / 18.1 and 16.8 / 22.9, 16384 x 4096 40.9 /
+// 54.7 and 55.8 / 80.1, 4099 x 2728 nearest 14.9 and 14.7).  Anything else is staged, except for the transposed index, whose
+// random bytes run down the columns.
 static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr)
 {
-    const bool staged = !(p.x_vec_ok == 2 && p.rng_aligned) && !(sr && (p.flags & FP4Q_INDEX_TRANSPOSED));
+    const bool staged = !(p.x_vec_ok && p.rng_aligned) && !(sr && (p.flags & FP4Q_INDEX_TRANSPOSED));
     const int which = (p.flags & FP4Q_BLOCK_16) ? 1 : (p.flags & FP4Q_BLOCK_64) ? 2 : 0;
     static const Quant2dKernel kernels[2][2][3] = {
         {{quantize2d_kernel<FP4Q_ROUND_NEAREST>, quantize2d_kernel<FP4Q_ROUND_NEAREST, 16>, quantize2d_kernel<FP4Q_ROUND_NEAREST, 64>},

@@ -240,3 +240,20 @@ def test_rows_that_start_anywhere(rows, cols, pitch, offset, mode, block):
         o_s = np.repeat(np.repeat(o_s, 2, 0), 2, 1)[:s.shape[0], :s.shape[1]]
     assert np.array_equal(s, o_s)
     assert np.array_equal(qt.q_rm.cpu().numpy()[:, :(cols + 1) // 2], o_rm) and np.array_equal(qt.q_t.cpu().numpy()[:, :(rows + 1) // 2], o_t)
+
+
+@pytest.mark.parametrize("rows,cols,pitch,offset", [(129, 256, 264, 0), (300, 400, 408, 8), (160, 128, 136, 24), (64, 1000, 1000, 0), (33, 136, 144, 8)])
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("flags", [0, binding.BLOCK_16, binding.BLOCK_64, binding.INDEX_TRANSPOSED])
+def test_rows_on_16_byte_boundaries(rows, cols, pitch, offset, mode, flags):
+    # 128-bit loads, whole tiles and ragged ones; with cols % 16 != 0 the stochastic ones are staged
+    g = torch.Generator(device="cuda").manual_seed(rows + cols)
+    flat = torch.full((offset + rows * pitch + 64,), float("nan"), device="cuda", dtype=torch.bfloat16)
+    x = flat[offset:offset + rows * pitch].view(rows, pitch)[:, :cols]
+    x.copy_(torch.randn(rows, cols, generator=g, device="cuda"))
+    assert x.data_ptr() % 16 == 0
+    strided, packed = (gpu_quantize(t, mode, seed=8, tensor_id=2, flags=flags) for t in (x, x.contiguous()))
+    assert torch.equal(strided.q_rm, packed.q_rm) and torch.equal(strided.q_t, packed.q_t) and torch.equal(strided.scale, packed.scale)
+    if not flags & (binding.BLOCK_16 | binding.BLOCK_64):
+        o_rm, o_t, o_s = oracle.quantize2d(workloads.bf16_bits(x), mode, 8, 2, flags)
+        assert np.array_equal(strided.q_rm.cpu().numpy()[:, :(cols + 1) // 2], o_rm) and np.array_equal(strided.scale.cpu().numpy(), o_s)
