@@ -40,7 +40,7 @@ constexpr int BM = 128, BN = 256;            // per-CTA accumulator: 128 rows x 
 constexpr int kMaxStages = 6;
 constexpr int kAStageBytes = BM * 128;
 constexpr int kMaxGroupsShared = 1023;       // grouped contraction: boundaries kept in shared memory up to this many groups
-constexpr int kMaxGroupsSorted = 256;        // grouped contraction: groups are taken longest first up to this many
+constexpr int kMaxGroupsSorted = 256;        // grouped contraction: up to this many groups may be taken longest first (launch_gemm_impl says when)
 constexpr int kMaxRowTilesShared = 2048;     // grouped rows: group of each 128-row tile kept in shared memory up to this many tiles
 constexpr int kSmemTail = 512;               // barriers, TMEM base, abort flag, scale scratch (one per loader warp)
 // 2D-block scales: the scale images of a whole unit (up to 16 stages = 4096 contraction elements of one tile) are
@@ -185,6 +185,7 @@ struct GemmParams {
     const int64_t *row_offsets;
     int32_t b_rows_per_group;        // grouped rows: B row offset per group (forward)
     int32_t b_k_per_group;           // grouped rows: B contraction offset per group (dgrad)
+    int32_t sort_groups;             // grouped contraction: take the groups longest first
     uint32_t *status;
     // quantizing epilogue (EPI_QUANT): the output leaves as a 2D-block FP4 tensor instead of BF16/FP32
     uint8_t *q_rm, *q_t, *q_scale;
@@ -1129,10 +1130,9 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             reinterpret_cast<uint16_t *>(goffs_smem)[i] = (uint16_t)find_group(p.row_offsets, nullptr, p.n_groups, (int64_t)i * BM);
     const int32_t *goffs = goffs_ok ? goffs_smem : nullptr;
     // Grouped contraction: the groups longest first.  Their tiles go round the CTAs in turn, so that in any other order a CTA
-    // that meets several of the long ones finishes last (expert layer, 128 groups of
-    // 256 .. 15616 tokens in four random orders: 235-262 -> 222-226 us).
+    // that meets several of the long ones finishes last.
     uint16_t *gorder = nullptr;
-    if (goffs_ok && p.mode == MODE_GROUPED_K && p.n_groups <= kMaxGroupsSorted) {
+    if (goffs_ok && p.sort_groups) {
         gorder = reinterpret_cast<uint16_t *>(goffs_smem + kMaxGroupsShared + 1);
         __syncthreads();
         for (int g = threadIdx.x; g < p.n_groups; g += kThreads) {
@@ -1884,11 +1884,21 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
             return FP4Q_ERR_CUDA;
         attr_set[dev] = true;
     }
-    int slots = sm_count(dev) / CTAS;
+    int slots = sm_count(dev) / CTAS;   // CTAs or pairs that run at a time
 #ifdef FP4Q_TRACE
     if (const char *g = getenv("FP4Q_DEBUG_SLOTS")) slots = atoi(g);   // development only: use fewer SMs
 #endif
     const int grid = CTAS * (p.n_tile_total < slots ? p.n_tile_total : slots);
+    constexpr int kElems = kind_fp4(KIND) ? 256 : 128;
+    const int64_t tile_stages = ceil_div(p.K, kElems);   // a grouped contraction: of one output tile over all groups
+    const int64_t n_stages = p.mode == MODE_GROUPED_K ? (int64_t)p.m_tiles * p.n_tiles * (tile_stages + p.n_groups) : p.n_tile_total * tile_stages;
+    // Longest first costs every CTA a sort before its first load, quadratic in the groups (1.8 us at 128, 4.4 us at 256), and runs
+    // the groups that are bound by MMAs apart from those that are bound by output.  It pays for groups of two stages and more
+    // on average in products that last: at least half a stage a slot for every group.  us, as they come and longest first,
+    // Zipf lengths: 139520 rows x 768 x 2048 in 128 groups 244-248 / 239, 32768 in 64 103 / 98, 16384 in 32 55-57 / 53;
+    // below the line 65536 x 256 x 512 in 128 38 / 41, 131072 x 256 x 512 in 256 65-69 / 76, 4096 x 128 x 256 in 256 12 / 16.
+    p.sort_groups = p.mode == MODE_GROUPED_K && p.n_groups <= kMaxGroupsSorted && p.K >= 512 * (int64_t)p.n_groups &&
+                    2 * n_stages >= (int64_t)p.n_groups * slots;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(kThreads);
@@ -1898,9 +1908,6 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     // microbatch of five calls 111 -> 106 us, 16 x 16 blocks at 8192 x 2048 x 2048 134 -> 129 us).  Long ones do not: their CTAs
     // would be placed as SMs fall free instead of in order, and tiles that share operands end up far apart (all three products of
     // 16384 x 11008 x 4096 with their quantizers 1039 -> 1084 us, 1D activations at 8192 x 5632 x 2048 241 -> 251 us).
-    constexpr int kElems = kind_fp4(KIND) ? 256 : 128;
-    const int64_t tile_stages = ceil_div(p.K, kElems);   // a grouped contraction: of one output tile over all groups
-    const int64_t n_stages = p.mode == MODE_GROUPED_K ? (int64_t)p.m_tiles * p.n_tiles * (tile_stages + p.n_groups) : p.n_tile_total * tile_stages;
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
     if (CTAS == 2) {

@@ -378,3 +378,22 @@ def test_accumulating_without_an_output_starts_from_zero(ws, grouped):
     got = binding.fp4q_gemm_wgrad(qd, qx, accumulate=True, row_offsets=offs, ws=ws)
     torch.cuda.synchronize()
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("counts,N,K", [([0, 128, 2944, 1152], 768, 768), ([2944, 1152, 0, 128], 768, 768),
+                                        ([100, 300, 1200, 900, 0, 700, 5, 1300] * 32, 1024, 1024)])
+def test_grouped_weight_gradient_longest_groups_first(ws, counts, N, K):
+    # lengths and widths at which the groups are sorted.  Every 32 x 32 block holds whole numbers of the format up to 6, so
+    # that quantization, products and FP32 sums (below 2^24) are exact
+    offs = workloads.padded_row_offsets(np.array(counts), 128)
+    rows = int(offs[-1])
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    values = torch.tensor([0, 1, 2, 3, 4, 6, -1, -2, -3, -4, -6], device="cuda", dtype=torch.bfloat16)
+    x, dy = (values[torch.randint(0, 11, (rows, n), generator=g, device="cuda")] for n in (K, N))
+    x[::32, ::32], dy[::32, ::32] = 6, -6
+    qx, qd = binding.fp4q_quantize2d(x), binding.fp4q_quantize2d(dy)
+    got = binding.fp4q_gemm_wgrad(qd, qx, row_offsets=torch.from_numpy(offs).cuda(), ws=ws)
+    for e in range(len(counts)):
+        a, z = int(offs[e]), int(offs[e + 1])
+        assert torch.equal(got[e * N:(e + 1) * N], dy[a:z].float().T @ x[a:z].float()), e
+    assert binding.fp4q_workspace_status(ws) == 0
