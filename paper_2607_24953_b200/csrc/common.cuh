@@ -24,16 +24,27 @@ struct Workspace {
 };
 
 // Short launches overlap their predecessor's end: quantizers of up to kShortGrid CTAs and short products (launch_gemm_impl says
-// which) are launched as the programmatic dependents of the kernel before them in their stream (after a copy or a foreign
-// kernel the attribute changes nothing), so their CTAs may be placed, and set up barriers and tensor memory, while the last
-// CTAs of that kernel still run.  Before it touches global memory - reads an input or writes an output - every thread
-// waits until that kernel has completed and its writes are visible: streams keep their order.  A kernel lets its own successor
-// in only after that wait, so that whoever skips the wait (the later tensors of a multi-tensor quantizer call) still
+// which) are launched as the programmatic dependents of the kernel before them in their stream (behind a copy, or a kernel that
+// admits nobody before it ends, the attribute changes nothing), so their CTAs may be placed, and set up barriers and tensor memory,
+// while the last CTAs of that kernel still run.  Before it touches global memory - reads an input or writes an output - every
+// thread waits until that kernel has completed and its writes are visible: streams keep their order.  A kernel lets its own
+// successor in only after that wait, so that whoever skips the wait (the later tensors of a multi-tensor quantizer call) still
 // runs behind everything before the call.  What the predecessor wrote is read with ordinary loads: the non-coherent path
 // (ld.global.nc, __ldg) is for memory that nothing writes while the kernel runs, and a dependent kernel runs before its
-// inputs are complete.  Long grids do not take part: in a dependent launch the wait costs every CTA of the
-// grid, not only the first ones (expert layer with all quantizers dependent 1662 -> 1844 us).
-constexpr int64_t kShortGrid = 2 * 4 * 148;   // two waves of four CTAs per SM
+// inputs are complete.
+// A dependent quantizer takes places on the SMs that its predecessor's last wave still wants, so the line is one CTA per SM.
+// Passes of quantizers and products, none / up to 148 / up to 1184 CTAs dependent, us: 128 x 256 x 256 36.0 / 33.3 / 33.3,
+// 2048 x 2048 x 2048 51.6 / 51.6 / 53.4, 4096 x 4096 x 4096 151.3 / 151.3 / 156.7, 1D activations 8192 x 5632 x 2048 251.3 / 251.3 /
+// 259.0, MXFP8 512 x 1024 x 1024 18.8 / 14.9 / 14.9.  In a captured graph, whose launches cost less, dependent quantizers lose
+// (256 x 512 x 1024 33.3 without and 36.1 us with, expert layer of 1024 tokens 34.5 and 36.3): there they are not.
+constexpr int64_t kShortGrid = 148;
+inline bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus st;
+    if (cudaStreamIsCapturing(stream, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();   // the legacy stream beside another stream's capture: the launch itself will report it
+    return true;
+}
 // A launch of `kernel` with one parameter block; always: as a dependent whatever its size.
 template <typename P>
 inline cudaError_t launch_dependent(void (*kernel)(const P), dim3 grid, int threads, cudaStream_t stream, const P &p, bool always = false)
@@ -46,7 +57,7 @@ inline cudaError_t launch_dependent(void (*kernel)(const P), dim3 grid, int thre
     cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = always || (int64_t)grid.x * grid.y <= kShortGrid ? 1 : 0;
+    cfg.numAttrs = always || ((int64_t)grid.x * grid.y <= kShortGrid && !capturing(stream)) ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 #ifdef __CUDACC__

@@ -1904,10 +1904,13 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = Cfg<KIND, CTAS>::kSmemBytes;
     cfg.stream = static_cast<cudaStream_t>(stream);
-    // Short products start beside their predecessor's end (up to 48 stages, about 25 us, per CTA or pair: a 2048 x 4096 x 4096
-    // microbatch of five calls 111 -> 106 us, 16 x 16 blocks at 8192 x 2048 x 2048 134 -> 129 us).  Long ones do not: their CTAs
-    // would be placed as SMs fall free instead of in order, and tiles that share operands end up far apart (all three products of
-    // 16384 x 11008 x 4096 with their quantizers 1039 -> 1084 us, 1D activations at 8192 x 5632 x 2048 241 -> 251 us).
+    // Short products start beside their predecessor's end: up to 48 stages, about 25 us, per CTA or pair.  Passes of quantizers
+    // and products, without and with, us: 2048 x 4096 x 4096 (28 stages) 102.8 / 97.6, 1D activations 2048 x 4096 x 4096 32.5 / 29.3,
+    // 16 x 16 blocks 8192 x 2048 x 2048 134 / 129; nothing changes from 4096 x 4096 x 4096 (55 stages) on, except that CTAs of long
+    // products are placed as SMs fall free instead of in order, and tiles that share operands end up far apart (all three
+    // products of 16384 x 11008 x 4096 with their quantizers 1039 / 1084).  In a captured graph the one-CTA products of the smallest
+    // layers lose (4 experts of 512 tokens in all 31.7 / 33.4, 128 x 256 x 256 31.0 / 31.9) while the pairs gain
+    // (512 x 1024 x 1024 36.3 / 34.3), so only these take part there.
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
     if (CTAS == 2) {
@@ -1917,7 +1920,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
         attr[0].val.clusterDim.z = 1;
         cfg.numAttrs = 1;
     }
-    if (n_stages <= 48 * (int64_t)slots) {
+    if (n_stages <= 48 * (int64_t)slots && !(CTAS == 1 && capturing(cfg.stream))) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     }
