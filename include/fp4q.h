@@ -156,9 +156,9 @@ size_t fp4q_workspace_bytes(void);
  * are unspecified; the context stays usable and later calls are unaffected. */
 fp4q_status fp4q_workspace_status(void *ws, void *stream);
 
-/* Every wait inside the GEMM kernels is bounded by a number of polls (default 2^22, far beyond
- * anything a healthy run needs; the one wait that spans a whole tile scales it with the tile's
- * contraction length).  This call stores another limit in the workspace (0 restores the default);
+/* Every wait inside the GEMM kernels is bounded by a number of polls of at most about one
+ * microsecond each (default 2^22, i.e. four seconds at the latest, far beyond anything a healthy
+ * run needs; the one wait that spans a whole tile scales it with the tile's contraction length).  This call stores another limit in the workspace (0 restores the default);
  * it applies to every later call that uses the workspace.  Synchronises `stream`. */
 fp4q_status fp4q_workspace_set_wait_limit(void *ws, uint32_t polls, void *stream);
 

@@ -265,7 +265,7 @@ def fp4q_workspace_status(ws: torch.Tensor, stream=None) -> int:
 
 
 def fp4q_workspace_set_wait_limit(ws: torch.Tensor, polls: int, stream=None):
-    """Poll limit of the kernels' bounded waits for every later call that uses ws (0 = default)."""
+    """Poll limit of the kernels' bounded waits for every later call that uses ws (0 = default); a poll takes up to about 1 us."""
     _check(lib().fp4q_workspace_set_wait_limit(ws.data_ptr(), int(polls), _stream(stream)), "fp4q_workspace_set_wait_limit")
 
 

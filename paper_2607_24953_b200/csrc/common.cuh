@@ -18,7 +18,7 @@ static inline bool aligned(const void *p, size_t a) { return (reinterpret_cast<u
 struct Workspace {
     uint32_t status;         // 0 = ok, otherwise an fp4q_status written by a kernel
     uint32_t detail;         // where the kernel gave up (role/stage), for diagnostics
-    uint32_t wait_limit;     // polls after which a bounded wait gives up; 0 = the kernels' default
+    uint32_t wait_limit;     // polls (of up to about 1 us) after which a bounded wait gives up; 0 = the kernels' default
     uint32_t withhold_load;  // development hook, 0 in production: n > 0 = CTA 0 leaves out its n-th stage load
     uint32_t pad[60];
 };

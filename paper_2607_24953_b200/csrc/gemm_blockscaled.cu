@@ -134,6 +134,9 @@ template <int KIND> struct SfCols { static constexpr int kStride = KIND == KIND_
 static_assert(kTmemSfBase + 5 * SfCols<KIND_MXF4>::kStride <= kTmemCols && kTmemSfBase + 4 * SfCols<KIND_MXF4B16>::kStride <= kTmemCols,
               "tensor memory budget: 256 accumulator columns + one scale slot per ring stage");
 constexpr uint32_t kWaitLimit = 1u << 22;       // default number of polls after which a wait gives up (workspace word 2 overrides it)
+// Longest suspension of one suspending poll: without it the limit is the system's, and a number of polls bounds nothing.  With
+// 2^22 polls a wait gives up after about four seconds at the latest.
+constexpr uint32_t kSuspendNs = 1000;
 constexpr int kRelaxedNs = 64, kLazyNs = 256;   // back-off between polls of roles with slack
 // Developer diagnostic (off by default): -DFP4Q_TRACE makes CTA 0 add up clock64() intervals of its roles in
 // registers and leave them in the workspace's padding words (status[16 + 2*slot], 64-bit each).
@@ -220,8 +223,8 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.b32 %0, 1, 0, p;\n}"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.b32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(kSuspendNs) : "memory");
     return ok != 0;
 }
 
@@ -246,9 +249,9 @@ __device__ __forceinline__ bool elect_one()
 __device__ __forceinline__ void named_sync(uint32_t id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 
 // Bounded wait.  Returns false when the limit ran out (the timeout is then recorded) or when another
-// role of this CTA has already given up.  Every poll of an mbarrier is a shared-memory transaction that
-// competes with the tensor core's operand reads and with the MMA thread's own waits, so roles that have
-// slack (everything but the MMA issuer) sleep between polls.
+// role of this CTA has already given up, which it looks for after every suspension and after every 256th probe.  Every poll
+// of an mbarrier is a shared-memory transaction that competes with the tensor core's operand reads and with the other
+// roles' waits: a suspended thread makes one in kSuspendNs at most.
 template <int BACKOFF_NS, bool PROBE = false>
 __device__ __forceinline__ bool mbar_wait_impl(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status,
                                                uint64_t limit, uint32_t where)
@@ -256,7 +259,7 @@ __device__ __forceinline__ bool mbar_wait_impl(uint32_t bar, uint32_t parity, vo
     for (uint64_t it = 0; it < limit; it++) {
         if (PROBE ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity)) return true;
         if (BACKOFF_NS > 0) __nanosleep(BACKOFF_NS);
-        if (((uint32_t)it & 255u) == 255u && *abort_flag) return false;
+        if ((!PROBE || ((uint32_t)it & 255u) == 255u) && *abort_flag) return false;
     }
     *abort_flag = 1u;
     if (atomicCAS(status, 0u, (uint32_t)FP4Q_ERR_TIMEOUT) == 0u) status[1] = where;
@@ -272,13 +275,14 @@ __device__ __noinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity, vo
 {
     return mbar_wait_impl<kRelaxedNs>(bar, parity, abort_flag, status, limit, where);
 }
-__device__ __noinline__ bool mbar_wait_lazy(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status,
-                                            uint64_t limit, uint32_t where)
+// For the end of an aborted launch, when the abort flag is set already: 256 polls, a third of a millisecond at most.
+__device__ __noinline__ void mbar_drain(uint32_t bar)
 {
-    return mbar_wait_impl<kLazyNs>(bar, parity, abort_flag, status, limit, where);
+    for (int it = 0; it < 256 && !mbar_try_wait(bar, 0u); it++) __nanosleep(kLazyNs);
 }
-// For barriers that another CTA of the cluster completes (a multicast tcgen05.commit): probe instead of try_wait,
-// whose suspended thread is not reliably woken early by a remote arrival.
+// The builder of 2D-block images in a pair, whose buffers the leader's multicast commits release: probes with a back-off.
+// (Whether a remote arrival wakes a suspended thread is not specified; where the other roles suspend on such barriers, they
+// look again after kSuspendNs at the latest.)
 __device__ __noinline__ bool mbar_poll_relaxed(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status,
                                                uint64_t limit, uint32_t where)
 {
@@ -1332,7 +1336,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             // this warp has run through them.  Wait (bounded) until the tensor pipe is idle before tensor memory is freed.
             if (issuer) tcgen05_commit<CTAS>(bar_drain);
             __syncwarp();
-            if (lane == 0) mbar_wait_lazy(bar_drain, 0u, abort_flag, p.status, wait_limit, 0x220u);   // gives up after 256 polls (abort is set)
+            if (lane == 0) mbar_drain(bar_drain);
             __syncwarp();
             // After an abort the stages were consumed without waiting for their operands, so loads of either CTA may
             // still be on their way: hold the pair (the other roles wait at the final barrier) until they have landed.

@@ -66,3 +66,56 @@ def test_status_decoding_of_a_workspace_word():
     assert binding.fp4q_workspace_status(ws) == FP4Q_ERR_TIMEOUT
     assert int(ws.view(torch.int32)[0]) == 0
     assert binding.fp4q_workspace_status(ws) == 0
+
+
+def _products(ws):
+    """Every kind of kernel, by name."""
+    x, w, dy = (torch.randn(512, n, device="cuda").to(torch.bfloat16) for n in (1024, 1024, 512))
+    small, wide = x[:128].contiguous(), torch.randn(1024, 256, device="cuda").to(torch.bfloat16)
+    q, q16 = binding.fp4q_quantize2d, lambda t: binding.fp4q_quantize2d(t, flags=binding.BLOCK_16)
+    xq, xs = binding.fp4q_quantize1d(x)
+    tq, ts = binding.fp4q_quantize1d_t(wide)
+    x8, xs8 = binding.fp4q_mxfp8_quantize1d(x[:, :512].contiguous())
+    w8, ws8 = binding.fp4q_mxfp8_quantize1d(w[:, :512].contiguous())
+    qx, qw, qs, qwide = q(x), q(w), q(small), q(wide)
+    offs, row_offs = torch.tensor([0, 1024], device="cuda"), torch.tensor([0, 256, 512], device="cuda")
+    stack = q(torch.cat([w[:256], w[256:512]]))
+    return {
+        "dense one-CTA": lambda: binding.fp4q_gemm_fwd(qs, qw, ws=ws),
+        "grouped rows one-CTA": lambda: binding.fp4q_gemm_fwd(qx, stack, row_offsets=row_offs, ws=ws),
+        "grouped rows on pairs": lambda: binding.fp4q_gemm_fwd(qx, stack, row_offsets=row_offs, row_alignment=256, ws=ws),
+        "grouped weight gradient": lambda: binding.fp4q_gemm_wgrad(qwide, qwide, row_offsets=offs, ws=ws),
+        "quantizing epilogue": lambda: binding.fp4q_gemm_fwd_quantized(qx, qw, ws=ws).q_rm,
+        "1D activations": lambda: binding.fp4q_gemm_fwd_act1d(xq, xs, 512, qw, ws=ws),
+        "1D activations one-CTA": lambda: binding.fp4q_gemm_fwd_act1d(xq[:128], xs[:128], 128, qw, ws=ws),
+        "1D weight gradient": lambda: binding.fp4q_gemm_wgrad_act1d(qwide, tq, ts, 256, ws=ws),
+        "16 x 16 blocks": lambda: binding.fp4q_gemm_fwd_b16(q16(x), q16(w), ws=ws),
+        "16 x 16 blocks one-CTA": lambda: binding.fp4q_gemm_fwd_b16(q16(small), q16(w), ws=ws),
+        "MXFP8": lambda: binding.fp4q_mxfp8_gemm(x8, xs8, w8, ws8, 512, 512, 512, ws=ws),
+        "MXFP8 one-CTA": lambda: binding.fp4q_mxfp8_gemm(x8[:128], xs8[:128], w8, ws8, 128, 512, 512, ws=ws)}
+
+
+@pytest.mark.parametrize("name", [
+    "dense one-CTA", "grouped rows one-CTA", "grouped rows on pairs", "grouped weight gradient", "quantizing epilogue", "1D activations",
+    "1D activations one-CTA", "1D weight gradient", "16 x 16 blocks", "16 x 16 blocks one-CTA", "MXFP8", "MXFP8 one-CTA"])
+def test_every_kernel_leaves_through_its_timeout_path(name):
+    # four ring stages per CTA and one tile each, the third load withheld: the stage never completes and is not used again
+    ws = binding.alloc_workspace("cuda")
+    call = _products(ws)[name]
+    want = call().clone()
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
+    binding.fp4q_workspace_set_wait_limit(ws, 1 << 12)
+    binding.fp4q_debug_withhold_load(ws, 3)
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    start.record()
+    call()
+    end.record()
+    torch.cuda.synchronize()
+    # 2^12 polls of about a microsecond, once per role that has something to wait for, and 0.6 ms of waiting for copies
+    assert start.elapsed_time(end) < 200.0
+    assert binding.fp4q_workspace_status(ws) == FP4Q_ERR_TIMEOUT
+    binding.fp4q_debug_withhold_load(ws, 0)
+    binding.fp4q_workspace_set_wait_limit(ws, 0)
+    assert torch.equal(call(), want)
+    assert binding.fp4q_workspace_status(ws) == 0
