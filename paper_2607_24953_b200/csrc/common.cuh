@@ -60,6 +60,14 @@ inline cudaError_t launch_dependent(void (*kernel)(const P), dim3 grid, int thre
     cfg.numAttrs = always || ((int64_t)grid.x * grid.y <= kShortGrid && !capturing(stream)) ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, p);
 }
+// The status of a launch that returned e.  Only this launch counts, not an error that an earlier call of somebody else's left
+// behind, and its own error is not left for the next caller to find.
+inline fp4q_status launched(cudaError_t e)
+{
+    if (e == cudaSuccess) return FP4Q_OK;
+    cudaGetLastError();
+    return FP4Q_ERR_CUDA;
+}
 #ifdef __CUDACC__
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // An ordinary load; it stays below wait_for_predecessor(), which clobbers memory.

@@ -1928,7 +1928,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     }
-    return cudaLaunchKernelEx(&cfg, gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH>, tmA, tmB, tmC, tmD, p) == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
+    return launched(cudaLaunchKernelEx(&cfg, gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH>, tmA, tmB, tmC, tmD, p));
 }
 
 // Argument checks common to every product: everything that can be refused is refused here, before any work is enqueued.

@@ -324,8 +324,7 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d(const void *x_bf16, int64_t rows, i
     const int64_t total = rows * (p.segs_per_row / 2);
     const int64_t n_cta = ceil_div(total, 256);
     if (n_cta > 0x7FFFFFFF) return FP4Q_ERR_UNSUPPORTED;
-    launch_dependent(mxfp8_quantize1d_kernel, dim3((unsigned)n_cta), 256, static_cast<cudaStream_t>(stream), p);
-    return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
+    return launched(launch_dependent(mxfp8_quantize1d_kernel, dim3((unsigned)n_cta), 256, static_cast<cudaStream_t>(stream), p));
 }
 
 extern "C" fp4q_status fp4q_mxfp8_quantize1d_t(const void *x_bf16, int64_t rows, int64_t cols, int64_t ld_x,
@@ -347,11 +346,9 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d_t(const void *x_bf16, int64_t rows,
     // full 128x128 tiles and aligned rows: the tile kernel (coalesced 128-byte column stores)
     if (rows % 128 == 0 && cols % 128 == 0 && aligned(x_bf16, 32) && ld_x % 16 == 0 && ld_s % 4 == 0 && aligned(scale, 4) &&
         (rows / 128) * (cols / 128) <= 0x7FFFFFFF) {
-        launch_dependent(mxfp8_quantize1d_t_tile_kernel, dim3((unsigned)((rows / 128) * (cols / 128))), 128, static_cast<cudaStream_t>(stream), p);
-        return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
+        return launched(launch_dependent(mxfp8_quantize1d_t_tile_kernel, dim3((unsigned)((rows / 128) * (cols / 128))), 128, static_cast<cudaStream_t>(stream), p));
     }
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;
-    launch_dependent(mxfp8_quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p);
-    return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
+    return launched(launch_dependent(mxfp8_quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p));
 }

@@ -339,9 +339,8 @@ extern "C" fp4q_status fp4q_quantize1d(const void *x_bf16, int64_t rows, int64_t
     const int64_t n_cta = ceil_div(rows * (p.segs_per_row / 2), 256);
     if (n_cta > 0x7FFFFFFF) return FP4Q_ERR_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (mode == FP4Q_ROUND_STOCHASTIC) launch_dependent(quantize1d_kernel<FP4Q_ROUND_STOCHASTIC>, dim3((unsigned)n_cta), 256, s, p);
-    else launch_dependent(quantize1d_kernel<FP4Q_ROUND_NEAREST>, dim3((unsigned)n_cta), 256, s, p);
-    return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
+    return launched(launch_dependent(mode == FP4Q_ROUND_STOCHASTIC ? quantize1d_kernel<FP4Q_ROUND_STOCHASTIC> : quantize1d_kernel<FP4Q_ROUND_NEAREST>,
+                                     dim3((unsigned)n_cta), 256, s, p));
 }
 
 extern "C" fp4q_status fp4q_quantize1d_t(const void *x_bf16, int64_t rows, int64_t cols, int64_t ld_x, uint8_t *q, int64_t ld_q,
@@ -360,11 +359,9 @@ extern "C" fp4q_status fp4q_quantize1d_t(const void *x_bf16, int64_t rows, int64
     // full 128x128 tiles and aligned rows: the tile kernel (coalesced 64-byte column stores)
     if (rows % 128 == 0 && cols % 128 == 0 && aligned(x_bf16, 32) && ld_x % 16 == 0 && ld_s % 4 == 0 && aligned(scale, 4) &&
         (rows / 128) * (cols / 128) <= 0x7FFFFFFF) {
-        launch_dependent(quantize1d_t_tile_kernel, dim3((unsigned)((rows / 128) * (cols / 128))), 128, static_cast<cudaStream_t>(stream), p);
-        return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
+        return launched(launch_dependent(quantize1d_t_tile_kernel, dim3((unsigned)((rows / 128) * (cols / 128))), 128, static_cast<cudaStream_t>(stream), p));
     }
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;
-    launch_dependent(quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p);
-    return cudaGetLastError() == cudaSuccess ? FP4Q_OK : FP4Q_ERR_CUDA;
+    return launched(launch_dependent(quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p));
 }

@@ -552,8 +552,7 @@ extern "C" fp4q_status fp4q_quantize2d(const void *x_bf16, int64_t rows, int64_t
     if (n_cta == 0) return FP4Q_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     p.waits = 1;
-    return launch_dependent(quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC), dim3((unsigned)n_cta), 128, s, p) == cudaSuccess
-               ? FP4Q_OK : FP4Q_ERR_CUDA;
+    return launched(launch_dependent(quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC), dim3((unsigned)n_cta), 128, s, p));
 }
 
 extern "C" fp4q_status fp4q_quantize2d_multi(const fp4q_quantize_job *jobs, int32_t n_jobs, fp4q_round mode, uint64_t seed,
@@ -581,8 +580,8 @@ extern "C" fp4q_status fp4q_quantize2d_multi(const fp4q_quantize_job *jobs, int3
                            jobs[j].flags, p, &n_cta);
         if (n_cta == 0) continue;
         p.waits = first;
-        if (launch_dependent(quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC), dim3((unsigned)n_cta), 128, s, p, !first) != cudaSuccess)
-            return FP4Q_ERR_CUDA;
+        if (fp4q_status st = launched(launch_dependent(quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC), dim3((unsigned)n_cta), 128, s, p, !first)))
+            return st;
         first = false;
     }
     return FP4Q_OK;
