@@ -189,10 +189,14 @@ def _host():
     global _native
     if _native is None:
         L = lib()
+        path = os.path.join(_HERE, "_host.so")
+        hint = "run `python -m paper_2607_24953_b200.build` (there is no fallback path)"
+        if not os.path.exists(path):
+            raise ImportError("_host.so is not built: " + hint)
         try:
             from . import _host as module
         except ImportError as exc:
-            raise ImportError("_host.so is not built: run `python -m paper_2607_24953_b200.build` (there is no fallback path)") from exc
+            raise ImportError("%s does not load (%s); if it was built for another Python or torch, %s" % (path, exc, hint)) from exc
         module.init({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in EXPORTS}, QTensor, _check)
         _native = module
     return _native
