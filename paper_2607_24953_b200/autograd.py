@@ -43,7 +43,7 @@ def fp4_linear(x: torch.Tensor, weight: torch.Tensor, seed: int = 0, tensor_id: 
     `seed` / `tensor_id` key the stochastic rounding of the incoming gradient (change one of them every step)."""
     if ws is None:
         ws = binding.alloc_workspace(x.device)
-    if x.dim() == 2:   # nothing to fold: two autograd nodes less
+    if x.dim() == 2 and x.shape[1] != 0:   # nothing to fold: two autograd nodes less (reshape refuses rows of nothing)
         return _FP4LinearFn.apply(x, weight, seed, tensor_id, ws)
     lead = x.shape[:-1]
     y = _FP4LinearFn.apply(x.reshape(-1, x.shape[-1]), weight, seed, tensor_id, ws)

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2607_24953_b200 import binding
+from paper_2607_24953_b200 import autograd, binding
 
 
 @pytest.mark.parametrize("number", [np.int64(3), np.int32(3), np.uint8(3), torch.tensor(3), True, -1, 2 ** 70])
@@ -23,6 +23,11 @@ def test_rounding_modes_of_any_whole_number_type(mode):
 def test_other_things_than_whole_numbers_are_refused(what, value):
     with pytest.raises(TypeError):
         binding.fp4q_quantize2d_multi([], stream=0, **{what: value})
+
+
+def test_a_linear_layer_of_no_inputs_is_refused():
+    with pytest.raises(RuntimeError, match="reshape"):
+        autograd.fp4_linear(torch.empty(3, 0), torch.empty(4, 0), ws=torch.empty(0))
 
 
 def test_lists_of_tensors_need_a_length():
