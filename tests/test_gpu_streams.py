@@ -52,10 +52,13 @@ def test_a_side_stream_does_not_wait_for_the_current_one_nor_share_its_memory(by
     side = torch.cuda.Stream()
     for name, call in calls.items():
         want = [t.clone() for t in _tensors(call(None))]
-        call(side)                                          # kernels loaded, the side stream's pool has blocks
-        torch.cuda.synchronize()
         # blocks that the current stream's pool would hand out next, with work on them still to come
         dirty = [torch.empty_like(t) for t in want] + [torch.empty(b.fp4q_workspace_bytes(), dtype=torch.uint8, device="cuda")]
+        # everything once before: the first use of a kernel loads it, the first allocation grows the pool, and both may wait
+        _on(side, _tensors(call(side)))
+        for t in dirty:
+            t.view(torch.uint8).fill_(0x5A)
+        torch.cuda.synchronize()
         torch.cuda._sleep(400_000_000)                      # about 0.2 s of the current stream
         for t in dirty:
             t.view(torch.uint8).fill_(0x5A)
