@@ -32,12 +32,15 @@ struct Workspace {
 // runs behind everything before the call.  What the predecessor wrote is read with ordinary loads: the non-coherent path
 // (ld.global.nc, __ldg) is for memory that nothing writes while the kernel runs, and a dependent kernel runs before its
 // inputs are complete.
-// A dependent quantizer takes places on the SMs that its predecessor's last wave still wants, so the line is one CTA per SM.
-// Passes of quantizers and products, none / up to 148 / up to 1184 CTAs dependent, us: 128 x 256 x 256 36.0 / 33.3 / 33.3,
-// 2048 x 2048 x 2048 51.6 / 51.6 / 53.4, 4096 x 4096 x 4096 151.3 / 151.3 / 156.7, 1D activations 8192 x 5632 x 2048 251.3 / 251.3 /
-// 259.0, MXFP8 512 x 1024 x 1024 18.8 / 14.9 / 14.9.  In a captured graph, whose launches cost less, dependent quantizers lose
-// (256 x 512 x 1024 33.3 without and 36.1 us with, expert layer of 1024 tokens 34.5 and 36.3): there they are not.
-constexpr int64_t kShortGrid = 148;
+// A product lets nobody in before it ends: its last wave leaves some SMs idle for microseconds, and a quantizer that
+// is admitted then is placed on those alone.  Passes of quantizers and products, us, products that admit early with quantizers
+// of up to 1184 and 148 CTAs dependent, and products that do not with up to 1184: 512 x 1024 x 1024 36.3 / 36.3 / 35.3,
+// 2048 x 2048 x 2048 49.3 / 48.8 / 45.4, 4096 x 4096 x 4096 151.5 / 147.3 / 142.8, 8192 x 2048 x 2048 quantized by one call 103.9 / 94.5 /
+// 92.4, experts of 1024 tokens 38.9 / 38.9 / 34.5, three ragged operands by one call 26.8 / 28.1 / 26.8.
+// Long grids do not take part: in a dependent launch the wait costs every CTA of the grid, not only the first ones.  Nor do
+// quantizers in a captured graph, whose launches cost less: there they lose (256 x 512 x 1024 33.3 without and 36.1 us with,
+// expert layer of 1024 tokens 34.5 and 36.3).
+constexpr int64_t kShortGrid = 2 * 4 * 148;   // two waves of four CTAs per SM
 inline bool capturing(cudaStream_t stream)
 {
     cudaStreamCaptureStatus st;

@@ -1114,9 +1114,9 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
         }
     }
-    // Everything above touches this CTA only; from here on the kernel reads what its predecessor in the stream wrote.
+    // Everything above touches this CTA only; from here on the kernel reads what its predecessor in the stream wrote.  Its own
+    // successor is let in by its end (launch_dependent says why).
     wait_for_predecessor();
-    admit_successor();
     // Poll limit of every bounded wait (workspace word 2; 0 = the default) and the development hook of word 3 (n > 0:
     // the producer of CTA 0 leaves out its n-th stage load, so that a test can watch a wait run out and the kernel
     // leave through its timeout path without anything faulting or spinning for long).
@@ -1908,13 +1908,12 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = Cfg<KIND, CTAS>::kSmemBytes;
     cfg.stream = static_cast<cudaStream_t>(stream);
-    // Short products start beside their predecessor's end: up to 48 stages, about 25 us, per CTA or pair.  Passes of quantizers
-    // and products, without and with, us: 2048 x 4096 x 4096 (28 stages) 102.8 / 97.6, 1D activations 2048 x 4096 x 4096 32.5 / 29.3,
-    // 16 x 16 blocks 8192 x 2048 x 2048 134 / 129; nothing changes from 4096 x 4096 x 4096 (55 stages) on, except that CTAs of long
-    // products are placed as SMs fall free instead of in order, and tiles that share operands end up far apart (all three
-    // products of 16384 x 11008 x 4096 with their quantizers 1039 / 1084).  In a captured graph the one-CTA products of the smallest
-    // layers lose (4 experts of 512 tokens in all 31.7 / 33.4, 128 x 256 x 256 31.0 / 31.9) while the pairs gain
-    // (512 x 1024 x 1024 36.3 / 34.3), so only these take part there.
+    // Short products start beside the end of a quantizer before them: up to 48 stages, about 25 us, per CTA or pair.  Passes of
+    // quantizers and products, without and with, us: 2048 x 4096 x 4096 (28 stages) 102.8 / 97.6, 1D activations 2048 x 4096 x 4096
+    // 32.5 / 29.3; nothing changes from 4096 x 4096 x 4096 (55 stages) on, except that CTAs of long products are placed as SMs
+    // fall free instead of in order, and tiles that share operands end up far apart (all three products of 16384 x 11008 x 4096
+    // with their quantizers 1039 / 1084).  In a captured graph the one-CTA products of the smallest layers lose (4 experts of 512
+    // tokens in all 31.7 / 33.4, 128 x 256 x 256 31.0 / 31.9), so only those on pairs take part there.
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
     if (CTAS == 2) {
