@@ -397,3 +397,16 @@ def test_grouped_weight_gradient_longest_groups_first(ws, counts, N, K):
         a, z = int(offs[e]), int(offs[e + 1])
         assert torch.equal(got[e * N:(e + 1) * N], dy[a:z].float().T @ x[a:z].float()), e
     assert binding.fp4q_workspace_status(ws) == 0
+
+
+@pytest.mark.parametrize("K", [1408, 2720, 416, 4512])      # 44 (words), 85, 13 and 141 blocks a row
+def test_mxfp8_scale_rows_on_any_word_or_byte(ws, K):
+    T, N = 300, 264
+    g = torch.Generator(device="cuda").manual_seed(K)
+    x = (torch.randn(T, K, generator=g, device="cuda") * torch.exp(2 * torch.randn(T, 1, generator=g, device="cuda"))).to(torch.bfloat16)
+    w = (torch.randn(N, K, generator=g, device="cuda") * 0.02).to(torch.bfloat16)
+    (xq, xs, xd), (wq, wsc, wd) = _mxfp8_operand(x), _mxfp8_operand(w)
+    y = binding.fp4q_mxfp8_gemm(xq, xs, wq, wsc, T, N, K, dt=binding.OUT_F32, ws=ws)
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
+    check(y, (torch.from_numpy(xd).cuda() @ torch.from_numpy(wd).cuda().T).cpu().numpy(), "MXFP8 product")
