@@ -18,6 +18,8 @@
  *     fp4q_workspace_set_wait_limit, fp4q_debug_withhold_load) copy a few bytes and DO
  *     synchronise `stream`.  The first call on a device creates per-device state (module load,
  *     driver entry point lookup, kernel attributes) and should be made outside stream capture.
+ *   - Calls on one stream keep their order.  Short kernels may be placed on the GPU beside the end of
+ *     the kernel before them in their stream, but touch memory only after it has completed.
  *   - Every function returns an fp4q_status; nothing throws, traps or aborts.  Argument
  *     errors are reported before any work is enqueued.  Device-side anomalies (a bounded
  *     wait that ran out) are recorded in the workspace status word and read back with
@@ -128,7 +130,8 @@ fp4q_status fp4q_quantize2d(const void *x_bf16, int64_t rows, int64_t cols, int6
  * bytes as one call per tensor; the rounding stream of tensor j is keyed on jobs[j].tensor_id).  The operands of a
  * layer do not depend on one another and many of them are small (a 4096 x 4096 weight is a few waves of CTAs), so the
  * call enqueues one kernel per tensor on `stream` with each kernel after the first configured as the programmatic
- * dependent of its predecessor: it starts beside the predecessor's last wave instead of after it and completes after
+ * dependent of its predecessor: the first waits for everything before the call, a later one starts beside the last wave of
+ * its predecessor instead of after it (it does not read what that one writes) and completes after
  * it, and whatever is enqueued after the call sees all tensors.  `jobs` is a HOST array of n_jobs descriptors, read
  * during the call; the pointers inside are device pointers as for fp4q_quantize2d.  32 x 32 blocks only (flags: 0 or
  * FP4Q_INDEX_TRANSPOSED).  The tensors must not overlap one another's outputs.  Every job is validated before anything

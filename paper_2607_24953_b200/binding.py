@@ -60,7 +60,8 @@ _lib = None
 
 
 def lib() -> ctypes.CDLL:
-    """Load libfp4q.so (built in-tree by paper_2607_24953_b200.build). Fails loudly if absent."""
+    """Load libfp4q.so (built in-tree by paper_2607_24953_b200.build). Fails loudly if absent.  The signatures are for
+    callers of the C interface through ctypes; the functions below reach the quantizers and products through _host."""
     global _lib
     if _lib is None:
         if not os.path.exists(LIB_PATH):

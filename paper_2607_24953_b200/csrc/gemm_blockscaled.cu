@@ -6,9 +6,9 @@
 //                   contraction block kb is scale[r/32][kb] or, for a transposed view, scale[kb][r/32].
 //   kind::mxf8f6f4  E4M3 payload, one UE8M0 scale per row and 32 contraction elements (MXFP8).
 //
-// Persistent kernel, one CTA per SM, 12 warps.  Dense FP4 products run as clusters of two CTAs that share a 256x256
-// tile through cta_group::2 MMAs (each CTA holds 128 rows of the accumulator, loads its own 128 A rows and half of
-// the B rows); grouped products and MXFP8 use one CTA per 128x256 tile.
+// Persistent kernel, one CTA per SM, 12 warps.  Dense products of more than 128 rows, grouped weight gradients and grouped rows
+// on 256-row boundaries run as clusters of two CTAs that share a 256x256 tile through cta_group::2 MMAs (each CTA holds 128
+// rows of the accumulator, loads its own 128 A rows and half of the B rows); everything else uses one CTA per 128x256 tile.
 //   warp 0      TMA producer: per stage the A tile (128 rows x 128 B) and the B tile (256 or 128 rows x 128 B),
 //               128B swizzle
 //   warp 1      MMA issuer: stays converged, one elected lane issues per stage 6 tcgen05.cp (scale images -> TMEM),
@@ -21,10 +21,10 @@
 //               images tcgen05.cp reads in place (double-buffered); 2D-block scales as replicated 8-row images,
 //               per-row scales as real 32-row images
 //   warps 4-11  epilogue: tcgen05.ld of the 128x256 FP32 accumulator (each warp 32 lanes x 128 columns),
-//               release of the accumulator as soon as it sits in registers, then convert and store (pair kernel:
-//               through staging rows and TMA stores; one CTA: 256-bit stores)
-// A ring of four (one CTA: 48 KB of operands per stage) or five (pair: 32 KB) shared-memory stages is guarded by
-// mbarriers; the scale columns in TMEM form a ring of the same depth.  Every mbarrier wait is bounded: when a limit
+//               release of the accumulator as soon as it sits in registers, then convert and store (through staging
+//               rows and TMA stores; one CTA with per-row scales: 256-bit stores)
+// A ring of three or four (one CTA: 48 KB of operands per stage) or four or five (pair: 32 KB) shared-memory stages, by kind
+// (Cfg), is guarded by mbarriers; the scale columns in TMEM form a ring of the same depth.  Every mbarrier wait is bounded: when a limit
 // is hit the CTA records FP4Q_ERR_TIMEOUT in the workspace, releases the MMA warp from its named barriers, stops
 // issuing work and leaves through the normal exit (TMEM is freed).
 #include <cstdlib>
@@ -123,7 +123,7 @@ struct Cfg {
 };
 // Dense products and grouped rows: row tiles per rasterisation group.  With grouped rows a group's A rows and the weights of the
 // few experts they belong to stay in L2 for the whole sweep over the columns (expert layer, 139520 rows, one group of all
-// row tiles -> groups of 16: 768 x 2048 fwd/dgrad 148/207 -> 132/170 us, 2048 x 768 201/149 -> 164/134 us; 8 and 32 within 2 %).
+// row tiles -> groups of 16: 768 x 2048 fwd/dgrad 142/207 -> 126/166 us, 2048 x 768 199/144 -> 158/128; 8 and 32 within 2 %).
 constexpr int kRasterM = 16;
 constexpr int kThreads = 384;
 constexpr int kTmemCols = 512;
