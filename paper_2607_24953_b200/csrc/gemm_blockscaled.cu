@@ -17,7 +17,7 @@
 //   warp 2      dense FP4 and MXFP8 pairs: watcher, polls the slots' "full" barriers (several at a time), the scale images
 //               and the accumulator's "empty" barrier and meets the MMA warp at a named barrier per stage (elsewhere the
 //               MMA warp looks for itself); per-row FP4 kinds: second scale image builder
-//   warp 3      scale image builder: per unit of 16 stages (4 or 2 with per-row images) gathers the scale bytes and writes the
+//   warp 3      scale image builder: per unit of 16 stages (4 or 2 with per-row images) loads the scale bytes and writes the
 //               images tcgen05.cp reads in place (double-buffered); 2D-block scales as replicated 8-row images,
 //               per-row scales as real 32-row images
 //   warps 4-11  epilogue: tcgen05.ld of the 128x256 FP32 accumulator (each warp 32 lanes x 128 columns),
@@ -56,8 +56,8 @@ constexpr int kUnitStagesMxf4 = kCacheChunks / 2;
 // pays for one more ring stage.
 constexpr int kUnitStagesMxf8 = 4;
 constexpr int kImageStageBytesMxf8 = 1536;
-constexpr int kCompactBytes = kCacheChunks * 48;
 constexpr int kImageStageBytes = 768;        // A chunk 0, A chunk 1, B chunk 0 (rows 0..127, 128..255), B chunk 1 (same)
+constexpr int kCompactBytes = kCacheChunks * 48;
 constexpr int kCacheBufBytes = kUnitStagesMxf4 * kImageStageBytes;
 // mxf4 with per-row scales: a stage has two chunks of four blocks; A 2 x 512 B, B (256 rows) 4 x 512 B per stage
 constexpr int kUnitStagesMxf4R = 4;
@@ -270,25 +270,11 @@ __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile u
 {
     return mbar_wait_impl<0>(bar, parity, abort_flag, status, limit, where);
 }
-__device__ __noinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status,
-                                               uint64_t limit, uint32_t where)
-{
-    return mbar_wait_impl<kRelaxedNs>(bar, parity, abort_flag, status, limit, where);
-}
 // For the end of an aborted launch, when the abort flag is set already: 256 polls, a third of a millisecond at most.
 __device__ __noinline__ void mbar_drain(uint32_t bar)
 {
     for (int it = 0; it < 256 && !mbar_try_wait(bar, 0u); it++) __nanosleep(kLazyNs);
 }
-// The builder of 2D-block images in a pair, whose buffers the leader's multicast commits release: probes with a back-off.
-// (Whether a remote arrival wakes a suspended thread is not specified; where the other roles suspend on such barriers, they
-// look again after kSuspendNs at the latest.)
-__device__ __noinline__ bool mbar_poll_relaxed(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status,
-                                               uint64_t limit, uint32_t where)
-{
-    return mbar_wait_impl<kRelaxedNs, true>(bar, parity, abort_flag, status, limit, where);
-}
-
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int32_t x, int32_t y, uint32_t bar)
 {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -309,13 +295,13 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+// What such an arrival announces lies in this CTA's own shared memory or tensor memory and was made visible to the asynchronous proxy
+// or fenced before; the other CTA only issues the instructions that read it here.  So release at the default scope is enough;
+// release at cluster scope kept the arrival back for another 400 ns (first MMA of 8192 x 2048 x 2048 1850 -> 1400 ns after the
+// first load).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_cluster_release(uint32_t cluster_bar)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
@@ -558,78 +544,128 @@ __device__ __forceinline__ uint4 transpose4x4_bytes(uint32_t w0, uint32_t w1, ui
 // mxf4 / 2D blocks: a stage covers 8 contraction blocks (two chunks of 4).  For 128 operand rows and one chunk the
 // scale image is 32 identical rows of 16 bytes [row tile 0..3][block 0..3]; A needs 2 such rows per stage (one per
 // chunk), B (256 rows) 4.
-// Gathers the scale bytes of n_chunks contraction chunks (4 blocks each) for 2^log2_rt consecutive row tiles into
-// dst[(chunk << log2_rt) + rt] as 32-bit words (byte k = block 4*chunk + k): the 16-byte image rows of the chunk.
-// One warp; each lane takes items lane, lane + 32, ...  Slots beyond the tensor read the pad byte.
-__device__ __forceinline__ void build_scale_cache(const ScaleView &v, int rt0, int kb0, int n_chunks, int log2_rt,
-                                                  uint32_t *dst, int lane)
+//
+// A unit has as many chunks as a warp has lanes: lane c loads the scale bytes of chunk c, four words for every four row tiles, and
+// holds whole image rows.  All of a unit's loads are in flight together, and the next unit's while a unit is written.  A product's
+// first MMA waits for its first unit, and a tile with a short contraction for its own: with the loads of A and B one after the
+// other, then a pass through shared memory, then stores that met in the same banks, the first unit took 3300-6700 cycles from
+// the first operand load on and every later one 4000-5000; now 1300-2800 and 1500.  One warp runs an instruction in about five
+// cycles, so their number counts as well.
+// w[i]: row-major scales: blocks kb..kb+3 of row tile rt0 + i; transposed view (stride_kb != 1): row tiles of group i / 4 of
+// block kb + i % 4.
+enum { SCALES_WHOLE = 0, SCALES_SHIFTED = 1, SCALES_GATHER = 2 };
+
+// Where word i of lane's chunk starts, and how many bytes exist from there on.  Rows and blocks beyond the tensor take the place of
+// ones that exist (their payload is zero, any finite scale will do).
+__device__ __forceinline__ const uint8_t *chunk_word(const ScaleView &v, int rt0, int kb, int kb0, int i, int &n)
 {
-    const bool aligned4 = (reinterpret_cast<uintptr_t>(v.ptr) & 3) == 0;
-    if (v.stride_row == 1 && v.stride_kb != 1 && aligned4 && (v.stride_kb & 3) == 0 && (rt0 & 3) == 0) {
-        // transposed view: the row-tile bytes of one block are contiguous.  An item is a chunk and a group of four
-        // row tiles: four 32-bit loads (one per block) and a 4x4 byte transpose give the group's four words.
-        const int log2_g = log2_rt - 2, n_items = n_chunks << log2_g;
-        for (int base = 0; base < n_items; base += 32 * 2) {
-            uint32_t w[2][4];
+    if (v.stride_kb != 1) {
+        const int rt = rt0 + (i & ~3) < v.n_row ? rt0 + (i & ~3) : rt0;
+        n = v.n_row - rt;
+        return v.ptr + min(kb + (i & 3), v.n_kb - 1) * v.stride_kb + rt;
+    }
+    if (kb >= v.n_kb) kb = kb0;
+    n = v.n_kb - kb;
+    return v.ptr + min(rt0 + i, v.n_row - 1) * v.stride_row + kb;
+}
+// An aligned word that reaches past an end of the scale matrix, which occupies the bytes lo .. hi - 1.
+__device__ __noinline__ uint32_t load_end_word(const uint8_t *src, const uint8_t *lo, const uint8_t *hi)
+{
+    uint32_t w = 0;
 #pragma unroll
-            for (int j = 0; j < 2; j++) {
-                const int q = base + 32 * j + lane;
-                const int chunk = q >> log2_g, rg = q & ((1 << log2_g) - 1);
-                const int row = rt0 + 4 * rg, kb = kb0 + 4 * chunk;
+    for (int e = 0; e < 4; e++)
+        if (src + e >= lo && src + e < hi) w |= (uint32_t)load_global(src + e) << (8 * e);
+    return w;
+}
+// Loads a unit's words of G groups of four row tiles: as they are, where all start on words and exist; otherwise up to two aligned
+// words each, which place_chunk_scales shifts into place when they are needed.  One lane a chunk, that is some four hundred
+// instructions whatever the unit's length; units whose words make one round of gather_scale_rows (12 a chunk, 128 a round) are
+// gathered by all lanes instead (SCALES_GATHER, nothing is loaded yet).  us, forward / input gradient / weight gradient, all
+// units one lane a chunk and all gathered: 300 x 777 x 1234 (10, 7 and 3 chunks) 10.3 / 10.9 / 11.6 and 10.0 / 9.7 / 11.0,
+// 1999 x 1003 x 2731 (22, 8 and 16) 12.8 / 14.4 / 13.7 and 14.9 / 12.3 / 14.2.
+constexpr int kGatherChunks = 10;
+template <int G>
+__device__ __forceinline__ int fetch_chunk_scales(const ScaleView &v, int rt0, int kb0, int n_real, int n_chunks, uint32_t (&w)[4 * G], uint32_t (&next)[4 * G], int lane)
+{
+    const bool tr = v.stride_kb != 1;
+    const int64_t pitch = tr ? v.stride_kb : v.stride_row;
+    const uint8_t *src = v.ptr + (tr ? kb0 * pitch + rt0 : rt0 * pitch + kb0);
+    if (((reinterpret_cast<uintptr_t>(src) | (uintptr_t)pitch) & 3) == 0 && rt0 + 4 * G <= v.n_row && kb0 + 4 * n_real <= v.n_kb) {
+        if (lane < n_chunks) {   // a whole number of stages: the chunk that fills up the last one takes the first chunk's scales
+            if (lane < n_real) src += 4 * lane * (tr ? pitch : 1);
 #pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    w[j][k] = kScalePad * 0x01010101u;
-                    if (q < n_items) {
-                        if (row + 4 <= v.n_row && kb + k < v.n_kb) {
-                            ldg_b32(v.ptr + (int64_t)(kb + k) * v.stride_kb + row, w[j][k]);
-                        } else {
-                            uint32_t b0, b1, b2, b3;
-                            load_scale(v, row, kb + k, b0);
-                            load_scale(v, row + 1, kb + k, b1);
-                            load_scale(v, row + 2, kb + k, b2);
-                            load_scale(v, row + 3, kb + k, b3);
-                            w[j][k] = b0 | (b1 << 8) | (b2 << 16) | (b3 << 24);
-                        }
-                    }
-                }
-            }
+            for (int i = 0; i < 4 * G; i++) ldg_b32(src + (tr ? (i & 3) : i) * pitch + (tr ? (i & ~3) : 0), w[i]);
+        }
+        return SCALES_WHOLE;
+    }
+    if (n_chunks <= kGatherChunks) return SCALES_GATHER;
+    const uint8_t *end = v.ptr + (tr ? (v.n_kb - 1) * pitch + v.n_row : (v.n_row - 1) * pitch + v.n_kb);
+    if (lane < n_chunks) {
 #pragma unroll
-            for (int j = 0; j < 2; j++) {
-                const int q = base + 32 * j + lane;
-                if (q < n_items) reinterpret_cast<uint4 *>(dst)[q] = transpose4x4_bytes(w[j][0], w[j][1], w[j][2], w[j][3]);
+        for (int i = 0; i < 4 * G; i++) {
+            int n;
+            const uint8_t *a = chunk_word(v, rt0, kb0 + 4 * lane, kb0, i, n);
+            const int mis = (int)(reinterpret_cast<uintptr_t>(a) & 3);
+            a -= mis;
+            next[i] = 0u;
+            if (a >= v.ptr && a + 4 <= end) ldg_b32(a, w[i]);
+            else w[i] = load_end_word(a, v.ptr, end);
+            if (mis + n > 4 && mis != 0) {
+                if (a + 8 <= end) ldg_b32(a + 4, next[i]);
+                else next[i] = load_end_word(a + 4, v.ptr, end);
             }
         }
-        return;
     }
-    const int n_items = n_chunks << log2_rt;
-    const bool along_k = v.stride_kb == 1 && aligned4 && (v.stride_row & 3) == 0 && (kb0 & 3) == 0;
-    for (int base = 0; base < n_items; base += 32 * 4) {
-        uint32_t w[4];
+    return SCALES_SHIFTED;
+}
+template <int G>
+__device__ __forceinline__ void place_chunk_scales(const ScaleView &v, int rt0, int kb0, uint32_t (&w)[4 * G], const uint32_t (&next)[4 * G], int lane)
+{
+#pragma unroll
+    for (int i = 0; i < 4 * G; i++) {
+        int n;
+        const uint8_t *a = chunk_word(v, rt0, kb0 + 4 * lane, kb0, i, n);
+        const uint32_t keep = n < 4 ? (1u << (8 * n)) - 1u : 0xFFFFFFFFu;
+        w[i] = (__funnelshift_r(w[i], next[i], 8 * (uint32_t)(reinterpret_cast<uintptr_t>(a) & 3)) & keep) | (kScalePad * 0x01010101u & ~keep);
+    }
+}
+// The 16-byte image row [row tile][block] of a group's four words.
+__device__ __forceinline__ uint4 chunk_image_row(const ScaleView &v, const uint32_t *w)
+{
+    return v.stride_kb != 1 ? transpose4x4_bytes(w[0], w[1], w[2], w[3]) : make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Short units at the ends of a scale matrix, or of scales that start on any byte.  The words of the operands that need it, item q a (chunk, row tile) of A's
+// four row tiles or, after them, of B's eight, spread over the lanes (one lane a chunk, 300 x 777 x 1234 took 0.7 to 1.5 us longer) and
+// gathered in shared memory as rows of 16 bytes.  Slots beyond the tensor hold the pad byte.
+__device__ __forceinline__ void gather_scale_rows(const GemmParams &p, const Tile &t, int k0, bool need_a, bool need_b, int n_chunks, uint32_t *dst, int lane)
+{
+    const int n_a = need_a ? 4 * n_chunks : 0, n = n_a + (need_b ? 8 * n_chunks : 0);
+    for (int base = 0; base < n; base += 32 * 4) {
+        uint32_t b[4][4];
 #pragma unroll
         for (int j = 0; j < 4; j++) {   // loads of four items in flight before anything is used
             const int q = base + 32 * j + lane;
-            const int chunk = q >> log2_rt, rt = q & ((1 << log2_rt) - 1);
-            const int row = rt0 + rt, kb = kb0 + 4 * chunk;
-            w[j] = 0;
-            if (q < n_items) {
-                if (along_k && row < v.n_row && kb + 4 <= v.n_kb) {
-                    ldg_b32(v.ptr + (int64_t)row * v.stride_row + kb, w[j]);
-                } else {
-                    uint32_t b0, b1, b2, b3;
-                    load_scale(v, row, kb, b0);
-                    load_scale(v, row, kb + 1, b1);
-                    load_scale(v, row, kb + 2, b2);
-                    load_scale(v, row, kb + 3, b3);
-                    w[j] = b0 | (b1 << 8) | (b2 << 16) | (b3 << 24);
-                }
+            const bool is_a = q < n_a;
+            const int i = is_a ? q : q - n_a, chunk = is_a ? i >> 2 : i >> 3, rt = is_a ? i & 3 : i & 7;
+            const ScaleView &v = is_a ? p.sfa : p.sfb;
+            const int row = ((is_a ? t.a_row0 : t.b_row0) >> 5) + rt, kb = (((is_a ? t.a_k0 : t.b_k0) + k0) >> 5) + 4 * chunk;
+            const uint8_t *src = v.ptr + (int64_t)row * v.stride_row + (int64_t)kb * v.stride_kb;
+            const int n_bytes = q < n && row < v.n_row ? v.n_kb - kb : 0;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                b[j][k] = kScalePad;
+                asm volatile("{\n .reg .pred p;\n setp.gt.s32 p, %2, %3;\n @p ld.global.u8 %0, [%1];\n}" : "+r"(b[j][k]) : "l"(src), "r"(n_bytes), "r"(k));
+                src += v.stride_kb;
             }
         }
 #pragma unroll
         for (int j = 0; j < 4; j++) {
             const int q = base + 32 * j + lane;
-            if (q < n_items) dst[q] = w[j];
+            if (q < n) dst[q < n_a ? q : 4 * kCacheChunks + q - n_a] = b[j][0] | b[j][1] << 8 | b[j][2] << 16 | b[j][3] << 24;
         }
     }
+    __syncwarp();
 }
 
 // Per-row scales (MXFP8): one 32-bit word = the four scale bytes of one row and one stage.
@@ -818,14 +854,17 @@ struct BufRing {
     __device__ __forceinline__ void next(uint32_t n) { if (++buf == n) { buf = 0; phase ^= 1u; } }
 };
 
-// The stream of scale units (kUnitStages stages of one tile) a CTA works through; per-row scales, dense products.
+// The stream of scale units (kUnitStages stages of one tile) a CTA works through.
+template <bool GROUPED>
 struct UnitIter {
     int tile, step, rank, k0;
     Tile t;
+    const int32_t *goffs = nullptr;
+    const uint16_t *gorder = nullptr;
     __device__ __forceinline__ void seek(const GemmParams &p)
     {
         while (tile < p.n_tile_total) {
-            decode_tile<false>(p, tile, rank, t, nullptr, nullptr);
+            decode_tile<GROUPED>(p, tile, rank, t, goffs, gorder);
             if (k0 < t.k_len) return;
             tile += step;
             k0 = 0;
@@ -1070,7 +1109,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *smem_a = smem;
     uint8_t *smem_b = smem + kStages * kAStageBytes;
-    uint8_t *smem_compact = smem + Cfg<KIND, CTAS>::kSmemOperands;   // 2D blocks: compact scale rows of the unit being built ...
+    uint8_t *smem_compact = smem + Cfg<KIND, CTAS>::kSmemOperands;   // 2D blocks: gathered scale rows of the unit being built ...
     uint8_t *smem_images = smem_compact + (Cfg<KIND, CTAS>::kRowImages ? 0 : kCompactBytes);   // ... and the buffers of ready scale images (any kind)
     uint8_t *smem_raw_scales = smem_images + Cfg<KIND, CTAS>::kImageBufs * kBufBytes;   // per-row scales: bytes in flight
     uint8_t *smem_staging = smem_compact + Cfg<KIND, CTAS>::kSmemScales;   // 1024-byte aligned (pair kernel only)
@@ -1338,10 +1377,10 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             // builders have finished to the leader, which issues the scale copies of both CTAs.
             bool fwd_ok = true;
             BufRing fr;
-            UnitIter un;
+            UnitIter<false> un;
             for (un.init(p, first_tile, tile_step, rank); fwd_ok && un.valid(p); un.next(p, kUnitStages * kStageElems), fr.next(kImageBufs)) {
                 fwd_ok = __all_sync(0xFFFFFFFFu, mbar_wait_impl<0>(bar_cache_full + 8 * fr.buf, fr.phase, abort_flag, p.status, wait_limit, 0x530u + fr.buf));
-                if (fwd_ok && issuer) mbar_arrive_cluster_release(cluster_addr(bar_peer_cache_full + 8 * fr.buf, 0));
+                if (fwd_ok && issuer) mbar_arrive_cluster(cluster_addr(bar_peer_cache_full + 8 * fr.buf, 0));
             }
             __syncwarp();
         }
@@ -1359,8 +1398,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         if (lane == 0) { TRACE_OUT(p, 2, c_acc); TRACE_OUT(p, 3, c_sync); TRACE_OUT(p, 4, c_issue); }
     } else if (warp == 3 || (warp == 2 && Cfg<KIND, CTAS>::kBuilders == 2)) {
         // ------------------------------------------------------------------ scale image builder
-        // 2D-block scales: per unit (up to 16 stages of one tile) gathers the compact scale bytes from global memory
-        // into 16-byte rows and replicates each row into its image; per-row scales: loads the unit's scale words and
+        // 2D-block scales: per unit (up to 16 stages of one tile) loads the scale bytes as 16-byte rows, one lane a chunk, and
+        // replicates each row into its image; per-row scales: loads the unit's scale words and
         // writes the 32-row images directly.  Two image buffers alternate, so the next unit is built while
         // the current one runs: all global-memory latency of the scale path is paid here, off the per-stage
         // critical path, and nothing has to be written per stage.  A buffer is free again once the MMA warp's
@@ -1374,7 +1413,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             constexpr int kBuilders = Cfg<KIND, CTAS>::kBuilders, kRawBytes = Cfg<KIND, CTAS>::kRawBytes, kSlotB = Cfg<KIND, CTAS>::kRawSlotB;
             constexpr int kOwnRaw = Cfg<KIND, CTAS>::kRawBufs > 0 ? Cfg<KIND, CTAS>::kRawBufs / kBuilders : 1;
             uint8_t *raw = smem_raw_scales + (3 - warp) * kOwnRaw * kRawBytes;
-            UnitIter ahead, cur;
+            UnitIter<false> ahead, cur;
             ahead.init(p, first_tile, tile_step, rank);
             cur.init(p, first_tile, tile_step, rank);
             if (warp == 2) {   // the second builder starts with the second unit
@@ -1430,45 +1469,76 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             }
             asm volatile("cp.async.wait_all;" ::: "memory");
         }
-        for (int tile = first_tile; KIND == KIND_MXF4 && ok && tile < p.n_tile_total; tile += tile_step) {
-            Tile t;
-            decode_tile<kGrouped>(p, tile, rank, t, goffs, gorder);
-            for (int k0 = 0; ok && k0 < t.k_len; k0 += kUnitStages * kStageElems, ring.next(kImageBufs)) {
+        if (KIND == KIND_MXF4) {
+            UnitIter<kGrouped> un;   // the unit whose scale bytes are being loaded
+            un.goffs = goffs;
+            un.gorder = gorder;
+            un.init(p, first_tile, tile_step, rank);
+            uint32_t wa[4] = {}, wb[8] = {};
+            uint32_t next_a[4] = {}, next_b[8] = {};
+            int how_a = SCALES_WHOLE, how_b = SCALES_WHOLE;
+            int n_chunks = 0;                // of the unit that is loaded; 0: none
+            // A unit is written while the next one's loads are in flight; the first is written before anything else is looked at.
+            // In a pair the leader's multicast commits release the buffers.  Whether a remote arrival wakes a suspended thread is not
+            // specified: this wait probes (where the other roles suspend on such barriers, they look again after kSuspendNs at the latest).
+            for (int unit = 0, fetched = 0;;) {
+                const int n = n_chunks;
+                uint4 row_a, row_b0, row_b1;
+                if (n > 0) {
+                    const int kb_a = (un.t.a_k0 + un.k0) >> 5, kb_b = (un.t.b_k0 + un.k0) >> 5;
+                    if (how_a == SCALES_SHIFTED) place_chunk_scales<1>(p.sfa, un.t.a_row0 >> 5, kb_a, wa, next_a, lane);
+                    if (how_b == SCALES_SHIFTED) place_chunk_scales<2>(p.sfb, un.t.b_row0 >> 5, kb_b, wb, next_b, lane);
+                    row_a = chunk_image_row(p.sfa, wa);
+                    row_b0 = chunk_image_row(p.sfb, wb);
+                    row_b1 = chunk_image_row(p.sfb, wb + 4);
+                    if (how_a == SCALES_GATHER || how_b == SCALES_GATHER) {
+                        gather_scale_rows(p, un.t, un.k0, how_a == SCALES_GATHER, how_b == SCALES_GATHER, n, reinterpret_cast<uint32_t *>(smem_compact), lane);
+                        const uint4 *gathered = reinterpret_cast<const uint4 *>(smem_compact);
+                        if (how_a == SCALES_GATHER) row_a = gathered[lane];
+                        if (how_b == SCALES_GATHER) { row_b0 = gathered[kCacheChunks + 2 * lane]; row_b1 = gathered[kCacheChunks + 2 * lane + 1]; }
+                        __syncwarp();
+                    }
+                }
+                n_chunks = 0;
+                if (n == 0 || unit > 0) {
+                    if (fetched++) un.next(p, kUnitStages * kStageElems);
+                    if (un.valid(p)) {
+                        const int n_real = min(kCacheChunks, (un.t.k_len - un.k0 + 127) >> 7);
+                        n_chunks = (n_real + 1) & ~1;   // whole stages
+                        how_a = fetch_chunk_scales<1>(p.sfa, un.t.a_row0 >> 5, (un.t.a_k0 + un.k0) >> 5, n_real, n_chunks, wa, next_a, lane);
+                        how_b = fetch_chunk_scales<2>(p.sfb, un.t.b_row0 >> 5, (un.t.b_k0 + un.k0) >> 5, n_real, n_chunks, wb, next_b, lane);
+                    } else if (n == 0) {
+                        break;
+                    }
+                }
+                if (n == 0) continue;
                 const int buf = ring.buf;
-                uint8_t *images = smem_images + buf * kBufBytes;
-                {
-                    const int n_chunks = min(kCacheChunks, (((t.k_len - k0 + 127) >> 7) + 1) & ~1);   // whole stages; pad rows beyond the tensor
-                    uint32_t *compact = reinterpret_cast<uint32_t *>(smem_compact);
-                    build_scale_cache(p.sfa, t.a_row0 >> 5, ((t.a_k0 + k0) >> 5), n_chunks, 2, compact, lane);
-                    build_scale_cache(p.sfb, t.b_row0 >> 5, ((t.b_k0 + k0) >> 5), n_chunks, 3, compact + kCacheChunks * 4, lane);
-                    __syncwarp();
-                    if (lane == 0)
-                        ok = CTAS == 2 ? mbar_poll_relaxed(bar_cache_empty + 8 * buf, ring.phase ^ 1u, abort_flag, p.status, wait_limit, 0x500u + buf)
-                                       : mbar_wait_relaxed(bar_cache_empty + 8 * buf, ring.phase ^ 1u, abort_flag, p.status, wait_limit, 0x500u + buf);
-                    ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+                if (unit >= kImageBufs) {   // the first units' buffers have never been used
+                    ok = mbar_wait_impl<kRelaxedNs, CTAS == 2>(bar_cache_empty + 8 * buf, ring.phase ^ 1u, abort_flag, p.status, wait_limit, 0x500u + buf);
+                    ok = __all_sync(0xFFFFFFFFu, ok);
                     if (!ok) break;
-                    const uint4 *rows = reinterpret_cast<const uint4 *>(smem_compact);
-                    for (int q = lane; q < 3 * n_chunks; q += 32) {
-                        uint4 row;
-                        uint8_t *dst;
-                        if (q < n_chunks) {                       // A, chunk q
-                            row = rows[q];
-                            dst = images + (q >> 1) * kImageStageBytes + (q & 1) * 128;
-                        } else {                                  // B, chunk (q - n_chunks) / 2, rows 0..127 or 128..255
-                            const int qb = q - n_chunks, chunk = qb >> 1;
-                            row = rows[kCacheChunks + qb];
-                            dst = images + (chunk >> 1) * kImageStageBytes + 256 + (chunk & 1) * 256 + (qb & 1) * 128;
-                        }
+                }
+                if (lane < n) {
+                    uint8_t *images = smem_images + buf * kBufBytes + (lane >> 1) * kImageStageBytes + (lane & 1) * 128;
+                    uint4 *img_a = reinterpret_cast<uint4 *>(images), *img_b = reinterpret_cast<uint4 *>(images + 256 + (lane & 1) * 128);
+                    // the lanes' images lie 128 bytes apart: each starts with another of the eight rows, so that eight lanes cover all banks
 #pragma unroll
-                        for (int r = 0; r < 8; r++) reinterpret_cast<uint4 *>(dst)[r] = row;
+                    for (int i = 0; i < 8; i++) {
+                        const int r = (i + lane) & 7;
+                        img_a[r] = row_a;
+                        img_b[r] = row_b0;
+                        img_b[8 + r] = row_b1;
                     }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tcgen05.cp
                 __syncwarp();
                 if (lane == 0) {   // 16-stage units leave time for the second CTA's own (slow) remote arrival
+                    TRACE_EV(5, unit);
                     if (CTAS == 1 || leader) mbar_arrive(bar_cache_full + 8 * buf);
-                    else mbar_arrive_cluster_release(cluster_addr(bar_peer_cache_full + 8 * buf, 0));
+                    else mbar_arrive_cluster(cluster_addr(bar_peer_cache_full + 8 * buf, 0));
                 }
+                ring.next(kImageBufs);
+                unit++;
             }
         }
     } else if (warp == 2) {

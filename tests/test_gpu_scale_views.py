@@ -1,0 +1,47 @@
+"""The scale matrices of 2D-block tensors at any pitch and start: the products read them as whole words, as pairs of words shifted
+into place, or byte by byte at the matrix's ends, by their alignment and the contraction's length.  Gaps between the rows hold
+0xFF, UE8M0's NaN, so that a byte that does not belong to the tensor shows."""
+import dataclasses
+
+import pytest
+import torch
+
+import oracle
+from paper_2607_24953_b200 import binding, workloads
+from tests.gpu_util import check_gemm, dequant_from_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def elsewhere(q, gap, start):
+    """q with its scale matrix `start` bytes into a buffer, its rows `gap` bytes further apart."""
+    rows, cols = q.scale.shape
+    buf = torch.full((start + rows * (cols + gap),), 0xFF, dtype=torch.uint8, device="cuda")
+    scale = buf.as_strided((rows, cols), (cols + gap, 1), start)
+    scale.copy_(q.scale)
+    return dataclasses.replace(q, scale=scale)
+
+
+# contractions of 1, 2, 5, 10, 11, 22, 31 and 33 chunks of 128 in one of the three products, row tiles at the tile's edge and beyond
+@pytest.mark.parametrize("T,N,K", [(100, 70, 200), (300, 777, 1234), (161, 1311, 2731), (257, 640, 1280), (520, 1400, 4200), (128, 256, 3968)])
+def test_products_do_not_depend_on_where_the_scales_lie(T, N, K):
+    g = torch.Generator(device="cuda").manual_seed(T + N + K)
+    scales = torch.exp2(torch.randint(-6, 7, (3,), generator=g, device="cuda").float())
+    x, w, dy = ((torch.randn(r, c, generator=g, device="cuda") * s * torch.exp2(torch.randint(-4, 5, (r, 1), generator=g, device="cuda").float())).to(torch.bfloat16)
+                for (r, c), s in zip(((T, K), (N, K), (T, N)), scales))
+    qx, qw, qdy = (binding.fp4q_quantize2d(t) for t in (x, w, dy))
+    ws = binding.alloc_workspace("cuda")
+
+    def products(x, w, dy):
+        return [binding.fp4q_gemm_fwd(x, w, dt=binding.OUT_F32, ws=ws), binding.fp4q_gemm_dgrad(dy, w, dt=binding.OUT_F32, ws=ws),
+                binding.fp4q_gemm_wgrad(dy, x, ws=ws)]
+
+    plain = products(qx, qw, qdy)
+    xd, wd, dyd = (dequant_from_gpu(q) for q in (qx, qw, qdy))
+    for got, ref, what in zip(plain, (oracle.gemm_fwd(xd, wd), oracle.gemm_dgrad(dyd, wd), oracle.gemm_wgrad(dyd, xd)), ("fwd", "dgrad", "wgrad")):
+        check_gemm(got, ref, what)
+    for gap, start in ((0, 1), (1, 0), (2, 3), (4 - qx.scale.shape[1] % 4, 4), (7, 2)):
+        for got, ref, what in zip(products(*(elsewhere(q, gap, start) for q in (qx, qw, qdy))), plain, ("fwd", "dgrad", "wgrad")):
+            assert torch.equal(got, ref), (what, gap, start)   # the same operands and order of sums
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
