@@ -9,6 +9,7 @@ products need are written by the same quantization call: nothing is re-quantized
 from __future__ import annotations
 
 import torch
+from torch.autograd import forward_ad
 
 from . import binding
 
@@ -38,15 +39,34 @@ class _FP4LinearFn(torch.autograd.Function):
         return dx, dw, None, None, None
 
 
+_TENSORS = (torch.Tensor, torch.nn.Parameter)
+
+
+def _plain(x, weight) -> bool:
+    """Ordinary tensors on one GPU and nothing that looks into a Python autograd function (transforms, tracers, modes,
+    forward-mode levels): the native node does the same in half the host's time.  Everything else, what is refused
+    included, goes through _FP4LinearFn."""
+    return (type(x) in _TENSORS and type(weight) in _TENSORS and x.is_cuda and weight.dim() == 2 and x.device == weight.device
+            and torch._C._functorch.peek_interpreter_stack() is None and torch._C._len_torch_dispatch_stack() == 0
+            and torch._C._len_torch_function_stack() == 0 and torch._C._get_tracing_state() is None
+            and forward_ad._current_level < 0 and not torch.compiler.is_compiling())
+
+
+def _linear(x, weight, seed, tensor_id, ws):
+    if _plain(x, weight):
+        return binding._host().linear(x, weight, int(seed), int(tensor_id), ws)
+    return _FP4LinearFn.apply(x, weight, seed, tensor_id, ws)
+
+
 def fp4_linear(x: torch.Tensor, weight: torch.Tensor, seed: int = 0, tensor_id: int = 0, ws=None) -> torch.Tensor:
     """y = x^ weight^^T with FP4 forward and backward products.  x [..., K] and weight [N, K] live on the GPU;
     `seed` / `tensor_id` key the stochastic rounding of the incoming gradient (change one of them every step)."""
     if ws is None:
         ws = binding.alloc_workspace(x.device)
     if x.dim() == 2 and x.shape[1] != 0:   # nothing to fold: two autograd nodes less (reshape refuses rows of nothing)
-        return _FP4LinearFn.apply(x, weight, seed, tensor_id, ws)
+        return _linear(x, weight, seed, tensor_id, ws)
     lead = x.shape[:-1]
-    y = _FP4LinearFn.apply(x.reshape(-1, x.shape[-1]), weight, seed, tensor_id, ws)
+    y = _linear(x.reshape(-1, x.shape[-1]), weight, seed, tensor_id, ws)
     return y.reshape(*lead, weight.shape[0])
 
 

@@ -17,6 +17,7 @@
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
+#include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "fp4q.h"
@@ -55,10 +56,11 @@ struct Ref {   // owned reference
     Ref &operator=(const Ref &) = delete;
 };
 
-// The interpreter lock is given up around allocations and library calls, as torch.empty and ctypes do.
+// The interpreter lock is given up around allocations and library calls, as torch.empty and ctypes do (the layer's passes run
+// without it altogether).
 struct Unlock {
-    PyThreadState *state = PyEval_SaveThread();
-    ~Unlock() { PyEval_RestoreThread(state); }
+    PyThreadState *state = PyGILState_Check() ? PyEval_SaveThread() : nullptr;
+    ~Unlock() { if (state) PyEval_RestoreThread(state); }
 };
 template <typename F, typename... A>
 fp4q_status unlocked(F fn, A... args)
@@ -106,6 +108,7 @@ struct OnStream {
     void *handle;
     std::optional<c10::cuda::CUDAStream> caller;
     std::optional<c10::cuda::CUDAStreamGuard> guard;
+    OnStream() : handle(c10::cuda::getCurrentCUDAStream().stream()) {}
     OnStream(PyObject *o, const at::Tensor *like)
     {
         if (o == Py_None) {
@@ -511,6 +514,135 @@ PyObject *mxfp8_qk(Args a, Py_ssize_t n)
     return PyTuple_Pack(2, q.p, k.p);
 }
 
+// ---- the straight-through layer of autograd.py as one native autograd node
+//
+// The layer's kernels run 20 to 90 us forward and backward at the sizes where layers are small; through a Python autograd
+// function and the calls above the interpreter took as long, forward in the caller's thread and backward, with the lock, in the
+// engine's (128 x 256 x 256, forward and backward, 122-139 -> 87 us, of which the engine's own change of threads is 36).
+void check_unlocked(fp4q_status st, const char *where)
+{
+    if (st == FP4Q_OK) return;
+    const PyGILState_STATE gil = PyGILState_Ensure();
+    python_error e;
+    try {
+        check(st, where);
+    } catch (const PyError &) {
+        e.persist();
+    }
+    PyGILState_Release(gil);
+    throw e;
+}
+struct LinearCall {
+    at::Tensor ws;
+    uint64_t seed;
+    uint32_t tensor_id;
+};
+// Places in one allocation, for the arrays of quantized tensors (pitches as in alloc_q): one by one, twelve allocations a step
+// would be a tenth of its host time.
+struct Block {
+    int64_t bytes = 0;
+    int64_t add(int64_t n)
+    {
+        const int64_t at = bytes;
+        bytes += ceil_to(n, 256) * 256;
+        return at;
+    }
+};
+struct Placed {   // a quantized [rows, cols]: where its arrays lie in their blocks
+    fp4q_tensor t = {};
+    int64_t rm = 0, tr = 0, sc = 0, n_rm, n_t, n_s;
+    Placed(int64_t rows, int64_t cols)
+    {
+        t.rows = rows; t.cols = cols;
+        t.ld_rm = std::max<int64_t>(pad16(ceil_to(cols, 32) * 16), 16);
+        t.ld_t = std::max<int64_t>(pad16(ceil_to(rows, 32) * 16), 16);
+        t.ld_s = std::max<int64_t>(ceil_to(cols, 32), 1);
+        n_rm = rows * t.ld_rm; n_t = cols * t.ld_t; n_s = ceil_to(rows, 32) * t.ld_s;
+    }
+    void place_rm(Block &b) { rm = b.add(n_rm); }
+    void place_t(Block &b) { tr = b.add(n_t); sc = b.add(n_s); }
+    void bind_rm(uint8_t *base) { t.q_rm = n_rm ? base + rm : nullptr; }
+    void bind_t(uint8_t *base) { t.q_t = n_t ? base + tr : nullptr; t.scale = n_s ? base + sc : nullptr; }
+};
+at::Tensor block(const Block &b, const at::Tensor &like) { return at::empty({b.bytes}, at::TensorOptions().dtype(at::kByte).device(like.device())); }
+at::Tensor as_bf16(const at::Tensor &t)
+{
+    const at::Tensor c = t.scalar_type() == at::kBFloat16 ? t : t.to(at::kBFloat16);
+    return c.is_contiguous() ? c : c.contiguous();
+}
+at::Tensor as_type(const at::Tensor &t, int64_t dtype) { return t.scalar_type() == (at::ScalarType)dtype ? t : t.to((at::ScalarType)dtype); }
+
+struct LinearNode : torch::autograd::Function<LinearNode> {
+    static at::Tensor forward(torch::autograd::AutogradContext *ctx, const at::Tensor &x, const at::Tensor &weight, const LinearCall &call)
+    {
+        const OnStream on;
+        const at::Tensor xb = as_bf16(x), wb = as_bf16(weight);
+        const int64_t T = xb.size(0), K = xb.size(1), N = wb.size(0);
+        Placed qx(T, K), qw(N, wb.size(1));
+        Block keep, drop;   // backward reads the transposed codes and the scales
+        qx.place_t(keep); qw.place_t(keep); qx.place_rm(drop); qw.place_rm(drop);
+        const at::Tensor kept = block(keep, xb), dropped = block(drop, xb);
+        for (Placed *q : {&qx, &qw}) { q->bind_t(bytes_of(kept)); q->bind_rm(bytes_of(dropped)); }
+        fp4q_quantize_job jobs[2] = {};
+        jobs[0].x_bf16 = xb.data_ptr(); jobs[0].rows = T; jobs[0].cols = K; jobs[0].ld_x = pitch(xb); jobs[0].out = &qx.t;
+        jobs[1].x_bf16 = wb.data_ptr(); jobs[1].rows = N; jobs[1].cols = wb.size(1); jobs[1].ld_x = pitch(wb); jobs[1].out = &qw.t;
+        check_unlocked(lib.quantize2d_multi(jobs, 2, FP4Q_ROUND_NEAREST, 0, on.handle), "fp4q_quantize2d");
+        const at::Tensor y = out_buffer(on, T, N, FP4Q_OUT_BF16, xb);
+        check_unlocked(lib.gemm_fwd(&qx.t, &qw.t, y.data_ptr(), out_pitch(y, N), FP4Q_OUT_BF16, nullptr, call.ws.data_ptr(), (size_t)call.ws.numel(), on.handle),
+                       "fp4q_gemm_fwd");
+        ctx->saved_data["kept"] = kept;
+        ctx->saved_data["ws"] = call.ws;
+        ctx->saved_data["numbers"] = std::vector<int64_t>{K, (int64_t)call.seed, (int64_t)call.tensor_id, (int64_t)x.scalar_type(), (int64_t)weight.scalar_type()};
+        return y.is_contiguous() ? y : y.contiguous();
+    }
+    static torch::autograd::variable_list backward(torch::autograd::AutogradContext *ctx, torch::autograd::variable_list grads)
+    {
+        TORCH_CHECK(!ctx->saved_data.empty(),
+                    "fp4_linear: the quantized operands are freed when backward has run; run the layer again instead of going through its graph a second time");
+        const OnStream on;
+        const at::Tensor kept = ctx->saved_data["kept"].toTensor(), ws = ctx->saved_data["ws"].toTensor(), dy = as_bf16(grads[0]);
+        const auto numbers = ctx->saved_data["numbers"].toIntVector();
+        const int64_t T = dy.size(0), N = dy.size(1), K = numbers[0];
+        Placed qx(T, K), qw(N, K), q(T, N);
+        Block keep, own;
+        qx.place_t(keep); qw.place_t(keep); q.place_rm(own); q.place_t(own);
+        const at::Tensor codes = block(own, dy);
+        qx.bind_t(bytes_of(kept)); qw.bind_t(bytes_of(kept));
+        q.bind_rm(bytes_of(codes)); q.bind_t(bytes_of(codes));
+        check_unlocked(lib.quantize2d(dy.data_ptr(), T, N, pitch(dy), &q.t, FP4Q_ROUND_STOCHASTIC, (uint64_t)numbers[1], (uint32_t)numbers[2], 0, on.handle),
+                       "fp4q_quantize2d");
+        at::Tensor dx, dw;
+        if (ctx->needs_input_grad(0)) {
+            dx = out_buffer(on, T, K, FP4Q_OUT_BF16, dy);
+            check_unlocked(lib.gemm_dgrad(&q.t, &qw.t, dx.data_ptr(), out_pitch(dx, K), FP4Q_OUT_BF16, nullptr, ws.data_ptr(), (size_t)ws.numel(), on.handle),
+                           "fp4q_gemm_dgrad");
+            dx = as_type(dx, numbers[3]);
+        }
+        if (ctx->needs_input_grad(1)) {
+            dw = out_buffer(on, N, K, FP4Q_OUT_F32, dy);
+            check_unlocked(lib.gemm_wgrad(&q.t, &qx.t, dw.data_ptr(), out_pitch(dw, K), FP4Q_OUT_F32, 0, nullptr, ws.data_ptr(), (size_t)ws.numel(), on.handle),
+                           "fp4q_gemm_wgrad");
+            dw = as_type(dw, numbers[4]);
+        }
+        ctx->saved_data.clear();
+        return {dx, dw, at::Tensor()};
+    }
+};
+
+// x [T, K], weight [N, K], seed, tensor_id, ws
+PyObject *linear(Args a, Py_ssize_t n)
+{
+    want(n, 5);
+    const at::Tensor x = as_tensor(a[0]), weight = as_tensor(a[1]);
+    const LinearCall call{as_tensor(a[4]), as_bits(a[2]), (uint32_t)as_bits(a[3])};
+    at::Tensor y;
+    {
+        Unlock u;
+        y = LinearNode::apply(x, weight, call);
+    }
+    return THPVariable_Wrap(y);
+}
+
 template <typename F>
 void set_entry(PyObject *addresses, const char *name, F &slot)
 {
@@ -576,6 +708,7 @@ PyMethodDef methods[] = {METHOD("init", init),
                          METHOD("gemm_wgrad_act1d", gemm_wgrad_act1d),
                          METHOD("mxfp8_gemm", mxfp8_gemm),
                          METHOD("mxfp8_qk", mxfp8_qk),
+                         METHOD("linear", linear),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_host", "argument marshalling of binding.py", -1, methods, nullptr, nullptr, nullptr, nullptr};
 
