@@ -31,7 +31,8 @@ EXPORTS = ["fp4q_quantize2d", "fp4q_gemm_fwd", "fp4q_gemm_dgrad", "fp4q_gemm_wgr
            "fp4q_status_string", "fp4q_version", "fp4q_gemm_fwd_static_workspace", "fp4q_workspace_set_wait_limit",
            "fp4q_debug_withhold_load", "fp4q_quantize1d", "fp4q_quantize1d_t", "fp4q_gemm_fwd_act1d", "fp4q_gemm_wgrad_act1d",
            "fp4q_mxfp8_quantize1d_t", "fp4q_mxfp8_gemm", "fp4q_gemm_fwd_quantized", "fp4q_gemm_dgrad_quantized",
-           "fp4q_gemm_fwd_b16", "fp4q_gemm_dgrad_b16", "fp4q_gemm_wgrad_b16", "fp4q_quantize2d_multi"]
+           "fp4q_gemm_fwd_b16", "fp4q_gemm_dgrad_b16", "fp4q_gemm_wgrad_b16", "fp4q_quantize2d_multi",
+           "fp4q_quantize2d_multi_f32"]
 
 
 class Fp4qError(RuntimeError):
@@ -119,6 +120,8 @@ def lib() -> ctypes.CDLL:
                                               ctypes.POINTER(_CTensor), ci, u64, u32, vp, vp, ctypes.c_size_t, vp]
         L.fp4q_quantize2d_multi.restype = ci
         L.fp4q_quantize2d_multi.argtypes = [ctypes.POINTER(_CQuantJob), ctypes.c_int32, ci, u64, vp]
+        L.fp4q_quantize2d_multi_f32.restype = ci
+        L.fp4q_quantize2d_multi_f32.argtypes = [ctypes.POINTER(_CQuantJob), ctypes.c_char_p, ctypes.c_int32, ci, u64, vp]
         b16_args = [ctypes.POINTER(_CTensor), ctypes.POINTER(_CTensor), vp, i64, ci, vp, ctypes.c_size_t, vp]
         L.fp4q_gemm_fwd_b16.restype = ci
         L.fp4q_gemm_fwd_b16.argtypes = b16_args
