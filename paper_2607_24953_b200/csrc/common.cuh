@@ -50,7 +50,7 @@ inline bool capturing(cudaStream_t stream)
 }
 // A launch of `kernel` with one parameter block; always: as a dependent whatever its size.
 template <typename P>
-inline cudaError_t launch_dependent(void (*kernel)(const P), dim3 grid, int threads, cudaStream_t stream, const P &p, bool always = false)
+inline cudaError_t launch_dependent(void (*kernel)(const P), dim3 grid, int threads, cudaStream_t stream, const P &p, bool always = false, int smem = 0)
 {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
@@ -58,6 +58,7 @@ inline cudaError_t launch_dependent(void (*kernel)(const P), dim3 grid, int thre
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = always || ((int64_t)grid.x * grid.y <= kShortGrid && !capturing(stream)) ? 1 : 0;

@@ -140,30 +140,46 @@ __device__ __forceinline__ void load_segment(const Quant2dParams &p, int64_t i, 
 //
 // Per-element 16-bit loads cost 128 load instructions a lane, and one Philox call per element sixteen times the
 // arithmetic.  Here a warp copies its 32 rows as aligned 16-byte pieces (17 cover 128 elements at any offset) into its own
-// staging rows with cp.async, each lane reads its segments back with three 128-bit shared loads a row and shifts them
-// into place; the nine Philox blocks that a row's 128 elements touch are drawn once per warp (9 per lane instead of 128)
-// into the same staging rows and shifted alike.  Measured on 4099 x 2731 (5.1 us at the
-// measured copy bandwidth): stochastic 102 -> 18.2 us, nearest 18.4 -> 13.3 us; 4099 x 1003, stochastic: 50.5 -> 9.9 us.
+// staging rows with cp.async and draws the nine Philox blocks that each row's 128 elements touch, once per warp, while they are on
+// their way; each lane reads its segments back with three 128-bit shared loads a row and shifts them, and their random bytes, into
+// place.  Bound by instructions and by the phases of a CTA, which only other CTAs overlap: with the copies waited for first, every
+// piece checked against the tensor's ends and the random blocks drawn afterwards into the same rows, us, nearest / stochastic:
+// 4099 x 2731 13.0 / 18.0 -> 12.2 / 16.4 (5.1 at the measured copy bandwidth), 16384 x 2731 41.3 / 58.7 -> 34.6 / 46.0,
+// 9001 x 8191 65.0 / 89.0 -> 52.1 / 70.6, 300 x 777 6.1 / 7.8 -> 6.0 / 7.4.
 constexpr int kStageRowBytes = 272;                        // 17 pieces
 constexpr int kStageRows4 = 4 * kStageRowBytes + 32;       // the rows r, 8 + r, 16 + r, 24 + r, which one load instruction reads
-constexpr int kRandomRowBytes = 160;                       // 9 blocks, padded: eight lanes' 16-byte reads fall into different banks
 constexpr int kStageWarpBytes = 8 * kStageRows4;
-static_assert(32 * kRandomRowBytes <= kStageWarpBytes, "random bytes reuse the staging rows");
 
 // Row r of row group rg.  The extra 32 bytes after the second of four rows make the offsets 0, 1, 4, 5 (in 16-byte units,
 // modulo 8), so that the eight lanes of one shared-memory pass (four row groups x two column halves, 32 bytes apart)
 // read eight different bank groups.
 __device__ __forceinline__ int stage_row_offset(int r, int rg) { return r * kStageRows4 + rg * kStageRowBytes + (rg >> 1) * 32; }
 
+// Starts the copies (the caller waits).  Tiles whose pieces all lie inside the tensor need no checks.
 __device__ __forceinline__ void stage_tile_rows(const Quant2dParams &p, int64_t tile_row0, int64_t tile_col0, uint8_t *stage, int lane)
 {
-    const int n_valid = (int)(p.cols - tile_col0 < 128 ? p.cols - tile_col0 : 128);
     const uintptr_t lo = reinterpret_cast<uintptr_t>(p.x), hi = reinterpret_cast<uintptr_t>(p.x + (p.rows - 1) * p.ld_x + p.cols);
+    const uintptr_t a0 = reinterpret_cast<uintptr_t>(p.x + tile_row0 * p.ld_x + tile_col0), pitch = 2 * (uintptr_t)p.ld_x;
+    const uint32_t dst0 = (uint32_t)__cvta_generic_to_shared(stage) + 16 * (lane & 15);
+    if (tile_row0 + 32 <= p.rows && tile_col0 + 128 <= p.cols && (a0 & ~(uintptr_t)15) >= lo && ((a0 + 31 * pitch) & ~(uintptr_t)15) + kStageRowBytes <= hi) {
+        uintptr_t a = a0 + (lane >> 4) * pitch;
+#pragma unroll
+        for (int k = 0; k < 16; k++) {   // two rows of 16 pieces per step, the 17th pieces of all rows last
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                         ::"r"(dst0 + stage_row_offset((2 * k) & 7, k >> 2) + (lane >> 4) * kStageRows4), "l"((a & ~(uintptr_t)15) + 16 * (lane & 15)) : "memory");
+            a += 2 * pitch;
+        }
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                     ::"r"((uint32_t)__cvta_generic_to_shared(stage) + stage_row_offset(lane & 7, lane >> 3) + 256), "l"(((a0 + lane * pitch) & ~(uintptr_t)15) + 256)
+                     : "memory");
+        return;
+    }
+    const int n_valid = (int)(p.cols - tile_col0 < 128 ? p.cols - tile_col0 : 128);
 #pragma unroll 1
-    for (int k = 0; k < 17; k++) {   // two rows of 16 pieces per step, the 17th pieces of all rows last
+    for (int k = 0; k < 17; k++) {
         const int row = k < 16 ? 2 * k + (lane >> 4) : lane, c = k < 16 ? lane & 15 : 16;
         if (tile_row0 + row >= p.rows) continue;
-        const uintptr_t a = reinterpret_cast<uintptr_t>(p.x + (tile_row0 + row) * p.ld_x + tile_col0);
+        const uintptr_t a = a0 + row * pitch;
         const uintptr_t g = (a & ~(uintptr_t)15) + 16 * c;
         if (g >= a + 2 * n_valid) continue;
         uint8_t *dst = stage + stage_row_offset(row & 7, row >> 3) + 16 * c;
@@ -177,8 +193,6 @@ __device__ __forceinline__ void stage_tile_rows(const Quant2dParams &p, int64_t 
             }
         }
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncwarp();
 }
 
 // One row's segment (16 elements) of the staged tile; off: the row's offset into its first piece, in bytes.
@@ -199,27 +213,26 @@ __device__ __forceinline__ void read_staged_segment(const uint8_t *src, uint32_t
     for (int k = 0; k < 8; k++) out[k] = __funnelshift_r(w[k], w[k + 1], 8 * (off & 2));
 }
 
-// The Philox blocks that the warp's 32 rows of 128 elements touch, nine per row, into the staging rows.
-__device__ __forceinline__ void stage_random_bytes(const Quant2dParams &p, int64_t tile_row0, int64_t tile_col0, uint8_t *stage, int lane)
+// The Philox blocks that the warp's 32 rows of 128 elements touch, nine per row: each lane draws the one in which its own segment
+// of each of its eight rows starts (`own`, 128 apart) and the ninth of the row that has its number (`ninth`).  A segment's bytes
+// run on into the block of its right neighbour, or into the ninth.
+__device__ __forceinline__ void draw_row_blocks(const Quant2dParams &p, int64_t tile_row0, int64_t tile_col0, int rg, int seg, uint4 *own, uint4 *ninth, int lane)
 {
-    const int n_valid = (int)(p.cols - tile_col0 < 128 ? p.cols - tile_col0 : 128);
+    uint64_t idx = (uint64_t)(tile_row0 + 8 * rg) * (uint64_t)p.cols + (uint64_t)tile_col0;
 #pragma unroll 1
-    for (int q = lane; q < 32 * 9; q += 32) {
-        const int row = q / 9, b = q - 9 * row;
-        const uint64_t idx = (uint64_t)(tile_row0 + row) * (uint64_t)p.cols + (uint64_t)tile_col0;
-        if (tile_row0 + row >= p.rows || 16 * b >= n_valid + (int)(idx & 15)) continue;
-        const uint64_t blk = (idx >> 4) + b;
+    for (int r = 0; r < 9; r++) {
+        if (r == 8) idx = (uint64_t)(tile_row0 + lane) * (uint64_t)p.cols + (uint64_t)tile_col0;
+        const uint64_t blk = (idx >> 4) + (r < 8 ? seg : 8);
         uint32_t R[4];
         philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), p.tensor_id, 0u, p.keys, R);
-        *reinterpret_cast<uint4 *>(stage + (4 * (row & 7) + (row >> 3)) * kRandomRowBytes + 16 * b) = make_uint4(R[0], R[1], R[2], R[3]);
+        *(r < 8 ? own + 128 * r : ninth + 4 * (lane & 7) + (lane >> 3)) = make_uint4(R[0], R[1], R[2], R[3]);
+        idx += (uint64_t)p.cols;
     }
-    __syncwarp();
 }
 
 // A segment's 16 random bytes; off: the row's offset into its first Philox block (0 .. 15).
-__device__ __forceinline__ void read_staged_random(const uint8_t *src, uint32_t off, uint32_t R[4])
+__device__ __forceinline__ void read_staged_random(const uint4 &a, const uint4 &b, uint32_t off, uint32_t R[4])
 {
-    const uint4 a = reinterpret_cast<const uint4 *>(src)[0], b = reinterpret_cast<const uint4 *>(src)[1];
     uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     const bool by2 = off & 8, by1 = off & 4;
 #pragma unroll
@@ -261,9 +274,9 @@ __device__ __forceinline__ void segment_random_bytes(const Quant2dParams &p, int
 // columns each), a 64x64 block sixteen lanes in each of two neighbouring warps, which exchange their maxima through
 // `xchg`.  With BLK = 64 the scale is still written once per 32x32 tile (four equal entries per block), so that the
 // tensor feeds the GEMMs as it stands; with BLK = 16 the scale matrix has one entry per 16x16 block.
-// STAGED = the tile goes through staging rows (above), of which `rnd_stage` then is the start.
+// STAGED = the tile goes through staging rows (above); the transposed payload's staging (qt_stage) then takes their place.
 template <int MODE, bool FAST, int BLK, bool STAGED = false, bool F32 = false>
-__device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_stage, uint4 *rnd_stage, uint32_t *xchg)
+__device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_stage, uint4 *rnd_stage, uint32_t *xchg, uint4 *staging = nullptr)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t = lane >> 3;          // which of the warp's four 32x32 blocks
@@ -302,8 +315,12 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
                            "=r"(raw[r][5]), "=r"(raw[r][6]), "=r"(raw[r][7])
                          : "l"(src + r * p.ld_x));
     } else if (STAGED) {
-        uint8_t *stage = reinterpret_cast<uint8_t *>(rnd_stage) + warp * kStageWarpBytes;
+        uint8_t *stage = reinterpret_cast<uint8_t *>(staging) + warp * kStageWarpBytes;
         stage_tile_rows(p, tile_row0, bx * 128, stage, lane);
+        if (MODE == FP4Q_ROUND_STOCHASTIC)   // while the copies are on their way
+            draw_row_blocks(p, tile_row0, bx * 128, rg, 2 * t + ch, rnd_stage + threadIdx.x, rnd_stage + 8 * 128 + 32 * warp, lane);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
 #pragma unroll
         for (int r = 0; r < 8; r++) {
             if (row0 + r < p.rows && col0 < p.cols) {
@@ -318,10 +335,6 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
 #pragma unroll
                 for (int k = 0; k < 8; k++) raw[r][k] = 0u;
             }
-        }
-        if (MODE == FP4Q_ROUND_STOCHASTIC) {
-            __syncwarp();   // every lane has read its elements: the rows are free
-            stage_random_bytes(p, tile_row0, bx * 128, stage, lane);
         }
     } else {
 #pragma unroll
@@ -440,9 +453,10 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
             uint32_t R[4] = {0u, 0u, 0u, 0u};
             if (MODE == FP4Q_ROUND_STOCHASTIC) {
                 if (STAGED) {
-                    const uint8_t *src = reinterpret_cast<const uint8_t *>(rnd_stage) + warp * kStageWarpBytes + (4 * r + rg) * kRandomRowBytes;
-                    const uint32_t off = (uint32_t)((uint64_t)i * (uint64_t)p.cols + (uint64_t)(bx * 128)) & 15u;
-                    read_staged_random(src + 16 * (2 * t + ch), off, R);
+                    const uint32_t off = ((uint32_t)i * (uint32_t)p.cols) & 15u;   // a tile starts on a multiple of 128
+                    const uint4 a = rnd_stage[r * 128 + threadIdx.x];
+                    const uint4 b = 2 * t + ch < 7 ? rnd_stage[r * 128 + threadIdx.x + (ch ? 7 : 1)] : rnd_stage[8 * 128 + 32 * warp + 4 * r + rg];
+                    read_staged_random(a, b, off, R);
                 } else if (FAST || p.rng_aligned) {
                     const uint4 v = rnd_stage[r * 128 + threadIdx.x];
                     R[0] = v.x; R[1] = v.y; R[2] = v.z; R[3] = v.w;
@@ -467,6 +481,7 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
 
     // transposed payload: per lane two 8x8 nibble blocks -> 16 words (one per column, 8 rows each)
     uint32_t *stage = reinterpret_cast<uint32_t *>(qt_stage);
+    if (STAGED) __syncthreads();   // every warp has read its rows
 #pragma unroll
     for (int g = 0; g < 2; g++) {
         uint32_t a[8];
@@ -512,17 +527,19 @@ __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_kernel(
     if (!p.waits) wait_for_predecessor();
 }
 
-// Every tile of a tensor whose rows start anywhere or whose segments straddle Philox blocks.  Static shared memory (44 KB with the
-// transposed payload's staging) and 128 registers allow four CTAs per SM, like the aligned kernel.
+// Every tile of a tensor whose rows start anywhere or whose segments straddle Philox blocks.  With the random blocks in memory of their
+// own they are drawn while the rows are on their way; the transposed payload's staging takes the place of the rows, so that 53 KB
+// and 128 registers allow four CTAs per SM, like the aligned kernel.
+template <int MODE> constexpr int kStagedSmem = 4 * kStageWarpBytes + (MODE == FP4Q_ROUND_STOCHASTIC ? (8 * 128 + 4 * 32) * 16 : 0);
+static_assert(4 * kStageWarpBytes >= 128 * 4 * 16, "the transposed payload's staging fits in the rows");
 template <int MODE, int BLK = 32>
 __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_staged_kernel(const __grid_constant__ Quant2dParams p)
 {
-    __shared__ uint4 qt_stage[128 * 4];
-    __shared__ uint4 stage[4 * kStageWarpBytes / 16];
+    extern __shared__ uint4 dynamic_stage[];
     __shared__ uint32_t xchg[BLK == 64 ? 16 : 1];
     if (p.waits) wait_for_predecessor();
     admit_successor();
-    quantize_tile<MODE, false, BLK, true>(p, qt_stage, stage, xchg);
+    quantize_tile<MODE, false, BLK, true>(p, dynamic_stage, dynamic_stage + 4 * kStageWarpBytes / 16, xchg, dynamic_stage);
     if (!p.waits) wait_for_predecessor();   // as in quantize2d_kernel
 }
 
@@ -550,7 +567,7 @@ typedef void (*Quant2dKernel)(const Quant2dParams);
 // (nearest / stochastic, us, direct and staged: 4096 x 4096 in a pitch of 4104 14.7 / 18.1 and 16.8 / 22.9, 16384 x 4096 40.9 /
 // 54.7 and 55.8 / 80.1, 4099 x 2728 nearest 14.9 and 14.7).  Anything else is staged, except for the transposed index, whose
 // random bytes run down the columns.
-static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr)
+static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr, int *smem)
 {
     const bool staged = !(p.x_vec_ok && p.rng_aligned) && !(sr && (p.flags & FP4Q_INDEX_TRANSPOSED));
     const int which = (p.flags & FP4Q_BLOCK_16) ? 1 : (p.flags & FP4Q_BLOCK_64) ? 2 : 0;
@@ -561,7 +578,15 @@ static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr)
           quantize2d_staged_kernel<FP4Q_ROUND_NEAREST, 64>},
          {quantize2d_staged_kernel<FP4Q_ROUND_STOCHASTIC>, quantize2d_staged_kernel<FP4Q_ROUND_STOCHASTIC, 16>,
           quantize2d_staged_kernel<FP4Q_ROUND_STOCHASTIC, 64>}}};
+    *smem = !staged ? 0 : sr ? kStagedSmem<FP4Q_ROUND_STOCHASTIC> : kStagedSmem<FP4Q_ROUND_NEAREST>;
     return kernels[staged][sr][which];
+}
+
+static fp4q_status launch_quantizer(Quant2dKernel kernel, int64_t n_cta, int smem, cudaStream_t stream, const Quant2dParams &p, bool later)
+{
+    // More than 48 KB are asked for by each launch: an attribute of the kernel on the current device, whose setting costs 0.2 us.
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return launched(cudaErrorUnknown);
+    return launched(launch_dependent(kernel, dim3((unsigned)n_cta), 128, stream, p, later, smem));
 }
 
 }  // namespace fp4q
@@ -614,7 +639,9 @@ extern "C" fp4q_status fp4q_quantize2d(const void *x_bf16, int64_t rows, int64_t
     if (n_cta == 0) return FP4Q_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     p.waits = 1;
-    return launched(launch_dependent(quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC), dim3((unsigned)n_cta), 128, s, p));
+    int smem;
+    const Quant2dKernel kernel = quantize2d_kernel_for(p, mode == FP4Q_ROUND_STOCHASTIC, &smem);
+    return launch_quantizer(kernel, n_cta, smem, s, p, false);
 }
 
 static fp4q_status quantize2d_jobs(const fp4q_quantize_job *jobs, const uint8_t *is_f32, int32_t n_jobs, fp4q_round mode, uint64_t seed, void *stream)
@@ -643,9 +670,10 @@ static fp4q_status quantize2d_jobs(const fp4q_quantize_job *jobs, const uint8_t 
             }
             if (pass == 0) continue;
             p.waits = first;
+            int smem = 0;
             const Quant2dKernel kernel = f32 ? (sr ? quantize2d_f32_kernel<FP4Q_ROUND_STOCHASTIC> : quantize2d_f32_kernel<FP4Q_ROUND_NEAREST>)
-                                             : quantize2d_kernel_for(p, sr);
-            if (fp4q_status st = launched(launch_dependent(kernel, dim3((unsigned)n_cta), 128, s, p, !first))) return st;
+                                             : quantize2d_kernel_for(p, sr, &smem);
+            if (fp4q_status st = launch_quantizer(kernel, n_cta, smem, s, p, !first)) return st;
             first = false;
         }
     }
