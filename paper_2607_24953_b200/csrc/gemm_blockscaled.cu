@@ -560,7 +560,7 @@ enum { SCALES_WHOLE = 0, SCALES_SHIFTED = 1, SCALES_GATHER = 2 };
 __device__ __forceinline__ const uint8_t *chunk_word(const ScaleView &v, int rt0, int kb, int kb0, int i, int &n)
 {
     if (v.stride_kb != 1) {
-        const int rt = rt0 + (i & ~3) < v.n_row ? rt0 + (i & ~3) : rt0;
+        const int rt = rt0 + (i & ~3) < v.n_row ? rt0 + (i & ~3) : rt0 < v.n_row ? rt0 : 0;   // 0: the second CTA of a pair, all of whose rows lie beyond
         n = v.n_row - rt;
         return v.ptr + min(kb + (i & 3), v.n_kb - 1) * v.stride_kb + rt;
     }

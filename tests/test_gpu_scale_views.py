@@ -22,8 +22,9 @@ def elsewhere(q, gap, start):
     return dataclasses.replace(q, scale=scale)
 
 
-# contractions of 1, 2, 5, 10, 11, 22, 31 and 33 chunks of 128 in one of the three products, row tiles at the tile's edge and beyond
-@pytest.mark.parametrize("T,N,K", [(100, 70, 200), (300, 777, 1234), (161, 1311, 2731), (257, 640, 1280), (520, 1400, 4200), (128, 256, 3968)])
+# contractions of 1, 2, 5, 10, 11, 12, 22, 31 and 33 chunks of 128 in one of the three products, row tiles at the tile's edge and beyond,
+# second CTAs of a pair that have no rows
+@pytest.mark.parametrize("T,N,K", [(100, 70, 200), (300, 777, 1234), (161, 1311, 2731), (257, 640, 1280), (520, 1400, 4200), (128, 256, 3968), (1500, 300, 70)])
 def test_products_do_not_depend_on_where_the_scales_lie(T, N, K):
     g = torch.Generator(device="cuda").manual_seed(T + N + K)
     scales = torch.exp2(torch.randint(-6, 7, (3,), generator=g, device="cuda").float())
