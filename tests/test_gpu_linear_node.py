@@ -145,3 +145,17 @@ def test_hooks_streams_and_threads():
     assert not errors
     for y, gx in out.values():
         assert torch.equal(y, want) and torch.equal(gx, b.grad)
+
+
+@pytest.mark.parametrize("which", [0, 1])
+@pytest.mark.parametrize("lazy", ["negative bit", "zeros without memory"])
+def test_fp32_operands_whose_memory_does_not_hold_their_values(which, lazy):
+    x, w, _ = leaves(20, 48, 64, torch.float32, torch.float32)
+    ops = [x, w]
+    ops[which] = torch._neg_view(ops[which]) if lazy == "negative bit" else torch._efficientzerotensor(ops[which].shape, device="cuda")
+    ws = binding.alloc_workspace("cuda")
+    y = autograd.fp4_linear(*ops, 0, 0, ws)
+    assert torch.equal(y, python_layer(*ops, 0, 0, ws))
+    plain = [x, w]
+    plain[which] = -plain[which] if lazy == "negative bit" else torch.zeros(plain[which].shape, device="cuda")
+    assert torch.equal(y, autograd.fp4_linear(*plain, 0, 0, ws))
