@@ -572,12 +572,12 @@ at::Tensor as_bf16(const at::Tensor &t)
     return c.is_contiguous() ? c : c.contiguous();
 }
 // What the quantizer reads of an operand: an FP32 one as it is, where its rows start on 16 bytes (a BF16 copy of a 2048 x 2048 weight
-// took 6 us, and 7 of host time); else BF16.  The copy is also what resolves a tensor whose memory does not hold its values: the
-// negative bit, and zeros without memory.
+// took 6 us, and 7 of host time); else BF16.  A single row is contiguous whatever its pitch, and the quantizer checks the pitch.  The
+// copy is also what resolves a tensor whose memory does not hold its values: the negative bit, and zeros without memory.
 at::Tensor as_source(const at::Tensor &t)
 {
-    const bool as_it_is = t.scalar_type() == at::kFloat && t.is_contiguous() && t.size(1) % 4 == 0 && !t.is_neg() && !t._is_zerotensor() &&
-                          reinterpret_cast<uintptr_t>(t.data_ptr()) % 16 == 0;
+    const bool as_it_is = t.scalar_type() == at::kFloat && t.is_contiguous() && t.size(1) % 4 == 0 && pitch(t) % 4 == 0 &&
+                          reinterpret_cast<uintptr_t>(t.data_ptr()) % 16 == 0 && !t.is_neg() && !t._is_zerotensor();
     return as_it_is ? t : as_bf16(t);
 }
 at::Tensor as_type(const at::Tensor &t, int64_t dtype) { return t.scalar_type() == (at::ScalarType)dtype ? t : t.to((at::ScalarType)dtype); }

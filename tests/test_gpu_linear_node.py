@@ -159,3 +159,28 @@ def test_fp32_operands_whose_memory_does_not_hold_their_values(which, lazy):
     plain = [x, w]
     plain[which] = -plain[which] if lazy == "negative bit" else torch.zeros(plain[which].shape, device="cuda")
     assert torch.equal(y, autograd.fp4_linear(*plain, 0, 0, ws))
+
+
+def both_layers(x, w, dy):
+    """Outputs and gradients of the native node and of the Python function for the same operands."""
+    ws, got = binding.alloc_workspace("cuda"), []
+    for layer in (autograd.fp4_linear, python_layer):
+        a, b = x.detach().requires_grad_(), w.detach().requires_grad_()
+        y = layer(a, b, 5, 3, ws)
+        y.backward(dy.to(y.dtype))
+        got.append((y.detach(), a.grad, b.grad))
+    assert type(y.grad_fn).__name__ == "_FP4LinearFnBackward"
+    return got
+
+
+@pytest.mark.parametrize("rows", [(1, 48), (20, 1), (1, 1)])   # one activation row, one output feature, both
+@pytest.mark.parametrize("pitch", [64, 70, 72, 257])
+@pytest.mark.parametrize("xd,wd", [(torch.float32, torch.float32), (torch.bfloat16, torch.float32), (torch.float32, torch.bfloat16)])
+def test_single_rows_cut_from_wider_buffers(rows, pitch, xd, wd):
+    T, N = rows
+    x, w, dy = leaves(20, 48, pitch, xd, wd)
+    x, w, dy = x[:T, :64], w[:N, :64], dy[:T, :N]
+    x, w = (x if T == 1 else x.contiguous()), (w if N == 1 else w.contiguous())
+    assert x.is_contiguous() and w.is_contiguous() and (x if T == 1 else w).stride(0) == pitch
+    for u, v in zip(*both_layers(x, w, dy)):
+        assert u.dtype == v.dtype and torch.equal(u, v)
