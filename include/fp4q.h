@@ -152,7 +152,8 @@ fp4q_status fp4q_quantize2d_multi(const fp4q_quantize_job *jobs, int32_t n_jobs,
  * fp4q_quantize2d_multi_f32 -- the same where is_f32[j] != 0 says that jobs[j].x_bf16 points to FP32 elements (ld_x in elements): a
  * master weight, without a BF16 copy of it being made first.  Every element is rounded to BF16 (nearest even) as it is read; the
  * result is that of fp4q_quantize2d on the BF16 copy.  FP32 sources are 16-byte aligned with ld_x a multiple of 4
- * (FP4Q_ERR_ALIGN otherwise).  is_f32 is a HOST array, as jobs is.
+ * (FP4Q_ERR_ALIGN otherwise).  is_f32 is a HOST array, as jobs is.  Stochastic rounding of FP32 sources is meant for columns in
+ * multiples of 16; with any other number a BF16 copy and its quantizer take a quarter of the time.
  */
 fp4q_status fp4q_quantize2d_multi_f32(const fp4q_quantize_job *jobs, const uint8_t *is_f32, int32_t n_jobs, fp4q_round mode,
                                       uint64_t seed, void *stream);

@@ -291,14 +291,24 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
     if (F32 && FAST) {
         const float *src = reinterpret_cast<const float *>(p.x) + row0 * p.ld_x + col0;
         uint32_t wide[8][16];
+        if (p.x_vec_ok == 2) {
 #pragma unroll
-        for (int r = 0; r < 8; r++)
+            for (int r = 0; r < 8; r++)
 #pragma unroll
-            for (int h = 0; h < 2; h++)
-                asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                             : "=r"(wide[r][8 * h]), "=r"(wide[r][8 * h + 1]), "=r"(wide[r][8 * h + 2]), "=r"(wide[r][8 * h + 3]),
-                               "=r"(wide[r][8 * h + 4]), "=r"(wide[r][8 * h + 5]), "=r"(wide[r][8 * h + 6]), "=r"(wide[r][8 * h + 7])
-                             : "l"(src + r * p.ld_x + 8 * h));
+                for (int h = 0; h < 2; h++)
+                    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                                 : "=r"(wide[r][8 * h]), "=r"(wide[r][8 * h + 1]), "=r"(wide[r][8 * h + 2]), "=r"(wide[r][8 * h + 3]),
+                                   "=r"(wide[r][8 * h + 4]), "=r"(wide[r][8 * h + 5]), "=r"(wide[r][8 * h + 6]), "=r"(wide[r][8 * h + 7])
+                                 : "l"(src + r * p.ld_x + 8 * h));
+        } else {   // rows on 16 bytes
+#pragma unroll
+            for (int r = 0; r < 8; r++)
+#pragma unroll
+                for (int h = 0; h < 4; h++)
+                    asm volatile("ld.global.v4.b32 {%0,%1,%2,%3}, [%4];"
+                                 : "=r"(wide[r][4 * h]), "=r"(wide[r][4 * h + 1]), "=r"(wide[r][4 * h + 2]), "=r"(wide[r][4 * h + 3])
+                                 : "l"(src + r * p.ld_x + 4 * h));
+        }
 #pragma unroll
         for (int r = 0; r < 8; r++)
 #pragma unroll
@@ -543,9 +553,13 @@ __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_staged_
     if (!p.waits) wait_for_predecessor();   // as in quantize2d_kernel
 }
 
-// FP32 source, rows on 16-byte boundaries: 5 bytes an element in one pass instead of 6 for a BF16 copy and 3 for its quantizer.  Sixteen
-// 256-bit loads a lane in flight take 128 registers beside everything else: three CTAs an SM instead of four.  The layer's pass, with
-// a BF16 copy of its FP32 weight and without: 128 x 256 x 256 84.6 -> 77.8 us, 8192 x 2048 x 2048 97.2 -> 95.0.
+// FP32 source, rows on 16-byte boundaries: 5 bytes an element in one pass instead of 6 for a BF16 copy and 3 for its quantizer.  The
+// loads of a lane's eight rows in flight take 128 registers beside everything else: three CTAs an SM instead of four.  The layer's
+// pass, with a BF16 copy of its FP32 weight and without: 128 x 256 x 256 84.6 -> 77.8 us, 8192 x 2048 x 2048 97.2 -> 95.0.  Rows on 16 but
+// not 32 bytes take 128-bit loads instead of 256-bit ones; through the body that checks every element they lost to the copy from
+// some 10 million elements on.  us, 32 activation rows and the weight, copy / checked / now: 2048 x 2052 10.8 / 8.5 / 8.1,
+// 4096 x 4100 31.9 / 29.8 / 20.3, 11008 x 4100 75.7 / 81.8 / 45.7.  The layer rounds its operands to nearest; stochastic rounding of rows
+// that straddle Philox blocks (cols % 16 != 0) draws a block per element here, and the copy is the faster way: 4096 x 4100 158.8 / 37.4.
 template <int MODE>
 __global__ void __launch_bounds__(128, 3) quantize2d_f32_kernel(const __grid_constant__ Quant2dParams p)
 {
@@ -554,7 +568,7 @@ __global__ void __launch_bounds__(128, 3) quantize2d_f32_kernel(const __grid_con
     if (p.waits) wait_for_predecessor();
     admit_successor();
     const int64_t bx = (int64_t)blockIdx.x % p.grid_x, by = (int64_t)blockIdx.x / p.grid_x;
-    const bool full = p.x_vec_ok == 2 && p.rng_aligned && (by + 1) * 128 <= p.rows && (bx + 1) * 128 <= p.cols;
+    const bool full = p.rng_aligned && (by + 1) * 128 <= p.rows && (bx + 1) * 128 <= p.cols;
     if (full) quantize_tile<MODE, true, 32, false, true>(p, qt_stage, rnd_stage, nullptr);
     else quantize_tile<MODE, false, 32, false, true>(p, qt_stage, rnd_stage, nullptr);
     if (!p.waits) wait_for_predecessor();   // as in quantize2d_kernel

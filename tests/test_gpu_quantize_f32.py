@@ -44,3 +44,19 @@ def test_unaligned_fp32_sources_are_refused():
     x = torch.zeros(64, 70, device="cuda")
     assert quantize_f32([x[:, 1:65]], [1], 0, 0)[0] == 3       # the address
     assert quantize_f32([x], [1], 0, 0)[0] == 3                # the pitch
+
+
+# Rows on 16 but not on 32 bytes, by the address or by the pitch: whole tiles and tiles at every edge.
+@pytest.mark.parametrize("rows,cols,pitch,start", [(128, 128, 128, 4), (256, 256, 260, 0), (257, 260, 260, 4), (384, 272, 276, 12), (160, 132, 132, 0), (129, 1028, 1028, 0)])
+@pytest.mark.parametrize("mode", [binding.ROUND_NEAREST, binding.ROUND_STOCHASTIC])
+def test_rows_on_16_bytes_match_their_bf16_copies(rows, cols, pitch, start, mode):
+    g = torch.Generator(device="cuda").manual_seed(rows * cols + start)
+    buf = torch.randn(start + rows * pitch, generator=g, device="cuda") * torch.exp2(torch.randint(-8, 9, (start + rows * pitch,), generator=g, device="cuda").float())
+    x = buf[start:].view(rows, pitch)[:, :cols]
+    x[rows - 1, cols - 1], x[0, cols // 2], x[rows // 2, 0] = 3.4e38, float("nan"), float("inf")
+    st, (q,) = quantize_f32([x], [1], mode, 5)
+    assert st == 0
+    want = binding.fp4q_quantize2d(x.to(torch.bfloat16).contiguous(), mode=mode, seed=5, tensor_id=0)
+    assert torch.equal(q.scale, want.scale)
+    assert torch.equal(q.q_rm[:, :(cols + 31) // 32 * 16], want.q_rm[:, :(cols + 31) // 32 * 16])
+    assert torch.equal(q.q_t[:, :(rows + 31) // 32 * 16], want.q_t[:, :(rows + 31) // 32 * 16])
