@@ -257,3 +257,11 @@ def test_rows_on_16_byte_boundaries(rows, cols, pitch, offset, mode, flags):
     if not flags & (binding.BLOCK_16 | binding.BLOCK_64):
         o_rm, o_t, o_s = oracle.quantize2d(workloads.bf16_bits(x), mode, 8, 2, flags)
         assert np.array_equal(strided.q_rm.cpu().numpy()[:, :(cols + 1) // 2], o_rm) and np.array_equal(strided.scale.cpu().numpy(), o_s)
+
+
+# Rows that start anywhere, in warps that have all of their 32 rows, some of them or none
+@pytest.mark.parametrize("rows", [1, 4, 7, 8, 9, 31, 32, 33, 64, 71, 127, 129])
+@pytest.mark.parametrize("cols", [1, 15, 17, 113, 129, 1000])
+def test_stochastic_bands_of_few_rows(rows, cols):
+    g = torch.Generator(device="cuda").manual_seed(1000 * rows + cols)
+    assert_matches_oracle(torch.randn(rows, cols, generator=g, device="cuda").to(torch.bfloat16), 1, seed=rows, tensor_id=cols)
