@@ -577,13 +577,12 @@ __device__ __noinline__ uint32_t load_end_word(const uint8_t *src, const uint8_t
         if (src + e >= lo && src + e < hi) w |= (uint32_t)load_global(src + e) << (8 * e);
     return w;
 }
-// Loads a unit's words of G groups of four row tiles: as they are, where all start on words and exist; otherwise up to two aligned
-// words each, which place_chunk_scales shifts into place when they are needed.  One lane a chunk, that is some four hundred
-// instructions whatever the unit's length; units whose words make one round of gather_scale_rows (12 a chunk, 128 a round) are
-// gathered by all lanes instead (SCALES_GATHER, nothing is loaded yet).  us, forward / input gradient / weight gradient, all
-// units one lane a chunk and all gathered: 300 x 777 x 1234 (10, 7 and 3 chunks) 10.3 / 10.9 / 11.6 and 10.0 / 9.7 / 11.0,
-// 1999 x 1003 x 2731 (22, 8 and 16) 12.8 / 14.4 / 13.7 and 14.9 / 12.3 / 14.2.
-constexpr int kGatherChunks = 10;
+// Loads a unit's words of G groups of four row tiles: as they are, where all start on words and exist; otherwise, of a full unit, up
+// to two aligned words each, which place_chunk_scales shifts into place when they are needed.  One lane a chunk, that is some
+// four hundred instructions whatever the unit's length, so units that are not full are gathered by all lanes instead (12 words a
+// chunk, 128 a round; SCALES_GATHER, nothing is loaded yet).  us, 161 x 2731, forward / input gradient, one lane a chunk and
+// gathered: contraction of 1281 (a unit of 12 chunks) 11.7 / 11.2 and 9.4 / 9.5, of 2305 (20) 12.9 / 12.6 and 11.2 / 11.3, of 3585 (30)
+// 14.7 / 14.4 and 13.7 / 13.8, of 4095 (32, full) 12.4 / 13.0 and 13.0 / 13.6.
 template <int G>
 __device__ __forceinline__ int fetch_chunk_scales(const ScaleView &v, int rt0, int kb0, int n_real, int n_chunks, uint32_t (&w)[4 * G], uint32_t (&next)[4 * G], int lane)
 {
@@ -598,7 +597,7 @@ __device__ __forceinline__ int fetch_chunk_scales(const ScaleView &v, int rt0, i
         }
         return SCALES_WHOLE;
     }
-    if (n_chunks <= kGatherChunks) return SCALES_GATHER;
+    if (n_chunks < kCacheChunks) return SCALES_GATHER;
     const uint8_t *end = v.ptr + (tr ? (v.n_kb - 1) * pitch + v.n_row : (v.n_row - 1) * pitch + v.n_kb);
     if (lane < n_chunks) {
 #pragma unroll
@@ -635,9 +634,9 @@ __device__ __forceinline__ uint4 chunk_image_row(const ScaleView &v, const uint3
     return v.stride_kb != 1 ? transpose4x4_bytes(w[0], w[1], w[2], w[3]) : make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Short units at the ends of a scale matrix, or of scales that start on any byte.  The words of the operands that need it, item q a (chunk, row tile) of A's
-// four row tiles or, after them, of B's eight, spread over the lanes (one lane a chunk, 300 x 777 x 1234 took 0.7 to 1.5 us longer) and
-// gathered in shared memory as rows of 16 bytes.  Slots beyond the tensor hold the pad byte.
+// Units at the ends of a scale matrix, or of scales that start on any byte, but for full ones.  The words of the operands that need it,
+// item q a (chunk, row tile) of A's four row tiles or, after them, of B's eight, spread over the lanes and gathered in shared
+// memory as rows of 16 bytes.  Slots beyond the tensor hold the pad byte.
 __device__ __forceinline__ void gather_scale_rows(const GemmParams &p, const Tile &t, int k0, bool need_a, bool need_b, int n_chunks, uint32_t *dst, int lane)
 {
     const int n_a = need_a ? 4 * n_chunks : 0, n = n_a + (need_b ? 8 * n_chunks : 0);
@@ -645,6 +644,7 @@ __device__ __forceinline__ void gather_scale_rows(const GemmParams &p, const Til
         uint32_t b[4][4];
 #pragma unroll
         for (int j = 0; j < 4; j++) {   // loads of four items in flight before anything is used
+            if (base + 32 * j >= n) break;   // a product of one stage a tile pays for every instruction: 8704 x 256 x 2080 in 8 groups, input gradient 16.6 -> 15.6 us
             const int q = base + 32 * j + lane;
             const bool is_a = q < n_a;
             const int i = is_a ? q : q - n_a, chunk = is_a ? i >> 2 : i >> 3, rt = is_a ? i & 3 : i & 7;
@@ -661,6 +661,7 @@ __device__ __forceinline__ void gather_scale_rows(const GemmParams &p, const Til
         }
 #pragma unroll
         for (int j = 0; j < 4; j++) {
+            if (base + 32 * j >= n) break;
             const int q = base + 32 * j + lane;
             if (q < n) dst[q < n_a ? q : 4 * kCacheChunks + q - n_a] = b[j][0] | b[j][1] << 8 | b[j][2] << 16 | b[j][3] << 24;
         }

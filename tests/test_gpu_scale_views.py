@@ -3,6 +3,7 @@ into place, or byte by byte at the matrix's ends, by their alignment and the con
 0xFF, UE8M0's NaN, so that a byte that does not belong to the tensor shows."""
 import dataclasses
 
+import numpy as np
 import pytest
 import torch
 
@@ -44,5 +45,47 @@ def test_products_do_not_depend_on_where_the_scales_lie(T, N, K):
     for gap, start in ((0, 1), (1, 0), (2, 3), (4 - qx.scale.shape[1] % 4, 4), (7, 2)):
         for got, ref, what in zip(products(*(elsewhere(q, gap, start) for q in (qx, qw, qdy))), plain, ("fwd", "dgrad", "wgrad")):
             assert torch.equal(got, ref), (what, gap, start)   # the same operands and order of sums
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
+
+
+# Units of the builder (32 chunks of 128) that are full, in each of the three products, and units of every other length up to that.
+@pytest.mark.parametrize("T,N,K", [(70, 100, 4100), (100, 4100, 70), (4100, 100, 70), (40, 3970, 3970), (3970, 130, 40), (1500, 1700, 1900), (2200, 2500, 2800), (3100, 3400, 3700)])
+def test_units_of_every_length(T, N, K):
+    test_products_do_not_depend_on_where_the_scales_lie(T, N, K)
+
+
+# Grouped products: every group's scales start somewhere else in the matrix.  Contractions of 12, 2, 33 and 34 chunks in the forward product,
+# of 1, 32 and 33 in the input gradient, and groups of up to 34 chunks, empty ones among them, in the weight gradient.
+@pytest.mark.parametrize("counts,N,K", [((4224, 0, 1400, 1), 96, 100), ((130, 0, 300), 128, 1440), ((129, 1, 0, 260), 64, 4250), ((200, 300), 4096, 160), ((1, 500, 3968), 4160, 100)])
+@pytest.mark.parametrize("alignment", [128, 256])
+def test_grouped_products_do_not_depend_on_where_the_scales_lie(counts, N, K, alignment):
+    counts = np.array(counts)
+    offs = workloads.padded_row_offsets(counts, alignment)
+    T, E = int(offs[-1]), len(counts)
+    g = torch.Generator(device="cuda").manual_seed(T + N + K)
+    x, dy = (workloads.zero_padding_rows((torch.randn(T, c, generator=g, device="cuda") * torch.exp2(torch.randint(-4, 5, (T, 1), generator=g, device="cuda").float())).to(torch.bfloat16),
+                                         counts, offs) for c in (K, N))
+    w = (torch.randn(E * N, K, generator=g, device="cuda") * torch.exp2(torch.randint(-4, 5, (E * N, 1), generator=g, device="cuda").float())).to(torch.bfloat16)
+    qx, qw, qdy = (binding.fp4q_quantize2d(t) for t in (x, w, dy))
+    ws, d_offs = binding.alloc_workspace("cuda"), torch.from_numpy(offs).cuda()
+    dgrad = N % 64 == 0   # a group's contraction ends between two instructions' shares otherwise, and is refused
+
+    def products(x, w, dy):
+        rows = dict(dt=binding.OUT_F32, row_offsets=d_offs, ws=ws, row_alignment=alignment)
+        dw = binding.fp4q_gemm_wgrad(dy, x, row_offsets=d_offs, ws=ws)
+        return [binding.fp4q_gemm_fwd(x, w, **rows), dw] + ([binding.fp4q_gemm_dgrad(dy, w, **rows)] if dgrad else [])
+
+    plain = products(qx, qw, qdy)
+    xd, wd, dyd = (dequant_from_gpu(q) for q in (qx, qw, qdy))
+    check_gemm(plain[0], oracle.grouped(oracle.gemm_fwd, xd, wd, offs), "fwd")
+    if dgrad:
+        check_gemm(plain[2], oracle.grouped(oracle.gemm_dgrad, dyd, wd, offs), "dgrad")
+    ref = oracle.grouped_wgrad(dyd, xd, offs)
+    for e in np.flatnonzero(counts):   # by expert: a small one is not hidden by a large one
+        check_gemm(plain[1][e * N:(e + 1) * N], ref[e * N:(e + 1) * N], "wgrad of expert %d" % e)
+    for gap, start in ((0, 1), (1, 0), (2, 3), (4 - qx.scale.shape[1] % 4, 4), (7, 2)):
+        for got, ref, what in zip(products(*(elsewhere(q, gap, start) for q in (qx, qw, qdy))), plain, ("fwd", "wgrad", "dgrad")):
+            assert torch.equal(got, ref), (what, gap, start)
     torch.cuda.synchronize()
     assert binding.fp4q_workspace_status(ws) == 0
