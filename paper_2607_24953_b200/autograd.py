@@ -42,14 +42,30 @@ class _FP4LinearFn(torch.autograd.Function):
 _TENSORS = (torch.Tensor, torch.nn.Parameter)
 
 
+def _find_observers():
+    """A function that says whether anything looks into Python autograd functions just now: tracers, transforms, modes, forward-mode
+    levels.  None where this torch lacks one of the names, which are not public."""
+    try:
+        compiling, tracing = torch.compiler.is_compiling, torch._C._get_tracing_state
+        transforms, dispatch, function = torch._C._functorch.peek_interpreter_stack, torch._C._len_torch_dispatch_stack, torch._C._len_torch_function_stack
+        forward_ad._current_level   # a variable: read at every call
+    except AttributeError:
+        return None
+
+    def observed() -> bool:
+        return (compiling() or transforms() is not None or dispatch() != 0 or function() != 0 or tracing() is not None
+                or forward_ad._current_level >= 0)
+    return observed
+
+
+_observed = _find_observers()
+
+
 def _plain(x, weight) -> bool:
-    """Ordinary tensors on one GPU and nothing that looks into a Python autograd function (transforms, tracers, modes,
-    forward-mode levels): the native node does the same in half the host's time.  Everything else, what is refused
-    included, goes through _FP4LinearFn."""
-    return (type(x) in _TENSORS and type(weight) in _TENSORS and x.is_cuda and weight.dim() == 2 and x.device == weight.device
-            and torch._C._functorch.peek_interpreter_stack() is None and torch._C._len_torch_dispatch_stack() == 0
-            and torch._C._len_torch_function_stack() == 0 and torch._C._get_tracing_state() is None
-            and forward_ad._current_level < 0 and not torch.compiler.is_compiling())
+    """Ordinary tensors on one GPU and nothing that looks into a Python autograd function: the native node does the same in half
+    the host's time.  Everything else, what is refused included, goes through _FP4LinearFn."""
+    return (_observed is not None and type(x) in _TENSORS and type(weight) in _TENSORS and x.is_cuda and weight.dim() == 2
+            and x.device == weight.device and not _observed())
 
 
 def _linear(x, weight, seed, tensor_id, ws):

@@ -27,14 +27,15 @@ def leaves(T, N, K, xd, wd, transposed=False):
 def test_outputs_and_gradients_are_the_python_functions(T, N, K, xd, wd, needs, transposed):
     x, w, dy = leaves(T, N, K, xd, wd, transposed)
     ws = binding.alloc_workspace("cuda")
-    got = []
+    got, nodes = [], []
     for layer in (autograd.fp4_linear, python_layer):
         a, b = x.detach().requires_grad_(needs[0]), w.detach().requires_grad_(needs[1])
         y = layer(a, b, 2 ** 63 + 5, 9, ws)
         assert y.dtype == torch.bfloat16 and y.is_contiguous() and y.requires_grad
+        nodes.append(type(y.grad_fn).__name__)
         y.backward(dy.to(y.dtype))
         got.append((y.detach(), a.grad, b.grad))
-    assert type(y.grad_fn).__name__ == "_FP4LinearFnBackward"
+    assert nodes[0] != "_FP4LinearFnBackward" and nodes[1] == "_FP4LinearFnBackward"   # two ways to the same result
     for u, v in zip(*got):
         assert (u is None) == (v is None)
         assert u is None or (u.dtype == v.dtype and u.shape == v.shape and torch.equal(u, v))
@@ -132,6 +133,7 @@ def test_hooks_streams_and_threads():
                 for _ in range(20):
                     c = x.detach().requires_grad_()
                     y = autograd.fp4_linear(c, w, 3, 4, own)
+                    assert type(y.grad_fn).__name__ != "_FP4LinearFnBackward"
                     y.backward((2 * dy.to(y.dtype)))
                 out[i] = (y.detach().clone(), c.grad.clone())
             stream.synchronize()
@@ -163,13 +165,14 @@ def test_fp32_operands_whose_memory_does_not_hold_their_values(which, lazy):
 
 def both_layers(x, w, dy):
     """Outputs and gradients of the native node and of the Python function for the same operands."""
-    ws, got = binding.alloc_workspace("cuda"), []
+    ws, got, nodes = binding.alloc_workspace("cuda"), [], []
     for layer in (autograd.fp4_linear, python_layer):
         a, b = x.detach().requires_grad_(), w.detach().requires_grad_()
         y = layer(a, b, 5, 3, ws)
+        nodes.append(type(y.grad_fn).__name__)
         y.backward(dy.to(y.dtype))
         got.append((y.detach(), a.grad, b.grad))
-    assert type(y.grad_fn).__name__ == "_FP4LinearFnBackward"
+    assert nodes[0] != "_FP4LinearFnBackward" and nodes[1] == "_FP4LinearFnBackward"
     return got
 
 
@@ -184,3 +187,17 @@ def test_single_rows_cut_from_wider_buffers(rows, pitch, xd, wd):
     assert x.is_contiguous() and w.is_contiguous() and (x if T == 1 else w).stride(0) == pitch
     for u, v in zip(*both_layers(x, w, dy)):
         assert u.dtype == v.dtype and torch.equal(u, v)
+
+
+def test_without_the_private_names_the_python_function_runs(monkeypatch):
+    x, w, dy = leaves(20, 48, 64, torch.bfloat16, torch.float32)
+    want = both_layers(x, w, dy)[1]
+    monkeypatch.delattr(torch._C, "_len_torch_function_stack")
+    monkeypatch.setattr(autograd, "_observed", autograd._find_observers())
+    a, b = x.detach().requires_grad_(), w.detach().requires_grad_()
+    y = autograd.fp4_linear(a, b, 5, 3, binding.alloc_workspace("cuda"))
+    assert type(y.grad_fn).__name__ == "_FP4LinearFnBackward"
+    monkeypatch.undo()
+    y.backward(dy.to(y.dtype))
+    for u, v in zip((y.detach(), a.grad, b.grad), want):
+        assert torch.equal(u, v)
