@@ -179,3 +179,30 @@ def test_grouped_fused_products_equal_product_then_quantize(mode):
         import ctypes
         binding._check(binding.lib().fp4q_gemm_fwd_quantized(ctypes.byref(cx), ctypes.byref(cw), ctypes.byref(cy), 0, 0, 0,
                                                              ctypes.byref(g128), ws.data_ptr(), ws.numel(), None), "fwd_quantized")
+
+
+@pytest.mark.parametrize("T,N,K", [(160, 192, 256), (300, 528, 1008)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_non_finite_products_are_quantized_as_by_the_quantizer(T, N, K, mode):
+    """Row tile 0 of the left operand is scaled up to the end of FP32's range, so that its blocks mix infinities, NaN (infinities
+    of both signs in one sum) and finite entries; one of its blocks in row tile 2 has UE8M0's NaN as its scale."""
+    qx, qw = binding.fp4q_quantize2d(workloads.weights(T, K, 730, "cuda")), binding.fp4q_quantize2d(workloads.weights(N, K, 731, "cuda"))
+    qdy = binding.fp4q_quantize2d(workloads.weights(T, N, 732, "cuda"))
+    qw.scale += 20   # room for the left operand's scale below its largest code
+    ws = binding.alloc_workspace("cuda")
+    for a, plain, fused, cols in ((qx, binding.fp4q_gemm_fwd, binding.fp4q_gemm_fwd_quantized, N),
+                                  (qdy, binding.fp4q_gemm_dgrad, binding.fp4q_gemm_dgrad_quantized, K)):
+        finite = plain(a, qw, dt=binding.OUT_F32, ws=ws)
+        up = 128 - int(torch.log2(finite[:32].abs().median()).floor())
+        a.scale[0] += up
+        a.scale[2, 1] = 0xFF
+        y = plain(a, qw, dt=binding.OUT_BF16, ws=ws)
+        head = y[:32].float()
+        assert head.isinf().any() and head.isfinite().any() and y[64:96].isnan().all() and y[32:64].isfinite().all()
+        want = binding.fp4q_quantize2d(y.contiguous(), mode=mode, seed=3, tensor_id=8)
+        got = fused(a, qw, mode=mode, seed=3, tensor_id=8, ws=ws)
+        compare_logical(got, *logical(want), T, cols)
+        if mode == 0:
+            compare_logical(got, *oracle.quantize2d(workloads.bf16_bits(y), mode, 3, 8), T, cols)
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
