@@ -277,7 +277,7 @@ __device__ __forceinline__ void segment_random_bytes(const Quant2dParams &p, int
 // `xchg`.  With BLK = 64 the scale is still written once per 32x32 tile (four equal entries per block), so that the
 // tensor feeds the GEMMs as it stands; with BLK = 16 the scale matrix has one entry per 16x16 block.
 // STAGED = the tile goes through staging rows (above); the transposed payload's staging (qt_stage) then takes their place.
-template <int MODE, bool FAST, int BLK, bool STAGED = false, bool F32 = false>
+template <int MODE, bool FAST, int BLK, bool STAGED = false, int F32 = 0>
 __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_stage, uint4 *rnd_stage, uint32_t *xchg, uint4 *staging = nullptr)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -293,23 +293,22 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
     if (F32 && FAST) {
         const float *src = reinterpret_cast<const float *>(p.x) + row0 * p.ld_x + col0;
         uint32_t wide[8][16];
-        if (p.x_vec_ok == 2) {
 #pragma unroll
-            for (int r = 0; r < 8; r++)
+        for (int r = 0; r < 8; r++) {
+            if (F32 == 2) {
 #pragma unroll
                 for (int h = 0; h < 2; h++)
                     asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                                  : "=r"(wide[r][8 * h]), "=r"(wide[r][8 * h + 1]), "=r"(wide[r][8 * h + 2]), "=r"(wide[r][8 * h + 3]),
                                    "=r"(wide[r][8 * h + 4]), "=r"(wide[r][8 * h + 5]), "=r"(wide[r][8 * h + 6]), "=r"(wide[r][8 * h + 7])
                                  : "l"(src + r * p.ld_x + 8 * h));
-        } else {   // rows on 16 bytes
-#pragma unroll
-            for (int r = 0; r < 8; r++)
+            } else {
 #pragma unroll
                 for (int h = 0; h < 4; h++)
                     asm volatile("ld.global.v4.b32 {%0,%1,%2,%3}, [%4];"
                                  : "=r"(wide[r][4 * h]), "=r"(wide[r][4 * h + 1]), "=r"(wide[r][4 * h + 2]), "=r"(wide[r][4 * h + 3])
                                  : "l"(src + r * p.ld_x + 4 * h));
+            }
         }
 #pragma unroll
         for (int r = 0; r < 8; r++)
@@ -562,7 +561,7 @@ __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_staged_
 // some 10 million elements on.  us, 32 activation rows and the weight, copy / checked / now: 2048 x 2052 10.8 / 8.5 / 8.1,
 // 4096 x 4100 31.9 / 29.8 / 20.3, 11008 x 4100 75.7 / 81.8 / 45.7.  The layer rounds its operands to nearest; stochastic rounding of rows
 // that straddle Philox blocks (cols % 16 != 0) draws a block per element here, and the copy is the faster way: 4096 x 4100 158.8 / 37.4.
-template <int MODE>
+template <int MODE, int ROWS>   // ROWS: 2 = rows on 32 bytes, 1 = on 16
 __global__ void __launch_bounds__(128, 3) quantize2d_f32_kernel(const __grid_constant__ Quant2dParams p)
 {
     __shared__ uint4 qt_stage[128 * 4];
@@ -571,8 +570,8 @@ __global__ void __launch_bounds__(128, 3) quantize2d_f32_kernel(const __grid_con
     admit_successor();
     const int64_t bx = (int64_t)blockIdx.x % p.grid_x, by = (int64_t)blockIdx.x / p.grid_x;
     const bool full = p.rng_aligned && (by + 1) * 128 <= p.rows && (bx + 1) * 128 <= p.cols;
-    if (full) quantize_tile<MODE, true, 32, false, true>(p, qt_stage, rnd_stage, nullptr);
-    else quantize_tile<MODE, false, 32, false, true>(p, qt_stage, rnd_stage, nullptr);
+    if (full) quantize_tile<MODE, true, 32, false, ROWS>(p, qt_stage, rnd_stage, nullptr);
+    else quantize_tile<MODE, false, 32, false, ROWS>(p, qt_stage, rnd_stage, nullptr);
     if (!p.waits) wait_for_predecessor();   // as in quantize2d_kernel
 }
 
@@ -687,8 +686,10 @@ static fp4q_status quantize2d_jobs(const fp4q_quantize_job *jobs, const uint8_t 
             if (pass == 0) continue;
             p.waits = first;
             int smem = 0;
-            const Quant2dKernel kernel = f32 ? (sr ? quantize2d_f32_kernel<FP4Q_ROUND_STOCHASTIC> : quantize2d_f32_kernel<FP4Q_ROUND_NEAREST>)
-                                             : quantize2d_kernel_for(p, sr, &smem);
+            static const Quant2dKernel f32_kernels[2][2] = {
+                {quantize2d_f32_kernel<FP4Q_ROUND_NEAREST, 1>, quantize2d_f32_kernel<FP4Q_ROUND_NEAREST, 2>},
+                {quantize2d_f32_kernel<FP4Q_ROUND_STOCHASTIC, 1>, quantize2d_f32_kernel<FP4Q_ROUND_STOCHASTIC, 2>}};
+            const Quant2dKernel kernel = f32 ? f32_kernels[sr][p.x_vec_ok - 1] : quantize2d_kernel_for(p, sr, &smem);
             if (fp4q_status st = launch_quantizer(kernel, n_cta, smem, s, p, !first)) return st;
             first = false;
         }
