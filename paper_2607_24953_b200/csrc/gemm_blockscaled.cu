@@ -637,6 +637,7 @@ __device__ __forceinline__ uint4 chunk_image_row(const ScaleView &v, const uint3
 // Units at the ends of a scale matrix, or of scales that start on any byte, but for full ones.  The words of the operands that need it,
 // item q a (chunk, row tile) of A's four row tiles or, after them, of B's eight, spread over the lanes and gathered in shared
 // memory as rows of 16 bytes.  Slots beyond the tensor hold the pad byte.
+template <bool GROUPED>
 __device__ __forceinline__ void gather_scale_rows(const GemmParams &p, const Tile &t, int k0, bool need_a, bool need_b, int n_chunks, uint32_t *dst, int lane)
 {
     const int n_a = need_a ? 4 * n_chunks : 0, n = n_a + (need_b ? 8 * n_chunks : 0);
@@ -644,7 +645,9 @@ __device__ __forceinline__ void gather_scale_rows(const GemmParams &p, const Til
         uint32_t b[4][4];
 #pragma unroll
         for (int j = 0; j < 4; j++) {   // loads of four items in flight before anything is used
-            if (base + 32 * j >= n) break;   // a product of one stage a tile pays for every instruction: 8704 x 256 x 2080 in 8 groups, input gradient 16.6 -> 15.6 us
+            // One item a lane is all of a short unit, and grouped products of one stage a tile pay for every instruction: 8704 x 256 x 2080 in
+            // 8 groups, input gradient 16.5 -> 15.4 us.  (Dense ones, 0.3 % slower with it, do without.)
+            if (GROUPED && j == 1 && base + 32 >= n) break;
             const int q = base + 32 * j + lane;
             const bool is_a = q < n_a;
             const int i = is_a ? q : q - n_a, chunk = is_a ? i >> 2 : i >> 3, rt = is_a ? i & 3 : i & 7;
@@ -661,7 +664,7 @@ __device__ __forceinline__ void gather_scale_rows(const GemmParams &p, const Til
         }
 #pragma unroll
         for (int j = 0; j < 4; j++) {
-            if (base + 32 * j >= n) break;
+            if (GROUPED && j == 1 && base + 32 >= n) break;
             const int q = base + 32 * j + lane;
             if (q < n) dst[q < n_a ? q : 4 * kCacheChunks + q - n_a] = b[j][0] | b[j][1] << 8 | b[j][2] << 16 | b[j][3] << 24;
         }
@@ -1493,7 +1496,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                     row_b0 = chunk_image_row(p.sfb, wb);
                     row_b1 = chunk_image_row(p.sfb, wb + 4);
                     if (how_a == SCALES_GATHER || how_b == SCALES_GATHER) {
-                        gather_scale_rows(p, un.t, un.k0, how_a == SCALES_GATHER, how_b == SCALES_GATHER, n, reinterpret_cast<uint32_t *>(smem_compact), lane);
+                        gather_scale_rows<kGrouped>(p, un.t, un.k0, how_a == SCALES_GATHER, how_b == SCALES_GATHER, n, reinterpret_cast<uint32_t *>(smem_compact), lane);
                         const uint4 *gathered = reinterpret_cast<const uint4 *>(smem_compact);
                         if (how_a == SCALES_GATHER) row_a = gathered[lane];
                         if (how_b == SCALES_GATHER) { row_b0 = gathered[kCacheChunks + 2 * lane]; row_b1 = gathered[kCacheChunks + 2 * lane + 1]; }
