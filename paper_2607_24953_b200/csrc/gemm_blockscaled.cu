@@ -296,9 +296,13 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
     return r;
 }
 // What such an arrival announces lies in this CTA's own shared memory or tensor memory and was made visible to the asynchronous proxy
-// or fenced before; the other CTA only issues the instructions that read it here.  So release at the default scope is enough;
-// release at cluster scope kept the arrival back for another 400 ns (first MMA of 8192 x 2048 x 2048 1850 -> 1400 ns after the
-// first load).
+// or fenced before; the other CTA only issues the instructions that read it here.  Release at the default scope, this CTA, orders the
+// two, as an assumption about the hardware: that an SM has performed its own stores and the fence behind them before a later
+// arrival of the same thread leaves it.  PTX's memory model does not promise it; there, only release and acquire that both
+// reach the cluster order one CTA's writes before another's reads, and the waits on these barriers have the default scope too.
+// Were it wrong, a pair's MMAs would read scale images of the second CTA that are not written yet, or overwrite an accumulator that is
+// still being read: wrong results and no error.  Release at cluster scope for the images costs a product 0.45 to 0.6 us (forward
+// 2048 x 2048 x 2048 9.9 -> 10.4, 8192 x 2048 x 2048 20.5 -> 21.0, 16384 x 4096 x 4096 94.5 -> 95.2; 16 x 16 blocks there 116.8 -> 121.5).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
@@ -1745,9 +1749,11 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                     const int col0 = t.c_col0 + 128 * half + 32 * j;
                     if (col0 >= p.N || row0_blk >= p.M) continue;   // warp-uniform
                     // The maximum as in the quantizer: packed |.| with NaN propagation (a fifth of the instructions of a comparison per
-                    // element), so that a non-finite entry shows in the result and sends the block through the careful pass.  us, forward / input
-                    // gradient, captured: 300 x 768 x 1232 12.7 / 13.4 -> 11.9 / 12.7, 8192 x 2048 x 2048 30.7 / 35.8 -> 28.7 / 33.3, 16384 x 4096 x 4096
-                    // 107.7 / 114.1 and 109.3 / 115.1 (a pass of both, launched one by one, 259.9 either way).
+                    // element), so that a non-finite entry shows in the result and sends the block through the careful pass.  us, the two
+                    // builds replayed in turn, forward nearest / stochastic: 300 x 768 x 1232 12.8 / 14.2 -> 12.1 / 13.4, 8192 x 2048 x 2048 31.5 /
+                    // 36.4 -> 28.5 / 33.2, 8192 x 5632 x 2048 70.2 / 80.6 -> 62.5 / 73.1.  From 16 stages a tile on the epilogue is hidden and the
+                    // gain with it: 16384 x 4096 x 4096 117.4 / 119.6 -> 117.8 / 119.4, and 16384 x 11008 x 4096 loses with stochastic rounding,
+                    // 280.8 / 320.3 -> 278.9 / 325.0, for a reason that is not known.
                     uint32_t raw[16];
                     __nv_bfloat162 m2 = __float2bfloat162_rn(0.0f);
 #pragma unroll
