@@ -270,10 +270,11 @@ template <int BACKOFF_NS, bool PROBE = false>
 __device__ __forceinline__ bool mbar_wait_impl(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status,
                                                uint64_t limit, uint32_t where)
 {
-    for (uint64_t it = 0; it < limit; it++) {
+    for (uint64_t it = 1; ; it++) {
         if (PROBE ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity)) return true;
         if (BACKOFF_NS > 0) __nanosleep(BACKOFF_NS);
-        if ((!PROBE || ((uint32_t)it & 255u) == 255u) && *abort_flag) return false;
+        if ((!PROBE || ((uint32_t)it & 255u) == 0u) && *abort_flag) return false;
+        if (it >= limit) break;   // after the first poll: a wait that need not wait does not wait for the limit's load either
     }
     *abort_flag = 1u;
     if (atomicCAS(status, 0u, (uint32_t)FP4Q_ERR_TIMEOUT) == 0u) status[1] = where;
@@ -330,6 +331,18 @@ __device__ __forceinline__ uint32_t cluster_ctarank()
 __device__ __forceinline__ void cluster_sync_all()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The kernel's first barrier, which every warp passes at a place of its own: behind it the mbarriers of the CTA, or of both CTAs of
+// a pair, exist.  In a pair warps arrive ahead of time (warp 4, which initializes them, after its fence.mbarrier_init), so that the
+// way from one CTA to the other is under way while a role prepares what needs nobody else.  In one CTA nobody waits for the
+// builders, which come late and have a barrier of their own with warp 4.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+template <int CTAS, int BUILDERS, bool BUILDER = false>
+__device__ __forceinline__ void start_sync()
+{
+    if (CTAS == 2) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else if (BUILDER) asm volatile("bar.sync 12, %0;" ::"n"(32 + 32 * BUILDERS) : "memory");
+    else asm volatile("bar.sync 13, %0;" ::"n"(kThreads - 32 * BUILDERS) : "memory");
 }
 
 // TMA stores out of shared memory (bulk async-group completion).
@@ -1159,27 +1172,37 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     const bool leader = rank == 0;
     const int first_tile = blockIdx.x / CTAS, tile_step = gridDim.x / CTAS;
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; s++) {
-            // The producer's expect_tx arrival (in a pair the leader's, which announces both CTAs' bytes: the second
-            // CTA's loads complete on the leader's barrier).  The watcher of the stage waits on it.
-            mbar_init(bar_full + 8 * s, 1);
-            mbar_init(bar_empty + 8 * s, 1);    // tcgen05.commit
-        }
-        mbar_init(bar_acc_full, 1);
-        mbar_init(bar_drain, 1);
-        mbar_init(bar_acc_empty, 8 * CTAS);     // one arrival per epilogue warp (of both CTAs of a pair)
-        for (int b = 0; b < Cfg<KIND, CTAS>::kImageBufs; b++) {
-            mbar_init(bar_cache_full + 8 * b, 1);
-            mbar_init(bar_cache_empty + 8 * b, 1);
-            mbar_init(bar_peer_cache_full + 8 * b, 1);
-        }
-        *abort_flag = 0u;
+    // Roles start as soon as each can.  With initialization, tensor memory, a barrier and only then decoding and loads one after the
+    // other, the first operand load left 2900 cycles after a pair's first instruction and the first MMA 6100; now 1500 and 5300.  us:
+    // 2048 x 2048 x 2048 9.6 / 9.9 / 11.2 -> 9.5 / 9.6 / 10.9, quantized output 12.6 -> 12.3, 1D activations 11.0 -> 10.4, 300 x 777 x 1234 9.1 / 8.9 /
+    // 9.8 -> 8.8 / 8.7 / 9.4.
+    constexpr int kBuilders = Cfg<KIND, CTAS>::kBuilders;
+    if (warp == 4) {   // an epilogue warp has time
+        // One barrier a lane.  A stage's "full" barrier takes the producer's expect_tx arrival (in a pair the leader's, which announces
+        // both CTAs' bytes: the second CTA's loads complete on the leader's barrier), the accumulator's "empty" barrier one
+        // arrival per epilogue warp (of both CTAs of a pair), every other one commit or one builder.
+        if (lane < 21 || lane >= 24) mbar_init(smem_u32(bars + lane), lane == 13 ? 8 * CTAS : 1);
+        if (lane < 4) mbar_init(smem_u32(bars + 32 + lane), 1);
+        if (lane == 0) *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
-        if (Cfg<KIND, CTAS>::kTmaStores) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmC) : "memory");
-        if (EPI == EPI_QUANT) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmD) : "memory");
+        __threadfence_block();   // the flag, ahead of the relaxed arrival
+        __syncwarp();
+        if (CTAS == 2) cluster_arrive_relaxed();
+        else asm volatile("bar.arrive 12, %0;" ::"n"(32 + 32 * kBuilders) : "memory");   // for the builders
+        if (lane == 0) {
+            if (Cfg<KIND, CTAS>::kTmaStores) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmC) : "memory");
+            if (EPI == EPI_QUANT) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmD) : "memory");
+        }
+        __syncwarp();
+    } else if (CTAS == 2) {
+        cluster_arrive_relaxed();
+    }
+    if (warp == 0) {
+        if (lane == 0) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
+        }
+        __syncwarp();
     }
     if (warp == 1) {
         if (CTAS == 1) {
@@ -1228,12 +1251,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             gorder[before] = (uint16_t)g;
         }
     }
-    tcgen05_fence_before();
-    __syncwarp();
-    if (CTAS == 2) cluster_sync_all();   // the peer's barriers must exist before anything is signalled across CTAs
-    else __syncthreads();
-    tcgen05_fence_after();
-    const uint32_t tmem_base = *tmem_base_slot;
+    if (goffs_ok) __syncthreads();
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -1246,11 +1264,14 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         TRACE_DECL(c_empty); TRACE_DECL(c_issue);
         TRACE_T0(tt);
         int ev_j = 0;
+        bool started = false;
         for (int tile = first_tile; ok && tile < p.n_tile_total; tile += tile_step) {
             Tile t;
             decode_tile<kGrouped>(p, tile, rank, t, goffs, gorder);
             const int n_it = (t.k_len + kStageElems - 1) / kStageElems;
             int xa = t.a_k0 / kElemsPerByte, xb = t.b_k0 / kElemsPerByte;
+            if (!started) start_sync<CTAS, kBuilders>();
+            started = true;
 #pragma unroll 1
             for (int it = 0; it < n_it; it++, xa += 128, xb += 128) {
                 ok = mbar_wait_impl<0>(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.status, wait_limit, 0x100u + stage);
@@ -1279,6 +1300,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 TRACE_ADD(c_issue, tt);
             }
         }
+        if (!started) start_sync<CTAS, kBuilders>();
         if (!ok) {   // give copies already in flight time to land before the CTA's shared memory is released
             for (int i = 0; i < 200; i++) __nanosleep(1000);
         }
@@ -1293,6 +1315,12 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         // barriers BEFORE it issues a stage and waits afterwards only if they were not complete.  All lanes wait: a
         // lane-0 branch around the wait costs as much as the wait.
         uint32_t stage = 0, full_phase = 0, acc_empty_phase = 0;
+        tcgen05_fence_before();
+        __syncwarp();
+        if (CTAS == 2) asm volatile("bar.arrive 14, 288;" ::: "memory");   // tensor memory is there: for the epilogue warps
+        start_sync<CTAS, kBuilders>();
+        tcgen05_fence_after();
+        const uint32_t tmem_base = *tmem_base_slot;
         bool mma_ok = true, ready = false;   // !WATCH: this warp's waits have not run out; the next stage has been seen complete
         BufRing ring;   // image buffer of the current unit
         const bool issuer = elect_one();
@@ -1435,7 +1463,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         if (KIND != KIND_MXF4) {
             // per-row scales: the raw bytes of the next kOwnRaw units are in flight (cp.async) while a unit is turned into
             // images.  Two builders take every other unit and have raw buffers of their own.
-            constexpr int kBuilders = Cfg<KIND, CTAS>::kBuilders, kRawBytes = Cfg<KIND, CTAS>::kRawBytes, kSlotB = Cfg<KIND, CTAS>::kRawSlotB;
+            constexpr int kRawBytes = Cfg<KIND, CTAS>::kRawBytes, kSlotB = Cfg<KIND, CTAS>::kRawSlotB;
             constexpr int kOwnRaw = Cfg<KIND, CTAS>::kRawBufs > 0 ? Cfg<KIND, CTAS>::kRawBufs / kBuilders : 1;
             uint8_t *raw = smem_raw_scales + (3 - warp) * kOwnRaw * kRawBytes;
             UnitIter<false> ahead, cur;
@@ -1469,6 +1497,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                     if (ahead.valid(p)) ahead.next(p, kUnitStages * kStageElems);
             };
             for (int i = 0; i < kOwnRaw; i++) fetch(i);
+            start_sync<CTAS, kBuilders, true>();
             while (cur.valid(p)) {
                 asm volatile("cp.async.wait_group %0;" ::"n"(kOwnRaw - 1) : "memory");   // this unit's bytes have landed
                 __syncwarp();
@@ -1506,6 +1535,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             // A unit is written while the next one's loads are in flight; the first is written before anything else is looked at.
             // In a pair the leader's multicast commits release the buffers.  Whether a remote arrival wakes a suspended thread is not
             // specified: this wait probes (where the other roles suspend on such barriers, they look again after kSuspendNs at the latest).
+            bool started = false;
             for (int unit = 0, fetched = 0;;) {
                 const int n = n_chunks;
                 uint4 row_a, row_b0, row_b1;
@@ -1536,6 +1566,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                         break;
                     }
                 }
+                if (!started) start_sync<CTAS, kBuilders, true>();   // the first unit's loads are on their way
+                started = true;
                 if (n == 0) continue;
                 const int buf = ring.buf;
                 if (unit >= kImageBufs) {   // the first units' buffers have never been used
@@ -1565,6 +1597,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 ring.next(kImageBufs);
                 unit++;
             }
+            if (!started) start_sync<CTAS, kBuilders, true>();
         }
     } else if (warp == 2) {
         // ------------------------------------------------------------------ watcher
@@ -1576,6 +1609,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         // to its end.
         StageIter sg;
         sg.init(p, first_tile, tile_step, rank, kStageElems);
+        start_sync<CTAS, kBuilders>();
         uint32_t stage = 0, phase = 0, acc_phase = 0;
         BufRing ring;   // image buffer of the current unit
         bool ok = true;
@@ -1693,6 +1727,10 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         // ------------------------------------------------------------------ epilogue
         const int quarter = warp & 3;            // TMEM lanes 32*quarter .. +31 (hardware: warp id mod 4)
         const int half = (warp - 4) >> 2;        // accumulator columns 128*half .. +127
+        start_sync<CTAS, kBuilders>();
+        if (CTAS == 2) asm volatile("bar.sync 14, 288;" ::: "memory");
+        tcgen05_fence_after();
+        const uint32_t tmem_base = *tmem_base_slot;
         uint32_t acc_phase = 0;
         bool ok = true;
         int ev_t = 0;
@@ -1884,6 +1922,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     else __syncthreads();
     if (warp == 1) {
         tcgen05_fence_after();
+        const uint32_t tmem_base = *tmem_base_slot;
         if (CTAS == 1)
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
         else
