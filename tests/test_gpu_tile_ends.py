@@ -1,5 +1,6 @@
-"""Where a CTA's stream of tiles ends: the last tile's output leaves through the operand ring, and row tiles are numbered in groups
-with a smaller last one."""
+"""Where a CTA's stream of tiles ends: the last tile's output leaves through the operand ring, row tiles are numbered in groups with a
+smaller last one, and groups of rows are looked up through a copy of their boundaries when these fill more than a cache line."""
+import numpy as np
 import pytest
 import torch
 
@@ -30,5 +31,25 @@ def test_last_tiles(T, N, K):
     once = dw.clone()
     binding.fp4q_gemm_wgrad(qdy, qx, out=dw, accumulate=True, ws=ws)
     assert torch.equal(dw, 2 * once)
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
+
+
+# one line of boundaries and more than one, more than the images' place holds, empty groups at both ends and in the middle
+@pytest.mark.parametrize("E", [15, 16, 17, 200, 6200])
+def test_groups_are_found(E):
+    ws = binding.alloc_workspace("cuda")
+    rng = np.random.default_rng(E)
+    tiles = rng.integers(0, 3, E) if E < 1000 else (rng.random(E) < 0.02).astype(np.int64)
+    tiles[[0, E // 2, E - 1]] = 0
+    offs = np.concatenate([[0], np.cumsum(128 * tiles)])
+    T, N, K = int(offs[-1]), 64, 64
+    qx, qw, qdy = operands((T, K), (E * N, K), (T, N))
+    x, w, dy = (dequant_from_gpu(q) for q in (qx, qw, qdy))
+    d = torch.from_numpy(offs).cuda()
+    y, dx = binding.fp4q_gemm_fwd(qx, qw, row_offsets=d, ws=ws), binding.fp4q_gemm_dgrad(qdy, qw, row_offsets=d, ws=ws)
+    groups = [(g, slice(int(offs[g]), int(offs[g + 1]))) for g in range(E) if tiles[g]]
+    check_gemm(y, np.concatenate([x[s] @ w[g * N:(g + 1) * N].T for g, s in groups]), "fwd")
+    check_gemm(dx, np.concatenate([dy[s] @ w[g * N:(g + 1) * N] for g, s in groups]), "dgrad")
     torch.cuda.synchronize()
     assert binding.fp4q_workspace_status(ws) == 0
