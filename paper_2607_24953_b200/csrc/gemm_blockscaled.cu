@@ -22,7 +22,7 @@
 //               per-row scales as real 32-row images
 //   warps 4-11  epilogue: tcgen05.ld of the 128x256 FP32 accumulator (each warp 32 lanes x 128 columns),
 //               release of the accumulator as soon as it sits in registers, then convert and store (through staging
-//               rows and TMA stores; one CTA with per-row scales: 256-bit stores)
+//               rows and TMA stores; one CTA with MXFP8: 256-bit stores)
 // A ring of three or four (one CTA: 48 KB of operands per stage) or four or five (pair: 32 KB) shared-memory stages, by kind
 // (Cfg), is guarded by mbarriers; the scale columns in TMEM form a ring of the same depth.  Every mbarrier wait is bounded: when a limit
 // is hit the CTA records FP4Q_ERR_TIMEOUT in the workspace, releases the MMA warp from its named barriers, stops
@@ -58,16 +58,14 @@ constexpr int kUnitStagesMxf8 = 4;
 constexpr int kImageStageBytesMxf8 = 1536;
 constexpr int kImageStageBytes = 768;        // A chunk 0, A chunk 1, B chunk 0 (rows 0..127, 128..255), B chunk 1 (same)
 constexpr int kCompactBytes = kCacheChunks * 48;
-constexpr int kCacheBufBytes = kUnitStagesMxf4 * kImageStageBytes;
-// mxf4 with per-row scales: a stage has two chunks of four blocks; A 2 x 512 B, B (256 rows) 4 x 512 B per stage
+// mxf4 with per-row scales: a stage has two chunks of four blocks.  The 1D-block operand has real images, A 2 x 512 B or B (256 rows)
+// 4 x 512 B per stage, the 2D-block operand replicated ones like above, B 4 x 128 B or A 2 x 128 B.
 constexpr int kUnitStagesMxf4R = 4;
-constexpr int kImageStageBytesMxf4R = 3072;
-static_assert(kUnitStagesMxf4R * kImageStageBytesMxf4R == kCacheBufBytes, "the FP4 kinds share the size of an image buffer");
+constexpr int kImageStageBytesMxf4RA = 1024 + 512, kImageStageBytesMxf4RB = 256 + 2048;
 // mxf4nvf4 with 16-element scale vectors (tensors quantized in 16 x 16 blocks): every MMA (64 contraction elements)
 // has its own image per 128 operand rows - four scale bytes per row - so a stage holds A 4 x 512 B and B 8 x 512 B
 constexpr int kUnitStagesMxf4B16 = 2;
 constexpr int kImageStageBytesMxf4B16 = 6144;
-static_assert(kUnitStagesMxf4B16 * kImageStageBytesMxf4B16 == kCacheBufBytes, "the FP4 kinds share the size of an image buffer");
 // Epilogue staging of the pair kernel: each of the 8 epilogue warps owns 32 rows x 128 bytes, written from registers
 // (128-byte swizzle: the 16-byte pieces of 8 rows fall into different banks) and drained by a TMA store, which keeps
 // the output off the load/store unit that the MMA warp's instructions also pass through.
@@ -77,40 +75,45 @@ constexpr int kStagingWarpBytes = 32 * 128;
 // tile through cta_group::2 MMAs; each CTA loads its own 128 A rows and half of the B rows, which halves the
 // B-operand shared-memory and L2 traffic per CTA and leaves room for two more ring stages.
 // KIND_MXF4: FP4 payloads, 2D-block scales on both operands (replicated scale images).  KIND_MXF8: E4M3 payloads,
-// per-row scales.  KIND_MXF4R: FP4 payloads with per-row scale images - an operand quantized in 1D blocks (the
-// paper's activation layout) next to a 2D-block operand, whose tile scale is then expanded to its 32 rows.
+// per-row scales.  KIND_MXF4RA, KIND_MXF4RB: FP4 payloads with per-row scale images for one operand - A or B quantized in 1D blocks (the
+// paper's activation layout) - next to a 2D-block operand with replicated ones: in row-major order (B of the forward product) and
+// seen transposed (A of the weight gradient).
 // KIND_MXF4B16: FP4 payloads of tensors quantized in 16 x 16 blocks (block-size study): 16-element scale vectors
-// (kind::mxf4nvf4, scale_vec::4X, UE8M0 scales), real images built like the per-row kinds' (row_shift 4).
-enum { KIND_MXF4 = 0, KIND_MXF8 = 1, KIND_MXF4R = 2, KIND_MXF4B16 = 3 };
+// (kind::mxf4nvf4, scale_vec::4X, UE8M0 scales), real images whose upper and lower 16 rows are equal.
+enum { KIND_MXF4 = 0, KIND_MXF8 = 1, KIND_MXF4RA = 2, KIND_MXF4RB = 3, KIND_MXF4B16 = 4 };
 __host__ __device__ constexpr bool kind_fp4(int kind) { return kind != KIND_MXF8; }
 
-// Per-row scale images are rebuilt every 4 stages (2 with 16 x 16 blocks) from 12 KB (MXFP8: 6 KB) of scale bytes, whose
-// global-memory latency under the operand traffic (about 3000 cycles) exceeds the time such a unit runs.  The kernels for
-// those kinds therefore fetch the bytes two units ahead with cp.async into raw buffers (no registers are held meanwhile);
-// the FP4 kinds pay for the buffers with one ring stage; the pair kernel also keeps a third image buffer, because the way
-// from "the MMAs have finished with a buffer" to "the leader may copy the next unit out of it" (commit to both
-// CTAs, build, report to the leader) is longer than one unit as well.
+// Per-row scale images are rebuilt every 4 stages (2 with 16 x 16 blocks), and the global-memory latency of the bytes they are made of
+// (about 3000 cycles under the operand traffic) exceeds the time such a unit runs.  The kernels for those kinds therefore fetch the
+// bytes two units ahead with cp.async into raw buffers (no registers are held meanwhile); the pair kernel also keeps a third image
+// buffer, because the way from "the MMAs have finished with a buffer" to "the leader may copy the next unit out of it" (commit to
+// both CTAs, build, report to the leader) is longer than one unit as well.
 template <int KIND, int CTAS>
 struct Cfg {
     static constexpr bool kRowImages = KIND != KIND_MXF4;
     // Image builder warps: the per-row FP4 kinds, whose units are 4 or 2 stages, have two that take turns (one warp needs
     // 1500-2500 cycles for a unit, all of it latency); their MMA warp waits for itself and needs no watcher.
-    static constexpr int kBuilders = (KIND == KIND_MXF4R || KIND == KIND_MXF4B16) ? 2 : 1;
+    static constexpr int kBuilders = kRowImages && KIND != KIND_MXF8 ? 2 : 1;
     static constexpr int kImageBufs = (CTAS == 2 && kRowImages) ? (KIND == KIND_MXF4B16 ? 4 : 3) : 2;
     static constexpr int kRawBufs = kRowImages ? (KIND == KIND_MXF4B16 ? 4 : 2) : 0;
     // The output leaves through staging rows and TMA stores wherever shared memory allows (everything but the
-    // one-CTA kernel of the per-row kinds).  In the one-CTA kernel of the 2D kind - grouped products with short
+    // one-CTA kernel of MXFP8).  In the one-CTA kernel of the 2D kind - grouped products with short
     // contractions - plain stores of the 64 KB tile filled the SM's path to L2 and the TMA loads issued meanwhile
     // took 6500-8000 cycles instead of 3000; the staging costs that kernel its fourth ring stage.
-    static constexpr bool kTmaStores = CTAS == 2 || !kRowImages;
-    static constexpr int kStages = (CTAS == 2 ? 5 : (kTmaStores ? 3 : 4)) - (kRowImages && KIND != KIND_MXF8 ? 1 : 0);
-    static constexpr int kBufBytes = KIND == KIND_MXF8 ? kUnitStagesMxf8 * kImageStageBytesMxf8 : kCacheBufBytes;   // an image buffer
-    static constexpr int kUnitBlocks = KIND == KIND_MXF8 ? 16 : 32;   // per-row kinds: contraction blocks of a unit = scale bytes of a row
-    // a raw buffer: 32 lanes' scale bytes per slot, 4 slots of A rows and 8 of B rows; with 16 x 16 blocks both operands are
-    // compact and need one slot each
-    static constexpr int kRawSlotB = KIND == KIND_MXF4B16 ? 1 : 4;
-    static constexpr int kRawBytes = (kRawSlotB + (KIND == KIND_MXF4B16 ? 1 : 8)) * 32 * kUnitBlocks;
-    static constexpr int kSmemCache = (kRowImages ? 0 : kCompactBytes) + kImageBufs * kBufBytes + kRawBufs * kRawBytes;
+    static constexpr bool kTmaStores = CTAS == 2 || KIND != KIND_MXF8;
+    static constexpr int kStages = CTAS == 2 ? (KIND == KIND_MXF4RB || KIND == KIND_MXF4B16 ? 4 : 5) : (kTmaStores ? 3 : 4);
+    static constexpr int kUnitStages = KIND == KIND_MXF4 ? kUnitStagesMxf4 : KIND == KIND_MXF8 ? kUnitStagesMxf8
+                                       : KIND == KIND_MXF4B16 ? kUnitStagesMxf4B16 : kUnitStagesMxf4R;   // stages whose scale images are built together
+    static constexpr int kImageStage = KIND == KIND_MXF4 ? kImageStageBytes : KIND == KIND_MXF8 ? kImageStageBytesMxf8 : KIND == KIND_MXF4B16 ? kImageStageBytesMxf4B16
+                                       : KIND == KIND_MXF4RA ? kImageStageBytesMxf4RA : kImageStageBytesMxf4RB;
+    static constexpr int kBufBytes = kUnitStages * kImageStage;   // an image buffer
+    // A raw buffer: A's bytes, then B's, in entries of one row each, a word longer than the row's bytes of a unit (RowFetch); a 2D-block
+    // operand's entries are its row tiles or, seen transposed, the unit's 32 blocks.
+    static constexpr int kRawA = KIND == KIND_MXF8 ? 128 * 20 : KIND == KIND_MXF4RA ? 128 * 36 : KIND == KIND_MXF4RB ? 32 * 8 : 32 * 12;
+    static constexpr int kRawB = KIND == KIND_MXF8 ? 256 * 20 : KIND == KIND_MXF4RA ? 8 * 36 + 32 : KIND == KIND_MXF4RB ? 256 * 36 : 32 * 20;
+    static constexpr int kRawBytes = kRawA + kRawB;
+    static constexpr int kSortedBytes = KIND == KIND_MXF4RA || KIND == KIND_MXF4RB ? 256 : KIND == KIND_MXF4B16 ? 768 : 0;   // a builder's 2D-block bytes as image rows
+    static constexpr int kSmemCache = kRowImages ? kImageBufs * kBufBytes + kRawBufs * kRawBytes + kBuilders * kSortedBytes : kCompactBytes + kImageBufs * kBufBytes;
     static constexpr int kBRows = CTAS == 2 ? 128 : 256;
     static constexpr int kBStageBytes = kBRows * 128;
     static constexpr int kSmemOperands = kStages * (kAStageBytes + kBStageBytes);
@@ -166,11 +169,10 @@ enum { MODE_DENSE = 0, MODE_GROUPED_ROWS = 1, MODE_GROUPED_K = 2 };
 
 struct ScaleView {
     const uint8_t *ptr;
-    int64_t stride_row;   // mxf4: bytes between consecutive 32-row tiles; mxf8: bytes between consecutive rows
+    int64_t stride_row;   // 2D blocks: bytes between consecutive row tiles (of 32 or 16 rows); per-row scales: between consecutive rows
     int64_t stride_kb;    // bytes between consecutive contraction blocks of 32
-    int32_t n_row;        // mxf4: number of row tiles; mxf8: number of rows
+    int32_t n_row;        // 2D blocks: number of row tiles; per-row scales: number of rows
     int32_t n_kb;         // number of contraction blocks
-    int32_t row_shift;    // per-row images only: operand row r reads scale row r >> row_shift (5: a 2D-block operand, n_row counts tiles)
 };
 
 // Division by a number that the launch knows, as a multiplication (Granlund and Montgomery, "Division by invariant integers using
@@ -519,19 +521,6 @@ __device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int r
 
 // ---------------------------------------------------------------------------------------- scale images
 
-// Scale slots beyond the tensor read this byte instead (their payload is zero, any finite scale will do).
-__device__ const uint8_t g_scale_pad[4] = {kScalePad, kScalePad, kScalePad, kScalePad};
-
-// One compact scale byte.  The bounds check selects the ADDRESS, not the value, so that nothing depends on
-// the loaded byte until it is written into the image several stages later (an in-order warp stalls at the
-// first use of a pending load).
-__device__ __forceinline__ void load_scale(const ScaleView &v, int row, int kb, uint32_t &dst)
-{
-    const uint8_t *ptr = (row < v.n_row && kb < v.n_kb) ? v.ptr + (int64_t)row * v.stride_row + (int64_t)kb * v.stride_kb
-                                                        : g_scale_pad;
-    asm volatile("ld.global.u8 %0, [%1];" : "=r"(dst) : "l"(ptr));
-}
-
 // The stream of ring stages one CTA of a dense product works through: its tiles in order, each with its contraction stages.
 struct StageIter {
     int tile, step, rank, it, n_it;
@@ -703,69 +692,6 @@ __device__ __forceinline__ void gather_scale_rows(const GemmParams &p, const Til
     __syncwarp();
 }
 
-// Per-row scales (MXFP8): one 32-bit word = the four scale bytes of one row and one stage.
-__device__ __forceinline__ void load_scale_word(const ScaleView &v, int row, int kb0, uint32_t &dst)
-{
-    const uint8_t *ptr = v.ptr + (int64_t)row * v.stride_row + kb0;
-    if (row < v.n_row && kb0 + 4 <= v.n_kb && v.stride_kb == 1 && (reinterpret_cast<uintptr_t>(ptr) & 3) == 0) {
-        asm volatile("ld.global.b32 %0, [%1];" : "=r"(dst) : "l"(ptr));   // the common case: nothing depends on it yet
-        return;
-    }
-    uint32_t word = 0;
-#pragma unroll
-    for (int kb = 0; kb < 4; kb++) {
-        uint32_t b;
-        load_scale(v, row, kb0 + kb, b);
-        word |= b << (8 * kb);
-    }
-    dst = word;
-}
-
-template <int KIND>
-__device__ __forceinline__ void store_row_scale_images(const uint32_t (&w)[12][KIND == KIND_MXF8 ? 4 : 8], int n_stages, uint8_t *images, int lane)
-{
-    if constexpr (KIND == KIND_MXF8) {
-#pragma unroll
-        for (int st = 0; st < 4; st++) {
-            if (st < n_stages) {
-                uint4 *img = reinterpret_cast<uint4 *>(images + st * kImageStageBytesMxf8);
-                img[lane] = make_uint4(w[0][st], w[1][st], w[2][st], w[3][st]);           // A
-                img[32 + lane] = make_uint4(w[4][st], w[5][st], w[6][st], w[7][st]);      // B rows 0..127
-                img[64 + lane] = make_uint4(w[8][st], w[9][st], w[10][st], w[11][st]);    // B rows 128..255
-            }
-        }
-    } else if constexpr (KIND == KIND_MXF4B16) {
-        // word j of a row = the four scale bytes of MMA j of the unit (stage j / 4, MMA j % 4)
-#pragma unroll
-        for (int st = 0; st < 2; st++) {
-            if (st < n_stages) {
-                uint4 *img = reinterpret_cast<uint4 *>(images + st * kImageStageBytesMxf4B16);
-#pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    const int j = 4 * st + i;
-                    img[32 * i + lane] = make_uint4(w[0][j], w[1][j], w[2][j], w[3][j]);                  // A, MMA i
-                    img[128 + 64 * i + lane] = make_uint4(w[4][j], w[5][j], w[6][j], w[7][j]);            // B rows 0..127
-                    img[160 + 64 * i + lane] = make_uint4(w[8][j], w[9][j], w[10][j], w[11][j]);          // B rows 128..255
-                }
-            }
-        }
-    } else {
-#pragma unroll
-        for (int st = 0; st < 4; st++) {
-            if (st < n_stages) {
-                uint4 *img = reinterpret_cast<uint4 *>(images + st * kImageStageBytesMxf4R);
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    const int j = 2 * st + c;
-                    img[32 * c + lane] = make_uint4(w[0][j], w[1][j], w[2][j], w[3][j]);                 // A, chunk c
-                    img[64 + 64 * c + lane] = make_uint4(w[4][j], w[5][j], w[6][j], w[7][j]);            // B rows 0..127
-                    img[96 + 64 * c + lane] = make_uint4(w[8][j], w[9][j], w[10][j], w[11][j]);          // B rows 128..255
-                }
-            }
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------------------- epilogue store
 
 // Transpose of a 32x32 matrix of nibbles held one row per lane (W[w] nibble n = column 8w + n of the lane's row): on
@@ -920,200 +846,291 @@ struct UnitIter {
     }
 };
 
-__device__ __forceinline__ void cp_async(uint32_t dst, const void *src, int bytes, int src_bytes)
+// ---- scale images of the per-row kinds
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const uint8_t *src, int src_bytes)
 {
-    if (bytes == 16) asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-    else if (bytes == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const uint8_t *src, int src_bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const uint8_t *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ uint32_t lds32(const uint8_t *p) { return *reinterpret_cast<const uint32_t *>(p); }
+
+// A row's bytes from src on, which may lie on any byte, as WORDS aligned words from the one that holds the first.  The matrix
+// occupies the bytes lo .. hi - 1 and src is one of them; INSIDE: so are all bytes of the words.
+template <int WORDS, bool INSIDE>
+__device__ __forceinline__ void fetch_row(uint32_t dst, const uint8_t *src, const uint8_t *lo, const uint8_t *hi)
+{
+    const uint8_t *a = src - (reinterpret_cast<uintptr_t>(src) & 3);
+    if (INSIDE) {
+#pragma unroll
+        for (int k = 0; k < WORDS; k++) cp_async4(dst + 4 * k, a + 4 * k);
+        return;
+    }
+    const int n = (int)min((int64_t)(4 * WORDS), (int64_t)(hi - a));   // bytes before the matrix's end
+    if (a < lo) asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst), "r"(load_end_word(a, lo, hi)) : "memory");
+    else cp_async4(dst, a, min(n, 4));
+#pragma unroll
+    for (int k = 1; k < WORDS; k++) cp_async4(dst + 4 * k, 4 * k < n ? a + 4 * k : a, max(0, min(n - 4 * k, 4)));
+}
+// Word k of such a row, whose first byte is byte `mis` of the first word; bytes from n_valid on are not the row's.
+__device__ __forceinline__ uint32_t row_word(uint32_t lo, uint32_t hi, uint32_t mis, int k, int n_valid)
+{
+    const int n = n_valid - 4 * k;
+    const uint32_t w = __funnelshift_r(lo, hi, 8 * mis);
+    return n >= 4 ? w : n <= 0 ? 0u : w & ((1u << (8 * n)) - 1u);
 }
 
-// Raw scale bytes of one unit (BLOCKS contraction blocks from k0: 32, or 16 for MXFP8), asynchronously into `raw`: slot q
-// (q < 4: A rows 32q.., q >= 4: B rows 32(q-4)..) holds BLOCKS bytes per lane, the scale bytes of the lane's operand row.
-// A 2D-block operand (row_shift 5) needs only 32 bytes per row tile: they are packed at the start of the operand's
-// first slot; if its view is transposed (blocks stride_kb apart, row tiles contiguous) lane l fetches block l's
-// bytes for the operand's 4 or 8 row tiles into the first 8 bytes of its entry of that slot.  With 16 x 16 blocks
-// (row_shift 4, KB_SHIFT 4: a block is 16 contraction elements and a row tile 16 rows) the unit still has 32 blocks but
-// the operand has 8 or 16 row tiles.  Bytes beyond the tensor arrive as zero.  Every lane commits exactly one
-// cp.async group per call.
-template <int KB_SHIFT, int BLOCKS, int SLOT_B>
-__device__ __forceinline__ void issue_raw_scales(const GemmParams &p, const Tile &t, int k0, uint8_t *raw, int lane)
-{
+// Per-row scales: BYTES scale bytes of each of the NQ x 32 rows from row0 on, row row0 + lane + 32 q one of lane's.  Rows on 16-byte
+// boundaries are copied as they are, others word by word in entries of one word more and shifted when they are read.  (Loads
+// by each piece, with a wait for it, were ten times the code and did not run ahead: MXFP8 forward 1999 x 1003 x 2731, 86 blocks a row, 68.4 ->
+// 18.2 us, 300 x 777 x 1234 35.3 -> 12.7, 1D activations there 21.5 / 22.9 -> 11.4 / 12.5 and 12.0 / 20.1 -> 8.3 / 10.4.)  Rows beyond the tensor take
+// the place of the last (their payload is zero, any finite scale will do), bytes beyond a row's last become zero.
+template <int NQ, int BYTES>
+struct RowFetch {
+    const uint8_t *src[NQ];
+    __device__ __forceinline__ static bool wide(const ScaleView &v) { return ((reinterpret_cast<uintptr_t>(v.ptr) | (uintptr_t)v.stride_row) & 15) == 0; }
+    __device__ __forceinline__ void set(const ScaleView &v, int row0, int lane)
+    {
 #pragma unroll
-    for (int op = 0; op < 2; op++) {
-        const ScaleView &v = op == 0 ? p.sfa : p.sfb;
-        const int nq = op == 0 ? 4 : 8, q0 = op == 0 ? 0 : SLOT_B;
-        const int row0 = op == 0 ? t.a_row0 : t.b_row0;
-        const int kb0 = ((op == 0 ? t.a_k0 : t.b_k0) + k0) >> KB_SHIFT;
-        const int n_tiles = v.row_shift != 0 ? nq << (5 - v.row_shift) : 0;   // row tiles of a 2D-block operand
-        if (BLOCKS == 32 && v.row_shift != 0 && v.stride_kb != 1) {
-            const int rt0 = row0 >> v.row_shift, kb = kb0 + lane, nbytes = n_tiles;   // 4 .. 16 row tiles, one byte each
-            uint8_t *dst = raw + q0 * 1024 + lane * 32;
-            const uint8_t *src = v.ptr + (int64_t)kb * v.stride_kb + rt0;
-            const int valid = kb < v.n_kb ? max(0, min(nbytes, v.n_row - rt0)) : 0;
-            if (v.stride_row == 1 && (reinterpret_cast<uintptr_t>(src) & (nbytes - 1)) == 0) {
-                cp_async(smem_u32(dst), valid > 0 ? src : v.ptr - (reinterpret_cast<uintptr_t>(v.ptr) & 15), nbytes, valid);
-            } else {
-                for (int r = 0; r < nbytes; r++) {
-                    uint32_t b;
-                    load_scale(v, rt0 + r, kb, b);
-                    dst[r] = (uint8_t)b;
+        for (int q = 0; q < NQ; q++) src[q] = v.ptr + (int64_t)min(row0 + lane + 32 * q, v.n_row - 1) * v.stride_row;
+    }
+    __device__ __forceinline__ void fetch(const ScaleView &v, int kb0, uint32_t raw, int lane) const
+    {
+        if (wide(v)) {
+#pragma unroll
+            for (int q = 0; q < NQ; q++)
+#pragma unroll
+                for (int h = 0; h < BYTES / 16; h++) {
+                    const int n = max(0, min(16, v.n_kb - kb0 - 16 * h));
+                    cp_async16(raw + (32 * q + lane) * BYTES + 16 * h, src[q] + kb0 + (n > 0 ? 16 * h : 0), n);
                 }
-            }
-            continue;
+            return;
         }
-        if (BLOCKS == 32 && v.row_shift != 0) {
-            // 2D-block operand, blocks contiguous: the 32 bytes of each of the operand's row tiles once (two lanes
-            // per row tile copy 16 bytes each), packed at the start of the operand's first slot
-            if (lane < 2 * n_tiles) {
-                const int rt = (row0 >> v.row_shift) + (lane >> 1), kb = kb0 + 16 * (lane & 1);
-                uint8_t *dst = raw + q0 * 1024 + lane * 16;
-                const uint8_t *src = v.ptr + (int64_t)rt * v.stride_row + kb;
-                if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-                    const int valid = rt < v.n_row ? max(0, min(16, v.n_kb - kb)) : 0;
-                    cp_async(smem_u32(dst), valid > 0 ? src : v.ptr - (reinterpret_cast<uintptr_t>(v.ptr) & 15), 16, valid);
-                } else {
+        constexpr int kWords = BYTES / 4 + 1;
+        const uint8_t *hi = v.ptr + (int64_t)(v.n_row - 1) * v.stride_row + v.n_kb;
+        raw += 4 * kWords * lane;
+        if (__all_sync(0xFFFFFFFFu, src[0] + kb0 >= v.ptr + 3 && src[NQ - 1] + kb0 + 4 * kWords <= hi)) {
 #pragma unroll
-                    for (int st = 0; st < 4; st++) {
-                        uint32_t word;
-                        load_scale_word(v, rt, kb + 4 * st, word);
-                        reinterpret_cast<uint32_t *>(dst)[st] = word;
-                    }
-                }
-            }
-            continue;
-        }
+            for (int q = 0; q < NQ; q++) fetch_row<kWords, true>(raw + 128 * kWords * q, src[q] + kb0, v.ptr, hi);
+        } else {
 #pragma unroll
-        for (int q = 0; q < nq; q++) {
-            const int row = row0 + lane + 32 * q;
-            uint8_t *dst = raw + (q0 + q) * 32 * BLOCKS + lane * BLOCKS;
-            const uint8_t *src = v.ptr + (int64_t)row * v.stride_row + kb0;
-            if (v.stride_kb == 1 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-                const int valid = row < v.n_row ? max(0, min(BLOCKS, v.n_kb - kb0)) : 0;
-                const uint8_t *safe = v.ptr - (reinterpret_cast<uintptr_t>(v.ptr) & 15);
-                cp_async(smem_u32(dst), valid > 0 ? src : safe, 16, min(valid, 16));
-                if (BLOCKS == 32) cp_async(smem_u32(dst + 16), valid > 16 ? src + 16 : safe, 16, max(valid - 16, 0));
-            } else {
-                // Rows that start on any word or byte: a piece's loads are all in flight before the first is used.  One word
-                // after the other (four byte loads, a wait, a store) MXFP8 at 8192 x 4096 x 2720, 85 blocks a row, took 1002 us.
-                const bool words = v.stride_kb == 1 && row < v.n_row && kb0 + BLOCKS <= v.n_kb && (reinterpret_cast<uintptr_t>(src) & 3) == 0;
-                uint32_t *out = reinterpret_cast<uint32_t *>(dst);
-                if (words) {
-                    uint32_t w[BLOCKS / 4];
-#pragma unroll
-                    for (int k = 0; k < BLOCKS / 4; k++) ldg_b32(src + 4 * k, w[k]);
-#pragma unroll
-                    for (int k = 0; k < BLOCKS / 4; k++) out[k] = w[k];
-                } else {
-#pragma unroll
-                    for (int h = 0; h < BLOCKS; h += 16) {
-                        uint32_t b[16];
-#pragma unroll
-                        for (int k = 0; k < 16; k++) load_scale(v, row, kb0 + h + k, b[k]);
-#pragma unroll
-                        for (int k = 0; k < 4; k++) out[h / 4 + k] = b[4 * k] | b[4 * k + 1] << 8 | b[4 * k + 2] << 16 | b[4 * k + 3] << 24;
-                    }
-                }
-            }
+            for (int q = 0; q < NQ; q++) fetch_row<kWords, false>(raw + 128 * kWords * q, src[q] + kb0, v.ptr, hi);
         }
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-// The unit's scale words from a raw buffer whose copies have completed: w[q][j] = the four scale bytes of the
-// lane's row of slot q for blocks 4j..4j+3.  Lanes read bytes other lanes copied: the caller synchronizes the warp
-// after its cp.async wait.
-template <int BLOCKS, int SLOT_B>
-__device__ __forceinline__ void read_raw_scales(const GemmParams &p, const uint8_t *raw, int lane, uint32_t (&w)[12][BLOCKS / 4])
-{
-    if constexpr (BLOCKS == 16) {
+    // w[q]: the words of row row0 + lane + 32 q, of any tile whose bytes have landed
+    __device__ __forceinline__ static void read(const ScaleView &v, int row0, int kb0, const uint8_t *raw, int lane, uint32_t (*w)[BYTES / 4])
+    {
+        if (wide(v)) {
 #pragma unroll
-        for (int q = 0; q < 12; q++) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(raw + q * 512 + lane * 16);
-            w[q][0] = v.x; w[q][1] = v.y; w[q][2] = v.z; w[q][3] = v.w;
+            for (int q = 0; q < NQ; q++)
+#pragma unroll
+                for (int h = 0; h < BYTES / 16; h++) {
+                    const uint4 x = reinterpret_cast<const uint4 *>(raw + (32 * q + lane) * BYTES)[h];
+                    w[q][4 * h] = x.x; w[q][4 * h + 1] = x.y; w[q][4 * h + 2] = x.z; w[q][4 * h + 3] = x.w;
+                }
+            return;
         }
-        return;
+        constexpr int kWords = BYTES / 4 + 1;
+#pragma unroll
+        for (int q = 0; q < NQ; q++) {
+            const uint32_t mis = ((uint32_t)reinterpret_cast<uintptr_t>(v.ptr) + (uint32_t)min(row0 + lane + 32 * q, v.n_row - 1) * (uint32_t)v.stride_row + (uint32_t)kb0) & 3;
+            const uint8_t *e = raw + 4 * kWords * (32 * q + lane);
+            uint32_t x[kWords];
+#pragma unroll
+            for (int k = 0; k < kWords; k++) x[k] = lds32(e + 4 * k);
+#pragma unroll
+            for (int k = 0; k < BYTES / 4; k++) w[q][k] = row_word(x[k], x[k + 1], mis, k, v.n_kb - kb0);
+        }
+    }
+};
+
+// 2D-block scales in a per-row kind: TILES row tiles by 32 blocks, an entry a row tile or, seen transposed, a block.  Like a per-row
+// operand's rows they are copied as they are where their entries start on 16 (transposed: TILES) bytes, otherwise word by word in entries of
+// one word more.
+template <int TILES, bool TR>
+__device__ __forceinline__ bool wide_blocks(const ScaleView &v)
+{
+    return ((reinterpret_cast<uintptr_t>(v.ptr) | (uintptr_t)(TR ? v.stride_kb : v.stride_row)) & (TR ? TILES - 1 : 15)) == 0;
+}
+template <int TILES, bool TR>
+__device__ __forceinline__ void fetch_blocks(const ScaleView &v, int rt0, int kb0, uint32_t raw, int lane)
+{
+    if (TR) {
+        const int n = max(0, min(TILES, v.n_row - rt0));
+        const uint8_t *src = v.ptr + (int64_t)min(kb0 + lane, v.n_kb - 1) * v.stride_kb + (n > 0 ? rt0 : 0);
+        if (wide_blocks<TILES, TR>(v)) asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(raw + lane * TILES), "l"(src), "n"(TILES), "r"(n) : "memory");
+        else fetch_row<TILES / 4 + 1, false>(raw + lane * (TILES + 4), src, v.ptr, v.ptr + (int64_t)(v.n_kb - 1) * v.stride_kb + v.n_row);
+    } else if (wide_blocks<TILES, TR>(v)) {
+        if (lane < 2 * TILES) {
+            const int h = 16 * (lane & 1), n = max(0, min(16, v.n_kb - kb0 - h));
+            cp_async16(raw + lane * 16, v.ptr + (int64_t)min(rt0 + (lane >> 1), v.n_row - 1) * v.stride_row + kb0 + (n > 0 ? h : 0), n);
+        }
+    } else if (lane < TILES) {
+        const uint8_t *src = v.ptr + (int64_t)min(rt0 + lane, v.n_row - 1) * v.stride_row + kb0;
+        fetch_row<9, false>(raw + lane * 36, src, v.ptr, v.ptr + (int64_t)(v.n_row - 1) * v.stride_row + v.n_kb);
+    }
+}
+// The same, landed, as words of four blocks: store(row tile, chunk of four blocks, word).
+template <int TILES, bool TR, typename F>
+__device__ __forceinline__ void sort_blocks(const ScaleView &v, int rt0, int kb0, const uint8_t *raw, int lane, F store)
+{
+    const uint32_t p0 = (uint32_t)reinterpret_cast<uintptr_t>(v.ptr);
+    const bool wide = wide_blocks<TILES, TR>(v);
+    if (TR) {   // a lane transposes four blocks' bytes of four row tiles
+        if (lane < 2 * TILES) {
+            const int h = lane % (TILES / 4), c = lane / (TILES / 4);
+            uint32_t m[4];
+            if (wide) {
+#pragma unroll
+                for (int i = 0; i < 4; i++) m[i] = lds32(raw + (4 * c + i) * TILES + 4 * h);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    const uint8_t *e = raw + (4 * c + i) * (TILES + 4) + 4 * h;
+                    const uint32_t mis = (p0 + (uint32_t)min(kb0 + 4 * c + i, v.n_kb - 1) * (uint32_t)v.stride_kb + (uint32_t)(rt0 < v.n_row ? rt0 : 0)) & 3;
+                    m[i] = row_word(lds32(e), lds32(e + 4), mis, h, v.n_row - rt0);
+                }
+            }
+            const uint4 t = transpose4x4_bytes(m[0], m[1], m[2], m[3]);
+            store(4 * h, c, t.x); store(4 * h + 1, c, t.y); store(4 * h + 2, c, t.z); store(4 * h + 3, c, t.w);
+        }
+    } else if (wide) {
+        if (lane < 2 * TILES) {
+            const int rt = lane >> 1, c = 4 * (lane & 1);
+            const uint4 x = *reinterpret_cast<const uint4 *>(raw + lane * 16);
+            store(rt, c, x.x); store(rt, c + 1, x.y); store(rt, c + 2, x.z); store(rt, c + 3, x.w);
+        }
     } else {
 #pragma unroll
-    for (int op = 0; op < 2; op++) {
-        const ScaleView &v = op == 0 ? p.sfa : p.sfb;
-        const int nq = op == 0 ? 4 : 8, q0 = op == 0 ? 0 : 4, s0 = op == 0 ? 0 : SLOT_B;
-        if (v.row_shift != 0 && v.stride_kb != 1) {
-            // lane l holds block l's bytes [row tile 0..]: words of four consecutive lanes, transposed as 4x4 bytes,
-            // are the four row tiles' words of one chunk
-            if (v.row_shift == 4) {
-                // 16-row tiles: 8 (A) or 16 (B) bytes per lane; operand rows l + 32 q of image row l lie in row tile
-                // 2 q + (l >> 4), so the two halves of the warp pick different tiles of each transposed word
-                const uint4 mine4 = *reinterpret_cast<const uint4 *>(raw + s0 * 1024 + lane * 32);
-                const bool hi = lane >= 16;
-#pragma unroll
-                for (int h = 0; h < (op == 0 ? 2 : 4); h++) {
-                    const uint32_t m = h == 0 ? mine4.x : h == 1 ? mine4.y : h == 2 ? mine4.z : mine4.w;
-#pragma unroll
-                    for (int j = 0; j < 8; j++) {
-                        const uint4 tr = transpose4x4_bytes(__shfl_sync(0xFFFFFFFFu, m, 4 * j), __shfl_sync(0xFFFFFFFFu, m, 4 * j + 1),
-                                                            __shfl_sync(0xFFFFFFFFu, m, 4 * j + 2), __shfl_sync(0xFFFFFFFFu, m, 4 * j + 3));
-                        w[q0 + 2 * h][j] = hi ? tr.y : tr.x;
-                        w[q0 + 2 * h + 1][j] = hi ? tr.w : tr.z;
-                    }
-                }
-                continue;
-            }
-            const uint2 mine = *reinterpret_cast<const uint2 *>(raw + s0 * 1024 + lane * 32);
-#pragma unroll
-            for (int h = 0; h < (op == 0 ? 1 : 2); h++) {
-                const uint32_t m = h == 0 ? mine.x : mine.y;
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    const uint4 tr = transpose4x4_bytes(__shfl_sync(0xFFFFFFFFu, m, 4 * j), __shfl_sync(0xFFFFFFFFu, m, 4 * j + 1),
-                                                        __shfl_sync(0xFFFFFFFFu, m, 4 * j + 2), __shfl_sync(0xFFFFFFFFu, m, 4 * j + 3));
-                    w[q0 + 4 * h + 0][j] = tr.x; w[q0 + 4 * h + 1][j] = tr.y; w[q0 + 4 * h + 2][j] = tr.z; w[q0 + 4 * h + 3][j] = tr.w;
-                }
-            }
-            continue;
+        for (int i = 0; i < TILES / 4; i++) {
+            const int rt = (lane + 32 * i) % TILES, c = (lane + 32 * i) / TILES;
+            const uint32_t mis = (p0 + (uint32_t)min(rt0 + rt, v.n_row - 1) * (uint32_t)v.stride_row + (uint32_t)kb0) & 3;
+            const uint8_t *e = raw + rt * 36 + 4 * c;
+            store(rt, c, row_word(lds32(e), lds32(e + 4), mis, c, v.n_kb - kb0));
         }
-#pragma unroll
-        for (int q = 0; q < nq; q++) {
-            const int tile = v.row_shift == 4 ? 2 * q + (lane >> 4) : q;   // row tile of operand row lane + 32 q
-            const uint4 *src = reinterpret_cast<const uint4 *>(v.row_shift != 0 ? raw + s0 * 1024 + tile * 32 : raw + (s0 + q) * 1024 + lane * 32);
-            const uint4 lo = src[0], hi = src[1];
-            w[q0 + q][0] = lo.x; w[q0 + q][1] = lo.y; w[q0 + q][2] = lo.z; w[q0 + q][3] = lo.w;
-            w[q0 + q][4] = hi.x; w[q0 + q][5] = hi.y; w[q0 + q][6] = hi.z; w[q0 + q][7] = hi.w;
-        }
-    }
     }
 }
 
-// MXFP8: the lane's twelve scale rows of a tile (4 of A, 8 of B).  A unit's fetch is then one 16-byte copy per row with
-// nothing to compute but the address step.
-struct RowFetch {
-    const uint8_t *src[12];
-    uint32_t valid;   // bit q: the row exists
-    bool fast;        // every copy starts on a 16-byte boundary
+// What bounds these kinds is how fast a warp, whose work is all latency, turns a unit's bytes into images.  A 2D-block operand's are
+// therefore transposed by one lane each (not all by every lane), and in KIND_MXF4RA / RB it has replicated images, whose 16-byte rows
+// are a quarter of the real images' bytes; that also pays for the fifth ring stage of RA.  us, 8192 x 5632 x 2048: 1D activations
+// forward / weight gradient 51.0 / 52.3 -> 47.7 / 48.4 (16384 x 4096 x 4096 121 / 130 -> 109 / 123), 16 x 16 blocks 53.5 / 47.6 / 55.1 -> 53.0 / 45.1 /
+// 50.8.  With the image rows read back from shared memory only when their buffer was free, 16 x 16 forward 2048 x 2048 x 2048 took 10.7 instead
+// of 10.0.
+// A builder's unit of a per-row kind, in three steps: fetch() starts the copies of a unit's bytes, read() takes them out of the raw
+// buffer into registers, write() makes the images, of which nothing but stores is left when their buffer falls free.  `sorted` is the
+// builder's own: 2D-block bytes as 16-byte image rows.
+template <int KIND, int CTAS>
+struct RowBuilder {
+    static constexpr int kRawA = Cfg<KIND, CTAS>::kRawA;
+    static constexpr bool kRowsA = KIND == KIND_MXF8 || KIND == KIND_MXF4RA, kRowsB = KIND == KIND_MXF8 || KIND == KIND_MXF4RB;
+    static constexpr int kBytes = KIND == KIND_MXF8 ? 16 : 32, kShift = KIND == KIND_MXF4B16 ? 4 : 5;   // a unit's blocks; log2 of a block's length
+    RowFetch<kRowsA ? 4 : 1, kBytes> a;
+    RowFetch<kRowsB ? 8 : 1, kBytes> b;
+    uint32_t w[KIND == KIND_MXF4B16 ? 1 : (kRowsA ? 4 : 0) + (kRowsB ? 8 : 0)][kBytes / 4];   // per-row operands, A's rows first
+    uint4 block_rows[KIND == KIND_MXF4B16 ? 24 : KIND == KIND_MXF4RA ? 4 : KIND == KIND_MXF4RB ? 2 : 1];   // 2D-block operands' image rows
+
     __device__ __forceinline__ void set(const GemmParams &p, const Tile &t, int lane)
     {
-        valid = 0;
-        fast = true;
-#pragma unroll
-        for (int q = 0; q < 12; q++) {
-            const ScaleView &v = q < 4 ? p.sfa : p.sfb;
-            const int row = q < 4 ? t.a_row0 + lane + 32 * q : t.b_row0 + lane + 32 * (q - 4), kb = (q < 4 ? t.a_k0 : t.b_k0) >> 5;
-            const bool ok = row < v.n_row;
-            valid |= ok ? 1u << q : 0u;
-            src[q] = ok ? v.ptr + (int64_t)row * v.stride_row + kb : v.ptr;
-            fast = fast && v.stride_kb == 1 && v.stride_row % 16 == 0 && (reinterpret_cast<uintptr_t>(v.ptr) & 15) == 0 && (kb & 15) == 0;
+        if (kRowsA) a.set(p.sfa, t.a_row0, lane);
+        if (kRowsB) b.set(p.sfb, t.b_row0, lane);
+    }
+    __device__ __forceinline__ void fetch(const GemmParams &p, const Tile &t, int k0, uint8_t *raw, int lane) const
+    {
+        const int kb0 = k0 >> kShift;
+        const uint32_t ra = smem_u32(raw), rb = ra + kRawA;
+        if (kRowsA) a.fetch(p.sfa, kb0, ra, lane);
+        if (kRowsB) b.fetch(p.sfb, kb0, rb, lane);
+        if (KIND == KIND_MXF4RA) fetch_blocks<8, false>(p.sfb, t.b_row0 >> 5, kb0, rb, lane);
+        if (KIND == KIND_MXF4RB) fetch_blocks<4, true>(p.sfa, t.a_row0 >> 5, kb0, ra, lane);
+        if (KIND == KIND_MXF4B16) {
+            if (p.sfa.stride_kb != 1) fetch_blocks<8, true>(p.sfa, t.a_row0 >> 4, kb0, ra, lane);
+            else fetch_blocks<8, false>(p.sfa, t.a_row0 >> 4, kb0, ra, lane);
+            if (p.sfb.stride_kb != 1) fetch_blocks<16, true>(p.sfb, t.b_row0 >> 4, kb0, rb, lane);
+            else fetch_blocks<16, false>(p.sfb, t.b_row0 >> 4, kb0, rb, lane);
         }
     }
-    __device__ __forceinline__ void issue(const GemmParams &p, const Tile &t, int k0, uint32_t raw, int lane) const
+    __device__ __forceinline__ void read(const GemmParams &p, const Tile &t, int k0, const uint8_t *raw, uint8_t *sorted, int lane)
     {
-        const int kb0 = k0 >> 5;   // both operands of an MXFP8 product have the same number of blocks
-        const int n = max(0, min(16, p.sfa.n_kb - (t.a_k0 >> 5) - kb0));
-#pragma unroll
-        for (int q = 0; q < 12; q++) {
-            const bool ok = (valid >> q & 1) && n > 0;
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(raw + q * 512 + lane * 16), "l"(ok ? src[q] + kb0 : src[q]),
-                         "r"(ok ? n : 0) : "memory");
+        const int kb0 = k0 >> kShift;
+        uint32_t *s = reinterpret_cast<uint32_t *>(sorted);
+        if (kRowsA) a.read(p.sfa, t.a_row0, kb0, raw, lane, w);
+        if (kRowsB) b.read(p.sfb, t.b_row0, kb0, raw + kRawA, lane, w + (kRowsA ? 4 : 0));
+        // [chunk][row tile], that is a chunk's one or two image rows
+        if (KIND == KIND_MXF4RA) sort_blocks<8, false>(p.sfb, t.b_row0 >> 5, kb0, raw + kRawA, lane, [&](int rt, int c, uint32_t x) { s[8 * c + rt] = x; });
+        if (KIND == KIND_MXF4RB) sort_blocks<4, true>(p.sfa, t.a_row0 >> 5, kb0, raw, lane, [&](int rt, int c, uint32_t x) { s[4 * c + rt] = x; });
+        if (KIND == KIND_MXF4B16) {
+            // operand rows l + 32 q of image row l lie in row tile 2 q + l / 16: [MMA][half of the lanes][q]
+            auto sa = [&](int rt, int c, uint32_t x) { s[8 * c + 4 * (rt & 1) + (rt >> 1)] = x; };
+            auto sb = [&](int rt, int c, uint32_t x) { s[64 + 16 * c + 8 * (rt & 1) + (rt >> 1)] = x; };
+            if (p.sfa.stride_kb != 1) sort_blocks<8, true>(p.sfa, t.a_row0 >> 4, kb0, raw, lane, sa);
+            else sort_blocks<8, false>(p.sfa, t.a_row0 >> 4, kb0, raw, lane, sa);
+            if (p.sfb.stride_kb != 1) sort_blocks<16, true>(p.sfb, t.b_row0 >> 4, kb0, raw + kRawA, lane, sb);
+            else sort_blocks<16, false>(p.sfb, t.b_row0 >> 4, kb0, raw + kRawA, lane, sb);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (KIND == KIND_MXF8) return;
+        __syncwarp();
+        const uint4 *rows = reinterpret_cast<const uint4 *>(sorted);
+        if (KIND == KIND_MXF4B16) {
+            const int hi = lane >> 4;
+#pragma unroll
+            for (int j = 0; j < 8; j++) {   // MMA j % 4 of stage j / 4
+                block_rows[3 * j] = rows[2 * j + hi];                       // A
+                block_rows[3 * j + 1] = rows[16 + 4 * j + 2 * hi];          // B rows 0..127
+                block_rows[3 * j + 2] = rows[16 + 4 * j + 2 * hi + 1];      // B rows 128..255
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < (KIND == KIND_MXF4RA ? 4 : 2); i++) block_rows[i] = rows[4 * i + (lane >> 3)];
+        }
+    }
+    __device__ __forceinline__ void write(int n_stages, uint8_t *images, int lane) const
+    {
+        constexpr int kStage = Cfg<KIND, CTAS>::kImageStage;
+        if (KIND == KIND_MXF4B16) {
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                if (j >= 4 * n_stages) break;
+                uint4 *img = reinterpret_cast<uint4 *>(images + (j >> 2) * kStage) + lane;
+                img[32 * (j & 3)] = block_rows[3 * j];
+                img[128 + 64 * (j & 3)] = block_rows[3 * j + 1];
+                img[160 + 64 * (j & 3)] = block_rows[3 * j + 2];
+            }
+            return;
+        }
+        if (KIND == KIND_MXF4RA || KIND == KIND_MXF4RB) {   // replicated images: lane writes one of the eight copies of every fourth row
+            constexpr int kRows = KIND == KIND_MXF4RA ? 2 : 1, kFirst = KIND == KIND_MXF4RA ? 1024 : 0;   // image rows per chunk
+#pragma unroll
+            for (int i = 0; i < 2 * kRows; i++) {
+                const int k = 4 * i + (lane >> 3), c = k / kRows;
+                *reinterpret_cast<uint4 *>(images + (c >> 1) * kStage + kFirst + (c & 1) * 128 * kRows + (k % kRows) * 128 + (lane & 7) * 16) = block_rows[i];
+            }
+        }
+#pragma unroll
+        for (int st = 0; st < 4; st++) {   // real images
+            if (st >= n_stages) break;
+            uint4 *img = reinterpret_cast<uint4 *>(images + st * kStage + (KIND == KIND_MXF4RB ? 256 : 0)) + lane;
+            if (KIND == KIND_MXF8) {
+                img[0] = make_uint4(w[0][st], w[1][st], w[2][st], w[3][st]);            // A
+                img[32] = make_uint4(w[4][st], w[5][st], w[6][st], w[7][st]);           // B rows 0..127
+                img[64] = make_uint4(w[8][st], w[9][st], w[10][st], w[11][st]);         // B rows 128..255
+            } else {
+#pragma unroll
+                for (int c = 0; c < 2; c++)
+#pragma unroll
+                    for (int r = 0; r < (KIND == KIND_MXF4RB ? 2 : 1); r++) {
+                        const int j = 2 * st + c, q = 4 * r;
+                        img[(KIND == KIND_MXF4RB ? 64 : 32) * c + 32 * r] = make_uint4(w[q][j], w[q + 1][j], w[q + 2][j], w[q + 3][j]);
+                    }
+            }
+        }
     }
 };
 
@@ -1135,12 +1152,9 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     constexpr int kElemsPerByte = kind_fp4(KIND) ? 2 : 1;
     constexpr int kStages = Cfg<KIND, CTAS>::kStages;
     constexpr int kBStageBytes = Cfg<KIND, CTAS>::kBStageBytes;
-    constexpr int kUnitStages = KIND == KIND_MXF4 ? kUnitStagesMxf4 : KIND == KIND_MXF8 ? kUnitStagesMxf8
-                                : KIND == KIND_MXF4R ? kUnitStagesMxf4R : kUnitStagesMxf4B16;   // stages whose scale images are built together
+    constexpr int kUnitStages = Cfg<KIND, CTAS>::kUnitStages, kImageStage = Cfg<KIND, CTAS>::kImageStage;
     constexpr int kBufBytes = Cfg<KIND, CTAS>::kBufBytes;
-    constexpr int kUnitBlocks = Cfg<KIND, CTAS>::kUnitBlocks;
     constexpr bool kGrouped = kGroupedKernel<KIND, WATCH>;
-    constexpr int kKbShift = KIND == KIND_MXF4B16 ? 4 : 5;    // log2 of the scale vector's length (contraction elements per scale byte)
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -1373,35 +1387,28 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 if (lane == 0) TRACE_EV(2, ev_j);
                 if (issuer) {
                     const uint32_t sf_tmem = tmem_base + kTmemSfBase + stage * SfCols<KIND>::kStride;
-                    if (KIND == KIND_MXF4) {
-                        const uint32_t img = smem_u32(smem_images + ring.buf * kBufBytes + (it & (kUnitStages - 1)) * kImageStageBytes);
-#pragma unroll
-                        for (int c = 0; c < 2; c++) {
-                            tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 4 * c, smem_desc_scale_image_rep(img + 128 * c));
-                            tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 8 + 8 * c, smem_desc_scale_image_rep(img + 256 + 256 * c));
-                            tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 12 + 8 * c, smem_desc_scale_image_rep(img + 384 + 256 * c));
-                        }
-                    } else if (KIND == KIND_MXF4B16) {
-                        const uint32_t img = smem_u32(smem_images + ring.buf * kBufBytes + (it & (kUnitStages - 1)) * kImageStageBytesMxf4B16);
+                    const uint32_t img = smem_u32(smem_images + ring.buf * kBufBytes + (it & (kUnitStages - 1)) * kImageStage);
+                    if (KIND == KIND_MXF4B16) {
 #pragma unroll
                         for (int i = 0; i < 4; i++) {
                             tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 4 * i, smem_desc_scale_image(img + 512 * i));
                             tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 16 + 8 * i, smem_desc_scale_image(img + 2048 + 1024 * i));
                             tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 20 + 8 * i, smem_desc_scale_image(img + 2560 + 1024 * i));
                         }
-                    } else if (KIND == KIND_MXF4R) {
-                        const uint32_t img = smem_u32(smem_images + ring.buf * kBufBytes + (it & (kUnitStages - 1)) * kImageStageBytesMxf4R);
-#pragma unroll
-                        for (int c = 0; c < 2; c++) {
-                            tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 4 * c, smem_desc_scale_image(img + 512 * c));
-                            tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 8 + 8 * c, smem_desc_scale_image(img + 1024 + 1024 * c));
-                            tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 12 + 8 * c, smem_desc_scale_image(img + 1536 + 1024 * c));
-                        }
-                    } else {
-                        const uint32_t img = smem_u32(smem_images + ring.buf * kBufBytes + (it & (kUnitStages - 1)) * kImageStageBytesMxf8);
+                    } else if (KIND == KIND_MXF8) {
                         tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem, smem_desc_scale_image(img));
                         tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 8, smem_desc_scale_image(img + 512));
                         tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 12, smem_desc_scale_image(img + 1024));
+                    } else {
+                        constexpr bool kRealA = KIND == KIND_MXF4RA, kRealB = KIND == KIND_MXF4RB;   // the other images are replicated
+                        constexpr uint32_t kA = kRealA ? 512 : 128, kB = kRealB ? 512 : 128;
+#pragma unroll
+                        for (int c = 0; c < 2; c++) {
+                            tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 4 * c, kRealA ? smem_desc_scale_image(img + kA * c) : smem_desc_scale_image_rep(img + kA * c));
+                            const uint32_t b = img + 2 * kA + 2 * kB * c;
+                            tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 8 + 8 * c, kRealB ? smem_desc_scale_image(b) : smem_desc_scale_image_rep(b));
+                            tcgen05_cp_32x128b_warpx4<CTAS>(sf_tmem + 12 + 8 * c, kRealB ? smem_desc_scale_image(b + kB) : smem_desc_scale_image_rep(b + kB));
+                        }
                     }
                     const uint64_t adesc = smem_desc_sw128(smem_u32(smem_a + stage * kAStageBytes));
                     const uint64_t bdesc = smem_desc_sw128(smem_u32(smem_b + stage * kBStageBytes));
@@ -1474,53 +1481,50 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         if (KIND != KIND_MXF4) {
             // per-row scales: the raw bytes of the next kOwnRaw units are in flight (cp.async) while a unit is turned into
             // images.  Two builders take every other unit and have raw buffers of their own.
-            constexpr int kRawBytes = Cfg<KIND, CTAS>::kRawBytes, kSlotB = Cfg<KIND, CTAS>::kRawSlotB;
+            constexpr int kRawBytes = Cfg<KIND, CTAS>::kRawBytes, kSorted = Cfg<KIND, CTAS>::kSortedBytes;
             constexpr int kOwnRaw = Cfg<KIND, CTAS>::kRawBufs > 0 ? Cfg<KIND, CTAS>::kRawBufs / kBuilders : 1;
-            uint8_t *raw = smem_raw_scales + (3 - warp) * kOwnRaw * kRawBytes;
+            uint8_t *raw = smem_raw_scales + (3 - warp) * (kOwnRaw * kRawBytes + kSorted);
             UnitIter<false> ahead, cur;
             ahead.init(p, first_tile, tile_step, rank);
-            cur.init(p, first_tile, tile_step, rank);
             if (warp == 2) {   // the second builder starts with the second unit
                 if (ahead.valid(p)) ahead.next(p, kUnitStages * kStageElems);
-                if (cur.valid(p)) cur.next(p, kUnitStages * kStageElems);
                 ring.next(kImageBufs);
             }
-            RowFetch rows;
+            cur = ahead;
+            RowBuilder<KIND, CTAS> rb;
             int rows_tile = -1;
             uint32_t raw_buf = 0;
             BufRing used;
             bool any = false;
-            auto fetch = [&](uint32_t buf) {   // the unit `ahead` points at, into raw buffer buf; one cp.async group in any case
-                if (!ahead.valid(p)) {
-                    asm volatile("cp.async.commit_group;" ::: "memory");
-                    return;
+#pragma unroll 1
+            for (int i = -kOwnRaw;; i++) {   // unit i of this builder is made, unit i + kOwnRaw is fetched
+                uint8_t *own = raw + raw_buf * kRawBytes;
+                if (++raw_buf == kOwnRaw) raw_buf = 0;
+                if (i >= 0) {
+                    if (!cur.valid(p)) break;
+                    asm volatile("cp.async.wait_group %0;" ::"n"(kOwnRaw - 1) : "memory");   // this unit's bytes have landed
+                    __syncwarp();
+                    rb.read(p, cur.t, cur.k0, own, raw + kOwnRaw * kRawBytes, lane);
+                    __syncwarp();   // the raw buffer and the sorted rows are free
                 }
-                if constexpr (KIND == KIND_MXF8) {
+                if (ahead.valid(p)) {
                     if (ahead.tile != rows_tile) {
-                        rows.set(p, ahead.t, lane);
+                        rb.set(p, ahead.t, lane);
                         rows_tile = ahead.tile;
                     }
-                    if (rows.fast) rows.issue(p, ahead.t, ahead.k0, smem_u32(raw + buf * kRawBytes), lane);
-                    else issue_raw_scales<kKbShift, kUnitBlocks, kSlotB>(p, ahead.t, ahead.k0, raw + buf * kRawBytes, lane);
-                } else {
-                    issue_raw_scales<kKbShift, kUnitBlocks, kSlotB>(p, ahead.t, ahead.k0, raw + buf * kRawBytes, lane);
+                    rb.fetch(p, ahead.t, ahead.k0, own, lane);
+                    for (int n = 0; n < kBuilders; n++)
+                        if (ahead.valid(p)) ahead.next(p, kUnitStages * kStageElems);
                 }
-#pragma unroll
-                for (int i = 0; i < kBuilders; i++)
-                    if (ahead.valid(p)) ahead.next(p, kUnitStages * kStageElems);
-            };
-            for (int i = 0; i < kOwnRaw; i++) fetch(i);
-            start_sync<CTAS, kBuilders, true>();
-            while (cur.valid(p)) {
-                asm volatile("cp.async.wait_group %0;" ::"n"(kOwnRaw - 1) : "memory");   // this unit's bytes have landed
-                __syncwarp();
-                uint32_t w[12][kUnitBlocks / 4];
-                read_raw_scales<kUnitBlocks, kSlotB>(p, raw + raw_buf * kRawBytes, lane, w);
+                asm volatile("cp.async.commit_group;" ::: "memory");   // one group in any case
+                if (i < 0) {
+                    if (i == -1) start_sync<CTAS, kBuilders, true>();
+                    continue;
+                }
                 ok = mbar_wait_impl<0>(bar_cache_empty + 8 * ring.buf, ring.phase ^ 1u, abort_flag, p.status, wait_limit, 0x500u + ring.buf);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
-                store_row_scale_images<KIND>(w, min(kUnitStages, (cur.t.k_len - cur.k0 + kStageElems - 1) / kStageElems),
-                                             smem_images + ring.buf * kBufBytes, lane);
+                rb.write(min(kUnitStages, (cur.t.k_len - cur.k0 + kStageElems - 1) / kStageElems), smem_images + ring.buf * kBufBytes, lane);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tcgen05.cp
                 __syncwarp();
                 // In the second CTA of a pair the arrival is forwarded to the leader by warp 1: the remote arrival
@@ -1528,10 +1532,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 if (lane == 0) mbar_arrive(bar_cache_full + 8 * ring.buf);
                 used = ring;
                 any = true;
-                fetch(raw_buf);   // the raw buffer just read is free
-                if (++raw_buf == kOwnRaw) raw_buf = 0;
-#pragma unroll
-                for (int i = 0; i < kBuilders; i++) {
+                for (int n = 0; n < kBuilders; n++) {
                     ring.next(kImageBufs);
                     if (cur.valid(p)) cur.next(p, kUnitStages * kStageElems);
                 }
@@ -2455,13 +2456,12 @@ extern "C" fp4q_status fp4q_gemm_fwd_act1d(const uint8_t *xq, int64_t ld_xq, con
     if (ldy < N || ld_xq < round_up(K, 32) / 2 || ld_xs < ceil_div(K, 32)) return FP4Q_ERR_SHAPE;
     Operand A, B = operand_rm(W);
     A.payload = xq; A.rows = T; A.row_bytes = round_up(K, 32) / 2; A.ld_bytes = ld_xq;
-    A.sf = ScaleView{xs, ld_xs, 1, (int32_t)T, (int32_t)ceil_div(K, 32), 0};
-    B.sf.row_shift = 5;
+    A.sf = ScaleView{xs, ld_xs, 1, (int32_t)T, (int32_t)ceil_div(K, 32)};
     GemmParams p = {};
     p.C = Y; p.ldc = ldy; p.M = (int32_t)T; p.N = (int32_t)N; p.K = (int32_t)K;
     p.out_f32 = dt == FP4Q_OUT_F32;
     dense_tiles(p);
-    return launch_gemm<KIND_MXF4R>(A, B, p, ws, ws_bytes, stream);
+    return launch_gemm<KIND_MXF4RA>(A, B, p, ws, ws_bytes, stream);
 }
 
 extern "C" fp4q_status fp4q_gemm_wgrad_act1d(const fp4q_tensor *dY, const uint8_t *xtq, int64_t ld_xtq, const uint8_t *xts,
@@ -2478,14 +2478,13 @@ extern "C" fp4q_status fp4q_gemm_wgrad_act1d(const fp4q_tensor *dY, const uint8_
     if (!dW || !dY->q_t || !dY->scale || !xtq || !xts) return FP4Q_ERR_NULL;
     if (ldw < K || ld_xtq < round_up(T, 32) / 2 || ld_xts < ceil_div(T, 32)) return FP4Q_ERR_SHAPE;
     Operand A = operand_t(dY), B;
-    A.sf.row_shift = 5;
     B.payload = xtq; B.rows = K; B.row_bytes = round_up(T, 32) / 2; B.ld_bytes = ld_xtq;
-    B.sf = ScaleView{xts, ld_xts, 1, (int32_t)K, (int32_t)ceil_div(T, 32), 0};
+    B.sf = ScaleView{xts, ld_xts, 1, (int32_t)K, (int32_t)ceil_div(T, 32)};
     GemmParams p = {};
     p.C = dW; p.ldc = ldw; p.M = (int32_t)N; p.N = (int32_t)K; p.K = (int32_t)T;
     p.out_f32 = dt == FP4Q_OUT_F32; p.accumulate = accumulate ? 1 : 0;
     dense_tiles(p);
-    return launch_gemm<KIND_MXF4R>(A, B, p, ws, ws_bytes, stream);
+    return launch_gemm<KIND_MXF4RB>(A, B, p, ws, ws_bytes, stream);
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -2496,13 +2495,13 @@ namespace fp4q {
 static Operand operand_rm16(const fp4q_tensor *t)
 {
     Operand o = operand_rm(t);
-    o.sf = ScaleView{t->scale, t->ld_s, 1, (int32_t)ceil_div(t->rows, 16), (int32_t)ceil_div(t->cols, 16), 4};
+    o.sf = ScaleView{t->scale, t->ld_s, 1, (int32_t)ceil_div(t->rows, 16), (int32_t)ceil_div(t->cols, 16)};
     return o;
 }
 static Operand operand_t16(const fp4q_tensor *t)
 {
     Operand o = operand_t(t);
-    o.sf = ScaleView{t->scale, 1, t->ld_s, (int32_t)ceil_div(t->cols, 16), (int32_t)ceil_div(t->rows, 16), 4};
+    o.sf = ScaleView{t->scale, 1, t->ld_s, (int32_t)ceil_div(t->cols, 16), (int32_t)ceil_div(t->rows, 16)};
     return o;
 }
 

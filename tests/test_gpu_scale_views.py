@@ -89,3 +89,41 @@ def test_grouped_products_do_not_depend_on_where_the_scales_lie(counts, N, K, al
             assert torch.equal(got, ref), (what, gap, start)
     torch.cuda.synchronize()
     assert binding.fp4q_workspace_status(ws) == 0
+
+
+def moved(scale, gap, start):
+    """A scale matrix `start` bytes into a buffer, its rows `gap` bytes further apart."""
+    rows, cols = scale.shape
+    buf = torch.full((start + rows * (cols + gap),), 0xFF, dtype=torch.uint8, device="cuda")
+    view = buf.as_strided((rows, cols), (cols + gap, 1), start)
+    view.copy_(scale)
+    return view
+
+
+# The per-row kinds fetch rows on 16 bytes as they are and others word by word: rows of 1, 3, 7, 8, 16, 17 and 86 blocks (twice that in 16 x 16
+# blocks), one unit and several, tiles with one row, with rows at the tile's edge and beyond, one CTA and pairs.
+@pytest.mark.parametrize("T,N,K", [(1, 1, 32), (100, 70, 200), (128, 256, 256), (300, 777, 1234), (161, 1311, 2731), (257, 512, 544), (512, 1024, 512), (700, 96, 2080)])
+def test_per_row_products_do_not_depend_on_where_the_scales_lie(T, N, K):
+    x, w, dy = (workloads.activations_student_t(r, c, i, "cuda") for i, (r, c) in enumerate(((T, K), (N, K), (T, N))))
+    ws = binding.alloc_workspace("cuda")
+    qw, qdy, q16 = binding.fp4q_quantize2d(w), binding.fp4q_quantize2d(dy), [binding.fp4q_quantize2d(t, flags=binding.BLOCK_16) for t in (x, w, dy)]
+    (xq, xs), (xtq, xts) = binding.fp4q_quantize1d(x), binding.fp4q_quantize1d_t(x)
+    (mq, ms), (nq, ns) = binding.fp4q_mxfp8_quantize1d(x), binding.fp4q_mxfp8_quantize1d(w)
+
+    def products(move, move_q):
+        w2, dy2, (x16, w16, dy16) = move_q(qw), move_q(qdy), [move_q(q) for q in q16]
+        return [binding.fp4q_gemm_fwd_act1d(xq, move(xs), T, w2, dt=binding.OUT_F32, ws=ws), binding.fp4q_gemm_wgrad_act1d(dy2, xtq, move(xts), K, ws=ws),
+                binding.fp4q_gemm_fwd_b16(x16, w16, dt=binding.OUT_F32, ws=ws), binding.fp4q_gemm_dgrad_b16(dy16, w16, dt=binding.OUT_F32, ws=ws),
+                binding.fp4q_gemm_wgrad_b16(dy16, x16, ws=ws), binding.fp4q_mxfp8_gemm(mq, move(ms), nq, move(ns), T, N, K, dt=binding.OUT_F32, ws=ws)]
+
+    plain = products(lambda s: s, lambda q: q)
+    xd = {k: torch.from_numpy(v).cuda() for k, v in dict(
+        x1=oracle.dequantize1d(xq.cpu().numpy()[:, :(K + 1) // 2].copy(), xs.cpu().numpy()[:, :(K + 31) // 32].copy(), T, K),
+        w=dequant_from_gpu(qw), dy=dequant_from_gpu(qdy)).items()}
+    check_gemm(plain[0], (xd["x1"] @ xd["w"].T).cpu().numpy(), "1D forward")
+    for gap, start in ((0, 0), (0, 1), (1, 0), (2, 3), (16 - xs.shape[1] % 16, 0), (16 - xs.shape[1] % 16, 4), (7, 2)):
+        got = products(lambda s: moved(s, gap, start), lambda q: dataclasses.replace(q, scale=moved(q.scale, gap, start)))
+        for i, (a, b) in enumerate(zip(got, plain)):
+            assert torch.equal(a, b), (i, gap, start)   # the same operands and order of sums
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
