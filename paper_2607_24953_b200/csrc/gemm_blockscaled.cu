@@ -7,7 +7,7 @@
 //   kind::mxf8f6f4  E4M3 payload, one UE8M0 scale per row and 32 contraction elements (MXFP8).
 //
 // Persistent kernel, one CTA per SM, 12 warps.  Dense products of more than 128 rows, grouped weight gradients and grouped rows
-// on 256-row boundaries run as clusters of two CTAs that share a 256x256 tile through cta_group::2 MMAs (each CTA holds 128
+// on 256-row boundaries, or on 128-row ones where that pays, run as clusters of two CTAs that share a 256x256 tile through cta_group::2 MMAs (each CTA holds 128
 // rows of the accumulator, loads its own 128 A rows and half of the B rows); everything else uses one CTA per 128x256 tile.
 //   warp 0      TMA producer: per stage the A tile (128 rows x 128 B) and the B tile (256 or 128 rows x 128 B),
 //               128B swizzle
@@ -41,6 +41,7 @@ constexpr int kMaxStages = 6;
 constexpr int kAStageBytes = BM * 128;
 constexpr int kMaxGroupsShared = 1023;       // grouped contraction: boundaries kept in shared memory up to this many groups
 constexpr int kMaxGroupsSorted = 256;        // grouped contraction: up to this many groups may be taken longest first (launch_gemm_impl says when)
+constexpr int kMaxGroupsPaired = 3071;       // paired rows: groups whose first tiles and numbers of pairs fit where the images will be
 constexpr int kMaxRowTilesShared = 2048;     // grouped rows: group of each 128-row tile kept in shared memory up to this many tiles
 constexpr int kSmemTail = 512;               // barriers, TMEM base, abort flag, scale scratch (one per loader warp)
 // 2D-block scales: the scale images of a whole unit (up to 16 stages = 4096 contraction elements of one tile) are
@@ -165,7 +166,9 @@ extern "C" int fp4q_debug_events(void *host) { return (int)cudaMemcpyFromSymbol(
 #endif
 constexpr uint8_t kScalePad = 127;           // UE8M0 code of 1.0 for scale slots beyond the tensor (their payload is 0)
 
-enum { MODE_DENSE = 0, MODE_GROUPED_ROWS = 1, MODE_GROUPED_K = 2 };
+// MODE_PAIRED_ROWS: grouped rows on pairs where groups start on multiples of 128 rows: two row tiles of one group a pair, the last alone if
+// the group has an odd number (the second CTA then loads nothing for A and stores nothing).
+enum { MODE_DENSE = 0, MODE_GROUPED_ROWS = 1, MODE_GROUPED_K = 2, MODE_PAIRED_ROWS = 3 };
 
 struct ScaleView {
     const uint8_t *ptr;
@@ -459,7 +462,8 @@ __device__ __forceinline__ uint32_t instr_desc(uint32_t a_sf_id, uint32_t b_sf_i
 // each): 4000 cycles per tile, more than a tile with a short contraction runs.  So the CTA fills a table in shared
 // memory before its roles start (`goffs`, 4 KB, null when the problem is too large for it or the kernel's
 // configuration has no room): with grouped rows the group of every 128-row tile as 16 bits (one load per tile),
-// with a grouped contraction a 32-bit copy of the boundaries.
+// with a grouped contraction a 32-bit copy of the boundaries, with paired rows a word for every pair: its first row tile (16 bits),
+// its group (15) and whether it has that tile only (1).
 
 __device__ __forceinline__ int find_group(const int64_t *offs, const int32_t *goffs, int n_groups, int64_t row)
 {
@@ -472,20 +476,23 @@ __device__ __forceinline__ int find_group(const int64_t *offs, const int32_t *go
     return lo;
 }
 
-// need_b = false leaves out the B operand's position: with grouped rows that is the group lookup, which only the
-// producer and the scale builder need - the MMA issuer, the watcher and the epilogue use the contraction length and
-// the output position alone, and a lookup in the MMA warp (shared-memory reads behind its pending MMAs) costs
-// about 1900 cycles per tile.
+// need: NEED_ALL; NEED_OUTPUT leaves out the B operand's position, with grouped rows the group lookup, which only the
+// producer and the scale builder need; NEED_LENGTH, the contraction length alone, is for the MMA issuer and the watcher: a lookup in
+// the MMA warp (shared-memory reads behind its pending MMAs) costs about 1900 cycles per tile.
+// m_tiles: p.m_tiles but for paired rows, whose number only the boundaries tell.
+enum { NEED_LENGTH = 0, NEED_OUTPUT = 1, NEED_ALL = 2 };
 // One warp runs an instruction in about five cycles and every role decodes its tiles.  us, with integer divisions and with multiplications:
 // 2048 x 2048 x 2048 10.4 / 10.6 / 11.9 -> 10.3 / 10.4 / 11.7, 16 groups of 9088 rows 768 x 1440 16.6 / 14.2 / 23.7 -> 16.0 / 13.4 / 22.9, quantized
 // output 8192 x 5632 x 2048 61.4 -> 58.2.
-// GROUPED = false: a kernel that only dense products use.  Their tiles are decoded without the group branches, which cost
-// the builders of the per-row kinds 3-8 % of a product (1D activations at 4096 x 4096 x 4096: 45.8 us without, 49.7 us with).
-template <bool GROUPED>
-__device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int rank, Tile &t, const int32_t *goffs, const uint16_t *gorder, bool need_b = true)
+// GROUPS: what a kernel is made for.  Dense products' tiles are decoded without the group branches, which cost the builders of the
+// per-row kinds 3-8 % of a product (1D activations at 4096 x 4096 x 4096: 45.8 us without, 49.7 us with), one CTA's smallest ones 0.3 us
+// (128 x 256 x 256 6.1 / 5.8) and quantized outputs 3-5 % (2048 x 2048 x 2048 12.4 / 11.7, 8192 x 5632 x 2048 56.6 / 55.2).
+enum { GROUPS_NONE = 0, GROUPS_ANY = 1, GROUPS_PAIRED = 2 };   // PAIRED: any, and paired rows
+template <int GROUPS>
+__device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int rank, Tile &t, int m_tiles, const int32_t *goffs, const uint16_t *gorder, int need = NEED_ALL)
 {
-    const int mode = GROUPED ? p.mode : MODE_DENSE;
-    const int per_problem = p.m_tiles * p.n_tiles;
+    const int mode = GROUPS != GROUPS_NONE ? p.mode : MODE_DENSE;
+    const int per_problem = m_tiles * p.n_tiles;
     const int nth = mode == MODE_GROUPED_K ? p.by_problem(tile) : 0, g = mode == MODE_GROUPED_K && gorder ? (int)gorder[nth] : nth;
     const int local = tile - nth * per_problem;
     // Tiles that run at the same time (consecutive indices) cover raster_m row tiles x a few column tiles, and
@@ -493,8 +500,8 @@ __device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int r
     // in L2 for the whole sweep instead of the whole A operand being streamed once per wave.
     const int per_group = p.raster_m * p.n_tiles;
     const int grp_m = p.by_group(local), in_grp = local - grp_m * per_group;
-    const int m0 = grp_m * p.raster_m, gsz = min(p.raster_m, p.m_tiles - m0);
-    const int n_blk = gsz == p.raster_m ? p.by_raster(in_grp) : p.by_tail(in_grp), m_blk = m0 + (in_grp - n_blk * gsz);
+    const int m0 = grp_m * p.raster_m, gsz = min(p.raster_m, m_tiles - m0);
+    const int n_blk = gsz == p.raster_m ? p.by_raster(in_grp) : GROUPS == GROUPS_PAIRED && mode == MODE_PAIRED_ROWS ? in_grp / gsz : p.by_tail(in_grp), m_blk = m0 + (in_grp - n_blk * gsz);
     t.a_row0 = (m_blk * p.ctas + rank) * BM;
     t.b_row0 = n_blk * BN;
     t.b_load_row0 = t.b_row0 + (p.ctas == 2 ? rank * 128 : 0);
@@ -504,8 +511,17 @@ __device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int r
     t.c_col0 = t.b_row0;
     t.m_valid = min(BM, p.M - t.a_row0);
     t.n_valid = min(BN, p.N - t.b_row0);
-    if (mode == MODE_GROUPED_ROWS) {
-        if (!need_b) return;
+    if (GROUPS == GROUPS_PAIRED && mode == MODE_PAIRED_ROWS) {
+        if (need == NEED_LENGTH) return;
+        const uint32_t e = (uint32_t)goffs[m_blk], alone = e >> 31;
+        t.a_row0 = t.c_row0 = ((int)(e & 0xFFFFu) + (alone ? 0 : rank)) * BM;
+        t.m_valid = alone && rank ? 0 : min(BM, p.M - t.a_row0);
+        const int grp = (int)(e >> 16 & 0x7FFFu);
+        t.b_row0 += grp * p.b_rows_per_group;
+        t.b_load_row0 += grp * p.b_rows_per_group;
+        t.b_k0 = grp * p.b_k_per_group;
+    } else if (mode == MODE_GROUPED_ROWS) {
+        if (need != NEED_ALL) return;
         const int grp = goffs ? (int)reinterpret_cast<const uint16_t *>(goffs)[t.a_row0 / BM]
                               : find_group(p.row_offsets, nullptr, p.n_groups, (int64_t)t.a_row0);
         t.b_row0 += grp * p.b_rows_per_group;
@@ -528,7 +544,7 @@ struct StageIter {
     __device__ __forceinline__ void seek(const GemmParams &p, int stage_elems)
     {
         while (tile < p.n_tile_total) {
-            decode_tile<false>(p, tile, rank, t, nullptr, nullptr, false);
+            decode_tile<GROUPS_NONE>(p, tile, rank, t, p.m_tiles, nullptr, nullptr, NEED_LENGTH);
             n_it = (t.k_len + stage_elems - 1) / stage_elems;
             if (n_it > 0) { it = 0; return; }
             tile += step;
@@ -818,27 +834,28 @@ struct BufRing {
 };
 
 // The stream of scale units (kUnitStages stages of one tile) a CTA works through.
-template <bool GROUPED>
+template <int GROUPS>
 struct UnitIter {
-    int tile, step, rank, k0;
+    int tile, step, rank, k0, m_tiles, n_total;
     Tile t;
     const int32_t *goffs = nullptr;
     const uint16_t *gorder = nullptr;
     __device__ __forceinline__ void seek(const GemmParams &p)
     {
-        while (tile < p.n_tile_total) {
-            decode_tile<GROUPED>(p, tile, rank, t, goffs, gorder);
+        while (tile < n_total) {
+            decode_tile<GROUPS>(p, tile, rank, t, m_tiles, goffs, gorder);
             if (k0 < t.k_len) return;
             tile += step;
             k0 = 0;
         }
     }
-    __device__ __forceinline__ void init(const GemmParams &p, int first, int step_, int rank_)
+    __device__ __forceinline__ void init(const GemmParams &p, int first, int step_, int rank_, int m_tiles_, int n_total_)
     {
+        m_tiles = m_tiles_; n_total = n_total_;
         tile = first; step = step_; rank = rank_; k0 = 0;
         seek(p);
     }
-    __device__ __forceinline__ bool valid(const GemmParams &p) const { return tile < p.n_tile_total; }
+    __device__ __forceinline__ bool valid(const GemmParams &p) const { return tile < n_total; }
     __device__ __forceinline__ void next(const GemmParams &p, int unit_elems)
     {
         k0 += unit_elems;
@@ -1136,12 +1153,10 @@ struct RowBuilder {
 
 // ---------------------------------------------------------------------------------------- kernel
 
-// Grouped products exist for 2D-block scales only, and their kernels have no watcher.
-template <int KIND, bool WATCH> constexpr bool kGroupedKernel = KIND == KIND_MXF4 && !WATCH;
-
 // WATCH: warp 2 looks at the ring's barriers for the MMA warp and the two meet at a named barrier per stage; otherwise the
 // MMA warp looks for itself, at the next stage's before it issues a stage.  launch_gemm() says which is used where.
-template <int KIND, int CTAS, int EPI, bool WATCH>
+// GROUPS: see decode_tile; grouped products exist for 2D-block scales only, and their kernels have no watcher.
+template <int KIND, int CTAS, int EPI, bool WATCH, int GROUPS>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmD,
@@ -1154,7 +1169,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     constexpr int kBStageBytes = Cfg<KIND, CTAS>::kBStageBytes;
     constexpr int kUnitStages = Cfg<KIND, CTAS>::kUnitStages, kImageStage = Cfg<KIND, CTAS>::kImageStage;
     constexpr int kBufBytes = Cfg<KIND, CTAS>::kBufBytes;
-    constexpr bool kGrouped = kGroupedKernel<KIND, WATCH>;
+    constexpr bool kGrouped = GROUPS != GROUPS_NONE;
+    static_assert(!kGrouped || (KIND == KIND_MXF4 && !WATCH), "grouped products");
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -1239,7 +1255,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     // grouped products: a 32-bit copy of the group boundaries for the per-tile lookups of every role
     const int n_row_tiles = (p.M + BM - 1) / BM;
     const bool goffs_ok = kGrouped && Cfg<KIND, CTAS>::kSmemGroups > 0 &&
-                          ((p.mode == MODE_GROUPED_K && p.n_groups <= kMaxGroupsShared) ||
+                          ((GROUPS == GROUPS_PAIRED && p.mode == MODE_PAIRED_ROWS) || (p.mode == MODE_GROUPED_K && p.n_groups <= kMaxGroupsShared) ||
                            (p.mode == MODE_GROUPED_ROWS && n_row_tiles <= kMaxRowTilesShared && p.n_groups <= 65535));
     if (goffs_ok && p.mode == MODE_GROUPED_K)
         for (int g = threadIdx.x; g <= p.n_groups; g += kThreads) goffs_smem[g] = (int32_t)load_global(p.row_offsets + g);
@@ -1255,6 +1271,39 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         }
         for (int i = threadIdx.x; i < n_row_tiles; i += kThreads)
             reinterpret_cast<uint16_t *>(goffs_smem)[i] = (uint16_t)find_group(p.row_offsets, copy ? bounds : nullptr, p.n_groups, (int64_t)i * BM);
+    }
+    int m_tiles = p.m_tiles, n_tile_total = p.n_tile_total;
+    if (GROUPS == GROUPS_PAIRED && p.mode == MODE_PAIRED_ROWS) {
+        // Groups' first row tiles, their numbers of pairs added up, then every pair looks its group up.  Offsets that are not as the caller
+        // states go to some tile or other, but to no other memory.
+        int32_t *start = reinterpret_cast<int32_t *>(smem_images), *first = start + p.n_groups + 1;
+        for (int g = threadIdx.x; g <= p.n_groups; g += kThreads)
+            start[g] = g == 0 ? 0 : g == p.n_groups ? n_row_tiles : (int32_t)max((int64_t)0, min((int64_t)n_row_tiles, (load_global(p.row_offsets + g) + BM - 1) / BM));
+        __syncthreads();
+        if (warp == 4) {
+            const int per_lane = (p.n_groups + 31) / 32, g0 = min(lane * per_lane, p.n_groups), g1 = min(g0 + per_lane, p.n_groups);
+            int sum = 0;
+            for (int g = g0; g < g1; g++) sum += (max(0, start[g + 1] - start[g]) + 1) >> 1;
+            int before = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int other = __shfl_up_sync(0xFFFFFFFFu, before, d);
+                if (lane >= d) before += other;
+            }
+            before -= sum;
+            for (int g = g0; g < g1; g++) {
+                first[g] = before;
+                before += (max(0, start[g + 1] - start[g]) + 1) >> 1;
+            }
+            if (lane == 31) first[p.n_groups] = min(before, kMaxGroupsShared + 1);
+        }
+        __syncthreads();
+        m_tiles = first[p.n_groups];
+        n_tile_total = m_tiles * p.n_tiles;
+        for (int i = threadIdx.x; i < m_tiles; i += kThreads) {
+            const int g = find_group(nullptr, first, p.n_groups, i), rt = start[g] + 2 * (i - first[g]);
+            goffs_smem[i] = (int32_t)((uint32_t)rt | (uint32_t)g << 16 | (rt + 1 >= start[g + 1] ? 0x80000000u : 0u));
+        }
     }
     const int32_t *goffs = goffs_ok ? goffs_smem : nullptr;
     // Grouped contraction: the groups longest first.  Their tiles go round the CTAs in turn, so that in any other order a CTA
@@ -1288,9 +1337,10 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         TRACE_T0(tt);
         int ev_j = 0;
         bool started = false;
-        for (int tile = first_tile; ok && tile < p.n_tile_total; tile += tile_step) {
+        for (int tile = first_tile; ok && tile < n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile<kGrouped>(p, tile, rank, t, goffs, gorder);
+            decode_tile<GROUPS>(p, tile, rank, t, m_tiles, goffs, gorder);
+            const int32_t ya = kGrouped && t.m_valid <= 0 ? p.M : t.a_row0;   // a CTA without rows: zeros from beyond the tensor
             const int n_it = (t.k_len + kStageElems - 1) / kStageElems;
             int xa = t.a_k0 / kElemsPerByte, xb = t.b_k0 / kElemsPerByte;
             if (!started) start_sync<CTAS, kBuilders>();
@@ -1306,14 +1356,14 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                     const uint32_t lbar = lbar0 + 8 * stage;
                     if (CTAS == 1) {
                         mbar_arrive_expect_tx(lbar, kAStageBytes + kBStageBytes);
-                        tma_load_2d(a0 + stage * kAStageBytes, &tmA, xa, t.a_row0, lbar);
+                        tma_load_2d(a0 + stage * kAStageBytes, &tmA, xa, ya, lbar);
                         tma_load_2d(b0 + stage * kBStageBytes, &tmB, xb, t.b_load_row0, lbar);
                     } else {
                         // Both CTAs' bytes are counted on the leader's barrier, which the leader arms for all of them.
                         // (A remote mbarrier.arrive per stage by a thread of the second CTA costs ~1200 cycles each
                         // and cannot be pipelined; letting the TMA unit signal the remote barrier costs nothing.)
                         if (leader) mbar_arrive_expect_tx(bar_full + 8 * stage, 2 * (kAStageBytes + kBStageBytes));
-                        tma_load_2d_pair(a0 + stage * kAStageBytes, &tmA, xa, t.a_row0, lbar);
+                        tma_load_2d_pair(a0 + stage * kAStageBytes, &tmA, xa, ya, lbar);
                         tma_load_2d_pair(b0 + stage * kBStageBytes, &tmB, xb, t.b_load_row0, lbar);
                     }
                 }
@@ -1350,9 +1400,9 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         int ev_j = 0;
         TRACE_DECL(c_acc); TRACE_DECL(c_sync); TRACE_DECL(c_issue);
         TRACE_T0(tt);
-        for (int tile = first_tile; leader && tile < p.n_tile_total; tile += tile_step) {
+        for (int tile = first_tile; leader && tile < n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile<kGrouped>(p, tile, rank, t, goffs, gorder, false);
+            decode_tile<GROUPS>(p, tile, rank, t, m_tiles, goffs, gorder, NEED_LENGTH);
             const int n_it = (t.k_len + kStageElems - 1) / kStageElems;
             if (n_it == 0) continue;
             TRACE_ADD(c_acc, tt);
@@ -1446,8 +1496,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             // builders have finished to the leader, which issues the scale copies of both CTAs.
             bool fwd_ok = true;
             BufRing fr;
-            UnitIter<false> un;
-            for (un.init(p, first_tile, tile_step, rank); fwd_ok && un.valid(p); un.next(p, kUnitStages * kStageElems), fr.next(kImageBufs)) {
+            UnitIter<GROUPS_NONE> un;
+            for (un.init(p, first_tile, tile_step, rank, m_tiles, n_tile_total); fwd_ok && un.valid(p); un.next(p, kUnitStages * kStageElems), fr.next(kImageBufs)) {
                 fwd_ok = __all_sync(0xFFFFFFFFu, mbar_wait_impl<0>(bar_cache_full + 8 * fr.buf, fr.phase, abort_flag, p.status, wait_limit, 0x530u + fr.buf));
                 if (fwd_ok && issuer) mbar_arrive_cluster(cluster_addr(bar_peer_cache_full + 8 * fr.buf, 0));
             }
@@ -1484,8 +1534,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             constexpr int kRawBytes = Cfg<KIND, CTAS>::kRawBytes, kSorted = Cfg<KIND, CTAS>::kSortedBytes;
             constexpr int kOwnRaw = Cfg<KIND, CTAS>::kRawBufs > 0 ? Cfg<KIND, CTAS>::kRawBufs / kBuilders : 1;
             uint8_t *raw = smem_raw_scales + (3 - warp) * (kOwnRaw * kRawBytes + kSorted);
-            UnitIter<false> ahead, cur;
-            ahead.init(p, first_tile, tile_step, rank);
+            UnitIter<GROUPS_NONE> ahead, cur;
+            ahead.init(p, first_tile, tile_step, rank, m_tiles, n_tile_total);
             if (warp == 2) {   // the second builder starts with the second unit
                 if (ahead.valid(p)) ahead.next(p, kUnitStages * kStageElems);
                 ring.next(kImageBufs);
@@ -1541,10 +1591,10 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             if (ok && any) mbar_wait_impl<0>(bar_cache_empty + 8 * used.buf, used.phase, abort_flag, p.status, wait_limit, 0x540u);
         }
         if (KIND == KIND_MXF4) {
-            UnitIter<kGrouped> un;   // the unit whose scale bytes are being loaded
+            UnitIter<GROUPS> un;   // the unit whose scale bytes are being loaded
             un.goffs = goffs;
             un.gorder = gorder;
-            un.init(p, first_tile, tile_step, rank);
+            un.init(p, first_tile, tile_step, rank, m_tiles, n_tile_total);
             uint32_t wa[4] = {}, wb[8] = {};
             uint32_t next_a[4] = {}, next_b[8] = {};
             int how_a = SCALES_WHOLE, how_b = SCALES_WHOLE;
@@ -1756,10 +1806,10 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         int ev_t = 0;
         TRACE_DECL(c_wait); TRACE_DECL(c_ld); TRACE_DECL(c_store);
         TRACE_T0(tt);
-        for (int tile = first_tile; ok && tile < p.n_tile_total; tile += tile_step) {
+        for (int tile = first_tile; ok && tile < n_tile_total; tile += tile_step) {
             Tile t;
-            decode_tile<kGrouped>(p, tile, rank, t, goffs, gorder, false);
-            const bool last = tile + tile_step >= p.n_tile_total;   // of this CTA
+            decode_tile<GROUPS>(p, tile, rank, t, m_tiles, goffs, gorder, NEED_OUTPUT);
+            const bool last = tile + tile_step >= n_tile_total;   // of this CTA
             const int row_in_tile = 32 * quarter + lane;
             const int64_t row = (int64_t)t.c_row0 + row_in_tile;
             const bool row_ok = row_in_tile < t.m_valid;
@@ -2067,11 +2117,18 @@ static int sm_count(int dev)
     return n[dev];
 }
 
-template <int KIND, int CTAS, int EPI, bool WATCH>
+// Most row tiles that pairs can have with grouped rows on multiples of 128: a group with an odd number has one alone.
+static int64_t paired_tiles(const GemmParams &p)
+{
+    const int64_t rows = ceil_div(p.M, BM);
+    return (rows + (p.n_groups < rows ? p.n_groups : rows)) / 2;
+}
+
+template <int KIND, int CTAS, int EPI, bool WATCH, int GROUPS = GROUPS_NONE>
 static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmParams &p, void *stream)
 {
     CUtensorMap tmA, tmB, tmC;
-    if (!kGroupedKernel<KIND, WATCH> && p.mode != MODE_DENSE) return FP4Q_ERR_UNSUPPORTED;
+    if (GROUPS == GROUPS_NONE && p.mode != MODE_DENSE) return FP4Q_ERR_UNSUPPORTED;
     const int64_t out_rows = p.mode == MODE_GROUPED_K ? (int64_t)p.n_groups * p.M : p.M;
     if (!make_operand_map(&tmA, A.payload, A.rows, A.row_bytes, A.ld_bytes, BM)) return FP4Q_ERR_CUDA;
     CUtensorMap tmD = tmA;   // second output map: only the quantizing epilogue has one
@@ -2086,6 +2143,11 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     p.m_tiles = (int32_t)ceil_div(p.M, BM * CTAS);
     p.n_tile_total = p.m_tiles * p.n_tiles * (p.mode == MODE_GROUPED_K ? p.n_groups : 1);
     p.raster_m = p.mode != MODE_GROUPED_K ? (p.m_tiles < kRasterM ? p.m_tiles : kRasterM) : p.m_tiles;
+    if (p.mode == MODE_PAIRED_ROWS) {   // as many as there can be
+        p.m_tiles = (int32_t)paired_tiles(p);
+        p.n_tile_total = p.m_tiles * p.n_tiles;
+        p.raster_m = kRasterM;
+    }
 #ifdef FP4Q_TRACE
     if (const char *g = getenv("FP4Q_DEBUG_RASTER")) { p.raster_m = atoi(g); if (p.raster_m > p.m_tiles) p.raster_m = p.m_tiles; }
 #endif
@@ -2099,7 +2161,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     if (dev < 0) return FP4Q_ERR_CUDA;
     static bool attr_set[kMaxDevices];   // the attribute is a property of (kernel, device): one flag per device and instantiation
     if (!attr_set[dev]) {
-        if (cudaFuncSetAttribute(gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  Cfg<KIND, CTAS>::kSmemBytes) != cudaSuccess)
             return FP4Q_ERR_CUDA;
         attr_set[dev] = true;
@@ -2143,7 +2205,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     }
-    return launched(cudaLaunchKernelEx(&cfg, gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH>, tmA, tmB, tmC, tmD, p));
+    return launched(cudaLaunchKernelEx(&cfg, gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH, GROUPS>, tmA, tmB, tmC, tmD, p));
 }
 
 // Argument checks common to every product: everything that can be refused is refused here, before any work is enqueued.
@@ -2155,6 +2217,21 @@ static fp4q_status check_gemm_args(const Operand &A, const Operand &B, const Gem
     const size_t esize = p.out_f32 ? 4 : 2;
     if (!aligned(p.C, 16) || (p.ldc * esize) % 16) return FP4Q_ERR_ALIGN;
     return FP4Q_OK;
+}
+
+// Whether grouped rows on multiples of 128 run on pairs.  A tile of a pair takes 0.83-0.9 of the time of one CTA's that does half as much (three
+// stages 2.5 / 3.0 us, eight 4.75 / 5.4; nothing is gained with one or two), the table of pairs 0.7 us, and a group with an odd number of
+// row tiles, every other one on average, a tile for half the work.  So the rounds of tiles are compared, 9 to 10.  us, one CTA and pairs,
+// forward / input gradient: 272 row tiles in 32 groups, 768 x 2048 39.0 / 46.2 -> 34.5 / 44.7, 263 in 16 37.5 / 43.7 -> 32.5 / 41.2, 260 in 8, 1408 x 1024
+// 38.4 / 36.9 -> 33.5 / 32.1, 36 in 8, 1408 x 1440 16.1 / 14.1 -> 13.9 / 13.1; left on one CTA: 327 in 128, 768 x 2048 50.0 / 62.8 and 49.9 / 64.4, 145 in 32,
+// 768 x 1700 21.3 / 24.6 and 22.0 / 26.8, 257 in 4, 512 x 512 13.3 / 13.2 and 14.3 / 14.2.
+static bool pairs_pay(const GemmParams &p)
+{
+    const int64_t rows = ceil_div(p.M, BM), groups = p.n_groups < rows ? p.n_groups : rows;
+    if (p.K <= 512 || p.n_groups > kMaxGroupsPaired || paired_tiles(p) > kMaxGroupsShared + 1) return false;
+    const int dev = current_device();
+    const int64_t sms = dev < 0 ? 148 : sm_count(dev), pairs = (2 * rows + groups + 3) / 4;
+    return 9 * ceil_div(pairs * p.n_tiles, sms / 2) + 2 <= 10 * ceil_div(rows * p.n_tiles, sms);
 }
 
 template <int KIND>
@@ -2169,21 +2246,24 @@ static fp4q_status launch_gemm(const Operand &A, const Operand &B, GemmParams &p
     p.status = reinterpret_cast<uint32_t *>(ws);
     // Dense products (FP4 and MXFP8) with more than one row tile run as cta_group::2 pairs: 256x256 tiles, each CTA
     // loads half of the B rows; so does the grouped weight gradient, whose groups cut the contraction axis, not the
-    // output rows of a tile.  FP4Q_CTA_PAIRS=0 in the environment (read once, before the first GEMM call) selects
-    // the one-CTA kernel instead; grouped forward / input-gradient products use one CTA per 128x256 tile unless the
-    // caller states that every token group starts on a multiple of 256 rows.
+    // output rows of a tile, and grouped rows where every group starts on a multiple of 256 or where paired rows pay.
+    // FP4Q_CTA_PAIRS=0 in the environment (read once, before the first GEMM call) selects the one-CTA kernel instead.
     static const bool use_pairs = [] { const char *e = getenv("FP4Q_CTA_PAIRS"); return !(e && e[0] == '0'); }();
-    const bool pair_mode = p.mode == MODE_DENSE || p.mode == MODE_GROUPED_K || (p.mode == MODE_GROUPED_ROWS && p.rows_pair_aligned);
     // The watcher pays in the dense FP4 and MXFP8 products on pairs (16384 x 4096 x 4096, with and without: FP4 weight gradient
     // 98.4 and 102.7 us, forward 100.7 both; MXFP8 forward 213 and 218 us, weight gradient 228 and 236 us).  Everything else is
     // faster without it: the short contractions of grouped products (expert weight gradients 222 and 225 us without, 228
     // and 230 us with), the quantizing epilogue, whose warps it competes with (113 and 116 us), and the per-row FP4
     // kinds, where its warp builds scale images instead.
     constexpr bool kWatchDense = KIND == KIND_MXF4 || KIND == KIND_MXF8;
-    if (use_pairs && pair_mode && p.M > BM) {
-        if (kWatchDense && p.mode == MODE_DENSE) return launch_gemm_impl<KIND, 2, EPI_STORE, kWatchDense>(A, B, p, stream);
-        return launch_gemm_impl<KIND, 2, EPI_STORE, KIND == KIND_MXF8>(A, B, p, stream);
+    if constexpr (KIND == KIND_MXF4) {
+        if (p.mode != MODE_DENSE) {
+            if (use_pairs && p.M > BM && p.mode == MODE_GROUPED_ROWS && !p.rows_pair_aligned && pairs_pay(p)) p.mode = MODE_PAIRED_ROWS;
+            const bool pairs = p.mode == MODE_GROUPED_K || p.mode == MODE_PAIRED_ROWS || p.rows_pair_aligned;
+            if (use_pairs && pairs && p.M > BM) return launch_gemm_impl<KIND, 2, EPI_STORE, false, GROUPS_PAIRED>(A, B, p, stream);
+            return launch_gemm_impl<KIND, 1, EPI_STORE, false, GROUPS_ANY>(A, B, p, stream);
+        }
     }
+    if (use_pairs && p.M > BM) return launch_gemm_impl<KIND, 2, EPI_STORE, kWatchDense>(A, B, p, stream);
     return launch_gemm_impl<KIND, 1, EPI_STORE, false>(A, B, p, stream);
 }
 
@@ -2309,6 +2389,7 @@ static fp4q_status launch_gemm_quantized(const Operand &A, const Operand &B, int
         p.rows_pair_aligned = 1;
         p.b_rows_per_group = b_rows_per_group; p.b_k_per_group = b_k_per_group;
     }
+    if (g) return launch_gemm_impl<KIND_MXF4, 2, EPI_QUANT, false, GROUPS_ANY>(A, B, p, stream);
     return launch_gemm_impl<KIND_MXF4, 2, EPI_QUANT, false>(A, B, p, stream);
 }
 

@@ -53,3 +53,27 @@ def test_groups_are_found(E):
     check_gemm(dx, np.concatenate([dy[s] @ w[g * N:(g + 1) * N] for g, s in groups]), "dgrad")
     torch.cuda.synchronize()
     assert binding.fp4q_workspace_status(ws) == 0
+
+
+# Groups on multiples of 128 rows on pairs: two row tiles of a group a pair, the last of an odd number alone; empty groups, one group, more
+# groups than tiles, a last tile that is not full, both types of output
+@pytest.mark.parametrize("E,rows", [(8, 60), (600, 60), (1, 61), (3, 62)])
+def test_paired_rows(E, rows):
+    ws = binding.alloc_workspace("cuda")
+    rng = np.random.default_rng(E)
+    tiles = rng.multinomial(rows, rng.dirichlet(np.full(E, 0.5)))
+    offs = np.concatenate([[0], np.cumsum(128 * tiles)])
+    T, N, K = int(offs[-1]) - 3, 640, 1056
+    qx, qw, qdy = operands((T, K), (E * N, K), (T, N))
+    d = torch.from_numpy(offs).cuda()
+    full = {dt: (binding.fp4q_gemm_fwd(qx, qw, dt=dt, row_offsets=d, ws=ws), binding.fp4q_gemm_dgrad(qdy, qw, dt=dt, row_offsets=d, ws=ws))
+            for dt in (binding.OUT_BF16, binding.OUT_F32)}
+    x, dy, w = (torch.from_numpy(dequant_from_gpu(q)) for q in (qx, qdy, qw))
+    groups = [(g, slice(int(offs[g]), min(T, int(offs[g + 1])))) for g in range(E) if tiles[g]]
+    y = torch.cat([x[s] @ w[g * N:(g + 1) * N].T for g, s in groups]).numpy()
+    dx = torch.cat([dy[s] @ w[g * N:(g + 1) * N] for g, s in groups]).numpy()
+    for dt in full:
+        check_gemm(full[dt][0], y, "fwd")
+        check_gemm(full[dt][1], dx, "dgrad")
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
