@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "quant_device.cuh"
 
 namespace fp4q {
 
@@ -84,15 +85,15 @@ __global__ void __launch_bounds__(256) mxfp8_quantize1d_kernel(const __grid_cons
     const int be = (int)(fm >> 7), m7 = (int)(fm & 0x7F);
     int code = be == 0 ? 0 : be - 8 + (m7 > 0x60 ? 1 : 0);
     code = code < 0 ? 0 : code;
-    const float inv = __uint_as_float((uint32_t)(254 - code) << 23);   // 2^(127-code) = 2^-e
+    const uint32_t inv2 = (uint32_t)(254 - code) * 0x00800080u;   // 2^(127-code) = 2^-e, twice as BF16
     p.scale[i * p.ld_s + blk] = (uint8_t)code;
 
     uint32_t out[8];
 #pragma unroll
     for (int w = 0; w < 8; w++) {
-        const uint32_t w0 = raw[2 * w], w1 = raw[2 * w + 1];
-        out[w] = cvt_rn_e4m3x2(__uint_as_float(w0 & 0xFFFF0000u) * inv, __uint_as_float(w0 << 16) * inv) |
-                 (cvt_rn_e4m3x2(__uint_as_float(w1 & 0xFFFF0000u) * inv, __uint_as_float(w1 << 16) * inv) << 16);
+        const uint32_t w0 = scale_pair(raw[2 * w], inv2), w1 = scale_pair(raw[2 * w + 1], inv2);
+        out[w] = cvt_rn_e4m3x2(__uint_as_float(w0 & 0xFFFF0000u), __uint_as_float(w0 << 16)) |
+                 (cvt_rn_e4m3x2(__uint_as_float(w1 & 0xFFFF0000u), __uint_as_float(w1 << 16)) << 16);
     }
     uint4 *dst = reinterpret_cast<uint4 *>(p.q + i * p.ld_q + j0);
     dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(128, 4) mxfp8_quantize1d_t_tile_kernel(const _
         }
     }
     uint32_t codes[4] = {0u, 0u, 0u, 0u};
-    float inv[16];
+    uint32_t inv2[8] = {};   // two columns' 2^-e as BF16
 #pragma unroll
     for (int c = 0; c < 16; c++) {
         const uint32_t fm = (m2[c >> 1] >> (16 * (c & 1))) & 0x7FFFu;
@@ -262,8 +263,12 @@ __global__ void __launch_bounds__(128, 4) mxfp8_quantize1d_t_tile_kernel(const _
         int code = be == 0 ? 0 : be - 8 + (m7 > 0x60 ? 1 : 0);   // smallest e with 448*2^e >= M
         code = code < 0 ? 0 : code;
         codes[c >> 2] |= (uint32_t)code << (8 * (c & 3));
-        inv[c] = __uint_as_float((uint32_t)(254 - code) << 23);
+        inv2[c >> 1] |= (uint32_t)(254 - code) << (16 * (c & 1) + 7);
     }
+#pragma unroll
+    for (int r = 0; r < 8; r++)
+#pragma unroll
+        for (int k = 0; k < 8; k++) raw[r][k] = scale_pair(raw[r][k], inv2[k]);
     if (rg == 0) {
         uint8_t *sc = reinterpret_cast<uint8_t *>(sc_stage);
 #pragma unroll
@@ -280,8 +285,8 @@ __global__ void __launch_bounds__(128, 4) mxfp8_quantize1d_t_tile_kernel(const _
             for (int e = 0; e < 2; e++) {
                 const int r = 4 * h + 2 * e;
                 const uint32_t w0 = raw[r][c >> 1], w1 = raw[r + 1][c >> 1];
-                const float v0 = __uint_as_float((c & 1) ? (w0 & 0xFFFF0000u) : (w0 << 16)) * inv[c];
-                const float v1 = __uint_as_float((c & 1) ? (w1 & 0xFFFF0000u) : (w1 << 16)) * inv[c];
+                const float v0 = __uint_as_float((c & 1) ? (w0 & 0xFFFF0000u) : (w0 << 16));
+                const float v1 = __uint_as_float((c & 1) ? (w1 & 0xFFFF0000u) : (w1 << 16));
                 acc |= cvt_rn_e4m3x2(v1, v0) << (16 * e);
             }
             w[h] = acc;

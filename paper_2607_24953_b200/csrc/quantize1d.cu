@@ -262,12 +262,18 @@ __global__ void __launch_bounds__(128, 4) quantize1d_t_tile_kernel(const __grid_
         }
     }
     uint32_t codes[4] = {0u, 0u, 0u, 0u};   // 16 scale codes, one byte each
-    float inv[16];
+    uint32_t inv2[8] = {};                   // two columns' 2^-e as BF16
 #pragma unroll
     for (int c = 0; c < 16; c++) {
         const int code = scale_code_from_max((m2[c >> 1] >> (16 * (c & 1))) & 0x7FFFu);
         codes[c >> 2] |= (uint32_t)code << (8 * (c & 3));
-        inv[c] = careful ? inv_scale_f16_aligned(code) : inv_scale(code);
+        inv2[c >> 1] |= (uint32_t)(254 - code) << (16 * (c & 1) + 7);
+    }
+    if (!careful) {
+#pragma unroll
+        for (int r = 0; r < 8; r++)
+#pragma unroll
+            for (int k = 0; k < 8; k++) raw[r][k] = scale_pair(raw[r][k], inv2[k]);
     }
     if (rg == 0) {
         uint8_t *sc = reinterpret_cast<uint8_t *>(sc_stage);
@@ -284,8 +290,8 @@ __global__ void __launch_bounds__(128, 4) quantize1d_t_tile_kernel(const __grid_
 #pragma unroll
             for (int e = 0; e < 4; e++) {
                 const uint32_t w0 = raw[2 * e][c >> 1], w1 = raw[2 * e + 1][c >> 1];
-                const float v0 = __uint_as_float((c & 1) ? (w0 & 0xFFFF0000u) : (w0 << 16)) * inv[c];
-                const float v1 = __uint_as_float((c & 1) ? (w1 & 0xFFFF0000u) : (w1 << 16)) * inv[c];
+                const float v0 = __uint_as_float((c & 1) ? (w0 & 0xFFFF0000u) : (w0 << 16));
+                const float v1 = __uint_as_float((c & 1) ? (w1 & 0xFFFF0000u) : (w1 << 16));
                 word |= cvt_rn_e2m1x2(v1, v0) << (8 * e);
             }
         } else {   // rare: kept small and out of the hot loop's instruction footprint
@@ -295,7 +301,7 @@ __global__ void __launch_bounds__(128, 4) quantize1d_t_tile_kernel(const __grid_
                 const uint32_t w0 = raw[2 * e][c >> 1], w1 = raw[2 * e + 1][c >> 1];
                 h[e] = (c & 1) ? ((w0 >> 16) | (w1 & 0xFFFF0000u)) : ((w0 & 0xFFFFu) | (w1 << 16));
             }
-            word = round_column_scalar(make_uint4(h[0], h[1], h[2], h[3]), inv[c]);
+            word = round_column_scalar(make_uint4(h[0], h[1], h[2], h[3]), inv_scale_f16_aligned((int)(codes[c >> 2] >> (8 * (c & 3)) & 0xFFu)));
         }
         const int col_local = 32 * t + 16 * ch + c;
         // word index inside the 64-byte row: 4*(source warp) + rg, with the 16-byte chunk index XORed by the
