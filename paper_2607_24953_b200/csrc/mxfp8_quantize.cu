@@ -5,6 +5,7 @@
 
 #include "common.cuh"
 #include "quant_device.cuh"
+#include "quantize1d_staged.cuh"
 
 namespace fp4q {
 
@@ -114,18 +115,22 @@ __global__ void __launch_bounds__(128) mxfp8_quantize1d_t_kernel(const __grid_co
     if (i0 >= p.rows || c0 >= p.cols) return;
     const bool two = c0 + 1 < p.cols;
     uint32_t raw[32];
-    if (p.x_vec_ok && two && i0 + 32 <= p.rows) {   // interior: 32 unconditional word loads, one address step each
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(p.x + i0 * p.ld_x + c0);
-        const int64_t step = p.ld_x >> 1;
+    const uint32_t *words = reinterpret_cast<const uint32_t *>(p.x + i0 * p.ld_x + c0);   // the launch has seen to rows on words
+    const int64_t step = p.ld_x >> 1;
+    if (two && i0 + 32 <= p.rows) {   // interior: 32 unconditional word loads, one address step each
 #pragma unroll
-        for (int r = 0; r < 32; r++) raw[r] = load_global(src + r * step);
+        for (int r = 0; r < 32; r++) raw[r] = load_global(words + r * step);
+    } else if (two) {
+        const int n = (int)(p.rows - i0);
+#pragma unroll
+        for (int r = 0; r < 32; r++) raw[r] = r < n ? load_global(words + r * step) : 0u;
     } else {
 #pragma unroll
         for (int r = 0; r < 32; r++) {
             raw[r] = 0u;
             if (i0 + r < p.rows) {
                 const uint16_t *src = p.x + (i0 + r) * p.ld_x + c0;
-                raw[r] = (uint32_t)load_global(src) | (two ? (uint32_t)load_global(src + 1) << 16 : 0u);
+                raw[r] = load_global(src);
             }
         }
     }
@@ -329,6 +334,8 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d(const void *x_bf16, int64_t rows, i
     const int64_t total = rows * (p.segs_per_row / 2);
     const int64_t n_cta = ceil_div(total, 256);
     if (n_cta > 0x7FFFFFFF) return FP4Q_ERR_UNSUPPORTED;
+    if (!p.x_vec_ok && rows * cols >= kStagedRowsFrom)
+        return launch_quantize1d_staged(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, true, false, static_cast<cudaStream_t>(stream));
     return launched(launch_dependent(mxfp8_quantize1d_kernel, dim3((unsigned)n_cta), 256, static_cast<cudaStream_t>(stream), p));
 }
 
@@ -355,5 +362,7 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d_t(const void *x_bf16, int64_t rows,
     }
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;
+    if (!p.x_vec_ok || rows * cols >= kStagedTransposeFrom)
+        return launch_quantize1d_staged(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, true, true, static_cast<cudaStream_t>(stream));
     return launched(launch_dependent(mxfp8_quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p));
 }

@@ -26,6 +26,7 @@
 
 #include "common.cuh"
 #include "quant_device.cuh"
+#include "staged_tile.cuh"
 
 namespace fp4q {
 
@@ -146,72 +147,6 @@ __device__ __forceinline__ void load_segment(const Quant2dParams &p, int64_t i, 
 // piece checked against the tensor's ends and the random blocks drawn afterwards into the same rows, us, nearest / stochastic:
 // 4099 x 2731 13.0 / 18.0 -> 12.2 / 16.4 (5.1 at the measured copy bandwidth), 16384 x 2731 41.3 / 58.7 -> 34.6 / 46.0,
 // 9001 x 8191 65.0 / 89.0 -> 52.1 / 70.6, 300 x 777 6.1 / 7.8 -> 6.0 / 7.4.
-constexpr int kStageRowBytes = 272;                        // 17 pieces
-constexpr int kStageRows4 = 4 * kStageRowBytes + 32;       // the rows r, 8 + r, 16 + r, 24 + r, which one load instruction reads
-constexpr int kStageWarpBytes = 8 * kStageRows4;
-
-// Row r of row group rg.  The extra 32 bytes after the second of four rows make the offsets 0, 1, 4, 5 (in 16-byte units,
-// modulo 8), so that the eight lanes of one shared-memory pass (four row groups x two column halves, 32 bytes apart)
-// read eight different bank groups.
-__device__ __forceinline__ int stage_row_offset(int r, int rg) { return r * kStageRows4 + rg * kStageRowBytes + (rg >> 1) * 32; }
-
-// Starts the copies (the caller waits).  Tiles whose pieces all lie inside the tensor need no checks.
-__device__ __forceinline__ void stage_tile_rows(const Quant2dParams &p, int64_t tile_row0, int64_t tile_col0, uint8_t *stage, int lane)
-{
-    const uintptr_t lo = reinterpret_cast<uintptr_t>(p.x), hi = reinterpret_cast<uintptr_t>(p.x + (p.rows - 1) * p.ld_x + p.cols);
-    const uintptr_t a0 = reinterpret_cast<uintptr_t>(p.x + tile_row0 * p.ld_x + tile_col0), pitch = 2 * (uintptr_t)p.ld_x;
-    const uint32_t dst0 = (uint32_t)__cvta_generic_to_shared(stage) + 16 * (lane & 15);
-    if (tile_row0 + 32 <= p.rows && tile_col0 + 128 <= p.cols && (a0 & ~(uintptr_t)15) >= lo && ((a0 + 31 * pitch) & ~(uintptr_t)15) + kStageRowBytes <= hi) {
-        uintptr_t a = a0 + (lane >> 4) * pitch;
-#pragma unroll
-        for (int k = 0; k < 16; k++) {   // two rows of 16 pieces per step, the 17th pieces of all rows last
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
-                         ::"r"(dst0 + stage_row_offset((2 * k) & 7, k >> 2) + (lane >> 4) * kStageRows4), "l"((a & ~(uintptr_t)15) + 16 * (lane & 15)) : "memory");
-            a += 2 * pitch;
-        }
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
-                     ::"r"((uint32_t)__cvta_generic_to_shared(stage) + stage_row_offset(lane & 7, lane >> 3) + 256), "l"(((a0 + lane * pitch) & ~(uintptr_t)15) + 256)
-                     : "memory");
-        return;
-    }
-    const int n_valid = (int)(p.cols - tile_col0 < 128 ? p.cols - tile_col0 : 128);
-#pragma unroll 1
-    for (int k = 0; k < 17; k++) {
-        const int row = k < 16 ? 2 * k + (lane >> 4) : lane, c = k < 16 ? lane & 15 : 16;
-        if (tile_row0 + row >= p.rows) continue;
-        const uintptr_t a = a0 + row * pitch;
-        const uintptr_t g = (a & ~(uintptr_t)15) + 16 * c;
-        if (g >= a + 2 * n_valid) continue;
-        uint8_t *dst = stage + stage_row_offset(row & 7, row >> 3) + 16 * c;
-        if (g >= lo && g + 16 <= hi) {
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(g) : "memory");
-        } else {   // the piece reaches past the tensor's first or last element: element by element
-#pragma unroll 1
-            for (int e = 0; e < 8; e++) {
-                const uintptr_t s = g + 2 * e;
-                if (s >= lo && s < hi) reinterpret_cast<uint16_t *>(dst)[e] = load_global(reinterpret_cast<const uint16_t *>(s));
-            }
-        }
-    }
-}
-
-// One row's segment (16 elements) of the staged tile; off: the row's offset into its first piece, in bytes.
-__device__ __forceinline__ void read_staged_segment(const uint8_t *src, uint32_t off, uint32_t out[8])
-{
-    uint32_t w[12];
-#pragma unroll
-    for (int q = 0; q < 3; q++) {
-        const uint4 v = reinterpret_cast<const uint4 *>(src)[q];
-        w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
-    }
-    const bool by2 = off & 8, by1 = off & 4;
-#pragma unroll
-    for (int k = 0; k < 10; k++) w[k] = by2 ? w[k + 2] : w[k];
-#pragma unroll
-    for (int k = 0; k < 9; k++) w[k] = by1 ? w[k + 1] : w[k];
-#pragma unroll
-    for (int k = 0; k < 8; k++) out[k] = __funnelshift_r(w[k], w[k + 1], 8 * (off & 2));
-}
 
 // The Philox blocks that the warp's 32 rows of 128 elements touch, nine per row: each lane draws the one in which its own segment
 // of each of its eight rows starts (`own`, 128 apart) and the ninth of the row that has its number (`ninth`).  A segment's bytes
@@ -333,20 +268,7 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
 #pragma unroll
-        for (int r = 0; r < 8; r++) {
-            if (row0 + r < p.rows && col0 < p.cols) {
-                const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(p.x + (row0 + r) * p.ld_x + bx * 128) & 15);
-                read_staged_segment(stage + stage_row_offset(r, rg) + 32 * (2 * t + ch), off, raw[r]);
-                if (col0 + 16 > p.cols) {   // what follows the row's last element belongs to the next row
-                    const int n = (int)(p.cols - col0);
-#pragma unroll
-                    for (int k = 0; k < 8; k++) raw[r][k] = 2 * k + 2 <= n ? raw[r][k] : 2 * k < n ? raw[r][k] & 0xFFFFu : 0u;
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 8; k++) raw[r][k] = 0u;
-            }
-        }
+        for (int r = 0; r < 8; r++) read_staged_row(p, tile_row0, bx * 128, stage, lane, r, raw[r]);
     } else {
 #pragma unroll
         for (int r = 0; r < 8; r++) load_segment(p, row0 + r, col0, raw[r]);
