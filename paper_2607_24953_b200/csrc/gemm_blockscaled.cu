@@ -208,6 +208,7 @@ struct GemmParams {
     int32_t b_rows_per_group;        // grouped rows: B row offset per group (forward)
     int32_t b_k_per_group;           // grouped rows: B contraction offset per group (dgrad)
     int32_t sort_groups;             // grouped contraction: take the groups longest first
+    int32_t warps_meet;              // grouped contraction: epilogue warps start a tile together
     uint32_t *status;
     // quantizing epilogue (EPI_QUANT): the output leaves as a 2D-block FP4 tensor instead of BF16/FP32
     uint8_t *q_rm, *q_t, *q_scale;
@@ -1824,15 +1825,24 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 // this wait spans a whole tile (every other one spans a few stages at most): its limit grows with the
                 // tile's contraction length, so that a very long contraction cannot run into it on a healthy run
                 const uint64_t tile_limit = wait_limit * (uint64_t)(1 + (t.k_len >> 12));
-                // One thread waits and the warps meet at a named barrier: eight lanes polling the barrier kept the shared-memory
-                // unit busy enough to slow every other role's waits (a probe took 475 cycles), 2-3 % of a dense product.
-                if (warp == 4 && lane == 0) {
+                // Every warp waits for itself (the suspending form: polling warps keep the shared-memory unit busy enough to slow every other
+                // role's waits).  With one thread waiting and the warps meeting at a named barrier behind it, us: 2048 x 4096 x 4096 quantized
+                // 20.5 / 19.7, 8192 x 2048 x 2048 19.3 / 19.4 / 16.8 -> 18.3 / 18.4 / 16.7, 1D activations there 20.2 / 19.5 -> 19.5 / 19.4, 16 x 16 blocks 23.2 / 23.1 /
+                // 20.0 -> 22.3 / 22.0 / 19.8, 16384 x 4096 x 4096 98.3 / 98.4 / 104.6 -> 94.7 / 94.7 / 103.8.  Weight gradients of short groups, bound by
+                // their writes, lose when warps drift apart (36352 rows in 128 groups, 1408 x 2048, 271 -> 316; 16640 in 128, 512 x 2048 99 ->
+                // 113), so there they still meet.
+                if (kGrouped && p.warps_meet) {
+                    if (warp == 4 && lane == 0) {
+                        ok = mbar_wait(bar_acc_full, acc_phase, abort_flag, p.status, tile_limit, 0x404u);
+                        acc_seen[acc_phase] = ok ? 1u : 0u;   // one word per phase: a warp is at most one tile behind
+                    }
+                    __syncwarp();
+                    asm volatile("bar.sync 15, 256;" ::: "memory");
+                    ok = acc_seen[acc_phase] != 0u;
+                } else {
                     ok = mbar_wait(bar_acc_full, acc_phase, abort_flag, p.status, tile_limit, 0x404u);
-                    acc_seen[acc_phase] = ok ? 1u : 0u;   // one word per phase: a warp is at most one tile behind
+                    ok = __all_sync(0xFFFFFFFFu, ok);
                 }
-                __syncwarp();
-                asm volatile("bar.sync 15, 256;" ::: "memory");
-                ok = acc_seen[acc_phase] != 0u;
                 TRACE_ADD(c_wait, tt);
                 if (lane == 0) TRACE_EV(7, 16 * ev_t + 2 * (warp - 4));
                 if (!ok) break;
@@ -2186,6 +2196,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     // below the line 65536 x 256 x 512 in 128 38 / 41, 131072 x 256 x 512 in 256 65-69 / 76, 4096 x 128 x 256 in 256 12 / 16.
     p.sort_groups = p.mode == MODE_GROUPED_K && p.n_groups <= kMaxGroupsSorted && p.K >= 512 * (int64_t)p.n_groups &&
                     2 * n_stages >= (int64_t)p.n_groups * slots;
+    p.warps_meet = p.mode == MODE_GROUPED_K && p.K < 512 * (int64_t)p.n_groups;   // two stages a group on average
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(kThreads);
