@@ -14,7 +14,7 @@
 //   warp 1      MMA issuer: stays converged, one elected lane issues per stage 6 tcgen05.cp (scale images -> TMEM),
 //               4 tcgen05.mma and the tcgen05.commit that frees the slot; in the second CTA of a pair it reports
 //               that CTA's per-row scale images to the leader
-//   warp 2      dense FP4 and MXFP8 pairs: watcher, polls the slots' "full" barriers (several at a time), the scale images
+//   warp 2      MXFP8 and long dense FP4 products on pairs: watcher, polls the slots' "full" barriers (several at a time), the scale images
 //               and the accumulator's "empty" barrier and meets the MMA warp at a named barrier per stage (elsewhere the
 //               MMA warp looks for itself); per-row FP4 kinds: second scale image builder
 //   warp 3      scale image builder: per unit of 16 stages (4 or 2 with per-row images) loads the scale bytes and writes the
@@ -129,6 +129,7 @@ struct Cfg {
 // few experts they belong to stay in L2 for the whole sweep over the columns (expert layer, 139520 rows, one group of all
 // row tiles -> groups of 16: 768 x 2048 fwd/dgrad 142/207 -> 126/166 us, 2048 x 768 199/144 -> 158/128; 8 and 32 within 2 %).
 constexpr int kRasterM = 16;
+constexpr int kShortStages = 48;   // a short product: up to so many ring stages per CTA or pair (launch_gemm, launch_gemm_impl)
 constexpr int kThreads = 384;
 constexpr int kTmemCols = 512;
 constexpr int kTmemSfBase = 256;
@@ -2217,7 +2218,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
         attr[0].val.clusterDim.z = 1;
         cfg.numAttrs = 1;
     }
-    if (n_stages <= 48 * (int64_t)slots && !(CTAS == 1 && capturing(cfg.stream))) {
+    if (n_stages <= kShortStages * (int64_t)slots && !(CTAS == 1 && capturing(cfg.stream))) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     }
@@ -2265,12 +2266,12 @@ static fp4q_status launch_gemm(const Operand &A, const Operand &B, GemmParams &p
     // output rows of a tile, and grouped rows where every group starts on a multiple of 256 or where paired rows pay.
     // FP4Q_CTA_PAIRS=0 in the environment (read once, before the first GEMM call) selects the one-CTA kernel instead.
     static const bool use_pairs = [] { const char *e = getenv("FP4Q_CTA_PAIRS"); return !(e && e[0] == '0'); }();
-    // The watcher pays in the dense FP4 and MXFP8 products on pairs (16384 x 4096 x 4096, with and without: FP4 weight gradient
-    // 98.4 and 102.7 us, forward 100.7 both; MXFP8 forward 213 and 218 us, weight gradient 228 and 236 us).  Everything else is
-    // faster without it: the short contractions of grouped products (expert weight gradients 222 and 225 us without, 228
-    // and 230 us with), the quantizing epilogue, whose warps it competes with (113 and 116 us), and the per-row FP4
-    // kinds, where its warp builds scale images instead.
-    constexpr bool kWatchDense = KIND == KIND_MXF4 || KIND == KIND_MXF8;
+    // The watcher pays in dense FP4 and MXFP8 products on pairs that last: with and without, 16384 x 4096 x 4096 FP4 102.6 / 103.5 / 98.0 and
+    // 103.9 / 104.5 / 101.3 us, MXFP8 199.7 and 207.0.  FP4 products of up to 48 stages a pair are faster without it (2048 x 2048 x 2048 8.5 / 8.6 / 9.6
+    // and 8.1 / 8.3 / 9.3, 512 x 1024 x 1024 6.8 / 6.6 / 7.2 and 6.5 / 6.3 / 7.0, 3000 x 3000 x 3000 16.8 / 16.9 / 18.5 and 16.5 / 16.7 / 18.2; from 55 stages on
+    // between -1.5 and +1.4 %, from 80 on slower), MXFP8 ones are level.  Everything else has none: the short contractions of grouped
+    // products (expert weight gradients 222 and 225 us without, 228 and 230 us with), the quantizing epilogue, whose warps it competes
+    // with (113 and 116 us), and the per-row FP4 kinds, where its warp builds scale images instead.
     if constexpr (KIND == KIND_MXF4) {
         if (p.mode != MODE_DENSE) {
             if (use_pairs && p.M > BM && p.mode == MODE_GROUPED_ROWS && !p.rows_pair_aligned && pairs_pay(p)) p.mode = MODE_PAIRED_ROWS;
@@ -2279,7 +2280,14 @@ static fp4q_status launch_gemm(const Operand &A, const Operand &B, GemmParams &p
             return launch_gemm_impl<KIND, 1, EPI_STORE, false, GROUPS_ANY>(A, B, p, stream);
         }
     }
-    if (use_pairs && p.M > BM) return launch_gemm_impl<KIND, 2, EPI_STORE, kWatchDense>(A, B, p, stream);
+    if (use_pairs && p.M > BM) {
+        if constexpr (KIND == KIND_MXF4) {
+            const int dev = current_device();
+            const int64_t pairs = dev < 0 ? 74 : sm_count(dev) / 2;
+            if (ceil_div(p.M, 2 * BM) * p.n_tiles * ceil_div(p.K, 256) <= kShortStages * pairs) return launch_gemm_impl<KIND, 2, EPI_STORE, false>(A, B, p, stream);
+        }
+        return launch_gemm_impl<KIND, 2, EPI_STORE, KIND == KIND_MXF4 || KIND == KIND_MXF8>(A, B, p, stream);
+    }
     return launch_gemm_impl<KIND, 1, EPI_STORE, false>(A, B, p, stream);
 }
 
