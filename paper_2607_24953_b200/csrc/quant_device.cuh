@@ -70,12 +70,22 @@ __device__ __forceinline__ float inv_scale_f16_aligned(int code)
 // 2^-e = 2^(127-code): always a normal FP32 for code in [0, 253].
 __device__ __forceinline__ float inv_scale(int code) { return __uint_as_float((uint32_t)(254 - code) << 23); }
 
-// Four FP32 -> four E2M1 nibbles (e0 in bits 3..0), stochastic rounding with the hardware's byte routing.
-__device__ __forceinline__ uint32_t cvt_rs_e2m1x4(float e3, float e2, float e1, float e0, uint32_t rbits)
+// Two pairs of FP32 -> E2M1 in nibbles 0, 2 and, of the second pair, 4, 6 (the others are zero), stochastic rounding with the hardware's byte routing.
+__device__ __forceinline__ uint32_t cvt_rs_e2m1x4x2(float d2, float d0, uint32_t rd, float c2, float c0, uint32_t rc)
 {
-    uint16_t d;
-    asm("cvt.rs.satfinite.e2m1x4.f32 %0, {%1, %2, %3, %4}, %5;" : "=h"(d) : "f"(e3), "f"(e2), "f"(e1), "f"(e0), "r"(rbits));
-    return d;
+    uint32_t w;
+    asm("{ .reg .b16 c, d; cvt.rs.satfinite.e2m1x4.f32 c, {%7, %1, %7, %2}, %3; cvt.rs.satfinite.e2m1x4.f32 d, {%7, %4, %7, %5}, %6; mov.b32 %0, {c, d}; }"
+        : "=r"(w) : "f"(c2), "f"(c0), "r"(rc), "f"(d2), "f"(d0), "r"(rd), "f"(0.0f));
+    return w;
+}
+// Eight FP32 -> eight E2M1 nibbles (v[0] in bits 3..0), round to nearest even.
+__device__ __forceinline__ uint32_t cvt_rn_e2m1x8(const float (&v)[8])
+{
+    uint32_t w;
+    asm("{ .reg .b8 a, b, c, d; cvt.rn.satfinite.e2m1x2.f32 a, %2, %1; cvt.rn.satfinite.e2m1x2.f32 b, %4, %3; cvt.rn.satfinite.e2m1x2.f32 c, %6, %5; "
+        "cvt.rn.satfinite.e2m1x2.f32 d, %8, %7; mov.b32 %0, {a, b, c, d}; }"
+        : "=r"(w) : "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]));
+    return w;
 }
 // Two FP32 -> two E2M1 nibbles (lo in bits 3..0), round to nearest even.
 __device__ __forceinline__ uint32_t cvt_rn_e2m1x2(float hi, float lo)
@@ -117,24 +127,21 @@ __device__ __forceinline__ void round_segment(const uint32_t raw[8], float inv, 
     const uint32_t inv2 = __byte_perm(__float_as_uint(inv), 0u, 0x3232);
 #pragma unroll
     for (int g = 0; g < 2; g++) {
-        uint32_t half[2];
+        float v[8];
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int q = 2 * g + h;                       // elements 4q .. 4q+3
-            const uint32_t w0 = scale_pair(raw[2 * q], inv2), w1 = scale_pair(raw[2 * q + 1], inv2);
-            const float v0 = __uint_as_float(w0 << 16), v1 = __uint_as_float(w0 & 0xFFFF0000u);
-            const float v2 = __uint_as_float(w1 << 16), v3 = __uint_as_float(w1 & 0xFFFF0000u);
-            if (MODE == FP4Q_ROUND_STOCHASTIC) {
-                // random bytes r0..r3 of the four elements; first convert: elements 0 and 2 (nibbles 0, 2),
-                // second convert: elements 1 and 3, merged one nibble higher
-                const uint32_t even = cvt_rs_e2m1x4(0.0f, v2, 0.0f, v0, __byte_perm(R[q], 0u, 0x2044));
-                const uint32_t odd = cvt_rs_e2m1x4(0.0f, v3, 0.0f, v1, __byte_perm(R[q], 0u, 0x3144));
-                half[h] = even | (odd << 4);
-            } else {
-                half[h] = cvt_rn_e2m1x2(v1, v0) | (cvt_rn_e2m1x2(v3, v2) << 8);
-            }
+        for (int k = 0; k < 4; k++) {
+            const uint32_t w = scale_pair(raw[4 * g + k], inv2);
+            v[2 * k] = __uint_as_float(w << 16);
+            v[2 * k + 1] = __uint_as_float(w & 0xFFFF0000u);
         }
-        W[g] = half[0] | (half[1] << 16);
+        if (MODE == FP4Q_ROUND_STOCHASTIC) {
+            // random bytes r0..r3 of four elements: elements 0 and 2 (nibbles 0, 2) and elements 1 and 3, merged one nibble higher
+            const uint32_t even = cvt_rs_e2m1x4x2(v[6], v[4], __byte_perm(R[2 * g + 1], 0u, 0x2044), v[2], v[0], __byte_perm(R[2 * g], 0u, 0x2044));
+            const uint32_t odd = cvt_rs_e2m1x4x2(v[7], v[5], __byte_perm(R[2 * g + 1], 0u, 0x3144), v[3], v[1], __byte_perm(R[2 * g], 0u, 0x3144));
+            W[g] = even + (odd << 4);
+        } else {
+            W[g] = cvt_rn_e2m1x8(v);
+        }
     }
 }
 
