@@ -20,14 +20,6 @@ struct Mxfp8QuantParams {
     int x_vec_ok;
 };
 
-// {hi, lo} -> two E4M3 bytes (hi in bits 15..8), round to nearest even, saturating to +-448.
-__device__ __forceinline__ uint32_t cvt_rn_e4m3x2(float hi, float lo)
-{
-    uint16_t d;
-    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(d) : "f"(hi), "f"(lo));
-    return d;
-}
-
 __global__ void __launch_bounds__(256) mxfp8_quantize1d_kernel(const __grid_constant__ Mxfp8QuantParams p)
 {
     wait_for_predecessor();
@@ -93,8 +85,7 @@ __global__ void __launch_bounds__(256) mxfp8_quantize1d_kernel(const __grid_cons
 #pragma unroll
     for (int w = 0; w < 8; w++) {
         const uint32_t w0 = scale_pair(raw[2 * w], inv2), w1 = scale_pair(raw[2 * w + 1], inv2);
-        out[w] = cvt_rn_e4m3x2(__uint_as_float(w0 & 0xFFFF0000u), __uint_as_float(w0 << 16)) |
-                 (cvt_rn_e4m3x2(__uint_as_float(w1 & 0xFFFF0000u), __uint_as_float(w1 << 16)) << 16);
+        out[w] = cvt_rn_e4m3x4(__uint_as_float(w1 & 0xFFFF0000u), __uint_as_float(w1 << 16), __uint_as_float(w0 & 0xFFFF0000u), __uint_as_float(w0 << 16));
     }
     uint4 *dst = reinterpret_cast<uint4 *>(p.q + i * p.ld_q + j0);
     dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
@@ -165,7 +156,7 @@ __global__ void __launch_bounds__(128) mxfp8_quantize1d_t_kernel(const __grid_co
     uint32_t A[8], B[8];   // the two columns' 32 payload bytes
 #pragma unroll
     for (int w = 0; w < 8; w++) {
-        uint32_t a = 0, b = 0;
+        float va[4], vb[4];
 #pragma unroll
         for (int e = 0; e < 2; e++) {
             const uint32_t w0 = raw[4 * w + 2 * e], w1 = raw[4 * w + 2 * e + 1];
@@ -176,11 +167,11 @@ __global__ void __launch_bounds__(128) mxfp8_quantize1d_t_kernel(const __grid_co
                 if ((lo1 & 0x7FFFFFFFu) > 0x7F800000u) lo1 = 0u;
                 if ((hi1 & 0x7FFFFFFFu) > 0x7F800000u) hi1 = 0u;
             }
-            a |= cvt_rn_e4m3x2(__uint_as_float(lo1) * inv[0], __uint_as_float(lo0) * inv[0]) << (16 * e);
-            b |= cvt_rn_e4m3x2(__uint_as_float(hi1) * inv[1], __uint_as_float(hi0) * inv[1]) << (16 * e);
+            va[2 * e] = __uint_as_float(lo0) * inv[0]; va[2 * e + 1] = __uint_as_float(lo1) * inv[0];
+            vb[2 * e] = __uint_as_float(hi0) * inv[1]; vb[2 * e + 1] = __uint_as_float(hi1) * inv[1];
         }
-        A[w] = a;
-        B[w] = b;
+        A[w] = cvt_rn_e4m3x4(va[3], va[2], va[1], va[0]);
+        B[w] = cvt_rn_e4m3x4(vb[3], vb[2], vb[1], vb[0]);
     }
     uint8_t *dst = p.q + c0 * p.ld_q + i0;
     reinterpret_cast<uint4 *>(dst)[0] = make_uint4(A[0], A[1], A[2], A[3]);
@@ -285,16 +276,10 @@ __global__ void __launch_bounds__(128, 4) mxfp8_quantize1d_t_tile_kernel(const _
         uint32_t w[2];
 #pragma unroll
         for (int h = 0; h < 2; h++) {
-            uint32_t acc = 0;
+            float v[4];
 #pragma unroll
-            for (int e = 0; e < 2; e++) {
-                const int r = 4 * h + 2 * e;
-                const uint32_t w0 = raw[r][c >> 1], w1 = raw[r + 1][c >> 1];
-                const float v0 = __uint_as_float((c & 1) ? (w0 & 0xFFFF0000u) : (w0 << 16));
-                const float v1 = __uint_as_float((c & 1) ? (w1 & 0xFFFF0000u) : (w1 << 16));
-                acc |= cvt_rn_e4m3x2(v1, v0) << (16 * e);
-            }
-            w[h] = acc;
+            for (int e = 0; e < 4; e++) v[e] = __uint_as_float((c & 1) ? (raw[4 * h + e][c >> 1] & 0xFFFF0000u) : (raw[4 * h + e][c >> 1] << 16));
+            w[h] = cvt_rn_e4m3x4(v[3], v[2], v[1], v[0]);
         }
         const int col_local = 32 * t + 16 * ch + c;
         const int chunk = (warp * 2 + (rg >> 1)) ^ ((col_local >> 4) & 7);

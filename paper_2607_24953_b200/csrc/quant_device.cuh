@@ -87,12 +87,14 @@ __device__ __forceinline__ uint32_t cvt_rn_e2m1x8(const float (&v)[8])
         : "=r"(w) : "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]));
     return w;
 }
-// Two FP32 -> two E2M1 nibbles (lo in bits 3..0), round to nearest even.
-__device__ __forceinline__ uint32_t cvt_rn_e2m1x2(float hi, float lo)
+
+// Four FP32 -> four E4M3 bytes (v0 in bits 7..0), round to nearest even, saturating to +-448.
+__device__ __forceinline__ uint32_t cvt_rn_e4m3x4(float v3, float v2, float v1, float v0)
 {
-    uint16_t d;
-    asm("{ .reg .b8 t; cvt.rn.satfinite.e2m1x2.f32 t, %1, %2; cvt.u16.u8 %0, t; }" : "=h"(d) : "f"(hi), "f"(lo));
-    return d;
+    uint32_t w;
+    asm("{ .reg .b16 a, b; cvt.rn.satfinite.e4m3x2.f32 a, %2, %1; cvt.rn.satfinite.e4m3x2.f32 b, %4, %3; mov.b32 %0, {a, b}; }"
+        : "=r"(w) : "f"(v0), "f"(v1), "f"(v2), "f"(v3));
+    return w;
 }
 
 // One element, scalar: used for blocks that contain non-finite values.

@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(128) quantize1d_t_kernel(const __grid_constant
     uint32_t A[4], B[4];   // the two columns' 32 nibbles
 #pragma unroll
     for (int g = 0; g < 4; g++) {
-        uint32_t a = 0, b = 0;
+        float va[8], vb[8];
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             uint32_t w0 = raw[8 * g + 2 * e], w1 = raw[8 * g + 2 * e + 1];
@@ -170,11 +170,11 @@ __global__ void __launch_bounds__(128) quantize1d_t_kernel(const __grid_constant
                 if ((lo1 & 0x7FFFFFFFu) > 0x7F800000u) lo1 = 0u;
                 if ((hi1 & 0x7FFFFFFFu) > 0x7F800000u) hi1 = 0u;
             }
-            a |= cvt_rn_e2m1x2(__uint_as_float(lo1) * inv0, __uint_as_float(lo0) * inv0) << (8 * e);
-            b |= cvt_rn_e2m1x2(__uint_as_float(hi1) * inv1, __uint_as_float(hi0) * inv1) << (8 * e);
+            va[2 * e] = __uint_as_float(lo0) * inv0; va[2 * e + 1] = __uint_as_float(lo1) * inv0;
+            vb[2 * e] = __uint_as_float(hi0) * inv1; vb[2 * e + 1] = __uint_as_float(hi1) * inv1;
         }
-        A[g] = a;
-        B[g] = b;
+        A[g] = cvt_rn_e2m1x8(va);
+        B[g] = cvt_rn_e2m1x8(vb);
     }
     *reinterpret_cast<uint4 *>(p.q + c0 * p.ld_q + (i0 >> 1)) = make_uint4(A[0], A[1], A[2], A[3]);
     p.scale[c0 * p.ld_s + rb] = (uint8_t)code0;
@@ -292,13 +292,10 @@ __global__ void __launch_bounds__(128, 4) quantize1d_t_tile_kernel(const __grid_
     for (int c = 0; c < 16; c++) {
         uint32_t word = 0;
         if (!careful) {
+            float v[8];
 #pragma unroll
-            for (int e = 0; e < 4; e++) {
-                const uint32_t w0 = raw[2 * e][c >> 1], w1 = raw[2 * e + 1][c >> 1];
-                const float v0 = __uint_as_float((c & 1) ? (w0 & 0xFFFF0000u) : (w0 << 16));
-                const float v1 = __uint_as_float((c & 1) ? (w1 & 0xFFFF0000u) : (w1 << 16));
-                word |= cvt_rn_e2m1x2(v1, v0) << (8 * e);
-            }
+            for (int r = 0; r < 8; r++) v[r] = __uint_as_float((c & 1) ? (raw[r][c >> 1] & 0xFFFF0000u) : (raw[r][c >> 1] << 16));
+            word = cvt_rn_e2m1x8(v);
         } else {   // rare: kept small and out of the hot loop's instruction footprint
             uint32_t h[4];
 #pragma unroll

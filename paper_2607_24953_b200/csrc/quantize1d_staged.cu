@@ -16,12 +16,6 @@
 
 namespace fp4q {
 
-__device__ __forceinline__ uint32_t cvt_rn_e4m3x2(float hi, float lo)
-{
-    uint16_t d;
-    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(d) : "f"(hi), "f"(lo));
-    return d;
-}
 template <bool FP8>
 __device__ __forceinline__ int scale_code(uint32_t mbits) { return FP8 ? e4m3_scale_code(mbits) : scale_code_from_max(mbits); }
 // Packed |.| maximum with NaN propagation: a non-finite entry shows in the result.
@@ -79,12 +73,15 @@ __device__ __forceinline__ void quantize_rows(const Staged1dParams &p, int64_t t
             if (FP8) {
                 uint32_t out[4];
 #pragma unroll
-                for (int w = 0; w < 4; w++) out[w] = cvt_rn_e4m3x2(high(v[2 * w]), low(v[2 * w])) | cvt_rn_e4m3x2(high(v[2 * w + 1]), low(v[2 * w + 1])) << 16;
+                for (int w = 0; w < 4; w++) out[w] = cvt_rn_e4m3x4(high(v[2 * w + 1]), low(v[2 * w + 1]), high(v[2 * w]), low(v[2 * w]));
                 *reinterpret_cast<uint4 *>(dst + col0) = make_uint4(out[0], out[1], out[2], out[3]);
             } else {
-                uint32_t out[2] = {0u, 0u};
+                uint32_t out[2];
 #pragma unroll
-                for (int k = 0; k < 8; k++) out[k >> 2] |= cvt_rn_e2m1x2(high(v[k]), low(v[k])) << (8 * (k & 3));
+                for (int w = 0; w < 2; w++) {
+                    const float f[8] = {low(v[4 * w]), high(v[4 * w]), low(v[4 * w + 1]), high(v[4 * w + 1]), low(v[4 * w + 2]), high(v[4 * w + 2]), low(v[4 * w + 3]), high(v[4 * w + 3])};
+                    out[w] = cvt_rn_e2m1x8(f);
+                }
                 *reinterpret_cast<uint2 *>(dst + (col0 >> 1)) = make_uint2(out[0], out[1]);
             }
             if (ch == 0) p.scale[row * p.ld_s + (col0 >> 5)] = (uint8_t)code;
@@ -158,21 +155,19 @@ __global__ void __launch_bounds__(128, 4) quantize1d_t_staged_kernel(const __gri
         }
     }
     __syncthreads();   // every warp has read its rows
-    // One convert takes the same column of two consecutive rows.  A column's codes are 64 or 128 bytes of staging, in 16-byte chunks XORed by
+    // A column's codes are 64 or 128 bytes of staging, in 16-byte chunks XORed by
     // the column's group so that a warp's stores spread over the banks.
 #pragma unroll
     for (int c = 0; c < 16; c++) {
         const int col_local = 32 * t + 16 * ch + c;
-        auto pair = [&](int r) {   // rows r + 1 and r
-            const uint32_t w0 = raw[r][c >> 1], w1 = raw[r + 1][c >> 1];
-            const float v0 = (c & 1) ? high(w0) : low(w0), v1 = (c & 1) ? high(w1) : low(w1);
-            return FP8 ? cvt_rn_e4m3x2(v1, v0) : cvt_rn_e2m1x2(v1, v0);
-        };
+        float v[8];
+#pragma unroll
+        for (int r = 0; r < 8; r++) v[r] = (c & 1) ? high(raw[r][c >> 1]) : low(raw[r][c >> 1]);
         if (FP8) {
             const int chunk = (warp * 2 + (rg >> 1)) ^ ((col_local >> 4) & 7);
-            reinterpret_cast<uint2 *>(stage)[(col_local * 8 + chunk) * 2 + (rg & 1)] = make_uint2(pair(0) | pair(2) << 16, pair(4) | pair(6) << 16);
+            reinterpret_cast<uint2 *>(stage)[(col_local * 8 + chunk) * 2 + (rg & 1)] = make_uint2(cvt_rn_e4m3x4(v[3], v[2], v[1], v[0]), cvt_rn_e4m3x4(v[7], v[6], v[5], v[4]));
         } else {
-            reinterpret_cast<uint32_t *>(stage)[col_local * 16 + (((warp ^ t) << 2) | rg)] = pair(0) | pair(2) << 8 | pair(4) << 16 | pair(6) << 24;
+            reinterpret_cast<uint32_t *>(stage)[col_local * 16 + (((warp ^ t) << 2) | rg)] = cvt_rn_e2m1x8(v);
         }
     }
     __syncthreads();
