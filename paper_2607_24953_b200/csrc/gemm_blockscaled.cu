@@ -265,10 +265,15 @@ __device__ __forceinline__ bool elect_one()
     asm volatile("{\n .reg .pred P;\n elect.sync _|P, 0xFFFFFFFF;\n selp.b32 %0, 1, 0, P;\n}" : "=r"(p));
     return p != 0;
 }
-// Named barrier on which the MMA warp and the warp that watches a ring slot for it meet (64 threads).  Both sides
-// use the waiting form: with a non-waiting arrival a watcher that releases stages unseen (after a timeout) could
-// complete a barrier phase on its own and leave the MMA warp without a partner.
-__device__ __forceinline__ void named_sync(uint32_t id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+// Named barrier on which the MMA warp and the warp that watches a ring slot for it meet (64 threads).  Both sides use the waiting
+// form: with a non-waiting arrival a watcher that has given up, and only counts the remaining stages, could complete a barrier phase on
+// its own and leave the MMA warp without a partner.  It says so with its arrival; returns whether the stage may be used.
+__device__ __forceinline__ bool named_meet(uint32_t id, bool usable)
+{
+    uint32_t r;
+    asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %2, 0;\n bar.red.and.pred q, %1, 64, p;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(r) : "r"(id), "r"((uint32_t)usable) : "memory");
+    return r != 0u;
+}
 
 // Bounded wait.  Returns false when the limit ran out (the timeout is then recorded) or when another
 // role of this CTA has already given up, which it looks for after every suspension and after every 256th probe.  Every poll
@@ -1413,7 +1418,11 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         start_sync<CTAS, kBuilders>();
         tcgen05_fence_after();
         const uint32_t tmem_base = *tmem_base_slot;
-        bool mma_ok = true, ready = false;   // !WATCH: this warp's waits have not run out; the next stage has been seen complete
+        // mma_ok: no wait for a stage has run out.  Afterwards the remaining stages are issued unseen, but their slots are not given back: the
+        // producers would announce a slot's next bytes on a barrier that still waits for the last ones, which is undefined.  (One
+        // predicate on that commit and the watcher's word with its arrival: within 0.3 % of a product; nothing issued at all, 0.5 to 1 %.)
+        bool mma_ok = true;
+        bool ready = false;   // !WATCH: the next stage has been seen complete
         BufRing ring;   // image buffer of the current unit
         const bool issuer = elect_one();
         int ev_j = 0;
@@ -1427,7 +1436,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             TRACE_ADD(c_acc, tt);
             for (int it = 0; it < n_it; it++) {
                 if (WATCH) {
-                    named_sync(1 + stage);   // the watcher has seen the operands and both scale images of this stage
+                    mma_ok = named_meet(1 + stage, true);   // the watcher has seen the operands and both scale images of this stage
                 } else {
                     if (it == 0) {
                         if (mma_ok) mma_ok = mbar_wait_impl<0>(bar_acc_empty, acc_empty_phase ^ 1u, abort_flag, p.status, wait_limit, 0x200u);
@@ -1498,7 +1507,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                                                                  sf_tmem + 8 + 8 * chunk, (it > 0 || i > 0) ? 1u : 0u);
                         }
                     }
-                    tcgen05_commit<CTAS>(bar_empty + 8 * stage);
+                    if (mma_ok) tcgen05_commit<CTAS>(bar_empty + 8 * stage);
                     if (it == n_it - 1) tcgen05_commit<CTAS>(bar_acc_full);
                     if ((it & (kUnitStages - 1)) == kUnitStages - 1 || it == n_it - 1)
                         tcgen05_commit<CTAS>(bar_cache_empty + 8 * ring.buf);   // the unit's images have been copied
@@ -1523,14 +1532,16 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             __syncwarp();
         }
         if (leader && *abort_flag) {
-            // Some role gave up: the watcher then releases every remaining stage unseen (or this warp has stopped waiting), and
-            // this warp has run through them.  Wait (bounded) until the tensor pipe is idle before tensor memory is freed.
+            // Some role gave up, and this warp has run through the remaining stages.  The second CTA, whose producer waits for slots that
+            // are not given back, is told; and before tensor memory is freed the tensor pipe is idle (a bounded wait).
+            if (CTAS == 2 && lane == 0)
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(smem_u32(const_cast<const uint32_t *>(abort_flag)), 1)), "r"(1u) : "memory");
             if (issuer) tcgen05_commit<CTAS>(bar_drain);
             __syncwarp();
             if (lane == 0) mbar_drain(bar_drain);
             __syncwarp();
-            // After an abort the stages were consumed without waiting for their operands, so loads of either CTA may
-            // still be on their way: hold the pair (the other roles wait at the final barrier) until they have landed.
+            // Loads of either CTA may still be on their way: hold the pair (the other roles wait at the final barrier) until they
+            // have landed.
             for (int i = 0; i < 200; i++) __nanosleep(1000);
         }
         if (lane == 0) { TRACE_OUT(p, 2, c_acc); TRACE_OUT(p, 3, c_sync); TRACE_OUT(p, 4, c_issue); }
@@ -1693,9 +1704,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         // Follows the stream of stages (one CTA, or the leader of a pair; the second CTA's warp idles).  For each
         // it waits for the ring slot's "full" barrier (the operand bytes of both CTAs), at the first stage of a
         // unit for the unit's scale images (of both CTAs), and at the first stage of a tile for the accumulator
-        // to be drained; then it meets the MMA warp at the slot's named barrier.  After a timeout every remaining
-        // stage is released unseen, so that the MMA warp, which cannot time out on a named barrier, always runs
-        // to its end.
+        // to be drained; then it meets the MMA warp at the slot's named barrier.  After a timeout they meet at every remaining
+        // stage all the same, so that the MMA warp, which cannot time out on a named barrier, always runs to its end.
         StageIter sg;
         sg.init(p, first_tile, tile_step, rank, kStageElems);
         start_sync<CTAS, kBuilders>();
@@ -1803,7 +1813,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             TRACE_ADD(c_poll, tt);
             if (lane == 0) TRACE_EV(6, ev_j);
             ev_j++;
-            named_sync(1 + stage);   // rendezvous: the MMA warp is at most one stage behind
+            named_meet(1 + stage, ok);   // rendezvous: the MMA warp is at most one stage behind
             TRACE_ADD(c_meet, tt);
             if (sg.it == 0) acc_phase ^= 1u;
             if ((sg.it & (kUnitStages - 1)) == kUnitStages - 1 || sg.it == sg.n_it - 1) ring.next(kImageBufs);

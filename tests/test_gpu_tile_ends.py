@@ -77,3 +77,25 @@ def test_paired_rows(E, rows):
         check_gemm(full[dt][1], dx, "dgrad")
     torch.cuda.synchronize()
     assert binding.fp4q_workspace_status(ws) == 0
+
+
+# 81 tiles of 43 and of 44 stages: both sides of the line (48 stages for each of 74 pairs) from which on a dense product runs with a
+# watcher between the loads and the MMAs; and that every role leaves there, too, when a load that it waits for never arrives
+@pytest.mark.parametrize("K", [43 * 256, 44 * 256])
+def test_short_and_long_products(K):
+    ws = binding.alloc_workspace("cuda")
+    qx, qw, qdy = operands((2304, K), (2304, K), (2304, 2304))
+    binding.fp4q_workspace_set_wait_limit(ws, 1 << 12)
+    binding.fp4q_debug_withhold_load(ws, 5)
+    binding.fp4q_gemm_fwd(qx, qw, ws=ws)
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 7
+    binding.fp4q_debug_withhold_load(ws, 0)
+    binding.fp4q_workspace_set_wait_limit(ws, 0)
+    rows = slice(5, None, 97)
+    x, w, dy = (dequant_from_gpu(q) for q in (qx, qw, qdy))
+    check_gemm(binding.fp4q_gemm_fwd(qx, qw, ws=ws)[rows], oracle.gemm_fwd(x[rows], w), "fwd")
+    check_gemm(binding.fp4q_gemm_dgrad(qdy, qw, ws=ws)[rows], oracle.gemm_dgrad(dy[rows], w), "dgrad")
+    check_gemm(binding.fp4q_gemm_wgrad(qdy, qx, ws=ws)[rows], oracle.gemm_wgrad(np.ascontiguousarray(dy[:, rows]), x), "wgrad")
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
