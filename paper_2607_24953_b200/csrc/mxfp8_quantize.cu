@@ -320,7 +320,7 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d(const void *x_bf16, int64_t rows, i
     const int64_t n_cta = ceil_div(total, 256);
     if (n_cta > 0x7FFFFFFF) return FP4Q_ERR_UNSUPPORTED;
     if (!p.x_vec_ok && rows * cols >= kStagedRowsFrom)
-        return launch_quantize1d_staged(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, true, false, static_cast<cudaStream_t>(stream));
+        return launch_quantize1d_staged<true>(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, false, static_cast<cudaStream_t>(stream));
     return launched(launch_dependent(mxfp8_quantize1d_kernel, dim3((unsigned)n_cta), 256, static_cast<cudaStream_t>(stream), p));
 }
 
@@ -348,6 +348,6 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d_t(const void *x_bf16, int64_t rows,
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;
     if (!p.x_vec_ok || rows * cols >= kStagedTransposeFrom)
-        return launch_quantize1d_staged(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, true, true, static_cast<cudaStream_t>(stream));
+        return launch_quantize1d_staged<true>(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, true, static_cast<cudaStream_t>(stream));
     return launched(launch_dependent(mxfp8_quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p));
 }

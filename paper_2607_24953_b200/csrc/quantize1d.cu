@@ -348,7 +348,7 @@ extern "C" fp4q_status fp4q_quantize1d(const void *x_bf16, int64_t rows, int64_t
     if (n_cta > 0x7FFFFFFF) return FP4Q_ERR_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!p.x_vec_ok && mode == FP4Q_ROUND_NEAREST && rows * cols >= kStagedRowsFrom)
-        return launch_quantize1d_staged(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, false, false, s);
+        return launch_quantize1d_staged<false>(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, false, s);
     return launched(launch_dependent(mode == FP4Q_ROUND_STOCHASTIC ? quantize1d_kernel<FP4Q_ROUND_STOCHASTIC> : quantize1d_kernel<FP4Q_ROUND_NEAREST>,
                                      dim3((unsigned)n_cta), 256, s, p));
 }
@@ -374,6 +374,6 @@ extern "C" fp4q_status fp4q_quantize1d_t(const void *x_bf16, int64_t rows, int64
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;
     if (!p.x_vec_ok || rows * cols >= kStagedTransposeFrom)
-        return launch_quantize1d_staged(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, false, true, static_cast<cudaStream_t>(stream));
+        return launch_quantize1d_staged<false>(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, true, static_cast<cudaStream_t>(stream));
     return launched(launch_dependent(quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p));
 }
