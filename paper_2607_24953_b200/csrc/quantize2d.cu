@@ -143,15 +143,16 @@ __device__ __forceinline__ void load_segment(const Quant2dParams &p, int64_t i, 
 // arithmetic.  Here a warp copies its 32 rows as aligned 16-byte pieces (17 cover 128 elements at any offset) into its own
 // staging rows with cp.async and draws the nine Philox blocks that each row's 128 elements touch, once per warp, while they are on
 // their way; each lane reads its segments back with three 128-bit shared loads a row and shifts them, and their random bytes, into
-// place.  Bound by instructions and by the phases of a CTA, which only other CTAs overlap: with the copies waited for first, every
-// piece checked against the tensor's ends and the random blocks drawn afterwards into the same rows, us, nearest / stochastic:
-// 4099 x 2731 13.0 / 18.0 -> 12.2 / 16.4 (5.1 at the measured copy bandwidth), 16384 x 2731 41.3 / 58.7 -> 34.6 / 46.0,
-// 9001 x 8191 65.0 / 89.0 -> 52.1 / 70.6, 300 x 777 6.1 / 7.8 -> 6.0 / 7.4.
+// place.  Bound by instructions (1537 and 2515 a warp with checks at every row, 714 and 1356 of the kernel for aligned rows) and by the
+// phases of a CTA, which only other CTAs overlap.  So no row is checked by itself: segments are read as they are staged, what lies
+// beyond the matrix is zeroed for all of a lane's rows at once where there is any, and only the stores ask.  us, nearest / stochastic, every row
+// checked and now: 4099 x 2731 11.4 / 15.5 -> 9.7 / 13.5 (5.1 at the measured copy bandwidth), 16384 x 2731 33.2 / 45.2 -> 28.9 / 39.7, 9001 x 8191
+// 50.7 / 70.0 -> 44.5 / 60.7, 300 x 777 5.5 / 6.9 -> 4.4 / 5.8, 7 x 7 4.4 / 5.9 -> 3.4 / 4.8.  (A body without checks for whole tiles beside the
+// checked one gains as much on large matrices but loses 2-11 % on small ones and ones of many edge tiles, whose SMs run both.)
 
 // The Philox blocks that the warp's 32 rows of 128 elements touch, nine per row: each lane draws the one in which its own segment
 // of each of its eight rows starts (`own`, 128 apart) and the ninth of the row that has its number (`ninth`).  A segment's bytes
-// run on into the block of its right neighbour, or into the ninth.  Warps without rows (in a tensor of 32 rows three of a CTA's four)
-// draw nothing: 32 x 1000001 84.3 -> 73.4 us, 4 x 65537 7.9 -> 6.8.  Loops that also stop at the last row cost whole tiles 1-2 %.
+// run on into the block of its right neighbour, or into the ninth.  Loops that also stop at the last row cost whole tiles 1-2 %.
 __device__ __forceinline__ void draw_row_blocks(const Quant2dParams &p, int64_t tile_row0, int64_t tile_col0, int rg, int seg, uint4 *own, uint4 *ninth, int lane)
 {
     if (tile_row0 >= p.rows) return;
@@ -223,7 +224,12 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
     const int64_t tile_row0 = by * 128 + warp * 32, tile_col0 = bx * 128 + t * 32;
     const int64_t row0 = tile_row0 + rg * 8, col0 = tile_col0 + ch * 16;
     const bool tile_exists = FAST || (tile_row0 < p.rows && tile_col0 < p.cols);
+    const int n_rows = FAST ? 8 : (int)max((int64_t)0, min((int64_t)8, p.rows - row0));   // of this lane's
 
+    // Staged tensors of few rows: warps without rows (in a tensor of 32 rows three of a CTA's four) only meet the others; us, nearest /
+    // stochastic, with everything done for them and now: 32 x 1000001 54.7 / 79.4 -> 42.5 / 56, 4 x 65537 6.6 / 8.6 -> 4.7 / 6.1; other sizes lose 1 %.
+    // And of one or two rows the other six are not rounded: 1 x 5001 stochastic 4.95 -> 4.37.
+    const bool idle = STAGED && tile_row0 >= p.rows, few = STAGED && p.rows <= 2;
     uint32_t raw[8][8];
     if (F32 && FAST) {
         const float *src = reinterpret_cast<const float *>(p.x) + row0 * p.ld_x + col0;
@@ -267,8 +273,11 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
             draw_row_blocks(p, tile_row0, bx * 128, rg, 2 * t + ch, rnd_stage + threadIdx.x, rnd_stage + 8 * 128 + 32 * warp, lane);
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
+        if (!idle) {
 #pragma unroll
-        for (int r = 0; r < 8; r++) read_staged_row(p, tile_row0, bx * 128, stage, lane, r, raw[r]);
+            for (int r = 0; r < 8; r++) read_staged_row_uncut(p, tile_row0, bx * 128, stage, lane, r, raw[r]);
+        }
+        cut_staged_rows(raw, n_rows, (int)max((int64_t)0, min((int64_t)16, p.cols - col0)));
     } else {
 #pragma unroll
         for (int r = 0; r < 8; r++) load_segment(p, row0 + r, col0, raw[r]);
@@ -361,19 +370,36 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
         p.scale[(tile_row0 >> 5) * p.ld_s + (tile_col0 >> 5)] = (uint8_t)code;
     }
 
+    const uint4 *next_block = rnd_stage + (2 * t + ch < 7 ? threadIdx.x + (ch ? 7 : 1) : 8 * 128 + 32 * warp + rg);
+    const int next_step = 2 * t + ch < 7 ? 128 : 4;
+    const uint32_t off0 = (uint32_t)row0 * (uint32_t)p.cols;   // a tile starts on a multiple of 128
+    auto staged_random = [&](int r, uint32_t R[4]) {
+        read_staged_random(rnd_stage[r * 128 + threadIdx.x], next_block[r * next_step], (off0 + r * (uint32_t)p.cols) & 15u, R);
+    };
     uint32_t W[8][2];
     uint8_t *dst_rm = p.q_rm + row0 * p.ld_rm + (col0 >> 1);
-    if (FAST && !nonfinite) {
-        // hot loop: no bounds checks, no path selection
+    if (idle) {   // nothing of it is written, transposed either
+    } else if ((FAST || STAGED) && !nonfinite) {
+        // hot loop: no path selection, and no bounds checks but at a staged row's store
+        const int n_store = tile_exists ? n_rows : 0;
 #pragma unroll
         for (int r = 0; r < 8; r++) {
+            if (STAGED && r == 2 && few) {
+#pragma unroll
+                for (int z = 2; z < 8; z++) W[z][0] = W[z][1] = 0u;
+                break;
+            }
             uint32_t R[4] = {0u, 0u, 0u, 0u};
             if (MODE == FP4Q_ROUND_STOCHASTIC) {
-                const uint4 v = rnd_stage[r * 128 + threadIdx.x];
-                R[0] = v.x; R[1] = v.y; R[2] = v.z; R[3] = v.w;
+                if (STAGED) {
+                    staged_random(r, R);
+                } else {
+                    const uint4 v = rnd_stage[r * 128 + threadIdx.x];
+                    R[0] = v.x; R[1] = v.y; R[2] = v.z; R[3] = v.w;
+                }
             }
             round_segment<MODE>(raw[r], inv, R, W[r]);
-            *reinterpret_cast<uint2 *>(dst_rm + r * p.ld_rm) = make_uint2(W[r][0], W[r][1]);
+            if (FAST || r < n_store) *reinterpret_cast<uint2 *>(dst_rm + r * p.ld_rm) = make_uint2(W[r][0], W[r][1]);
         }
     } else {
 #pragma unroll
@@ -386,10 +412,7 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
             uint32_t R[4] = {0u, 0u, 0u, 0u};
             if (MODE == FP4Q_ROUND_STOCHASTIC) {
                 if (STAGED) {
-                    const uint32_t off = ((uint32_t)i * (uint32_t)p.cols) & 15u;   // a tile starts on a multiple of 128
-                    const uint4 a = rnd_stage[r * 128 + threadIdx.x];
-                    const uint4 b = 2 * t + ch < 7 ? rnd_stage[r * 128 + threadIdx.x + (ch ? 7 : 1)] : rnd_stage[8 * 128 + 32 * warp + 4 * r + rg];
-                    read_staged_random(a, b, off, R);
+                    staged_random(r, R);
                 } else if (FAST || p.rng_aligned) {
                     const uint4 v = rnd_stage[r * 128 + threadIdx.x];
                     R[0] = v.x; R[1] = v.y; R[2] = v.z; R[3] = v.w;
@@ -415,6 +438,7 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
     // transposed payload: per lane two 8x8 nibble blocks -> 16 words (one per column, 8 rows each)
     uint32_t *stage = reinterpret_cast<uint32_t *>(qt_stage);
     if (STAGED) __syncthreads();   // every warp has read its rows
+    if (!idle)
 #pragma unroll
     for (int g = 0; g < 2; g++) {
         uint32_t a[8];

@@ -83,6 +83,26 @@ __device__ __forceinline__ void read_staged_segment(const uint8_t *src, uint32_t
     for (int k = 0; k < 8; k++) out[k] = __funnelshift_r(w[k], w[k + 1], 8 * (off & 2));
 }
 
+// Segment r of lane's eight as it is staged, without a look at the matrix's ends: cut_staged_rows does that for all eight at once.
+template <typename P>
+__device__ __forceinline__ void read_staged_row_uncut(const P &p, int64_t tile_row0, int64_t tile_col0, const uint8_t *stage, int lane, int r, uint32_t out[8])
+{
+    const int seg = 2 * (lane >> 3) + (lane & 1), rg = (lane >> 1) & 3;
+    const uint32_t a = (uint32_t)reinterpret_cast<uintptr_t>(p.x + tile_row0 * p.ld_x + tile_col0) + 16 * rg * (uint32_t)p.ld_x;
+    read_staged_segment(stage + stage_row_offset(r, rg) + 32 * seg, (a + 2 * r * (uint32_t)p.ld_x) & 15, out);
+}
+// Zeros in place of what lies beyond the matrix; n_rows (0 .. 8), n_cols (0 .. 16): what there is of this lane's.
+__device__ __forceinline__ void cut_staged_rows(uint32_t (&raw)[8][8], int n_rows, int n_cols)
+{
+    if (n_rows == 8 && n_cols == 16) return;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const uint32_t keep = 2 * k + 2 <= n_cols ? 0xFFFFFFFFu : 2 * k < n_cols ? 0xFFFFu : 0u;
+#pragma unroll
+        for (int r = 0; r < 8; r++) raw[r][k] = r < n_rows ? raw[r][k] & keep : 0u;
+    }
+}
+
 // Segment r of lane's eight (rows rg * 8 + r, columns 32 t + 16 ch .. + 15; t = lane / 8, rg = lane / 2 % 4, ch = lane % 2) of the staged tile;
 // what lies beyond the matrix reads as zero.
 template <typename P>
