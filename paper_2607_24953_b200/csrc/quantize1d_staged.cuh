@@ -7,7 +7,7 @@
 // memory, and code that runs once on an SM takes about ten cycles an instruction.  So the loop over a lane's rows is not unrolled where a row
 // is all that is needed (1999 x 2731 FP4 unrolled 8.2 us, rolled 7.1; reading rows twice to roll the other form's loop loses, 8.3 / 10.4).  us, FP4 /
 // MXFP8, element-wise loads before and now: 1999 x 2731 12.1 / 12.1 -> 7.2 / 7.1, 4099 x 5001 38.8 / 38.9 -> 14.9 / 14.8 (8.0 / 9.5 at the measured copy
-// bandwidth); transposed 11.3 / 12.9 -> 7.8 / 7.9, 23.4 / 32.4 -> 18.2 / 19.5.
+// bandwidth); transposed 11.3 / 12.9 -> 7.2 / 7.5, 23.4 / 32.4 -> 17.2 / 17.8 (7.5 / 7.7 and 17.9 / 19.0 with every row checked by itself).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -148,7 +148,8 @@ __global__ void __launch_bounds__(128, 4) quantize1d_t_staged_kernel(const __gri
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
 #pragma unroll
-    for (int r = 0; r < 8; r++) read_staged_row(p, tile_row0, bx * 128, stage + warp * kStageWarpBytes, lane, r, raw[r]);
+    for (int r = 0; r < 8; r++) read_staged_row_uncut(p, tile_row0, bx * 128, stage + warp * kStageWarpBytes, lane, r, raw[r]);
+    cut_staged_rows(raw, (int)max((int64_t)0, min((int64_t)8, p.rows - tile_row0 - 8 * rg)), (int)max((int64_t)0, min((int64_t)16, p.cols - bx * 128 - 32 * t - 16 * ch)));
     bool nonfinite = false;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
