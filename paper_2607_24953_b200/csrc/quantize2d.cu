@@ -524,13 +524,15 @@ __global__ void __launch_bounds__(128, 3) quantize2d_f32_kernel(const __grid_con
 typedef void (*Quant2dKernel)(const Quant2dParams);
 
 // Rows on vector boundaries and, with stochastic rounding, segments on Philox blocks are read directly: on 32-byte boundaries
-// by the check-free body, on 16-byte ones by the general body's 128-bit loads.  Staging costs those more than it gives
-// (nearest / stochastic, us, direct and staged: 4096 x 4096 in a pitch of 4104 14.7 / 18.1 and 16.8 / 22.9, 16384 x 4096 40.9 /
-// 54.7 and 55.8 / 80.1, 4099 x 2728 nearest 14.9 and 14.7).  Anything else is staged, except for the transposed index, whose
-// random bytes run down the columns.
+// by the check-free body, on 16-byte ones by the general body's 128-bit loads, where these reach the rows' ends.  us, nearest / stochastic,
+// direct and staged: 4096 x 4096 in a pitch of 4104 10.8 / 15.0 and 11.4 / 16.8, 2048 x 2048 in 2056 4.7 / 6.5 and 5.1 / 7.0, 16384 x 4096 40.5 / 54.2 and
+// 39.0 / 54.5; with a last segment that is not full, which the general body reads by elements: 4099 x 2728 nearest 11.9 and 9.9, 300 x 776 5.7 and
+// 4.4, 16 x 10008 5.9 and 3.9, 1 x 10008 2.9 and 3.3.  Anything else is staged, except for the transposed index, whose random bytes run down
+// the columns.
 static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr, int *smem)
 {
-    const bool staged = !(p.x_vec_ok && p.rng_aligned) && !(sr && (p.flags & FP4Q_INDEX_TRANSPOSED));
+    const bool direct = p.x_vec_ok && p.rng_aligned && (p.x_vec_ok == 2 || p.cols % 16 == 0 || p.rows <= 2);
+    const bool staged = !direct && !(sr && (p.flags & FP4Q_INDEX_TRANSPOSED));
     const int which = (p.flags & FP4Q_BLOCK_16) ? 1 : (p.flags & FP4Q_BLOCK_64) ? 2 : 0;
     static const Quant2dKernel kernels[2][2][3] = {
         {{quantize2d_kernel<FP4Q_ROUND_NEAREST>, quantize2d_kernel<FP4Q_ROUND_NEAREST, 16>, quantize2d_kernel<FP4Q_ROUND_NEAREST, 64>},

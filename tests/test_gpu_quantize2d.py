@@ -265,3 +265,17 @@ def test_rows_on_16_byte_boundaries(rows, cols, pitch, offset, mode, flags):
 def test_stochastic_bands_of_few_rows(rows, cols):
     g = torch.Generator(device="cuda").manual_seed(1000 * rows + cols)
     assert_matches_oracle(torch.randn(rows, cols, generator=g, device="cuda").to(torch.bfloat16), 1, seed=rows, tensor_id=cols)
+
+
+# Rows on 16-byte boundaries whose last segment is not full (staged from three rows on) and rows that start anywhere, with entries that
+# are not finite beside a matrix's ends: what is beyond them must not count
+@pytest.mark.parametrize("rows", [1, 2, 3, 130])
+@pytest.mark.parametrize("cols,pitch", [(120, 120), (136, 152), (1000, 1000), (127, 129)])
+@pytest.mark.parametrize("mode", MODES)
+def test_rows_that_end_inside_a_segment(rows, cols, pitch, mode):
+    g = torch.Generator(device="cuda").manual_seed(rows * cols)
+    x = torch.full((rows + 1, pitch), float("inf"), device="cuda", dtype=torch.bfloat16)[:rows, :cols]
+    x.copy_(torch.randn(rows, cols, generator=g, device="cuda"))
+    x[rows - 1, cols - 1] = float("nan")
+    x[0, 0] = float("-inf")
+    assert_matches_oracle(x, mode, seed=rows, tensor_id=cols)
