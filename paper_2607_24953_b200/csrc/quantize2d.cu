@@ -213,7 +213,12 @@ __device__ __forceinline__ void segment_random_bytes(const Quant2dParams &p, int
 // `xchg`.  With BLK = 64 the scale is still written once per 32x32 tile (four equal entries per block), so that the
 // tensor feeds the GEMMs as it stands; with BLK = 16 the scale matrix has one entry per 16x16 block.
 // STAGED = the tile goes through staging rows (above); the transposed payload's staging (qt_stage) then takes their place.
-template <int MODE, bool FAST, int BLK, bool STAGED = false, int F32 = 0>
+// EDGES = a tile of a tensor that is read directly and not made of whole 32-byte aligned tiles only: rows are not checked one by one
+// here either.  us, nearest / stochastic, every row checked and now: 300 x 768 3.6 / 4.9 -> 2.8 / 3.7, 1000 x 2048 3.8 / 5.4 -> 3.05 / 4.0, 3000 x 3008
+// 5.1 / 7.8 -> 4.7 / 6.6, 4099 x 2720 6.6 / 9.3 -> 6.0 / 8.5, on 16-byte boundaries 16384 x 4096 40.4 / 54.0 -> 35.6 / 47.6.  Tensors of whole tiles keep a
+// kernel with the checked body beside them: the body for whole tiles rounds stochastically 3 % slower when compiled beside the other
+// one, and 1 % alone (16384 x 11008 84.9, 87.9 and 86.4).
+template <int MODE, bool FAST, int BLK, bool STAGED = false, int F32 = 0, bool EDGES = false>
 __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_stage, uint4 *rnd_stage, uint32_t *xchg, uint4 *staging = nullptr)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -278,6 +283,29 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
             for (int r = 0; r < 8; r++) read_staged_row_uncut(p, tile_row0, bx * 128, stage, lane, r, raw[r]);
         }
         cut_staged_rows(raw, n_rows, (int)max((int64_t)0, min((int64_t)16, p.cols - col0)));
+    } else if (EDGES && p.x_vec_ok && col0 + 16 <= p.cols) {
+        const uint16_t *src = p.x + row0 * p.ld_x + col0;
+#pragma unroll
+        for (int r = 0; r < 8; r++)
+#pragma unroll
+            for (int k = 0; k < 8; k++) raw[r][k] = 0u;
+        if (p.x_vec_ok == 2) {
+#pragma unroll
+            for (int r = 0; r < 8; r++)
+                if (r < n_rows)
+                    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                                 : "=r"(raw[r][0]), "=r"(raw[r][1]), "=r"(raw[r][2]), "=r"(raw[r][3]), "=r"(raw[r][4]),
+                                   "=r"(raw[r][5]), "=r"(raw[r][6]), "=r"(raw[r][7])
+                                 : "l"(src + r * p.ld_x));
+        } else {
+#pragma unroll
+            for (int r = 0; r < 8; r++)
+                if (r < n_rows) {
+                    const uint4 a = load_global(reinterpret_cast<const uint4 *>(src + r * p.ld_x)), b = load_global(reinterpret_cast<const uint4 *>(src + r * p.ld_x) + 1);
+                    raw[r][0] = a.x; raw[r][1] = a.y; raw[r][2] = a.z; raw[r][3] = a.w;
+                    raw[r][4] = b.x; raw[r][5] = b.y; raw[r][6] = b.z; raw[r][7] = b.w;
+                }
+        }
     } else {
 #pragma unroll
         for (int r = 0; r < 8; r++) load_segment(p, row0 + r, col0, raw[r]);
@@ -379,8 +407,8 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
     uint32_t W[8][2];
     uint8_t *dst_rm = p.q_rm + row0 * p.ld_rm + (col0 >> 1);
     if (idle) {   // nothing of it is written, transposed either
-    } else if ((FAST || STAGED) && !nonfinite) {
-        // hot loop: no path selection, and no bounds checks but at a staged row's store
+    } else if ((FAST || STAGED || EDGES) && !nonfinite) {
+        // hot loop: no path selection, and no bounds checks but at the store
         const int n_store = tile_exists ? n_rows : 0;
 #pragma unroll
         for (int r = 0; r < 8; r++) {
@@ -413,7 +441,7 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
             if (MODE == FP4Q_ROUND_STOCHASTIC) {
                 if (STAGED) {
                     staged_random(r, R);
-                } else if (FAST || p.rng_aligned) {
+                } else if (FAST || EDGES || p.rng_aligned) {
                     const uint4 v = rnd_stage[r * 128 + threadIdx.x];
                     R[0] = v.x; R[1] = v.y; R[2] = v.z; R[3] = v.w;
                 } else {
@@ -466,7 +494,8 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
     }
 }
 
-template <int MODE, int BLK = 32>
+// EDGES: see quantize_tile; what comes here otherwise is made of whole tiles, or has the transposed index.
+template <int MODE, int BLK, bool EDGES>
 __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_kernel(const __grid_constant__ Quant2dParams p)
 {
     __shared__ uint4 qt_stage[128 * 4];   // 128 transposed rows x 64 B (four 16-byte chunks, XOR-swizzled)
@@ -477,7 +506,7 @@ __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_kernel(
     const int64_t bx = (int64_t)blockIdx.x % p.grid_x, by = (int64_t)blockIdx.x / p.grid_x;
     const bool full = p.x_vec_ok == 2 && p.rng_aligned && (by + 1) * 128 <= p.rows && (bx + 1) * 128 <= p.cols;
     if (full) quantize_tile<MODE, true, BLK>(p, qt_stage, rnd_stage, xchg);
-    else quantize_tile<MODE, false, BLK>(p, qt_stage, rnd_stage, xchg);
+    else quantize_tile<MODE, false, BLK, false, 0, EDGES>(p, qt_stage, rnd_stage, xchg);
     // The later tensors of a multi-tensor call do not read what the call's earlier ones wrote, so they did not wait; they
     // wait here, after their own stores, so that the grids still COMPLETE in launch order and whatever is enqueued after the
     // call sees every tensor of it.
@@ -524,25 +553,27 @@ __global__ void __launch_bounds__(128, 3) quantize2d_f32_kernel(const __grid_con
 typedef void (*Quant2dKernel)(const Quant2dParams);
 
 // Rows on vector boundaries and, with stochastic rounding, segments on Philox blocks are read directly: on 32-byte boundaries
-// by the check-free body, on 16-byte ones by the general body's 128-bit loads, where these reach the rows' ends.  us, nearest / stochastic,
-// direct and staged: 4096 x 4096 in a pitch of 4104 10.8 / 15.0 and 11.4 / 16.8, 2048 x 2048 in 2056 4.7 / 6.5 and 5.1 / 7.0, 16384 x 4096 40.5 / 54.2 and
-// 39.0 / 54.5; with a last segment that is not full, which the general body reads by elements: 4099 x 2728 nearest 11.9 and 9.9, 300 x 776 5.7 and
+// by the check-free body, on 16-byte ones by 128-bit loads, where these reach the rows' ends.  us, nearest / stochastic,
+// direct and staged: 4096 x 4096 in a pitch of 4104 10.6 / 13.6 and 11.4 / 16.8, 2048 x 2048 in 2056 4.4 / 5.5 and 5.1 / 7.0, 16384 x 4096 35.6 / 47.6 and
+// 39.0 / 54.5; with a last segment that is not full, which is read by elements: 4099 x 2728 nearest 11.9 and 9.9, 300 x 776 5.7 and
 // 4.4, 16 x 10008 5.9 and 3.9, 1 x 10008 2.9 and 3.3.  Anything else is staged, except for the transposed index, whose random bytes run down
 // the columns.
 static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr, int *smem)
 {
     const bool direct = p.x_vec_ok && p.rng_aligned && (p.x_vec_ok == 2 || p.cols % 16 == 0 || p.rows <= 2);
-    const bool staged = !direct && !(sr && (p.flags & FP4Q_INDEX_TRANSPOSED));
+    const bool transposed_index = sr && (p.flags & FP4Q_INDEX_TRANSPOSED), staged = !direct && !transposed_index;
+    const bool edges = direct && !transposed_index && (p.x_vec_ok != 2 || p.rows % 128 != 0 || p.cols % 128 != 0);
     const int which = (p.flags & FP4Q_BLOCK_16) ? 1 : (p.flags & FP4Q_BLOCK_64) ? 2 : 0;
-    static const Quant2dKernel kernels[2][2][3] = {
-        {{quantize2d_kernel<FP4Q_ROUND_NEAREST>, quantize2d_kernel<FP4Q_ROUND_NEAREST, 16>, quantize2d_kernel<FP4Q_ROUND_NEAREST, 64>},
-         {quantize2d_kernel<FP4Q_ROUND_STOCHASTIC>, quantize2d_kernel<FP4Q_ROUND_STOCHASTIC, 16>, quantize2d_kernel<FP4Q_ROUND_STOCHASTIC, 64>}},
-        {{quantize2d_staged_kernel<FP4Q_ROUND_NEAREST>, quantize2d_staged_kernel<FP4Q_ROUND_NEAREST, 16>,
-          quantize2d_staged_kernel<FP4Q_ROUND_NEAREST, 64>},
-         {quantize2d_staged_kernel<FP4Q_ROUND_STOCHASTIC>, quantize2d_staged_kernel<FP4Q_ROUND_STOCHASTIC, 16>,
-          quantize2d_staged_kernel<FP4Q_ROUND_STOCHASTIC, 64>}}};
+    constexpr int N = FP4Q_ROUND_NEAREST, S = FP4Q_ROUND_STOCHASTIC;
+    static const Quant2dKernel kernels[3][2][3] = {
+        {{quantize2d_kernel<N, 32, false>, quantize2d_kernel<N, 16, false>, quantize2d_kernel<N, 64, false>},
+         {quantize2d_kernel<S, 32, false>, quantize2d_kernel<S, 16, false>, quantize2d_kernel<S, 64, false>}},
+        {{quantize2d_kernel<N, 32, true>, quantize2d_kernel<N, 16, true>, quantize2d_kernel<N, 64, true>},
+         {quantize2d_kernel<S, 32, true>, quantize2d_kernel<S, 16, true>, quantize2d_kernel<S, 64, true>}},
+        {{quantize2d_staged_kernel<N>, quantize2d_staged_kernel<N, 16>, quantize2d_staged_kernel<N, 64>},
+         {quantize2d_staged_kernel<S>, quantize2d_staged_kernel<S, 16>, quantize2d_staged_kernel<S, 64>}}};
     *smem = !staged ? 0 : sr ? kStagedSmem<FP4Q_ROUND_STOCHASTIC> : kStagedSmem<FP4Q_ROUND_NEAREST>;
-    return kernels[staged][sr][which];
+    return kernels[staged ? 2 : edges][sr][which];
 }
 
 static fp4q_status launch_quantizer(Quant2dKernel kernel, int64_t n_cta, int smem, cudaStream_t stream, const Quant2dParams &p, bool later)

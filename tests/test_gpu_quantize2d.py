@@ -267,10 +267,10 @@ def test_stochastic_bands_of_few_rows(rows, cols):
     assert_matches_oracle(torch.randn(rows, cols, generator=g, device="cuda").to(torch.bfloat16), 1, seed=rows, tensor_id=cols)
 
 
-# Rows on 16-byte boundaries whose last segment is not full (staged from three rows on) and rows that start anywhere, with entries that
-# are not finite beside a matrix's ends: what is beyond them must not count
+# Rows on 16-byte boundaries whose last segment is not full (staged from three rows on), rows that start anywhere, and tiles that end
+# with a segment, with entries that are not finite beside a matrix's ends: what is beyond them must not count
 @pytest.mark.parametrize("rows", [1, 2, 3, 130])
-@pytest.mark.parametrize("cols,pitch", [(120, 120), (136, 152), (1000, 1000), (127, 129)])
+@pytest.mark.parametrize("cols,pitch", [(120, 120), (136, 152), (1000, 1000), (127, 129), (144, 160), (272, 280), (1008, 1008)])
 @pytest.mark.parametrize("mode", MODES)
 def test_rows_that_end_inside_a_segment(rows, cols, pitch, mode):
     g = torch.Generator(device="cuda").manual_seed(rows * cols)
