@@ -98,7 +98,7 @@ typedef struct {
  * hold zeros (the boundary-block rule of the appendix then makes them inert).  Groups may be
  * empty.  row_alignment is the caller's statement about the offsets: 0 or 128 = multiples of 128 (the general
  * case); 256 = every offset is a multiple of 256, which lets the grouped forward and input-gradient products
- * run on the 256-row CTA-pair tiles of the dense products (a wrong statement gives wrong results for the rows
+ * always run on the 256-row CTA-pair tiles of the dense products (a wrong statement gives wrong results for the rows
  * of a tile that straddles two groups, nothing worse).  Other values: FP4Q_ERR_UNSUPPORTED.
  */
 typedef struct {
