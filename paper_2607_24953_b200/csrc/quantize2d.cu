@@ -515,11 +515,12 @@ __global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_kernel(
 
 // Every tile of a tensor whose rows start anywhere or whose segments straddle Philox blocks.  With the random blocks in memory of their
 // own they are drawn while the rows are on their way; the transposed payload's staging takes the place of the rows, so that 53 KB
-// and 128 registers allow four CTAs per SM, like the aligned kernel.
+// and 128 registers allow four CTAs per SM, like the aligned kernel.  To nearest 36 KB and 96 registers allow five: us, four and five,
+// 4099 x 2731 9.7 and 8.7, 16384 x 2731 29.0 and 28.2, 9001 x 8191 44.6 and 43.1, 32 x 1000001 42.2 and 37.8, 300 x 777 4.33 and 4.29 (six spill).
 template <int MODE> constexpr int kStagedSmem = 4 * kStageWarpBytes + (MODE == FP4Q_ROUND_STOCHASTIC ? (8 * 128 + 4 * 32) * 16 : 0);
 static_assert(4 * kStageWarpBytes >= 128 * 4 * 16, "the transposed payload's staging fits in the rows");
 template <int MODE, int BLK = 32>
-__global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_staged_kernel(const __grid_constant__ Quant2dParams p)
+__global__ void __launch_bounds__(128, MODE == FP4Q_ROUND_NEAREST ? 5 : 4) quantize2d_staged_kernel(const __grid_constant__ Quant2dParams p)
 {
     extern __shared__ uint4 dynamic_stage[];
     __shared__ uint32_t xchg[BLK == 64 ? 16 : 1];
