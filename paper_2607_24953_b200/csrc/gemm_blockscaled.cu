@@ -2251,7 +2251,7 @@ static ScaleView scale_view(ScaleView v)
 {
     const bool tr = v.stride_kb != 1;
     const int64_t pitch = tr ? v.stride_kb : v.stride_row, n = tr ? v.n_kb : v.n_row;
-    v.words = aligned(v.ptr, 4) && pitch % 4 == 0 && pitch <= 0xFFFFFFFFll / (n + 16);
+    v.words = aligned(v.ptr, 4) && pitch % 4 == 0 && pitch >= 0 && pitch <= 0xFFFFFFFFll / (n + 16);
     return v;
 }
 
