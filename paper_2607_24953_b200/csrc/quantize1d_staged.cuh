@@ -7,7 +7,8 @@
 // memory, and code that runs once on an SM takes about ten cycles an instruction.  So the loop over a lane's rows is not unrolled where a row
 // is all that is needed (1999 x 2731 FP4 unrolled 8.2 us, rolled 7.1; reading rows twice to roll the other form's loop loses, 8.3 / 10.4).  us, FP4 /
 // MXFP8, element-wise loads before and now: 1999 x 2731 12.1 / 12.1 -> 7.2 / 7.1, 4099 x 5001 38.8 / 38.9 -> 14.9 / 14.8 (8.0 / 9.5 at the measured copy
-// bandwidth); transposed 11.3 / 12.9 -> 7.2 / 7.5, 23.4 / 32.4 -> 17.2 / 17.8 (7.5 / 7.7 and 17.9 / 19.0 with every row checked by itself).
+// bandwidth); transposed 11.3 / 12.9 -> 7.0 / 7.5, 23.4 / 32.4 -> 15.9 / 17.2 (17.9 / 19.0 with every row checked by itself,
+// 17.2 / 17.9 with four CTAs an SM instead of five).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(128) quantize1d_staged_kernel(const __grid_con
 
 // Blocks along the columns: one column of the warp's 32 rows, which four lanes hold.
 template <bool FP8>
-__global__ void __launch_bounds__(128, 4) quantize1d_t_staged_kernel(const __grid_constant__ Staged1dParams p)
+__global__ void __launch_bounds__(128, 5) quantize1d_t_staged_kernel(const __grid_constant__ Staged1dParams p)
 {
     __shared__ __align__(16) uint8_t stage[4 * kStageWarpBytes];   // the rows, then the codes of 128 columns
     __shared__ uint32_t sc_stage[128];                             // a column's four scale codes

@@ -556,7 +556,7 @@ typedef void (*Quant2dKernel)(const Quant2dParams);
 // Rows on vector boundaries and, with stochastic rounding, segments on Philox blocks are read directly: on 32-byte boundaries
 // by the check-free body, on 16-byte ones by 128-bit loads, where these reach the rows' ends.  us, nearest / stochastic,
 // direct and staged: 4096 x 4096 in a pitch of 4104 10.6 / 13.6 and 11.4 / 16.8, 2048 x 2048 in 2056 4.4 / 5.5 and 5.1 / 7.0, 16384 x 4096 35.6 / 47.6 and
-// 39.0 / 54.5; with a last segment that is not full, which is read by elements: 4099 x 2728 nearest 11.9 and 9.9, 300 x 776 5.7 and
+// 39.0 / 54.5; with a last segment that is not full, which is read by elements: 4099 x 2728 nearest 11.9 and 8.7, 300 x 776 5.7 and
 // 4.4, 16 x 10008 5.9 and 3.9, 1 x 10008 2.9 and 3.3.  Anything else is staged, except for the transposed index, whose random bytes run down
 // the columns.
 static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr, int *smem)
