@@ -208,7 +208,10 @@ __device__ __noinline__ uint32_t round_column_scalar(uint4 rows, float inv)
 // byte is a payload byte as it stands), and the payload leaves through swizzled staging rows as 64 contiguous bytes
 // per column; the four scale bytes of a column (one per warp) leave as
 // one 32-bit store.
-__global__ void __launch_bounds__(128, 4) quantize1d_t_tile_kernel(const __grid_constant__ Quant1dParams p)
+// CTAS: an SM.  Five are better where four on 148 SMs do not hold the grid; us, four and five: 16384 x 4096 32.5 and 30.5, 4096 x 4096 8.7 and
+// 8.35, but 2048 x 2048 (256 CTAs) 3.7 and 3.8.
+template <int CTAS>
+__global__ void __launch_bounds__(128, CTAS) quantize1d_t_tile_kernel(const __grid_constant__ Quant1dParams p)
 {
     wait_for_predecessor();
     admit_successor();
@@ -369,7 +372,7 @@ extern "C" fp4q_status fp4q_quantize1d_t(const void *x_bf16, int64_t rows, int64
     // full 128x128 tiles and aligned rows: the tile kernel (coalesced 64-byte column stores)
     if (rows % 128 == 0 && cols % 128 == 0 && aligned(x_bf16, 32) && ld_x % 16 == 0 && ld_s % 4 == 0 && aligned(scale, 4) &&
         (rows / 128) * (cols / 128) <= 0x7FFFFFFF) {
-        return launched(launch_dependent(quantize1d_t_tile_kernel, dim3((unsigned)((rows / 128) * (cols / 128))), 128, static_cast<cudaStream_t>(stream), p));
+        return launched(launch_dependent((rows / 128) * (cols / 128) > 592 ? quantize1d_t_tile_kernel<5> : quantize1d_t_tile_kernel<4>, dim3((unsigned)((rows / 128) * (cols / 128))), 128, static_cast<cudaStream_t>(stream), p));
     }
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;

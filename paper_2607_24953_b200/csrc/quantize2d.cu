@@ -202,10 +202,6 @@ __device__ __forceinline__ void segment_random_bytes(const Quant2dParams &p, int
     }
 }
 
-#ifndef FP4Q_QUANT_MIN_BLOCKS
-#define FP4Q_QUANT_MIN_BLOCKS 4
-#endif
-
 // FAST = the CTA's 128x128 tile lies fully inside the tensor, rows are 32-byte aligned (256-bit loads) and
 // one Philox block covers each 16-element segment: no per-row bounds or path checks remain in the hot loop.
 // BLK = block size: 32 (the method), or 16 / 64 for the block-size study.  A 16x16 block is two lanes (8 rows x 16
@@ -495,8 +491,8 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
 }
 
 // EDGES: see quantize_tile; what comes here otherwise is made of whole tiles, or has the transposed index.
-template <int MODE, int BLK, bool EDGES>
-__global__ void __launch_bounds__(128, FP4Q_QUANT_MIN_BLOCKS) quantize2d_kernel(const __grid_constant__ Quant2dParams p)
+template <int MODE, int BLK, bool EDGES, int CTAS = 4>   // CTAS: an SM
+__global__ void __launch_bounds__(128, CTAS) quantize2d_kernel(const __grid_constant__ Quant2dParams p)
 {
     __shared__ uint4 qt_stage[128 * 4];   // 128 transposed rows x 64 B (four 16-byte chunks, XOR-swizzled)
     __shared__ uint4 rnd_stage[MODE == FP4Q_ROUND_STOCHASTIC ? 8 * 128 : 1];   // per thread: 8 rows x 16 random bytes
@@ -573,7 +569,14 @@ static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr, int 
          {quantize2d_kernel<S, 32, true>, quantize2d_kernel<S, 16, true>, quantize2d_kernel<S, 64, true>}},
         {{quantize2d_staged_kernel<N>, quantize2d_staged_kernel<N, 16>, quantize2d_staged_kernel<N, 64>},
          {quantize2d_staged_kernel<S>, quantize2d_staged_kernel<S, 16>, quantize2d_staged_kernel<S, 64>}}};
+    // Nearest, where the grid is more than one or two rounds of four CTAs on 148 SMs: five.  us, four and five: edges 4099 x 2720 6.0 and 5.3, 4099 x 4096
+    // 7.8 and 7.4, 16384 x 4096 in a pitch of 4104 35.6 and 34.6, but 3000 x 3008 (576 CTAs) 4.6 and 4.7, 300 x 768 2.8 and 2.9; whole tiles 8192 x 4096
+    // 15.9 and 15.0, 4096 x 11008 24.2 and 23.0, 16384 x 4096 32.6 and 31.9, but 4096 x 4096 (1024), everything in L2, 6.9 and 7.2.
+    const int64_t n_cta = ceil_div(p.rows, 128) * ceil_div(p.cols, 128);
+    static const Quant2dKernel five[2][2] = {{quantize2d_kernel<N, 32, false, 5>, quantize2d_kernel<N, 16, false, 5>},
+                                             {quantize2d_kernel<N, 32, true, 5>, quantize2d_kernel<N, 16, true, 5>}};
     *smem = !staged ? 0 : sr ? kStagedSmem<FP4Q_ROUND_STOCHASTIC> : kStagedSmem<FP4Q_ROUND_NEAREST>;
+    if (!staged && !sr && which < 2 && n_cta > (edges ? 592 : 1184)) return five[edges][which];
     return kernels[staged ? 2 : edges][sr][which];
 }
 

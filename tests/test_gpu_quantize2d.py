@@ -279,3 +279,23 @@ def test_rows_that_end_inside_a_segment(rows, cols, pitch, mode):
     x[rows - 1, cols - 1] = float("nan")
     x[0, 0] = float("-inf")
     assert_matches_oracle(x, mode, seed=rows, tensor_id=cols)
+
+
+# More CTAs than four on each SM run in kernels of their own when rounded to nearest: whole tiles, and tiles at the edges; and the transposing 1D quantizer
+@pytest.mark.parametrize("rows,cols,pitch", [(8192, 2560, 2560), (4100, 2720, 2720), (4100, 2720, 2728)])
+@pytest.mark.parametrize("flags", [0, binding.BLOCK_16])
+def test_large_grids_equal_their_bands(rows, cols, pitch, flags):
+    x = workloads.activations_student_t(rows, pitch, 3, "cuda")[:, :cols]
+    whole = binding.fp4q_quantize2d(x, flags=flags)
+    b = 32 // (2 if flags else 1)
+    for r0 in range(0, rows, 1024):
+        band = binding.fp4q_quantize2d(x[r0:r0 + 1024], flags=flags)
+        n = min(1024, rows - r0)
+        assert torch.equal(whole.q_rm[r0:r0 + n, :cols // 2], band.q_rm[:, :cols // 2])
+        assert torch.equal(whole.q_t[:, r0 // 2:(r0 + n) // 2], band.q_t[:, :n // 2])
+        assert torch.equal(whole.scale[r0 // b:-(-(r0 + n) // b), :-(-cols // b)], band.scale[:-(-n // b), :-(-cols // b)])
+    if rows % 128 == 0:
+        q, s = binding.fp4q_quantize1d_t(x)
+        for r0 in range(0, rows, 1024):
+            bq, bs = binding.fp4q_quantize1d_t(x[r0:r0 + 1024])
+            assert torch.equal(q[:, r0 // 2:r0 // 2 + 512], bq) and torch.equal(s[:, r0 // 32:r0 // 32 + 32], bs)
