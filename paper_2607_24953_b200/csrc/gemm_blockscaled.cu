@@ -343,8 +343,12 @@ __device__ __forceinline__ uint32_t cluster_ctarank()
 }
 // The kernel's first barrier, which every warp passes at a place of its own: behind it the mbarriers of the CTA, or of both CTAs of
 // a pair, exist.  In a pair warps arrive ahead of time (warp 4, which initializes them, after its fence.mbarrier_init), so that the
-// way from one CTA to the other is under way while a role prepares what needs nobody else.  In one CTA nobody waits for the
-// builders, which come late and have a barrier of their own with warp 4.
+// way from one CTA to the other is under way while a role prepares what needs nobody else.  Only warp 1 arrives late: behind its
+// allocation of tensor memory, with release, because the leader's scale copies and MMAs write the other CTA's tensor memory and
+// nothing else puts them behind that CTA's allocation.  us, that arrival ahead of the allocation too and behind it: FP4 products level
+// (2048 x 2048 x 2048 8.1 / 8.3 / 9.3 and 8.1 / 8.1 / 9.2), per-row kinds 1 to 1.5 % for small ones (16 x 16 blocks 8192 x 2048 x 2048 22.6 / 22.2 / 19.7 and
+// 22.9 / 22.4 / 20.0, MXFP8 there 29.8 and 30.2).  In one CTA nobody waits for the builders, which come late and have a barrier of
+// their own with warp 4.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
@@ -1247,7 +1251,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             if (EPI == EPI_QUANT) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmD) : "memory");
         }
         __syncwarp();
-    } else if (CTAS == 2) {
+    } else if (CTAS == 2 && warp != 1) {
         cluster_arrive_relaxed();
     }
     if (warp == 0) {
@@ -1266,6 +1270,8 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_slot)),
                          "r"(kTmemCols) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+            tcgen05_fence_before();
+            cluster_arrive();
         }
     }
     // Everything above touches this CTA only; from here on the kernel reads what its predecessor in the stream wrote.  Its own
@@ -1879,7 +1885,10 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 tcgen05_fence_before();
                 __syncwarp();
                 // The accumulator now lives in registers.  Behind the last one nobody waits for the accumulator, and this warp has nothing
-                // to do with the other CTA any more: it lets the pair go while its output leaves.
+                // to do with the other CTA any more: it lets the pair go while its output leaves.  The arrival is relaxed: all that has to be
+                // over before tensor memory is freed is this warp's reads of it, which wait::ld has completed and which the tcgen05
+                // fences before the arrival and before the deallocation order (PTX's own examples pair these fences with relaxed
+                // arrivals).  Release costs products of 8 us 2 % (2048 x 2048 x 2048 8.1 / 8.1 / 9.15 -> 8.3 / 8.3 / 9.4).
                 if (last) {
                     if (CTAS == 2) cluster_arrive_relaxed();
                     else asm volatile("bar.arrive 14, 288;" ::: "memory");
