@@ -499,7 +499,7 @@ enum { NEED_LENGTH = 0, NEED_OUTPUT = 1, NEED_ALL = 2 };
 // GROUPS: what a kernel is made for.  Dense products' tiles are decoded without the group branches, which cost the builders of the
 // per-row kinds 3-8 % of a product (1D activations at 4096 x 4096 x 4096: 45.8 us without, 49.7 us with), one CTA's smallest ones 0.3 us
 // (128 x 256 x 256 6.1 / 5.8) and quantized outputs 3-5 % (2048 x 2048 x 2048 12.4 / 11.7, 8192 x 5632 x 2048 56.6 / 55.2).
-enum { GROUPS_NONE = 0, GROUPS_ANY = 1, GROUPS_PAIRED = 2 };   // PAIRED: any, and paired rows
+enum { GROUPS_NONE = 0, GROUPS_ANY = 1, GROUPS_PAIRED = 2, GROUPS_CUT = 3 };   // PAIRED: any, and paired rows; CUT: weight gradients of experts whose rows end within a box of 32
 template <int GROUPS>
 __device__ __forceinline__ void decode_tile(const GemmParams &p, int tile, int rank, Tile &t, int m_tiles, const int32_t *goffs, const uint16_t *gorder, int need = NEED_ALL)
 {
@@ -771,8 +771,13 @@ __device__ __forceinline__ void transpose_staged_codes(uint32_t stg, int jp, int
 
 // One round of the epilogue: 32 words per lane (this lane's row, 128 bytes) into the warp's swizzled staging rows, then one
 // TMA store (kind 0: BF16 bytes, 1: FP32 bytes, 2: FP32 add-reduction) of the 32 x 128 B box; fresh: staging rows that no store reads.
-__device__ __forceinline__ void stage_and_store(const CUtensorMap *map, const uint32_t *w, uint32_t stg_row, uint32_t swz,
-                                                uint32_t stg, int col, int32_t y, int kind, int lane, bool fresh)
+// CUT: n_rows of the box may be fewer than 32, with other rows of the output behind them (a grouped weight gradient is a stack of
+// matrices of any number of rows).  Such a box leaves by the lanes' own stores, in kernels that nothing else runs: compiled into those
+// of all grouped products they took 0.7 % on average, input gradients of ragged widths 1-3 %.  (So did a map with the group
+// as its outermost dimension, which clips the box: input gradients 38.0 -> 39.8, 24.6 -> 25.5 us.)
+template <bool CUT>
+__device__ __forceinline__ void stage_and_store(const GemmParams &p, const CUtensorMap *map, const uint32_t *w, uint32_t stg_row, uint32_t swz,
+                                                uint32_t stg, int col, int32_t y, int kind, int lane, bool fresh, int n_rows)
 {
     if (!fresh) {
         if (lane == 0) bulk_wait_read_all();   // the previous round's store has read the staging rows
@@ -782,6 +787,26 @@ __device__ __forceinline__ void stage_and_store(const CUtensorMap *map, const ui
     for (int c = 0; c < 8; c++)
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stg_row + ((c ^ swz) << 4)), "r"(w[4 * c]), "r"(w[4 * c + 1]),
                      "r"(w[4 * c + 2]), "r"(w[4 * c + 3]) : "memory");
+    if (CUT && n_rows < 32) {
+        __syncwarp();
+        const int c = col + (kind == 0 ? 2 : 1) * lane, n = p.N - c;   // this lane's word of a row, and what there is of its columns
+#pragma unroll 1
+        for (int r = 0; r < n_rows; r++) {
+            uint32_t x;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(stg + r * 128 + ((((uint32_t)lane >> 2) ^ (r & 7)) << 4) + 4 * (lane & 3)) : "memory");
+            const int64_t at = ((int64_t)y + r) * p.ldc + c;
+            if (kind == 0) {
+                if (n > 0) static_cast<uint16_t *>(p.C)[at] = (uint16_t)x;
+                if (n > 1) static_cast<uint16_t *>(p.C)[at + 1] = (uint16_t)(x >> 16);
+            } else if (n > 0) {
+                float *dst = static_cast<float *>(p.C) + at;
+                if (kind == 2) atomicAdd(dst, __uint_as_float(x));
+                else *dst = __uint_as_float(x);
+            }
+        }
+        __syncwarp();
+        return;
+    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> TMA store
     __syncwarp();
     if (lane == 0) {
@@ -2009,13 +2034,14 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                     const uint32_t stg0 = last ? smem_u32(smem) + (warp - 4) * 4 * kStagingWarpBytes : smem_u32(smem_staging) + (warp - 4) * kStagingWarpBytes;
                     const uint32_t swz = (uint32_t)(lane & 7);
                     const int32_t y = t.c_row0 + 32 * quarter;
+                    const int n_rows = t.m_valid - 32 * quarter;
                     if (p.out_f32) {
 #pragma unroll
                         for (int h = 0; h < 4; h++) {
                             const int col_in_tile = 128 * half + 32 * h;
                             const uint32_t stg = last ? stg0 + h * kStagingWarpBytes : stg0;
                             if (col_in_tile < t.n_valid)
-                                stage_and_store(&tmC, v[h], stg + lane * 128, swz, stg, t.c_col0 + col_in_tile, y, p.accumulate ? 2 : 1, lane, last);
+                                stage_and_store<GROUPS == GROUPS_CUT>(p, &tmC, v[h], stg + lane * 128, swz, stg, t.c_col0 + col_in_tile, y, p.accumulate ? 2 : 1, lane, last, n_rows);
                         }
                     } else {
 #pragma unroll
@@ -2030,7 +2056,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                                 w[e] = *reinterpret_cast<const uint32_t *>(&b);
                             }
                             const uint32_t stg = last ? stg0 + h * kStagingWarpBytes : stg0;
-                            stage_and_store(&tmC, w, stg + lane * 128, swz, stg, t.c_col0 + col_in_tile, y, 0, lane, last);
+                            stage_and_store<GROUPS == GROUPS_CUT>(p, &tmC, w, stg + lane * 128, swz, stg, t.c_col0 + col_in_tile, y, 0, lane, last, n_rows);
                         }
                     }
                 }
@@ -2314,6 +2340,10 @@ static fp4q_status launch_gemm(const Operand &A, const Operand &B, GemmParams &p
     if constexpr (KIND == KIND_MXF4) {
         if (p.mode != MODE_DENSE) {
             if (use_pairs && p.M > BM && p.mode == MODE_GROUPED_ROWS && !p.rows_pair_aligned && pairs_pay(p)) p.mode = MODE_PAIRED_ROWS;
+            if (p.mode == MODE_GROUPED_K && p.M % 32 != 0) {
+                if (use_pairs && p.M > BM) return launch_gemm_impl<KIND, 2, EPI_STORE, false, GROUPS_CUT>(A, B, p, stream);
+                return launch_gemm_impl<KIND, 1, EPI_STORE, false, GROUPS_CUT>(A, B, p, stream);
+            }
             const bool pairs = p.mode == MODE_GROUPED_K || p.mode == MODE_PAIRED_ROWS || p.rows_pair_aligned;
             if (use_pairs && pairs && p.M > BM) return launch_gemm_impl<KIND, 2, EPI_STORE, false, GROUPS_PAIRED>(A, B, p, stream);
             return launch_gemm_impl<KIND, 1, EPI_STORE, false, GROUPS_ANY>(A, B, p, stream);

@@ -79,6 +79,33 @@ def test_paired_rows(E, rows):
     assert binding.fp4q_workspace_status(ws) == 0
 
 
+# Weight gradients of experts whose rows do not end with a box of 32: one CTA (up to 128 rows) and pairs, a box within one expert and over several,
+# empty experts in every place, both types of output, added to what is there, rows beside the stack untouched
+@pytest.mark.parametrize("N", [1, 9, 48, 100, 129, 272, 300])
+def test_experts_of_any_number_of_rows(N):
+    ws = binding.alloc_workspace("cuda")
+    tiles = np.array([0, 2, 1, 0, 0, 3, 1, 5, 0])
+    offs = np.concatenate([[0], np.cumsum(128 * tiles)])
+    E, T, K = len(tiles), int(offs[-1]), 200
+    qx, qdy = operands((T, K), (T, N))
+    d = torch.from_numpy(offs).cuda()
+    x, dy = (dequant_from_gpu(q) for q in (qx, qdy))
+    want = np.concatenate([dy[offs[g]:offs[g + 1]].T @ x[offs[g]:offs[g + 1]] for g in range(E)])
+    for dt, dtype in ((binding.OUT_F32, torch.float32), (binding.OUT_BF16, torch.bfloat16)):
+        buf = torch.full((E * N + 40, K), 7.0, dtype=dtype, device="cuda")
+        check_gemm(binding.fp4q_gemm_wgrad(qdy, qx, out=buf[:E * N], dt=dt, row_offsets=d, ws=ws), want, "wgrad")
+        for g in np.flatnonzero(tiles == 0):
+            assert not buf[g * N:(g + 1) * N].any()
+        assert (buf[E * N:] == 7.0).all()
+    dw = torch.zeros(E * N + 40, K, device="cuda")
+    for _ in range(2):
+        binding.fp4q_gemm_wgrad(qdy, qx, out=dw[:E * N], accumulate=True, row_offsets=d, ws=ws)
+    check_gemm(dw[:E * N], 2 * want, "wgrad, added")
+    assert not dw[E * N:].any()
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
+
+
 # 81 tiles of 43 and of 44 stages: both sides of the line (48 stages for each of 74 pairs) from which on a dense product runs with a
 # watcher between the loads and the MMAs; and that every role leaves there, too, when a load that it waits for never arrives
 @pytest.mark.parametrize("K", [43 * 256, 44 * 256])
