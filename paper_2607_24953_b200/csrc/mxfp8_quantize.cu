@@ -96,6 +96,8 @@ __global__ void __launch_bounds__(256) mxfp8_quantize1d_kernel(const __grid_cons
 // (the contraction axis of the backward products).  A warp owns 32 rows x 64 columns: each row is one coalesced
 // 128-byte load, a lane keeps its two columns' 32 values in registers, and writes 32 contiguous payload bytes per
 // column (one whole sector each).
+// WORDS: rows on words; others are read element by element.
+template <bool WORDS>
 __global__ void __launch_bounds__(128) mxfp8_quantize1d_t_kernel(const __grid_constant__ Mxfp8QuantParams p)
 {
     wait_for_predecessor();
@@ -106,12 +108,12 @@ __global__ void __launch_bounds__(128) mxfp8_quantize1d_t_kernel(const __grid_co
     if (i0 >= p.rows || c0 >= p.cols) return;
     const bool two = c0 + 1 < p.cols;
     uint32_t raw[32];
-    const uint32_t *words = reinterpret_cast<const uint32_t *>(p.x + i0 * p.ld_x + c0);   // the launch has seen to rows on words
+    const uint32_t *words = reinterpret_cast<const uint32_t *>(p.x + i0 * p.ld_x + c0);
     const int64_t step = p.ld_x >> 1;
-    if (two && i0 + 32 <= p.rows) {   // interior: 32 unconditional word loads, one address step each
+    if (WORDS && two && i0 + 32 <= p.rows) {   // interior: 32 unconditional word loads, one address step each
 #pragma unroll
         for (int r = 0; r < 32; r++) raw[r] = load_global(words + r * step);
-    } else if (two) {
+    } else if (WORDS && two) {
         const int n = (int)(p.rows - i0);
 #pragma unroll
         for (int r = 0; r < 32; r++) raw[r] = r < n ? load_global(words + r * step) : 0u;
@@ -121,7 +123,7 @@ __global__ void __launch_bounds__(128) mxfp8_quantize1d_t_kernel(const __grid_co
             raw[r] = 0u;
             if (i0 + r < p.rows) {
                 const uint16_t *src = p.x + (i0 + r) * p.ld_x + c0;
-                raw[r] = load_global(src);
+                raw[r] = (uint32_t)load_global(src) | (!WORDS && two ? (uint32_t)load_global(src + 1) << 16 : 0u);
             }
         }
     }
@@ -319,7 +321,7 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d(const void *x_bf16, int64_t rows, i
     const int64_t total = rows * (p.segs_per_row / 2);
     const int64_t n_cta = ceil_div(total, 256);
     if (n_cta > 0x7FFFFFFF) return FP4Q_ERR_UNSUPPORTED;
-    if (!p.x_vec_ok && rows * cols >= kStagedRowsFrom)
+    if (!p.x_vec_ok && staged_rows_pay(rows, cols))
         return launch_quantize1d_staged<true>(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, false, static_cast<cudaStream_t>(stream));
     return launched(launch_dependent(mxfp8_quantize1d_kernel, dim3((unsigned)n_cta), 256, static_cast<cudaStream_t>(stream), p));
 }
@@ -347,7 +349,7 @@ extern "C" fp4q_status fp4q_mxfp8_quantize1d_t(const void *x_bf16, int64_t rows,
     }
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;
-    if (!p.x_vec_ok || rows * cols >= kStagedTransposeFrom)
+    if (staged_transpose_pays(rows, cols, p.x_vec_ok, true))
         return launch_quantize1d_staged<true>(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, true, static_cast<cudaStream_t>(stream));
-    return launched(launch_dependent(mxfp8_quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p));
+    return launched(launch_dependent(p.x_vec_ok ? mxfp8_quantize1d_t_kernel<true> : mxfp8_quantize1d_t_kernel<false>, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p));
 }

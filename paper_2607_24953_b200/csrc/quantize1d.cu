@@ -107,6 +107,8 @@ __global__ void __launch_bounds__(256) quantize1d_kernel(const __grid_constant__
 
 // The encoding of x^T, nearest rounding.  A warp owns 32 rows x 64 columns: each row is one coalesced 128-byte load,
 // a lane keeps its two columns' 32 values in registers, and writes the 16 payload bytes of each column's block.
+// WORDS: rows on words; others are read element by element.
+template <bool WORDS>
 __global__ void __launch_bounds__(128) quantize1d_t_kernel(const __grid_constant__ Quant1dParams p)
 {
     wait_for_predecessor();
@@ -117,12 +119,12 @@ __global__ void __launch_bounds__(128) quantize1d_t_kernel(const __grid_constant
     if (i0 >= p.rows || c0 >= p.cols) return;
     const bool two = c0 + 1 < p.cols;
     uint32_t raw[32];
-    const uint32_t *words = reinterpret_cast<const uint32_t *>(p.x + i0 * p.ld_x + c0);   // the launch has seen to rows on words
+    const uint32_t *words = reinterpret_cast<const uint32_t *>(p.x + i0 * p.ld_x + c0);
     const int64_t step = p.ld_x >> 1;
-    if (two && i0 + 32 <= p.rows) {   // interior: 32 unconditional word loads, one address step each
+    if (WORDS && two && i0 + 32 <= p.rows) {   // interior: 32 unconditional word loads, one address step each
 #pragma unroll
         for (int r = 0; r < 32; r++) raw[r] = load_global(words + r * step);
-    } else if (two) {
+    } else if (WORDS && two) {
         const int n = (int)(p.rows - i0);
 #pragma unroll
         for (int r = 0; r < 32; r++) raw[r] = r < n ? load_global(words + r * step) : 0u;
@@ -132,7 +134,7 @@ __global__ void __launch_bounds__(128) quantize1d_t_kernel(const __grid_constant
             raw[r] = 0u;
             if (i0 + r < p.rows) {
                 const uint16_t *src = p.x + (i0 + r) * p.ld_x + c0;
-                raw[r] = load_global(src);
+                raw[r] = (uint32_t)load_global(src) | (!WORDS && two ? (uint32_t)load_global(src + 1) << 16 : 0u);
             }
         }
     }
@@ -350,7 +352,7 @@ extern "C" fp4q_status fp4q_quantize1d(const void *x_bf16, int64_t rows, int64_t
     const int64_t n_cta = ceil_div(rows * (p.segs_per_row / 2), 256);
     if (n_cta > 0x7FFFFFFF) return FP4Q_ERR_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (!p.x_vec_ok && mode == FP4Q_ROUND_NEAREST && rows * cols >= kStagedRowsFrom)
+    if (!p.x_vec_ok && mode == FP4Q_ROUND_NEAREST && staged_rows_pay(rows, cols))
         return launch_quantize1d_staged<false>(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, false, s);
     return launched(launch_dependent(mode == FP4Q_ROUND_STOCHASTIC ? quantize1d_kernel<FP4Q_ROUND_STOCHASTIC> : quantize1d_kernel<FP4Q_ROUND_NEAREST>,
                                      dim3((unsigned)n_cta), 256, s, p));
@@ -376,7 +378,7 @@ extern "C" fp4q_status fp4q_quantize1d_t(const void *x_bf16, int64_t rows, int64
     }
     const int64_t gx = ceil_div(cols, 64), gy = ceil_div(ceil_div(rows, 32), 4);
     if (gx > 0x7FFFFFFF || gy > 65535) return FP4Q_ERR_UNSUPPORTED;
-    if (!p.x_vec_ok || rows * cols >= kStagedTransposeFrom)
+    if (staged_transpose_pays(rows, cols, p.x_vec_ok, false))
         return launch_quantize1d_staged<false>(Staged1dParams{p.x, rows, cols, ld_x, q, ld_q, scale, ld_s}, true, static_cast<cudaStream_t>(stream));
-    return launched(launch_dependent(quantize1d_t_kernel, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p));
+    return launched(launch_dependent(p.x_vec_ok ? quantize1d_t_kernel<true> : quantize1d_t_kernel<false>, dim3((unsigned)gx, (unsigned)gy), 128, static_cast<cudaStream_t>(stream), p));
 }

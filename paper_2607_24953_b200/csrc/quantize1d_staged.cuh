@@ -29,11 +29,23 @@ struct Staged1dParams {
     int64_t grid_x;   // tiles along the columns; set by the launch
 };
 
-// Which matrices come here, by their elements.  Rows that start anywhere, blocks along the rows: reading them element by element takes 2.2 us and
-// 2 a million elements, staged tiles 5 and 0.45 (300 x 777 3.4 / 5.1, 1999 x 1003 6.2 / 5.4, 4099 x 5001 38.8 / 14.6).  The transpose of what is not made
-// of whole tiles: rows on words have a kernel that is the better one for matrices that are over soon (2048 x 2752 5.7 / 7.6, 3000 x 3000
-// 12.5 / 10.0); others 300 x 777 8.3 / 5.4, 1999 x 2731 11.3 / 8.3.
-constexpr int64_t kStagedRowsFrom = 3 << 19, kStagedTransposeFrom = 6 << 20;
+// Which matrices come here.  The work goes by tiles of 128 x 128, whatever is in them: 5 us and 0.45 a million elements of the tiles.  us, the other
+// kernels and this one:
+// Rows off 16 bytes, blocks along the rows.  Reading them element by element takes 2.2 us and 2 a million elements of long rows, 1 of rows of a few
+// hundred, however few rows there are: 300 x 777 3.4 / 5.1, 1999 x 1003 6.2 / 5.4, 3001 x 3001 18.7 / 8.4; 1 x 2000001 6.2 / 27, 8 x 300001 6.3 / 11.8, 17 x 150001
+// 8.3 / 8.7, 20 x 100001 6.2 / 5.6, 28 x 100001 8.4 / 5.9; 60000 x 33 3.9 / 8.9, 20001 x 193 6.5 / 7.4, 10001 x 301 5.2 / 6.2, 10001 x 361 6.6 / 6.3, 30001 x 385
+// 19.0 / 13.5 (but 30001 x 301 10.6 / 9.9).
+inline bool staged_rows_pay(int64_t rows, int64_t cols) { return rows >= 20 && cols >= 360 && rows * cols >= 3 << 19; }
+// The transpose of what is not made of whole tiles, rows on words: a kernel that reads words, FP4 12000 x 6002 46.6 / 50.0, 16000 x 11010 118 / 113, MXFP8
+// 5000 x 7002 28.6 / 29.6, 6000 x 6002 32.1 / 30.1, 16000 x 4002 56.1 / 49.5; in tiles that are not nearly full 32 x 300002 6.0 / 19.5, 129 x 60002 5.5 / 10.5.
+// Others, element by element or here: 300 x 777 7.7 / 4.7, 3001 x 3001 12.9 / 8.8, 5001 x 31 7.8 / 5.2; 1 x 2000001 34 / 114, 1 x 5001 2.4 / 3.8, 8 x 70001 3.9 / 6.8,
+// 16 x 151937 6.6 / 12.9, 20 x 5001 5.5 / 4.6, 33 x 60001 8.3 / 7.5, 600001 x 3 22.6 / 51, 70001 x 3 5.0 / 8.3, 200001 x 17 16.4 / 19.4, 60000 x 33 8.8 / 8.5.
+inline bool staged_transpose_pays(int64_t rows, int64_t cols, bool words, bool fp8)
+{
+    const int64_t elements = rows * cols, tiles = ceil_div(rows, 128) * ceil_div(cols, 128), area = tiles * 128 * 128;
+    if (words) return elements >= (fp8 ? 34 << 20 : 96 << 20) && 8 * elements >= 7 * area;
+    return rows >= 16 && cols >= 8 && (tiles <= 400 || 17 * elements >= 4 * area);
+}
 
 // UE8M0 code of MXFP8's truncation-free scale: the smallest e with 448 * 2^e >= M, from the BF16 magnitude bits of M.
 __device__ __forceinline__ int e4m3_scale_code(uint32_t mbits)
@@ -127,6 +139,7 @@ __global__ void __launch_bounds__(128) quantize1d_staged_kernel(const __grid_con
     admit_successor();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t by = (int64_t)blockIdx.x / p.grid_x, bx = (int64_t)blockIdx.x - by * p.grid_x, tile_row0 = by * 128 + 32 * warp;
+    if (tile_row0 >= p.rows) return;   // 33 x 200001 11.3 -> 9.5 us
     stage_tile_rows(p, tile_row0, bx * 128, rows + warp * kStageWarpBytes, lane);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();

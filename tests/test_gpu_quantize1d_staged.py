@@ -3,6 +3,7 @@ along the rows and along the columns, on both sides of the sizes at which the st
 import numpy as np
 import pytest
 import torch
+from torch.profiler import ProfilerActivity, profile
 
 import oracle
 from paper_2607_24953_b200 import binding, workloads
@@ -38,3 +39,33 @@ def test_any_rows(rows, cols, pitch, start):
         assert np.array_equal(s.cpu().numpy()[:, :(length + 31) // 32], want_s), quantize.__name__
         assert np.array_equal(got_q[:, :n], want_q), quantize.__name__
         assert not got_q[:, n:(length + 31) // 32 * 32 // per_byte].any(), quantize.__name__   # block padding
+
+
+# Few rows or few columns, where tiles are mostly empty: the element-wise kernels whatever the number of elements, along the rows below 20 rows or 360
+# columns, along the columns below 16 rows or 8 columns or in more than 400 tiles that are less than a quarter full; rows on words in tiles that are not
+# nearly full; and what goes through tiles just beside these
+@pytest.mark.parametrize("rows,cols,pitch,start", [(1, 1600001, 1600001, 1), (19, 83001, 83001, 0), (20, 83001, 83001, 3), (33, 50001, 50001, 0), (15, 60001, 60001, 0),
+                                                    (16, 60001, 60001, 0), (16, 9001, 9001, 1), (32, 60001, 60001, 0), (60001, 33, 33, 1), (200001, 17, 17, 0), (4400, 359, 359, 0),
+                                                    (4400, 361, 361, 0), (70001, 7, 7, 0), (4001, 8, 9, 0), (33, 1100002, 1100002, 0)])
+def test_few_rows_or_columns(rows, cols, pitch, start):
+    test_any_rows(rows, cols, pitch, start)
+
+
+def kernels(call):
+    call()
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as p:
+        call()
+        torch.cuda.synchronize()
+    return " ".join(e.key for e in p.key_averages())
+
+
+# one row, a few, narrow ones: as many tiles as a matrix of 128 times the elements has; and what is made of full tiles
+@pytest.mark.parametrize("rows,cols,along_rows,along_columns", [(1, 2000001, False, False), (16, 151937, False, False), (60000, 33, False, True), (600001, 3, False, False),
+                                                                (33, 60001, True, True), (1999, 1003, True, True)])
+def test_work_is_counted_in_tiles(rows, cols, along_rows, along_columns):
+    x = torch.zeros(rows * cols + 1, dtype=torch.bfloat16, device="cuda")[1:].view(rows, cols)
+    for quantize, staged in ((binding.fp4q_quantize1d, along_rows), (binding.fp4q_mxfp8_quantize1d, along_rows),
+                             (binding.fp4q_quantize1d_t, along_columns), (binding.fp4q_mxfp8_quantize1d_t, along_columns)):
+        names = kernels(lambda: quantize(x))
+        assert "quantize1d" in names and ("staged" in names) == staged, (quantize.__name__, names)
