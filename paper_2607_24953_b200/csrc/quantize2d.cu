@@ -490,7 +490,7 @@ __device__ __forceinline__ void quantize_tile(const Quant2dParams &p, uint4 *qt_
     }
 }
 
-// EDGES: see quantize_tile; what comes here otherwise is made of whole tiles, or has the transposed index.
+// EDGES: see quantize_tile; what comes here otherwise is made of whole tiles, has the transposed index or is a few rows.
 template <int MODE, int BLK, bool EDGES, int CTAS = 4>   // CTAS: an SM
 __global__ void __launch_bounds__(128, CTAS) quantize2d_kernel(const __grid_constant__ Quant2dParams p)
 {
@@ -555,11 +555,17 @@ typedef void (*Quant2dKernel)(const Quant2dParams);
 // 39.0 / 54.5; with a last segment that is not full, which is read by elements: 4099 x 2728 nearest 11.9 and 8.7, 300 x 776 5.7 and
 // 4.4, 16 x 10008 5.9 and 3.9, 1 x 10008 2.9 and 3.3.  Anything else is staged, except for the transposed index, whose random bytes run down
 // the columns.
+// A few rows in many tiles are read directly too, in the kernel whose body checks every row and rounds only those that exist; us, nearest /
+// stochastic, all eight of a lane (or staged) and checked: 1 x 1000016 33.9 / 65.6 -> 28.0 / 52.8, 3 x 1000008 38.6 / 63.6 -> 31.2 / 63.6, 5 x 1000016
+// 34.2 / 65.9 -> 32.8 / 62.5, 2 x 100016 5.6 / 9.1 -> 5.2 / 8.2, 1 x 10016 2.9 / 3.9 -> 2.8 / 3.6, but 7 x 1000016 34.4 / 66.1 and 35.9 / 67.5, 5 x 100016
+// 5.65 / 9.1 and 6.0 / 9.7, 3 x 10016 2.9 / 3.8 and 3.0 / 4.0.
 static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr, int *smem)
 {
-    const bool direct = p.x_vec_ok && p.rng_aligned && (p.x_vec_ok == 2 || p.cols % 16 == 0 || p.rows <= 2);
+    const int64_t n_cta = ceil_div(p.rows, 128) * ceil_div(p.cols, 128);
+    const bool few = p.rows == 1 || (p.rows <= 5 && 300 * p.rows <= n_cta);
+    const bool direct = p.x_vec_ok && p.rng_aligned && (p.x_vec_ok == 2 || p.cols % 16 == 0 || p.rows <= 2 || few);
     const bool transposed_index = sr && (p.flags & FP4Q_INDEX_TRANSPOSED), staged = !direct && !transposed_index;
-    const bool edges = direct && !transposed_index && (p.x_vec_ok != 2 || p.rows % 128 != 0 || p.cols % 128 != 0);
+    const bool edges = direct && !transposed_index && !few && (p.x_vec_ok != 2 || p.rows % 128 != 0 || p.cols % 128 != 0);
     const int which = (p.flags & FP4Q_BLOCK_16) ? 1 : (p.flags & FP4Q_BLOCK_64) ? 2 : 0;
     constexpr int N = FP4Q_ROUND_NEAREST, S = FP4Q_ROUND_STOCHASTIC;
     static const Quant2dKernel kernels[3][2][3] = {
@@ -571,8 +577,8 @@ static Quant2dKernel quantize2d_kernel_for(const Quant2dParams &p, bool sr, int 
          {quantize2d_staged_kernel<S>, quantize2d_staged_kernel<S, 16>, quantize2d_staged_kernel<S, 64>}}};
     // Nearest, where the grid is more than one or two rounds of four CTAs on 148 SMs: five.  us, four and five: edges 4099 x 2720 6.0 and 5.3, 4099 x 4096
     // 7.8 and 7.4, 16384 x 4096 in a pitch of 4104 35.6 and 34.6, but 3000 x 3008 (576 CTAs) 4.6 and 4.7, 300 x 768 2.8 and 2.9; whole tiles 8192 x 4096
-    // 15.9 and 15.0, 4096 x 11008 24.2 and 23.0, 16384 x 4096 32.6 and 31.9, but 4096 x 4096 (1024), everything in L2, 6.9 and 7.2.
-    const int64_t n_cta = ceil_div(p.rows, 128) * ceil_div(p.cols, 128);
+    // 15.9 and 15.0, 4096 x 11008 24.2 and 23.0, 16384 x 4096 32.6 and 31.9, but 4096 x 4096 (1024), everything in L2, 6.9 and 7.2.  64 x 64 blocks, which only
+    // the study of block sizes uses, have not been tried with five.
     static const Quant2dKernel five[2][2] = {{quantize2d_kernel<N, 32, false, 5>, quantize2d_kernel<N, 16, false, 5>},
                                              {quantize2d_kernel<N, 32, true, 5>, quantize2d_kernel<N, 16, true, 5>}};
     *smem = !staged ? 0 : sr ? kStagedSmem<FP4Q_ROUND_STOCHASTIC> : kStagedSmem<FP4Q_ROUND_NEAREST>;

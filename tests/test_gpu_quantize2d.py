@@ -1,7 +1,10 @@
 """GPU parity: fp4q_quantize2d against the CPU oracle, bit for bit, through the C ABI."""
+import re
+
 import numpy as np
 import pytest
 import torch
+from torch.profiler import ProfilerActivity, profile
 
 import oracle
 from paper_2607_24953_b200 import binding, workloads
@@ -299,3 +302,33 @@ def test_large_grids_equal_their_bands(rows, cols, pitch, flags):
         for r0 in range(0, rows, 1024):
             bq, bs = binding.fp4q_quantize1d_t(x[r0:r0 + 1024])
             assert torch.equal(q[:, r0 // 2:r0 // 2 + 512], bq) and torch.equal(s[:, r0 // 32:r0 // 32 + 32], bs)
+
+
+def kernels(call):
+    call()
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as p:
+        call()
+        torch.cuda.synchronize()
+    return " ".join(e.key for e in p.key_averages())
+
+
+# One row, and up to five in 300 tiles a row: the kernel that rounds only the rows that exist; one tile fewer, or a row more: all of a lane's rows (or staged)
+@pytest.mark.parametrize("rows,cols,few", [(1, 16, True), (1, 1000, True), (1, 38416, True), (2, 76816, True), (2, 76656, False), (3, 115208, True), (5, 191888, True), (5, 191776, False),
+                                           (6, 230416, False)])
+@pytest.mark.parametrize("mode,flags", [(0, 0), (1, 0), (0, binding.BLOCK_16), (0, binding.BLOCK_64)])
+def test_few_rows(rows, cols, few, mode, flags):
+    g = torch.Generator(device="cuda").manual_seed(rows + cols)
+    x = torch.randn(rows, cols, generator=g, device="cuda").to(torch.bfloat16)
+    x[rows - 1, cols - 1] = float("inf")
+    if flags == 0:
+        assert_matches_oracle(x, mode, seed=rows, tensor_id=3)
+    else:   # the blocks of the oracle's other sizes: equal to the same rows on top of a taller tensor of zeros
+        tall = torch.zeros(8, cols, dtype=torch.bfloat16, device="cuda")
+        tall[:rows] = x
+        a, b = binding.fp4q_quantize2d(x, flags=flags), binding.fp4q_quantize2d(tall, flags=flags)
+        assert torch.equal(a.q_rm[:, :cols // 2], b.q_rm[:rows, :cols // 2]) and torch.equal(a.scale, b.scale)
+        assert torch.equal(a.q_t[:, :16], b.q_t[:, :16])
+    if mode == 0 or cols % 16 == 0:
+        names = kernels(lambda: binding.fp4q_quantize2d(x, mode=mode, flags=flags))
+        assert bool(re.search(r"quantize2d_kernel<\d+, \d+, false", names)) == few, names
