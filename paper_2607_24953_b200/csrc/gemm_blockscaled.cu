@@ -27,6 +27,7 @@
 // (Cfg), is guarded by mbarriers; the scale columns in TMEM form a ring of the same depth.  Every mbarrier wait is bounded: when a limit
 // is hit the CTA records FP4Q_ERR_TIMEOUT in the workspace, releases the MMA warp from its named barriers, stops
 // issuing work and leaves through the normal exit (TMEM is freed).
+#include <atomic>
 #include <cstdlib>
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -2109,16 +2110,12 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 
 static EncodeTiledFn encode_tiled_fn()
 {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const EncodeTiledFn fn = [] {   // several threads may make their first product at the same time: all but one wait
         void *ptr = nullptr;
         cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(ptr);
-    }
+        const bool found = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess && qres == cudaDriverEntryPointSuccess;
+        return found ? reinterpret_cast<EncodeTiledFn>(ptr) : nullptr;
+    }();
     return fn;
 }
 
@@ -2173,7 +2170,7 @@ struct Operand {
     ScaleView sf;
 };
 
-constexpr int kMaxDevices = 64;   // per-device host state (attributes set, SM counts, static workspace address)
+constexpr int kMaxDevices = 64;   // per-device host state (attributes set, SM counts, static workspace address); threads that find it unset all set the same
 
 static int current_device()
 {
@@ -2184,9 +2181,13 @@ static int current_device()
 
 static int sm_count(int dev)
 {
-    static int n[kMaxDevices];
-    if (n[dev] == 0 && (cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n[dev] <= 0)) n[dev] = 148;
-    return n[dev];
+    static std::atomic<int> known[kMaxDevices];
+    int n = known[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
+        known[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
 }
 
 // Most row tiles that pairs can have with grouped rows on multiples of 128: a group with an odd number has one alone.
@@ -2231,12 +2232,12 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
     p.by_tail = divisor(tail != 0 ? tail : 1);
     const int dev = current_device();
     if (dev < 0) return FP4Q_ERR_CUDA;
-    static bool attr_set[kMaxDevices];   // the attribute is a property of (kernel, device): one flag per device and instantiation
-    if (!attr_set[dev]) {
+    static std::atomic<bool> attr_set[kMaxDevices];   // the attribute is a property of (kernel, device): one flag per device and instantiation
+    if (!attr_set[dev].load(std::memory_order_relaxed)) {
         if (cudaFuncSetAttribute(gemm_block_scaled_kernel<KIND, CTAS, EPI, WATCH, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  Cfg<KIND, CTAS>::kSmemBytes) != cudaSuccess)
             return FP4Q_ERR_CUDA;
-        attr_set[dev] = true;
+        attr_set[dev].store(true, std::memory_order_relaxed);
     }
     int slots = sm_count(dev) / CTAS;   // CTAs or pairs that run at a time
 #ifdef FP4Q_TRACE
@@ -2737,7 +2738,7 @@ namespace fp4q {
 constexpr size_t kStaticWorkspaceBytes = 1024;   // stated maximum; the kernel's workspace must fit in it
 static __device__ __align__(256) unsigned char g_static_workspace[kStaticWorkspaceBytes];
 
-static void *g_static_workspace_addr[kMaxDevices];   // device address of the array, per device
+static std::atomic<void *> g_static_workspace_addr[kMaxDevices];   // device address of the array, per device
 
 // In host code the array's name is only a handle: the device address has to be asked for, once per device,
 // with that device current.
