@@ -2118,50 +2118,54 @@ static EncodeTiledFn encode_tiled_fn()
     }();
     return fn;
 }
+// The encoder wants a context on the calling thread, which the runtime binds with the thread's first call that needs one; a thread whose first
+// call is a product has made none.
+static bool encode_tiled(CUtensorMap *map, CUtensorMapDataType type, int rank, void *base, const cuuint64_t *dims, const cuuint64_t *strides,
+                         const cuuint32_t *box, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion promotion)
+{
+    const EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    const cuuint32_t estr[5] = {1u, 1u, 1u, 1u, 1u};
+    auto encode = [&] {
+        return fn(map, type, (cuuint32_t)rank, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, promotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    CUresult r = encode();
+    int dev;
+    if (r == CUDA_ERROR_INVALID_CONTEXT && cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = encode();
+    return r == CUDA_SUCCESS;
+}
 
 // Operand tile map: a [rows, row_bytes] byte matrix with pitch ld_bytes, box = 128 B x box_rows, 128B swizzle.
 static bool make_operand_map(CUtensorMap *map, const void *base, int64_t rows, int64_t row_bytes, int64_t ld_bytes,
                              int box_rows)
 {
-    EncodeTiledFn fn = encode_tiled_fn();
-    if (!fn) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)row_bytes, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)ld_bytes};
     const cuuint32_t box[2] = {128u, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1u, 1u};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(base), dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 
-// Output map for the pair kernel's TMA stores: box = 128 bytes x 32 rows, 128-byte swizzle.  Plain stores address the
+// Output map for the TMA stores: box = 128 bytes x 32 rows, 128-byte swizzle.  Plain stores address the
 // output as bytes; accumulation uses the TMA add-reduction, which needs the element type (FP32, 32 per box row).
 static bool make_output_map(CUtensorMap *map, void *base, int64_t rows, int64_t cols, int64_t ld, bool f32, bool reduce)
 {
-    EncodeTiledFn fn = encode_tiled_fn();
-    if (!fn) return false;
     const int64_t esize = f32 ? 4 : 2;
     const cuuint64_t dims[2] = {(cuuint64_t)(reduce ? cols : cols * esize), (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)(ld * esize)};
     const cuuint32_t box[2] = {reduce ? 32u : 128u, 32u};
-    const cuuint32_t estr[2] = {1u, 1u};
-    return fn(map, reduce ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_tiled(map, reduce ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_NONE);
 }
 
 // Plain byte matrix [rows, row_bytes] with pitch ld_bytes as a store target.
 static bool make_byte_map(CUtensorMap *map, void *base, int64_t rows, int64_t row_bytes, int64_t ld_bytes, int box_bytes,
                           int box_rows, CUtensorMapSwizzle swizzle)
 {
-    EncodeTiledFn fn = encode_tiled_fn();
-    if (!fn) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)row_bytes, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)ld_bytes};
     const cuuint32_t box[2] = {(cuuint32_t)box_bytes, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1u, 1u};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
-              CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE);
 }
 
 struct Operand {

@@ -50,3 +50,22 @@ def test_first_products_of_several_threads(library):
     # all come while the first of them looks for the driver's entry point
     L = ctypes.CDLL(library)
     assert in_threads(8, lambda: product(L, True)) == [0] * 8
+
+
+def test_a_threads_first_call_is_a_product(library):
+    # nothing has bound the thread to a device: the encoder refuses it, the product binds it and goes on
+    L = ctypes.CDLL(library)
+    assert in_threads(2, lambda: (product(L, False), L.fake_bound())) == [(0, 1)] * 2
+
+
+@pytest.mark.gpu
+def test_a_threads_first_call_is_a_product_on_the_device():
+    import torch
+    from paper_2607_24953_b200 import workloads
+    qx, qw = (binding.fp4q_quantize2d(workloads.activations_student_t(rows, 256, rows, "cuda")) for rows in (512, 300))
+    ws, out = binding.alloc_workspace("cuda"), torch.zeros(2, 512, 304, dtype=torch.bfloat16, device="cuda")[:, :, :300]
+    binding.fp4q_gemm_fwd(qx, qw, out=out[0], ws=ws)
+    torch.cuda.synchronize()
+    in_threads(1, lambda: binding.fp4q_gemm_fwd(qx, qw, out=out[1], ws=ws))
+    torch.cuda.synchronize()
+    assert out[0].any() and torch.equal(out[0], out[1])
