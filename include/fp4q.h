@@ -187,6 +187,7 @@ fp4q_status fp4q_debug_withhold_load(void *ws, uint32_t nth_load, void *stream);
  * Reads X.q_rm and W.q_rm (both contraction-contiguous) with scales X.scale[t/32, k/32] and
  * W.scale[n/32, k/32].  Y is BF16 or FP32 (dt), leading dimension ldy in elements; Y must be
  * 16-byte aligned and ldy*sizeof(element) a multiple of 16.  T, N arbitrary; K = X.cols = W.cols.
+ * Of Y, here and in every product, only the N columns of each row are written.
  * Grouped form (g != NULL): X is the permuted token matrix, W the expert stack [n_groups*N, K];
  * row t of group g is multiplied by rows g*N .. g*N+N-1 of the stack.
  */

@@ -204,6 +204,7 @@ struct GemmParams {
     int32_t raster_m;                // tile order: groups of raster_m row tiles, within a group row tile fastest
     Divisor by_problem, by_group, by_raster, by_tail;   // m_tiles * n_tiles; raster_m * n_tiles; raster_m; row tiles of the last group if it is smaller
     int32_t out_f32, accumulate;
+    int32_t tail_col;                // TMA stores: first column of a row's last bytes, fewer than 16, which they do not write; INT32_MIN: none
     int32_t wide_stores;             // output base and row pitch are 32-byte aligned: 256-bit stores (whole sectors)
     int32_t mode, n_groups;
     int32_t rows_pair_aligned;       // grouped rows: every group starts on a multiple of 256 rows (caller's statement)
@@ -221,7 +222,7 @@ struct GemmParams {
     PhiloxRoundKeys q_keys;
 };
 
-enum { EPI_STORE = 0, EPI_QUANT = 1 };
+enum { EPI_STORE = 0, EPI_QUANT = 1, EPI_TAIL = 2 };   // TAIL: rows of the output end inside 16 bytes, which TMA stores would fill
 
 struct Tile {
     int32_t a_row0, b_row0, b_load_row0, a_k0, b_k0, k_len, c_row0, c_col0, m_valid, n_valid;
@@ -772,11 +773,12 @@ __device__ __forceinline__ void transpose_staged_codes(uint32_t stg, int jp, int
 
 // One round of the epilogue: 32 words per lane (this lane's row, 128 bytes) into the warp's swizzled staging rows, then one
 // TMA store (kind 0: BF16 bytes, 1: FP32 bytes, 2: FP32 add-reduction) of the 32 x 128 B box; fresh: staging rows that no store reads.
+// TAIL: a box of nothing but a row's last elements (store_row_tail) is not stored.
 // CUT: n_rows of the box may be fewer than 32, with other rows of the output behind them (a grouped weight gradient is a stack of
 // matrices of any number of rows).  Such a box leaves by the lanes' own stores, in kernels that nothing else runs: compiled into those
 // of all grouped products they took 0.7 % on average, input gradients of ragged widths 1-3 %.  (So did a map with the group
 // as its outermost dimension, which clips the box: input gradients 38.0 -> 39.8, 24.6 -> 25.5 us.)
-template <bool CUT>
+template <bool CUT, bool TAIL>
 __device__ __forceinline__ void stage_and_store(const GemmParams &p, const CUtensorMap *map, const uint32_t *w, uint32_t stg_row, uint32_t swz,
                                                 uint32_t stg, int col, int32_t y, int kind, int lane, bool fresh, int n_rows)
 {
@@ -810,10 +812,38 @@ __device__ __forceinline__ void stage_and_store(const GemmParams &p, const CUten
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> TMA store
     __syncwarp();
-    if (lane == 0) {
+    if (lane == 0 && !(TAIL && col == p.tail_col)) {
         if (kind == 2) tma_reduce_add_2d(map, col, y, stg);                 // x in FP32 elements
         else tma_store_2d(map, col * (kind == 1 ? 4 : 2), y, stg);          // x in bytes
         bulk_commit();
+    }
+}
+
+// A row's last elements, n (1 .. 7) from column p.tail_col on, out of the 16 bytes of staging that hold them.  A TMA store writes whole pieces of 16 bytes,
+// whatever the map's element type: with a map that ended inside one, it wrote zeros over what follows the row's last column.  Kernels of
+// their own (EPI_TAIL), since the few instructions behind a tile cost others up to 3 %; us, with those zeros and without: 1999 x 1003 x 2731 forward
+// 10.5 / 10.8, 16384 x 1003 x 2721 24.6 / 25.2, 9001 x 4095 x 2049 43.8 / 44.7, 849 x 67 x 169 5.7 / 6.0.
+__device__ __forceinline__ void store_row_tail(const GemmParams &p, int64_t row, uint32_t src)
+{
+    uint32_t x[4];
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(src) : "memory");
+    const int n = p.N - p.tail_col;
+    const int64_t at = row * p.ldc + p.tail_col;   // on 16 bytes
+    if (p.out_f32) {
+        float *dst = static_cast<float *>(p.C) + at;
+        if (p.accumulate) {
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+                if (i < n) atomicAdd(dst + i, __uint_as_float(x[i]));
+        } else {
+            if (n & 2) *reinterpret_cast<uint2 *>(dst) = make_uint2(x[0], x[1]);
+            if (n & 1) dst[n - 1] = __uint_as_float(n & 2 ? x[2] : x[0]);
+        }
+    } else {
+        uint16_t *dst = static_cast<uint16_t *>(p.C) + at;
+        if (n & 4) *reinterpret_cast<uint2 *>(dst) = make_uint2(x[0], x[1]);
+        if (n & 2) *reinterpret_cast<uint32_t *>(dst + (n & 4)) = n & 4 ? x[2] : x[0];
+        if (n & 1) dst[n - 1] = (uint16_t)(n & 4 ? (n & 2 ? x[3] : x[2]) : (n & 2 ? x[1] : x[0]));
     }
 }
 
@@ -2042,7 +2072,7 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                             const int col_in_tile = 128 * half + 32 * h;
                             const uint32_t stg = last ? stg0 + h * kStagingWarpBytes : stg0;
                             if (col_in_tile < t.n_valid)
-                                stage_and_store<GROUPS == GROUPS_CUT>(p, &tmC, v[h], stg + lane * 128, swz, stg, t.c_col0 + col_in_tile, y, p.accumulate ? 2 : 1, lane, last, n_rows);
+                                stage_and_store<GROUPS == GROUPS_CUT, EPI == EPI_TAIL>(p, &tmC, v[h], stg + lane * 128, swz, stg, t.c_col0 + col_in_tile, y, p.accumulate ? 2 : 1, lane, last, n_rows);
                         }
                     } else {
 #pragma unroll
@@ -2057,8 +2087,14 @@ gemm_block_scaled_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                                 w[e] = *reinterpret_cast<const uint32_t *>(&b);
                             }
                             const uint32_t stg = last ? stg0 + h * kStagingWarpBytes : stg0;
-                            stage_and_store<GROUPS == GROUPS_CUT>(p, &tmC, w, stg + lane * 128, swz, stg, t.c_col0 + col_in_tile, y, 0, lane, last, n_rows);
+                            stage_and_store<GROUPS == GROUPS_CUT, EPI == EPI_TAIL>(p, &tmC, w, stg + lane * 128, swz, stg, t.c_col0 + col_in_tile, y, 0, lane, last, n_rows);
                         }
+                    }
+                    // The last box of a row is the one that lies in the staging rows now (or in its own place of the ring).
+                    const uint32_t tail = (uint32_t)p.tail_col - (uint32_t)(t.c_col0 + 128 * half);
+                    if (EPI == EPI_TAIL && tail < 128u && row_ok && !(GROUPS == GROUPS_CUT && n_rows < 32)) {
+                        const uint32_t byte = tail << (p.out_f32 ? 2 : 1);
+                        store_row_tail(p, row, stg0 + (last ? byte >> 7 : 0u) * kStagingWarpBytes + lane * 128 + (((byte >> 4 & 7u) ^ swz) << 4));
                     }
                 }
             } else if (row_ok) {
@@ -2147,11 +2183,13 @@ static bool make_operand_map(CUtensorMap *map, const void *base, int64_t rows, i
 }
 
 // Output map for the TMA stores: box = 128 bytes x 32 rows, 128-byte swizzle.  Plain stores address the
-// output as bytes; accumulation uses the TMA add-reduction, which needs the element type (FP32, 32 per box row).
+// output as bytes; accumulation uses the TMA add-reduction, which needs the element type (FP32, 32 per box row).  cols: whole
+// pieces of 16 bytes (store_row_tail has the rest), or none, and then no store uses the map.
 static bool make_output_map(CUtensorMap *map, void *base, int64_t rows, int64_t cols, int64_t ld, bool f32, bool reduce)
 {
     const int64_t esize = f32 ? 4 : 2;
-    const cuuint64_t dims[2] = {(cuuint64_t)(reduce ? cols : cols * esize), (cuuint64_t)rows};
+    const cuuint64_t row_bytes = (cuuint64_t)(cols > 0 ? cols * esize : 16);
+    const cuuint64_t dims[2] = {reduce ? row_bytes / 4 : row_bytes, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)(ld * esize)};
     const cuuint32_t box[2] = {reduce ? 32u : 128u, 32u};
     return encode_tiled(map, reduce ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -2214,7 +2252,11 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
         // [N, ceil32(T)/2] bytes, box 16 B x 128 rows
         if (!make_byte_map(&tmC, p.q_rm, p.M, round_up(p.N, 32) / 2, p.q_ld_rm, 64, 32, CU_TENSOR_MAP_SWIZZLE_64B)) return FP4Q_ERR_CUDA;
         if (p.q_t && !make_byte_map(&tmD, p.q_t, p.N, round_up(p.M, 32) / 2, p.q_ld_t, 16, 128, CU_TENSOR_MAP_SWIZZLE_NONE)) return FP4Q_ERR_CUDA;
-    } else if (!make_output_map(&tmC, p.C, out_rows, p.N, p.ldc, p.out_f32 != 0, p.accumulate != 0)) return FP4Q_ERR_CUDA;
+    } else {
+        const int32_t whole = p.N / (p.out_f32 ? 4 : 8) * (p.out_f32 ? 4 : 8);   // columns in whole pieces of 16 bytes
+        p.tail_col = whole < p.N ? whole : INT32_MIN;
+        if (!make_output_map(&tmC, p.C, out_rows, whole, p.ldc, p.out_f32 != 0, p.accumulate != 0)) return FP4Q_ERR_CUDA;
+    }
     if (!make_operand_map(&tmB, B.payload, B.rows, B.row_bytes, B.ld_bytes, Cfg<KIND, CTAS>::kBRows)) return FP4Q_ERR_CUDA;
     p.ctas = CTAS;
     p.m_tiles = (int32_t)ceil_div(p.M, BM * CTAS);
@@ -2321,6 +2363,16 @@ static bool pairs_pay(const GemmParams &p)
     return 9 * ceil_div(pairs * p.n_tiles, sms / 2) + 2 <= 10 * ceil_div(rows * p.n_tiles, sms);
 }
 
+// With the epilogue that the output's rows ask for.
+template <int KIND, int CTAS, bool WATCH, int GROUPS = GROUPS_NONE>
+static fp4q_status launch_store(const Operand &A, const Operand &B, GemmParams &p, void *stream)
+{
+    if constexpr (Cfg<KIND, CTAS>::kTmaStores)
+        if (GROUPS == GROUPS_CUT || p.N % (p.out_f32 ? 4 : 8) != 0) return launch_gemm_impl<KIND, CTAS, EPI_TAIL, WATCH, GROUPS>(A, B, p, stream);
+    if constexpr (GROUPS == GROUPS_CUT) return FP4Q_ERR_UNSUPPORTED;
+    else return launch_gemm_impl<KIND, CTAS, EPI_STORE, WATCH, GROUPS>(A, B, p, stream);
+}
+
 template <int KIND>
 static fp4q_status launch_gemm(const Operand &A, const Operand &B, GemmParams &p, void *ws, size_t ws_bytes, void *stream)
 {
@@ -2346,23 +2398,23 @@ static fp4q_status launch_gemm(const Operand &A, const Operand &B, GemmParams &p
         if (p.mode != MODE_DENSE) {
             if (use_pairs && p.M > BM && p.mode == MODE_GROUPED_ROWS && !p.rows_pair_aligned && pairs_pay(p)) p.mode = MODE_PAIRED_ROWS;
             if (p.mode == MODE_GROUPED_K && p.M % 32 != 0) {
-                if (use_pairs && p.M > BM) return launch_gemm_impl<KIND, 2, EPI_STORE, false, GROUPS_CUT>(A, B, p, stream);
-                return launch_gemm_impl<KIND, 1, EPI_STORE, false, GROUPS_CUT>(A, B, p, stream);
+                if (use_pairs && p.M > BM) return launch_store<KIND, 2, false, GROUPS_CUT>(A, B, p, stream);
+                return launch_store<KIND, 1, false, GROUPS_CUT>(A, B, p, stream);
             }
             const bool pairs = p.mode == MODE_GROUPED_K || p.mode == MODE_PAIRED_ROWS || p.rows_pair_aligned;
-            if (use_pairs && pairs && p.M > BM) return launch_gemm_impl<KIND, 2, EPI_STORE, false, GROUPS_PAIRED>(A, B, p, stream);
-            return launch_gemm_impl<KIND, 1, EPI_STORE, false, GROUPS_ANY>(A, B, p, stream);
+            if (use_pairs && pairs && p.M > BM) return launch_store<KIND, 2, false, GROUPS_PAIRED>(A, B, p, stream);
+            return launch_store<KIND, 1, false, GROUPS_ANY>(A, B, p, stream);
         }
     }
     if (use_pairs && p.M > BM) {
         if constexpr (KIND == KIND_MXF4) {
             const int dev = current_device();
             const int64_t pairs = dev < 0 ? 74 : sm_count(dev) / 2;
-            if (ceil_div(p.M, 2 * BM) * p.n_tiles * ceil_div(p.K, 256) <= kShortStages * pairs) return launch_gemm_impl<KIND, 2, EPI_STORE, false>(A, B, p, stream);
+            if (ceil_div(p.M, 2 * BM) * p.n_tiles * ceil_div(p.K, 256) <= kShortStages * pairs) return launch_store<KIND, 2, false>(A, B, p, stream);
         }
-        return launch_gemm_impl<KIND, 2, EPI_STORE, KIND == KIND_MXF4 || KIND == KIND_MXF8>(A, B, p, stream);
+        return launch_store<KIND, 2, KIND == KIND_MXF4 || KIND == KIND_MXF8>(A, B, p, stream);
     }
-    return launch_gemm_impl<KIND, 1, EPI_STORE, false>(A, B, p, stream);
+    return launch_store<KIND, 1, false>(A, B, p, stream);
 }
 
 static bool tensor_ok(const fp4q_tensor *t) { return t && t->rows >= 0 && t->cols >= 0; }

@@ -106,6 +106,46 @@ def test_experts_of_any_number_of_rows(N):
     assert binding.fp4q_workspace_status(ws) == 0
 
 
+# A row's last elements, in 16 bytes that the output fills only in part: all kinds, one CTA and pairs, both types; nothing is written beyond them
+@pytest.mark.parametrize("T", [1, 128, 300])
+@pytest.mark.parametrize("N,K", [(1, 300), (3, 65), (7, 129), (9, 130), (131, 257), (257, 1), (1003, 63), (515, 70)])
+def test_outputs_end_with_their_last_column(T, N, K):
+    ws = binding.alloc_workspace("cuda")
+    x, w, dy = (workloads.activations_student_t(r, c, 7 + i, "cuda") for i, (r, c) in enumerate([(T, K), (N, K), (T, N)]))
+    (qx, qw, qdy), (bx, bw, bdy) = ([binding.fp4q_quantize2d(t, flags=flags) for t in (x, w, dy)] for flags in (0, binding.BLOCK_16))
+    x1, xt1, x8, w8 = binding.fp4q_quantize1d(x), binding.fp4q_quantize1d_t(x), binding.fp4q_mxfp8_quantize1d(x), binding.fp4q_mxfp8_quantize1d(w)
+
+    def mxfp8(dt, ws, out=None):   # through the C interface, whose output may be any buffer
+        out = torch.empty(T, (N + 7) // 8 * 8, dtype=(torch.bfloat16, torch.float32)[dt], device="cuda")[:, :N] if out is None else out
+        operands = [v for (q, sc), rows in ((x8, T), (w8, N)) for v in (q.data_ptr(), q.stride(0), sc.data_ptr(), sc.stride(0), rows)]
+        assert binding.lib().fp4q_mxfp8_gemm(*operands, K, out.data_ptr(), out.stride(0), dt, ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream) == 0
+        return out
+
+    products = [((T, N), False, lambda **k: binding.fp4q_gemm_fwd(qx, qw, **k)), ((T, K), False, lambda **k: binding.fp4q_gemm_dgrad(qdy, qw, **k)),
+                ((N, K), True, lambda **k: binding.fp4q_gemm_wgrad(qdy, qx, **k)),
+                ((T, N), False, lambda **k: binding.fp4q_gemm_fwd_b16(bx, bw, **k)), ((T, K), False, lambda **k: binding.fp4q_gemm_dgrad_b16(bdy, bw, **k)),
+                ((N, K), True, lambda **k: binding.fp4q_gemm_wgrad_b16(bdy, bx, **k)), ((T, N), False, lambda **k: binding.fp4q_gemm_fwd_act1d(*x1, T, qw, **k)),
+                ((N, K), True, lambda **k: binding.fp4q_gemm_wgrad_act1d(qdy, *xt1, K, **k)), ((T, N), False, mxfp8)]
+    if T % 128 == 0:   # one group
+        products.append(((N, K), True, lambda **k: binding.fp4q_gemm_wgrad(qdy, qx, row_offsets=torch.tensor([0, T], device="cuda"), **k)))
+    for i, ((rows, cols), adds, product) in enumerate(products):
+        for dt, dtype in ((binding.OUT_F32, torch.float32), (binding.OUT_BF16, torch.bfloat16)):
+            whole = product(dt=dt, ws=ws)
+            buf = torch.full((rows + 3, (cols + 15) // 8 * 8), 7.0, dtype=dtype, device="cuda")
+            product(dt=dt, ws=ws, out=buf[:rows, :cols])
+            assert torch.equal(buf[:rows, :cols], whole), (i, dtype)
+            assert (buf[:rows, cols:] == 7.0).all() and (buf[rows:] == 7.0).all(), (i, dtype)
+        if adds:
+            once = product(dt=binding.OUT_F32, ws=ws)
+            buf = torch.full((rows + 3, (cols + 15) // 8 * 8), -0.0, device="cuda")
+            for _ in range(2):
+                product(dt=binding.OUT_F32, ws=ws, out=buf[:rows, :cols], accumulate=True)
+            assert torch.equal(buf[:rows, :cols], 2 * once), i
+            assert torch.signbit(buf[:rows, cols:]).all() and torch.signbit(buf[rows:]).all(), i
+    torch.cuda.synchronize()
+    assert binding.fp4q_workspace_status(ws) == 0
+
+
 # 81 tiles of 43 and of 44 stages: both sides of the line (48 stages for each of 74 pairs) from which on a dense product runs with a
 # watcher between the loads and the MMAs; and that every role leaves there, too, when a load that it waits for never arrives
 @pytest.mark.parametrize("K", [43 * 256, 44 * 256])
