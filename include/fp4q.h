@@ -52,7 +52,9 @@ typedef enum {
     FP4Q_ROUND_STOCHASTIC = 1  /* stochastic rounding (gradient tensors in the backward pass) */
 } fp4q_round;
 
-typedef enum { FP4Q_OUT_BF16 = 0, FP4Q_OUT_F32 = 1 } fp4q_out;
+/* FP4Q_OUT_PADDED, added to either type: the bytes from a row's last column up to the next multiple of 16 are padding that the
+ * call may write (zeros; nothing is added to them that changes them).  It saves rows that end inside 16 bytes stores of their own. */
+typedef enum { FP4Q_OUT_BF16 = 0, FP4Q_OUT_F32 = 1, FP4Q_OUT_PADDED = 0x100 } fp4q_out;
 
 /* fp4q_quantize2d flag: key the stochastic-rounding stream on the element's index in the
  * TRANSPOSED tensor (j*rows + i instead of i*cols + j), so that quantize(A^T) with this flag
@@ -187,7 +189,7 @@ fp4q_status fp4q_debug_withhold_load(void *ws, uint32_t nth_load, void *stream);
  * Reads X.q_rm and W.q_rm (both contraction-contiguous) with scales X.scale[t/32, k/32] and
  * W.scale[n/32, k/32].  Y is BF16 or FP32 (dt), leading dimension ldy in elements; Y must be
  * 16-byte aligned and ldy*sizeof(element) a multiple of 16.  T, N arbitrary; K = X.cols = W.cols.
- * Of Y, here and in every product, only the N columns of each row are written.
+ * Of Y, here and in every product, only the N columns of each row are written (but see FP4Q_OUT_PADDED).
  * Grouped form (g != NULL): X is the permuted token matrix, W the expert stack [n_groups*N, K];
  * row t of group g is multiplied by rows g*N .. g*N+N-1 of the stack.
  */

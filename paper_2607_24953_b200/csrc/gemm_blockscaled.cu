@@ -204,7 +204,8 @@ struct GemmParams {
     int32_t raster_m;                // tile order: groups of raster_m row tiles, within a group row tile fastest
     Divisor by_problem, by_group, by_raster, by_tail;   // m_tiles * n_tiles; raster_m * n_tiles; raster_m; row tiles of the last group if it is smaller
     int32_t out_f32, accumulate;
-    int32_t tail_col;                // TMA stores: first column of a row's last bytes, fewer than 16, which they do not write; INT32_MIN: none
+    int32_t padded;                  // the output's rows may be filled up to 16 bytes
+    int32_t tail_col;                // EPI_TAIL: first column of a row's last bytes, fewer than 16, which TMA stores do not write; INT32_MIN: none
     int32_t wide_stores;             // output base and row pitch are 32-byte aligned: 256-bit stores (whole sectors)
     int32_t mode, n_groups;
     int32_t rows_pair_aligned;       // grouped rows: every group starts on a multiple of 256 rows (caller's statement)
@@ -820,9 +821,10 @@ __device__ __forceinline__ void stage_and_store(const GemmParams &p, const CUten
 }
 
 // A row's last elements, n (1 .. 7) from column p.tail_col on, out of the 16 bytes of staging that hold them.  A TMA store writes whole pieces of 16 bytes,
-// whatever the map's element type: with a map that ended inside one, it wrote zeros over what follows the row's last column.  Kernels of
-// their own (EPI_TAIL), since the few instructions behind a tile cost others up to 3 %; us, with those zeros and without: 1999 x 1003 x 2731 forward
-// 10.5 / 10.8, 16384 x 1003 x 2721 24.6 / 25.2, 9001 x 4095 x 2049 43.8 / 44.7, 849 x 67 x 169 5.7 / 6.0.
+// whatever the map's element type: with a map that ends inside one, it writes zeros over what follows the row's last column.  Kernels of
+// their own (EPI_TAIL), since the few instructions behind a tile cost others up to 3 %, and only for outputs whose padding is not theirs to
+// fill; us, with those zeros and without: 1999 x 1003 x 2731 forward 10.5 / 10.8, 16384 x 1003 x 2721 24.6 / 25.2, 9001 x 4095 x 2049 43.8 / 44.7, 849 x 67 x 169
+// 5.7 / 6.0; where the output is not in L2, sectors that are written in part cost more (7296 x 490 x 1664 8.4 / 9.6).
 __device__ __forceinline__ void store_row_tail(const GemmParams &p, int64_t row, uint32_t src)
 {
     uint32_t x[4];
@@ -2183,8 +2185,8 @@ static bool make_operand_map(CUtensorMap *map, const void *base, int64_t rows, i
 }
 
 // Output map for the TMA stores: box = 128 bytes x 32 rows, 128-byte swizzle.  Plain stores address the
-// output as bytes; accumulation uses the TMA add-reduction, which needs the element type (FP32, 32 per box row).  cols: whole
-// pieces of 16 bytes (store_row_tail has the rest), or none, and then no store uses the map.
+// output as bytes; accumulation uses the TMA add-reduction, which needs the element type (FP32, 32 per box row).  cols: where
+// rows must not be filled up to 16 bytes, whole pieces of these (store_row_tail has the rest), or none, and then no store uses the map.
 static bool make_output_map(CUtensorMap *map, void *base, int64_t rows, int64_t cols, int64_t ld, bool f32, bool reduce)
 {
     const int64_t esize = f32 ? 4 : 2;
@@ -2253,7 +2255,7 @@ static fp4q_status launch_gemm_impl(const Operand &A, const Operand &B, GemmPara
         if (!make_byte_map(&tmC, p.q_rm, p.M, round_up(p.N, 32) / 2, p.q_ld_rm, 64, 32, CU_TENSOR_MAP_SWIZZLE_64B)) return FP4Q_ERR_CUDA;
         if (p.q_t && !make_byte_map(&tmD, p.q_t, p.N, round_up(p.M, 32) / 2, p.q_ld_t, 16, 128, CU_TENSOR_MAP_SWIZZLE_NONE)) return FP4Q_ERR_CUDA;
     } else {
-        const int32_t whole = p.N / (p.out_f32 ? 4 : 8) * (p.out_f32 ? 4 : 8);   // columns in whole pieces of 16 bytes
+        const int32_t whole = EPI == EPI_TAIL ? p.N / (p.out_f32 ? 4 : 8) * (p.out_f32 ? 4 : 8) : p.N;   // columns in whole pieces of 16 bytes
         p.tail_col = whole < p.N ? whole : INT32_MIN;
         if (!make_output_map(&tmC, p.C, out_rows, whole, p.ldc, p.out_f32 != 0, p.accumulate != 0)) return FP4Q_ERR_CUDA;
     }
@@ -2368,7 +2370,7 @@ template <int KIND, int CTAS, bool WATCH, int GROUPS = GROUPS_NONE>
 static fp4q_status launch_store(const Operand &A, const Operand &B, GemmParams &p, void *stream)
 {
     if constexpr (Cfg<KIND, CTAS>::kTmaStores)
-        if (GROUPS == GROUPS_CUT || p.N % (p.out_f32 ? 4 : 8) != 0) return launch_gemm_impl<KIND, CTAS, EPI_TAIL, WATCH, GROUPS>(A, B, p, stream);
+        if (GROUPS == GROUPS_CUT || (!p.padded && p.N % (p.out_f32 ? 4 : 8) != 0)) return launch_gemm_impl<KIND, CTAS, EPI_TAIL, WATCH, GROUPS>(A, B, p, stream);
     if constexpr (GROUPS == GROUPS_CUT) return FP4Q_ERR_UNSUPPORTED;
     else return launch_gemm_impl<KIND, CTAS, EPI_STORE, WATCH, GROUPS>(A, B, p, stream);
 }
@@ -2451,6 +2453,18 @@ static Operand operand_t(const fp4q_tensor *t)
     return o;
 }
 
+static bool out_type_ok(fp4q_out dt)
+{
+    const int type = (int)dt & ~(int)FP4Q_OUT_PADDED;
+    return type == FP4Q_OUT_BF16 || type == FP4Q_OUT_F32;
+}
+static bool out_type_f32(fp4q_out dt) { return ((int)dt & ~(int)FP4Q_OUT_PADDED) == FP4Q_OUT_F32; }
+static void set_out_type(GemmParams &p, fp4q_out dt)
+{
+    p.out_f32 = out_type_f32(dt);
+    p.padded = ((int)dt & (int)FP4Q_OUT_PADDED) != 0;
+}
+
 static void dense_tiles(GemmParams &p)
 {
     p.m_tiles = (int32_t)ceil_div(p.M, BM);
@@ -2471,7 +2485,7 @@ static fp4q_status prepare_fwd(const fp4q_tensor *X, const fp4q_tensor *W, void 
     *noop = false;
     if (!tensor_ok(X) || !tensor_ok(W)) return X && W ? FP4Q_ERR_SHAPE : FP4Q_ERR_NULL;
     if (fp4q_status s = check_groups(g)) return s;
-    if (dt != FP4Q_OUT_BF16 && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
+    if (!out_type_ok(dt)) return FP4Q_ERR_UNSUPPORTED;
     if (X->cols != W->cols) return FP4Q_ERR_SHAPE;
     const int64_t T = X->rows, K = X->cols;
     const int64_t N = g ? W->rows / g->n_groups : W->rows;
@@ -2482,7 +2496,7 @@ static fp4q_status prepare_fwd(const fp4q_tensor *X, const fp4q_tensor *W, void 
     if (ldy < N) return FP4Q_ERR_SHAPE;
     p = GemmParams{};
     p.C = Y; p.ldc = ldy; p.M = (int32_t)T; p.N = (int32_t)N; p.K = (int32_t)K;
-    p.out_f32 = dt == FP4Q_OUT_F32; p.accumulate = 0;
+    set_out_type(p, dt); p.accumulate = 0;
     dense_tiles(p);
     if (g) {
         p.mode = MODE_GROUPED_ROWS; p.n_groups = g->n_groups; p.row_offsets = g->row_offsets;
@@ -2571,7 +2585,7 @@ extern "C" fp4q_status fp4q_gemm_dgrad(const fp4q_tensor *dY, const fp4q_tensor 
 {
     if (!tensor_ok(dY) || !tensor_ok(W)) return dY && W ? FP4Q_ERR_SHAPE : FP4Q_ERR_NULL;
     if (fp4q_status s = check_groups(g)) return s;
-    if (dt != FP4Q_OUT_BF16 && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
+    if (!out_type_ok(dt)) return FP4Q_ERR_UNSUPPORTED;
     const int64_t T = dY->rows, N = dY->cols, K = W->cols;
     if (g ? (W->rows != N * g->n_groups) : (W->rows != N)) return FP4Q_ERR_SHAPE;
     if (g && N % 64) return FP4Q_ERR_UNSUPPORTED;   // a group's contraction range must end on an MMA boundary
@@ -2581,7 +2595,7 @@ extern "C" fp4q_status fp4q_gemm_dgrad(const fp4q_tensor *dY, const fp4q_tensor 
     if (ldx < K) return FP4Q_ERR_SHAPE;
     GemmParams p = {};
     p.C = dX; p.ldc = ldx; p.M = (int32_t)T; p.N = (int32_t)K; p.K = (int32_t)N;
-    p.out_f32 = dt == FP4Q_OUT_F32; p.accumulate = 0;
+    set_out_type(p, dt); p.accumulate = 0;
     dense_tiles(p);
     if (g) {
         p.mode = MODE_GROUPED_ROWS; p.n_groups = g->n_groups; p.row_offsets = g->row_offsets;
@@ -2596,8 +2610,8 @@ extern "C" fp4q_status fp4q_gemm_wgrad(const fp4q_tensor *dY, const fp4q_tensor 
 {
     if (!tensor_ok(dY) || !tensor_ok(X)) return dY && X ? FP4Q_ERR_SHAPE : FP4Q_ERR_NULL;
     if (fp4q_status s = check_groups(g)) return s;
-    if (dt != FP4Q_OUT_BF16 && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
-    if (accumulate && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
+    if (!out_type_ok(dt)) return FP4Q_ERR_UNSUPPORTED;
+    if (accumulate && !out_type_f32(dt)) return FP4Q_ERR_UNSUPPORTED;
     if (dY->rows != X->rows) return FP4Q_ERR_SHAPE;
     const int64_t T = dY->rows, N = dY->cols, K = X->cols;
     if (T > kMaxDim || N > kMaxDim || K > kMaxDim) return FP4Q_ERR_UNSUPPORTED;
@@ -2607,7 +2621,7 @@ extern "C" fp4q_status fp4q_gemm_wgrad(const fp4q_tensor *dY, const fp4q_tensor 
     if (ldw < K) return FP4Q_ERR_SHAPE;
     GemmParams p = {};
     p.C = dW; p.ldc = ldw; p.M = (int32_t)N; p.N = (int32_t)K; p.K = (int32_t)T;
-    p.out_f32 = dt == FP4Q_OUT_F32; p.accumulate = accumulate ? 1 : 0;
+    set_out_type(p, dt); p.accumulate = accumulate ? 1 : 0;
     dense_tiles(p);
     if (g) {
         p.mode = MODE_GROUPED_K; p.n_groups = g->n_groups; p.row_offsets = g->row_offsets;
@@ -2622,7 +2636,7 @@ extern "C" fp4q_status fp4q_mxfp8_qk(const uint8_t *xq, int64_t ld_xq, const uin
                                      void *K_out, int64_t ldo, fp4q_out dt, void *ws, size_t ws_bytes, void *stream)
 {
     if (T < 0 || N < 0 || Kdim < 0) return FP4Q_ERR_SHAPE;
-    if (dt != FP4Q_OUT_BF16 && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
+    if (!out_type_ok(dt)) return FP4Q_ERR_UNSUPPORTED;
     if (T > kMaxDim || N > kMaxDim || Kdim > kMaxDim) return FP4Q_ERR_UNSUPPORTED;
     if (T == 0 || N == 0) return FP4Q_OK;
     if (!xq || !xs) return FP4Q_ERR_NULL;
@@ -2642,7 +2656,7 @@ extern "C" fp4q_status fp4q_mxfp8_qk(const uint8_t *xq, int64_t ld_xq, const uin
         B.sf = ScaleView{wsf[i], ld_ws, 1, (int32_t)N, (int32_t)nkb};
         GemmParams p = {};
         p.C = out[i]; p.ldc = ldo; p.M = (int32_t)T; p.N = (int32_t)N; p.K = (int32_t)Kdim;
-        p.out_f32 = dt == FP4Q_OUT_F32;
+        set_out_type(p, dt);
         dense_tiles(p);
         if (fp4q_status s = launch_gemm<KIND_MXF8>(A, B, p, ws, ws_bytes, stream)) return s;
     }
@@ -2655,7 +2669,7 @@ extern "C" fp4q_status fp4q_mxfp8_gemm(const uint8_t *aq, int64_t ld_aq, const u
                                        void *stream)
 {
     if (M < 0 || N < 0 || Kdim < 0) return FP4Q_ERR_SHAPE;
-    if (dt != FP4Q_OUT_BF16 && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
+    if (!out_type_ok(dt)) return FP4Q_ERR_UNSUPPORTED;
     if (M > kMaxDim || N > kMaxDim || Kdim > kMaxDim) return FP4Q_ERR_UNSUPPORTED;
     if (M == 0 || N == 0) return FP4Q_OK;
     if (!aq || !as || !bq || !bs || !C) return FP4Q_ERR_NULL;
@@ -2668,7 +2682,7 @@ extern "C" fp4q_status fp4q_mxfp8_gemm(const uint8_t *aq, int64_t ld_aq, const u
     B.sf = ScaleView{bs, ld_bs, 1, (int32_t)N, (int32_t)nkb};
     GemmParams p = {};
     p.C = C; p.ldc = ldc; p.M = (int32_t)M; p.N = (int32_t)N; p.K = (int32_t)Kdim;
-    p.out_f32 = dt == FP4Q_OUT_F32;
+    set_out_type(p, dt);
     dense_tiles(p);
     return launch_gemm<KIND_MXF8>(A, B, p, ws, ws_bytes, stream);
 }
@@ -2679,7 +2693,7 @@ extern "C" fp4q_status fp4q_gemm_fwd_act1d(const uint8_t *xq, int64_t ld_xq, con
 {
     if (!tensor_ok(W)) return W ? FP4Q_ERR_SHAPE : FP4Q_ERR_NULL;
     if (T < 0) return FP4Q_ERR_SHAPE;
-    if (dt != FP4Q_OUT_BF16 && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
+    if (!out_type_ok(dt)) return FP4Q_ERR_UNSUPPORTED;
     const int64_t N = W->rows, K = W->cols;
     if (T > kMaxDim || N > kMaxDim || K > kMaxDim) return FP4Q_ERR_UNSUPPORTED;
     if (T == 0 || N == 0) return FP4Q_OK;
@@ -2690,7 +2704,7 @@ extern "C" fp4q_status fp4q_gemm_fwd_act1d(const uint8_t *xq, int64_t ld_xq, con
     A.sf = ScaleView{xs, ld_xs, 1, (int32_t)T, (int32_t)ceil_div(K, 32)};
     GemmParams p = {};
     p.C = Y; p.ldc = ldy; p.M = (int32_t)T; p.N = (int32_t)N; p.K = (int32_t)K;
-    p.out_f32 = dt == FP4Q_OUT_F32;
+    set_out_type(p, dt);
     dense_tiles(p);
     return launch_gemm<KIND_MXF4RA>(A, B, p, ws, ws_bytes, stream);
 }
@@ -2701,8 +2715,8 @@ extern "C" fp4q_status fp4q_gemm_wgrad_act1d(const fp4q_tensor *dY, const uint8_
 {
     if (!tensor_ok(dY)) return dY ? FP4Q_ERR_SHAPE : FP4Q_ERR_NULL;
     if (K < 0) return FP4Q_ERR_SHAPE;
-    if (dt != FP4Q_OUT_BF16 && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
-    if (accumulate && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
+    if (!out_type_ok(dt)) return FP4Q_ERR_UNSUPPORTED;
+    if (accumulate && !out_type_f32(dt)) return FP4Q_ERR_UNSUPPORTED;
     const int64_t T = dY->rows, N = dY->cols;
     if (T > kMaxDim || N > kMaxDim || K > kMaxDim) return FP4Q_ERR_UNSUPPORTED;
     if (N == 0 || K == 0) return FP4Q_OK;
@@ -2713,7 +2727,7 @@ extern "C" fp4q_status fp4q_gemm_wgrad_act1d(const fp4q_tensor *dY, const uint8_
     B.sf = ScaleView{xts, ld_xts, 1, (int32_t)K, (int32_t)ceil_div(T, 32)};
     GemmParams p = {};
     p.C = dW; p.ldc = ldw; p.M = (int32_t)N; p.N = (int32_t)K; p.K = (int32_t)T;
-    p.out_f32 = dt == FP4Q_OUT_F32; p.accumulate = accumulate ? 1 : 0;
+    set_out_type(p, dt); p.accumulate = accumulate ? 1 : 0;
     dense_tiles(p);
     return launch_gemm<KIND_MXF4RB>(A, B, p, ws, ws_bytes, stream);
 }
@@ -2742,8 +2756,8 @@ static fp4q_status gemm_b16(int which, const fp4q_tensor *a, const fp4q_tensor *
                             void *ws, size_t ws_bytes, void *stream)
 {
     if (!tensor_ok(a) || !tensor_ok(b)) return a && b ? FP4Q_ERR_SHAPE : FP4Q_ERR_NULL;
-    if (dt != FP4Q_OUT_BF16 && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
-    if (accumulate && dt != FP4Q_OUT_F32) return FP4Q_ERR_UNSUPPORTED;
+    if (!out_type_ok(dt)) return FP4Q_ERR_UNSUPPORTED;
+    if (accumulate && !out_type_f32(dt)) return FP4Q_ERR_UNSUPPORTED;
     int64_t M, N, K;
     if (which == 0) { if (a->cols != b->cols) return FP4Q_ERR_SHAPE; M = a->rows; N = b->rows; K = a->cols; }
     else if (which == 1) { if (a->cols != b->rows) return FP4Q_ERR_SHAPE; M = a->rows; N = b->cols; K = a->cols; }
@@ -2755,7 +2769,7 @@ static fp4q_status gemm_b16(int which, const fp4q_tensor *a, const fp4q_tensor *
     if (ldc < N) return FP4Q_ERR_SHAPE;
     GemmParams p = {};
     p.C = C; p.ldc = ldc; p.M = (int32_t)M; p.N = (int32_t)N; p.K = (int32_t)K;
-    p.out_f32 = dt == FP4Q_OUT_F32; p.accumulate = accumulate ? 1 : 0;
+    set_out_type(p, dt); p.accumulate = accumulate ? 1 : 0;
     dense_tiles(p);
     return launch_gemm<KIND_MXF4B16>(which == 2 ? operand_t16(a) : operand_rm16(a), which == 0 ? operand_rm16(b) : operand_t16(b), p, ws,
                                      ws_bytes, stream);

@@ -228,6 +228,9 @@ at::Tensor out_buffer(const OnStream &on, int64_t rows, int64_t cols, int dt, co
     on.returned(t);
     return ld == cols ? t : t.slice(1, 0, cols);
 }
+// The type as the library takes it: an output that was allocated here is padded, a caller's is written up to its last column.  (Callers of this
+// module name types 0 and 1 only; the library refuses anything else.)
+fp4q_out out_type(int dt, bool ours) { return (fp4q_out)(dt & FP4Q_OUT_PADDED ? 0xFF : ours ? dt | FP4Q_OUT_PADDED : dt); }
 int64_t out_pitch(const at::Tensor &out, int64_t cols) { return out.numel() ? out.stride(0) : cols; }
 
 struct Groups {
@@ -383,8 +386,8 @@ PyObject *gemm(Args a, Py_ssize_t n)
     const at::Tensor ws = workspace(a[10], like);
     const int64_t ld = out_pitch(out, cols);
     const fp4q_status s =
-        which == 2 ? unlocked(lib.gemm_wgrad, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, accumulate, g.ptr, ws.data_ptr(), (size_t)ws.numel(), on.handle)
-                   : unlocked(which == 1 ? lib.gemm_dgrad : lib.gemm_fwd, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, g.ptr, ws.data_ptr(),
+        which == 2 ? unlocked(lib.gemm_wgrad, &ta, &tb, out.data_ptr(), ld, out_type(dt, a[5] == Py_None), accumulate, g.ptr, ws.data_ptr(), (size_t)ws.numel(), on.handle)
+                   : unlocked(which == 1 ? lib.gemm_dgrad : lib.gemm_fwd, &ta, &tb, out.data_ptr(), ld, out_type(dt, a[5] == Py_None), g.ptr, ws.data_ptr(),
                                                                   (size_t)ws.numel(), on.handle);
     check(s, names[which]);
     return a[5] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[5]);
@@ -405,8 +408,8 @@ PyObject *gemm_b16(Args a, Py_ssize_t n)
     const at::Tensor ws = workspace(a[8], like);
     const int64_t ld = out_pitch(out, cols);
     const fp4q_status s =
-        which == 2 ? unlocked(lib.gemm_wgrad_b16, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, accumulate, ws.data_ptr(), (size_t)ws.numel(), on.handle)
-                   : unlocked(which == 1 ? lib.gemm_dgrad_b16 : lib.gemm_fwd_b16, &ta, &tb, out.data_ptr(), ld, (fp4q_out)dt, ws.data_ptr(),
+        which == 2 ? unlocked(lib.gemm_wgrad_b16, &ta, &tb, out.data_ptr(), ld, out_type(dt, a[5] == Py_None), accumulate, ws.data_ptr(), (size_t)ws.numel(), on.handle)
+                   : unlocked(which == 1 ? lib.gemm_dgrad_b16 : lib.gemm_fwd_b16, &ta, &tb, out.data_ptr(), ld, out_type(dt, a[5] == Py_None), ws.data_ptr(),
                                                                           (size_t)ws.numel(), on.handle);
     check(s, names[which]);
     return a[5] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[5]);
@@ -449,7 +452,7 @@ PyObject *gemm_fwd_act1d(Args a, Py_ssize_t n)
     const at::Tensor out = a[4] == Py_None ? out_buffer(on, T, as_i64(wr.p), dt, xq) : as_tensor(a[4]);
     const fp4q_tensor w = from_qtensor(a[3], 32);
     const at::Tensor ws = workspace(a[6], xq);
-    check(unlocked(lib.gemm_fwd_act1d, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), T, &w, out.data_ptr(), out.stride(0), (fp4q_out)dt,
+    check(unlocked(lib.gemm_fwd_act1d, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), T, &w, out.data_ptr(), out.stride(0), out_type(dt, a[4] == Py_None),
                              ws.data_ptr(), (size_t)ws.numel(), on.handle), "fp4q_gemm_fwd_act1d");
     return a[4] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[4]);
 }
@@ -467,7 +470,7 @@ PyObject *gemm_wgrad_act1d(Args a, Py_ssize_t n)
     if (a[4] == Py_None && accumulate) out.zero_();
     const fp4q_tensor d = from_qtensor(a[0], 32);
     const at::Tensor ws = workspace(a[7], xq);
-    check(unlocked(lib.gemm_wgrad_act1d, &d, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), K, out.data_ptr(), out.stride(0), (fp4q_out)dt,
+    check(unlocked(lib.gemm_wgrad_act1d, &d, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), K, out.data_ptr(), out.stride(0), out_type(dt, a[4] == Py_None),
                                accumulate, ws.data_ptr(), (size_t)ws.numel(), on.handle), "fp4q_gemm_wgrad_act1d");
     return a[4] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[4]);
 }
@@ -484,7 +487,7 @@ PyObject *mxfp8_gemm(Args a, Py_ssize_t n)
     const at::Tensor ws = workspace(a[8], aq);
     const int64_t per16 = dt == FP4Q_OUT_BF16 ? 8 : 4, ld = std::max(ceil_to(N, per16) * per16, per16);
     check(unlocked(lib.mxfp8_gemm, bytes_of(aq), aq.stride(0), bytes_of(as), as.stride(0), M, bytes_of(bq), bq.stride(0), bytes_of(bs), bs.stride(0), N,
-                         K, out.data_ptr(), ld, (fp4q_out)dt, ws.data_ptr(), (size_t)ws.numel(), on.handle), "fp4q_mxfp8_gemm");
+                         K, out.data_ptr(), ld, out_type(dt, true), ws.data_ptr(), (size_t)ws.numel(), on.handle), "fp4q_mxfp8_gemm");
     return THPVariable_Wrap(out);
 }
 
@@ -509,7 +512,7 @@ PyObject *mxfp8_qk(Args a, Py_ssize_t n)
     if (!wref.defined() || !sref.defined()) { PyErr_SetString(PyExc_AttributeError, "'NoneType' object has no attribute 'stride'"); throw PyError(); }
     const at::Tensor ws = workspace(a[10], xq);
     check(unlocked(lib.mxfp8_qk, bytes_of(xq), xq.stride(0), bytes_of(xs), xs.stride(0), T, K, p[0], p[1], p[2], p[3], wref.stride(0), sref.stride(0), N,
-                       out[0].defined() ? out[0].data_ptr() : nullptr, out[1].defined() ? out[1].data_ptr() : nullptr, ld, (fp4q_out)dt,
+                       out[0].defined() ? out[0].data_ptr() : nullptr, out[1].defined() ? out[1].data_ptr() : nullptr, ld, out_type(dt, true),
                        ws.data_ptr(), (size_t)ws.numel(), on.handle), "fp4q_mxfp8_qk");
     Ref q(out[0].defined() ? THPVariable_Wrap(out[0]) : Py_NewRef(Py_None)), k(out[1].defined() ? THPVariable_Wrap(out[1]) : Py_NewRef(Py_None));
     return PyTuple_Pack(2, q.p, k.p);
@@ -599,7 +602,7 @@ struct LinearNode : torch::autograd::Function<LinearNode> {
         const uint8_t is_f32[2] = {xb.scalar_type() == at::kFloat, wb.scalar_type() == at::kFloat};
         check_unlocked(lib.quantize2d_multi_f32(jobs, is_f32, 2, FP4Q_ROUND_NEAREST, 0, on.handle), "fp4q_quantize2d");
         const at::Tensor y = out_buffer(on, T, N, FP4Q_OUT_BF16, xb);
-        check_unlocked(lib.gemm_fwd(&qx.t, &qw.t, y.data_ptr(), out_pitch(y, N), FP4Q_OUT_BF16, nullptr, call.ws.data_ptr(), (size_t)call.ws.numel(), on.handle),
+        check_unlocked(lib.gemm_fwd(&qx.t, &qw.t, y.data_ptr(), out_pitch(y, N), out_type(FP4Q_OUT_BF16, true), nullptr, call.ws.data_ptr(), (size_t)call.ws.numel(), on.handle),
                        "fp4q_gemm_fwd");
         ctx->saved_data["kept"] = kept;
         ctx->saved_data["ws"] = call.ws;
@@ -625,13 +628,13 @@ struct LinearNode : torch::autograd::Function<LinearNode> {
         at::Tensor dx, dw;
         if (ctx->needs_input_grad(0)) {
             dx = out_buffer(on, T, K, FP4Q_OUT_BF16, dy);
-            check_unlocked(lib.gemm_dgrad(&q.t, &qw.t, dx.data_ptr(), out_pitch(dx, K), FP4Q_OUT_BF16, nullptr, ws.data_ptr(), (size_t)ws.numel(), on.handle),
+            check_unlocked(lib.gemm_dgrad(&q.t, &qw.t, dx.data_ptr(), out_pitch(dx, K), out_type(FP4Q_OUT_BF16, true), nullptr, ws.data_ptr(), (size_t)ws.numel(), on.handle),
                            "fp4q_gemm_dgrad");
             dx = as_type(dx, numbers[3]);
         }
         if (ctx->needs_input_grad(1)) {
             dw = out_buffer(on, N, K, FP4Q_OUT_F32, dy);
-            check_unlocked(lib.gemm_wgrad(&q.t, &qx.t, dw.data_ptr(), out_pitch(dw, K), FP4Q_OUT_F32, 0, nullptr, ws.data_ptr(), (size_t)ws.numel(), on.handle),
+            check_unlocked(lib.gemm_wgrad(&q.t, &qx.t, dw.data_ptr(), out_pitch(dw, K), out_type(FP4Q_OUT_F32, true), 0, nullptr, ws.data_ptr(), (size_t)ws.numel(), on.handle),
                            "fp4q_gemm_wgrad");
             dw = as_type(dw, numbers[4]);
         }

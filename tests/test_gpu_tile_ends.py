@@ -1,5 +1,7 @@
 """Where a CTA's stream of tiles ends: the last tile's output leaves through the operand ring, row tiles are numbered in groups with a
 smaller last one, and groups of rows are looked up through a copy of their boundaries when these fill more than a cache line."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -144,6 +146,21 @@ def test_outputs_end_with_their_last_column(T, N, K):
             assert torch.signbit(buf[:rows, cols:]).all() and torch.signbit(buf[rows:]).all(), i
     torch.cuda.synchronize()
     assert binding.fp4q_workspace_status(ws) == 0
+
+
+# An output whose rows are padded may be filled up to 16 bytes, and no further; the binding says so of its own outputs only
+def test_padded_outputs():
+    ws = binding.alloc_workspace("cuda")
+    qx, qw = operands((300, 100), (131, 100))
+    want = binding.fp4q_gemm_fwd(qx, qw, ws=ws)
+    buf = torch.full((300, 160), 7.0, dtype=torch.bfloat16, device="cuda")
+    cx, cw = qx.c_struct(), qw.c_struct()
+    assert binding.lib().fp4q_gemm_fwd(ctypes.byref(cx), ctypes.byref(cw), buf.data_ptr(), 160, 0x100 | binding.OUT_BF16, None, ws.data_ptr(), ws.numel(),
+                                       torch.cuda.current_stream().cuda_stream) == 0
+    assert torch.equal(buf[:, :131], want) and (buf[:, 136:] == 7.0).all()
+    for dt in (0x100, 0x101, 2, 0xFF):
+        with pytest.raises(binding.Fp4qError):
+            binding.fp4q_gemm_fwd(qx, qw, dt=dt, ws=ws)
 
 
 # 81 tiles of 43 and of 44 stages: both sides of the line (48 stages for each of 74 pairs) from which on a dense product runs with a
